@@ -180,8 +180,7 @@ def _lists(c, seed):
         out["selected"] = ctx.astype(np.int64)
     elif c["how"] == "refs":
         out["lines"], out["refs"], out["line_start"] = zip(*(_lines_of_request(r, c, int(n)) for n in ctx))
-        spans = [[(0, c["prefix"]), (st, int(n))] + [ln for lo, hi in rf for ln in li[lo:hi + 1]]
-                 for li, rf, st, n in zip(out["lines"], out["refs"], out["line_start"], ctx)]
+        spans = [_request_spans(c, out, b) for b in range(c["B"])]
     else:
         spans = out["spans"] = [_spans_of_request(r, c, b, int(n)) for b, n in enumerate(ctx)]
     if "selected" not in out:
@@ -362,3 +361,58 @@ def tolerance(case):
     if case["dtype"] == "f16":
         return {"rel": 8e-4, "max": 2e-3}
     return {"rel": 6e-3, "max": 1.6e-2}
+
+
+# ---- the same in 64 bits ----------------------------------------------------------------------------------------
+def exact(case, seed):
+    """What run() returns for these inputs: softmax(q K^T / sqrt(D)) V over each request's selected positions in
+    64 bits, and the lists as they stand."""
+    c, L, s = case, _lists(case, seed), prepare(case, seed)
+    B, H, D, how = c["B"], c["H"], c["D"], c["how"]
+    q = s["q"].double().reshape(B, H * c["n_q"], D)
+    group = H * c["n_q"] // c["H_kv"]
+    rows, lse, chosen = torch.empty_like(q), torch.empty(q.shape[:2], dtype=torch.float64, device="cuda"), []
+    for b in range(B):
+        n = int(L["ctx"][b])
+        if how in ("dense", "multiq"):
+            hit = np.ones(n, bool)
+        else:
+            hit = np.zeros(n, bool)
+            for st, e in _request_spans(c, L, b):
+                hit[st:e] = True
+        at = np.flatnonzero(hit)
+        chosen.append(at)
+        pos = _dev(at)
+        if how == "paged":
+            ps = c["page_size"]
+            pool = s["table"][b].long()[pos // ps] * ps + pos % ps
+            k, v = (s[t].reshape(-1, c["H_kv"], D)[pool].transpose(0, 1) for t in "kv")
+        else:
+            k, v = (s[t][b].view(torch.uint8 if s[t].element_size() == 1 else s[t].dtype)[:, pos].view(s[t].dtype) for t in "kv")
+        scores = q[b].view(c["H_kv"], group, D) @ k.double().transpose(1, 2) / math.sqrt(D)
+        top = torch.logsumexp(scores, -1, keepdim=True)
+        rows[b] = (torch.exp(scores - top) @ v.double()).reshape(-1, D)
+        lse[b] = top.reshape(-1)
+    out = [rows.view(s["out"].shape), lse.view(s["lse"].shape)]
+    if how in ("step", "host_step", "refs"):
+        index, counts = np.full(tuple(s["index"].shape), -1, np.int32), np.zeros(B, np.int32)
+        for b, at in enumerate(chosen):
+            index[b, :len(at)], counts[b] = at, len(at)
+        out += [index, counts]
+    elif how == "blockmask":
+        bs = c["block_size"]
+        idx = np.full(tuple(s["block_idx"].shape), -1, np.int32)
+        mask, counts = np.zeros(tuple(s["block_mask"].shape), np.uint32), np.zeros(B, np.int32)
+        for b, at in enumerate(chosen):
+            blocks, slot = np.unique(at // bs, return_inverse=True)
+            idx[b, :len(blocks)], counts[b] = blocks, len(blocks)
+            np.bitwise_or.at(mask[b], (slot, at % bs // 32), (np.uint32(1) << (at % 32).astype(np.uint32)))
+        out += [idx, mask.view(np.int32), counts]
+    return tuple(out)
+
+
+def _request_spans(c, L, b):
+    if c["how"] != "refs":
+        return L["spans"][b]
+    named = [ln for lo, hi in L["refs"][b] for ln in L["lines"][b][lo:hi + 1]]
+    return [(0, c["prefix"]), (L["line_start"][b], int(L["ctx"][b]))] + named
