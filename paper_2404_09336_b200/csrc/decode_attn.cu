@@ -78,7 +78,7 @@ struct DecodeParams {
   uint32_t k_row_bytes, v_row_bytes;   // token stride of the cache in bytes
   int32_t H, max_ctx, index_stride, max_selected, chunk, n_chunks, out_f32, early_release;
   int32_t kv_group;         // query heads per K/V head (1: multi-head attention)
-  int32_t gqa_wide;         // row-sharing kernel with eight warps per block
+  int32_t gqa_wide;         // row-sharing kernel, one large block per SM
   // paged cache (page_table != nullptr): logical position t of request b is row
   // page_table[b * page_table_stride + (t >> page_shift)] << page_shift | (t & page_mask) of the pool
   const int32_t* page_table;
@@ -540,12 +540,12 @@ namespace ssa {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool wide; };   // wide: eight-warp row-sharing blocks
+struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool wide; };   // wide: one large row-sharing block per SM
 
 // Grouped query heads go to the kernel that reads a K/V row once for the whole group.
 static bool shares_rows(const ssa_attn_desc* d) {
   const int group = d->H_kv > 0 ? d->H / d->H_kv : 1;
-  return d->D == 128 && group >= 2 && group <= kGqaHeads && d->kv_dtype != SSA_FP8_E4M3;   // mma takes 16-bit rows
+  return d->D == 128 && group >= 2 && group <= kGqaHeads;
 }
 
 static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
@@ -564,7 +564,7 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
   else while (chunk > 64 && units * ((max_selected + chunk - 1) / chunk) < want) chunk >>= 1;
   pl->wide = false;
   if (shares_rows(d) && 2 * units > sms && units <= sms && max_selected <= 2048) {
-    // One unit for most SMs and a short list: the whole list is one eight-warp block's work, and the second pass
+    // One unit for most SMs and a short list: the whole list is one large block's work, and the second pass
     // (about 3 us in the stream) is not needed (32 query heads over 4 K/V heads, 32 requests, 819 rows: 15.2 vs
     // 18.0 us).  With fewer units (2 K/V heads: 64) too many SMs would idle: 15.2 vs 14.4 us with four chunks.
     pl->wide = true;
@@ -572,7 +572,9 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
   } else if (shares_rows(d)) {
     // The row-sharing kernel leaves G triples per chunk, its blocks stream (a ring of tiles per warp) and two of
     // them fit an SM: about one block per resident slot, i.e. as few chunks as keep the SMs busy (measured,
-    // B*H_kv = 64..256, context 8192: within 3 % of the best split for groups of 4, 8 and 16 heads).
+    // B*H_kv = 64..256, context 8192: within 3 % of the best split for groups of 4, 8 and 16 heads).  Ragged batches
+    // would rather have shorter chunks (17 requests of 1001..8190 rows, 16 heads: 62 instead of 73 us with chunks of
+    // 1024), batches of like lengths pay for them (all 8190: 102 instead of 90 us), and the host knows no lengths.
     const long long target = sms * 2;
     long long n = target / units;                              // rounded down: never one block over a full wave
     n = std::max<long long>(1, std::min<long long>(n, (max_selected + 255) / 256));
@@ -636,27 +638,22 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
   size_t dynamic_smem = 0;
   unsigned block_threads = kThreads;
   bool share = false;
-  if constexpr (!kFp8) {                                // the row-sharing kernel feeds 16-bit rows to the tensor cores
-    share = D == 128 && p.kv_group >= 2 && p.kv_group <= kGqaHeads && mode != kBlockMask;
+  if constexpr (D == 128) {
+    share = p.kv_group >= 2 && p.kv_group <= kGqaHeads && mode != kBlockMask;
     if (share) {
       grid.y = (unsigned)(p.H / p.kv_group);            // one block per K/V head
       const bool hi = p.kv_group > 8;
-      constexpr int kW8 = kGqaWideWarps;
-      if (p.gqa_wide) {
-        if (mode == kIndex)
-          kernel = hi ? decode_partial_gqa_kernel<T, kIndex, true, kW8> : decode_partial_gqa_kernel<T, kIndex, false, kW8>;
-        else if (mode == kSpans)
-          kernel = hi ? decode_partial_gqa_kernel<T, kSpans, true, kW8> : decode_partial_gqa_kernel<T, kSpans, false, kW8>;
-        else
-          kernel = hi ? decode_partial_gqa_kernel<T, kDense, true, kW8> : decode_partial_gqa_kernel<T, kDense, false, kW8>;
-        block_threads = kW8 * 32;
-      } else if (mode == kIndex)
-        kernel = hi ? decode_partial_gqa_kernel<T, kIndex, true> : decode_partial_gqa_kernel<T, kIndex, false>;
-      else if (mode == kSpans)
-        kernel = hi ? decode_partial_gqa_kernel<T, kSpans, true> : decode_partial_gqa_kernel<T, kSpans, false>;
-      else
-        kernel = hi ? decode_partial_gqa_kernel<T, kDense, true> : decode_partial_gqa_kernel<T, kDense, false>;
-      dynamic_smem = (size_t)(block_threads / 32) * kStagedWarpBytes;
+      auto pick = [&](auto hi_tag, auto wide_tag) {
+        constexpr bool kHi = decltype(hi_tag)::value, kWide = decltype(wide_tag)::value;
+        using Shape = GqaShape<T, kHi, kWide>;
+        block_threads = Shape::kWarps * 32;
+        dynamic_smem = Shape::kSmemBytes;
+        kernel = mode == kIndex   ? decode_partial_gqa_kernel<T, kIndex, kHi, kWide>
+                 : mode == kSpans ? decode_partial_gqa_kernel<T, kSpans, kHi, kWide>
+                                  : decode_partial_gqa_kernel<T, kDense, kHi, kWide>;
+      };
+      if (hi) p.gqa_wide ? pick(std::true_type{}, std::true_type{}) : pick(std::true_type{}, std::false_type{});
+      else p.gqa_wide ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{});
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_smem) != cudaSuccess)
         return SSA_ERR_CUDA;
     }

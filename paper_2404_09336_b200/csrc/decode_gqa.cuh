@@ -8,11 +8,19 @@
 // slots before it runs out of HBM bandwidth, so here the two contractions go
 // to the tensor cores.  The shapes are far too small for tcgen05 tiles (G x 16
 // rows x 128), so they are warp-level mma.sync.m16n8k16 (16-bit inputs, fp32
-// accumulation) with the M dimension holding the query heads:
-//   S[16 heads, 16 rows]  = Q . K_tile^T : A = Q (registers, loaded once),
-//                           B = K tile via ldmatrix (rows are the n index);
-//   O[16 heads, 128 dims] += P . V_tile  : A = P from the accumulators of S,
-//                           B = V tile via ldmatrix.trans (rows are the k index).
+// accumulation) with the N dimension holding eight query heads:
+//   S^T[16 rows, 8 heads] = K_tile . Q^T : A = K tile (16 rows), B = Q
+//                           (registers, loaded once);
+//   O^T[16 dims, 8 heads] += V_tile^T . P^T : A = V tile, transposed, B = P
+//                           from the accumulators of S, transposed by movmatrix.
+// Groups of up to eight heads take one head tile, larger ones two (kHi): with
+// the heads in the M dimension instead, a group of up to eight heads paid for
+// sixteen, twice the matrix instructions.
+// 16-bit tiles come out of shared memory with ldmatrix (.trans for V).  8-bit
+// rows (e4m3) are read with plain 16-byte loads and converted in registers,
+// exactly: K to bf16 (the type of its queries), V to fp16; which lane holds
+// which dimension is free as long as Q (for K) and the output (for V) follow,
+// so a lane takes whole 16-byte pieces of a row.
 // The rows travel global -> shared memory by asynchronous 16-byte copies
 // (cp.async, evict-first in L2) into a ring of tiles that every warp keeps for
 // itself, and the fragments come out of that ring with ldmatrix.  The bytes in
@@ -29,6 +37,9 @@
 // The softmax weights are the fp32 accumulators of S; they enter the second
 // contraction as a 16-bit value plus a 16-bit residual (two mma passes), so
 // the result keeps fp32-level accuracy instead of the 2^-9 of a bf16 weight.
+// Over an 8-bit cache they are fp16 pairs of 2^13 times the weight: 22 bits
+// for the large ones and an absolute error below 2^-37 of the largest for the
+// rest.
 // Included by decode_attn.cu after DecodeParams and its helpers.
 #pragma once
 
@@ -55,7 +66,7 @@ template <>
 __device__ __forceinline__ void mma_16816<__nv_bfloat16>(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                                          uint32_t a3, uint32_t b0, uint32_t b1,
                                                          const float (&c)[4]) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                "{%10,%11,%12,%13};"
                : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
@@ -63,7 +74,7 @@ __device__ __forceinline__ void mma_16816<__nv_bfloat16>(float (&d)[4], uint32_t
 template <>
 __device__ __forceinline__ void mma_16816<__half>(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                   uint32_t b0, uint32_t b1, const float (&c)[4]) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                "{%10,%11,%12,%13};"
                : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
@@ -71,26 +82,40 @@ __device__ __forceinline__ void mma_16816<__half>(float (&d)[4], uint32_t a0, ui
 
 constexpr int kGqaRows = 16;            // rows per warp per iteration
 constexpr int kGqaHeads = 16;           // M of the mma: most query heads one block serves
-constexpr int kGqaPad = 4;              // floats of padding per head row of the block-level combine
+// floats per head row of the block-level combine, dim d at d + 2 (d / 16): lanes that hold dims 16 apart (8-bit rows)
+// or one apart (16-bit rows) and heads two apart store to different banks
+constexpr int kGqaPitch = 148;
+__device__ __forceinline__ int gqa_column(int d) { return d + 2 * (d >> 4); }
 
-constexpr int kStagedDepth = 3;                          // tiles per warp in the ring
-constexpr int kStagedTileBytes = kGqaRows * 256;         // one tensor's tile
-constexpr int kStagedWarpBytes = kStagedDepth * 2 * kStagedTileBytes;
-constexpr int kStagedSmemBytes = kWarps * kStagedWarpBytes;   // four-warp blocks: 96 KB, two blocks per SM
-constexpr int kGqaWideWarps = 8;                         // eight-warp blocks (192 KB, one per SM) for short lists of few units
-// A chunk is worked through in windows: the block's warps meet at every window's end (and, for lists, stage
-// the next window's positions).  Meeting often keeps the four warps on neighbouring rows, which the memory
-// system rewards (full context at 32 query heads over 8 / 4 / 2 K/V heads: 6.9 / 6.3 / 5.4 TB/s with windows
-// of 256 rows, 6.7 / 6.2 / 5.4 with 512, 6.5 / 6.0 / 5.4 with 1024, 6.3 / 5.8 / 5.2 without windows), but each
-// meeting lets the ring run empty once (windows of 64 rows: 5.7 / 5.2 / 4.6 TB/s).
+// Warps and ring of a block.  A team of warps shares one ring of tiles: one warp for up to eight heads, two - one per
+// head tile - for more (one warp with both head tiles had twice the instructions per tile in one dependent stream,
+// and with eight such warps per SM that stream, not the memory, was what a tile waited for).  Four teams with 24 KB
+// each make a block, two blocks fit an SM; 8-bit rows, whose tiles are half as large and cost more instructions
+// (conversions), take twice the teams with half the ring.  Wide blocks have twice the teams, one block per SM.
+template <typename T, bool kHi, bool kWide>
+struct GqaShape {
+  static constexpr int kTeam = kHi ? 2 : 1;
+  static constexpr int kRingBytes = (kIsFp8<T> && !kHi ? 12 : 24) * 1024;
+  static constexpr int kSmemBytes = (kWide ? 192 : 96) * 1024;
+  static constexpr int kTeams = kSmemBytes / kRingBytes;
+  static constexpr int kWarps = kTeam * kTeams;
+  static constexpr int kDenseWindow = kHi ? 1024 : kIsFp8<T> ? 512 : 256;   // see below
+};
+// A chunk is worked through in windows: for lists, the block's warps meet and stage the next window's positions; over
+// a full context, each team lets its ring run empty.  Short windows keep the teams on neighbouring rows, which the
+// memory system rewards, long ones keep more in flight.  Measured with windows of 256 / 512 / 1024 rows, full context:
+// 4 heads, 32 requests of 8192: 152 / 158 / 158 us; 16 heads, 26 x 3287: 62.8 / 61.4 / 60.3 us, 17 requests of
+// 1001..8190: 75.8 / 74.0 / 72.7 us, 17 x 8190: 89.2 / 92.2 / 93.4 us.  8-bit rows have twice the teams: 512.
 constexpr int kStagedWindow = 512;                       // list entries staged at a time ...
 constexpr int kStagedShortList = 1024;                   // ... unless the whole chunk fits this many: then one window
-constexpr int kStagedDenseWindow = 256;                  // full context: rows between two meetings of the warps
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // 16-byte asynchronous copy global -> shared, not kept in L1, evict-first in L2; src_bytes = 0 writes zeros.
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, uint32_t src_bytes, uint64_t policy) {
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, uint64_t policy) {
+  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
+}
+__device__ __forceinline__ void cp_async_16_or_zero(uint32_t dst, const void* src, uint32_t src_bytes, uint64_t policy) {
   asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;"
                ::"r"(dst), "l"(src), "r"(src_bytes), "l"(policy)
                : "memory");
@@ -110,38 +135,82 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t add
                : "r"(addr));
 }
 
+// 8x8 transpose of 16-bit values across a warp (lane 4r + c holds columns 2c, 2c + 1 of row r).
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t v) {
+  uint32_t r;
+  asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+  return r;
+}
+
+__device__ __forceinline__ uint4 lds_16B(uint32_t addr) {
+  uint4 r;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr) : "memory");
+  return r;
+}
+
+// Two e4m3 values (low 16 bits) -> two fp16 or two bf16 (both exact).
+__device__ __forceinline__ uint32_t e4m3x2_to_half2(uint32_t pair) {
+  uint32_t h2;
+  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((unsigned short)pair));
+  return h2;
+}
+__device__ __forceinline__ uint32_t e4m3x2_to_bf162(uint32_t pair) {
+  const float2 f = e4m3x2_to_float2(pair);
+  return pack2<__nv_bfloat16>(f.x, f.y);
+}
+
+// 8-bit tiles, [16 rows][128 B]: 16-byte chunk `chunk` of a row.  The XOR keeps the eight lanes that a 16-byte
+// shared load serves at a time on different banks: K reads take chunks 0-3 (4-7) of two neighbouring rows, V reads
+// chunks 2i, 2i + 1 of rows 0, 2, 4, 6 (1, 3, 5, 7).
+__device__ __forceinline__ uint32_t tile8_offset_k(int row, int chunk) {
+  return (uint32_t)(row * 128 + ((chunk ^ ((row & 1) << 2)) << 4));
+}
+__device__ __forceinline__ uint32_t tile8_offset_v(int row, int chunk) {
+  return (uint32_t)(row * 128 + ((chunk ^ (row & 6)) << 4));
+}
+
 // byte offset of 16-byte chunk `chunk` of row `row` inside a swizzled [16][256 B] tile
 __device__ __forceinline__ uint32_t tile_offset(int row, int chunk) {
   return (uint32_t)(row * 256 + ((chunk ^ (row & 7)) << 4));
 }
 
-// kW: warps per block.  Four is the rule (two blocks per SM).  Eight serve launches with at most one unit (request x
-// K/V head) per SM and short lists: a whole list is then one block's work - no second pass - and eight warps stream it.
-template <typename T, int kMode, bool kHi, int kW = kWarps>
-__global__ void __launch_bounds__(kW * 32, kW == kWarps ? 2 : 1)
+// kWide serves launches with at most one unit (request x K/V head) per SM and short lists: a whole list is then one
+// block's work, no second pass.
+template <typename T, int kMode, bool kHi, bool kWide>
+__global__ void __launch_bounds__(GqaShape<T, kHi, kWide>::kWarps * 32, kWide ? 1 : 2)
 decode_partial_gqa_kernel(const DecodeParams p) {
-  constexpr int kWarps = kW, kThreads = kW * 32;      // hide the library-wide four-warp constants in here
+  using Shape = GqaShape<T, kHi, kWide>;
+  constexpr int kWarps = Shape::kWarps, kThreads = kWarps * 32;   // hide the library-wide four-warp constants in here
+  constexpr int kTeam = Shape::kTeam, kTeams = Shape::kTeams;
   constexpr int D = 128;
   constexpr bool kSparse = kMode != kDense;
-  constexpr int kLiveHeads = kHi ? 16 : 8;
+  constexpr bool kFp8 = kIsFp8<T>;
+  using TQ = typename Storage<T>::Query;                // type of the query rows and of a stored output
+  using TP = typename std::conditional<kFp8, __half, T>::type;   // type of the weights in the second contraction
+  constexpr float kUp = kFp8 ? 8192.f : 1.f;            // weights (and all they enter) are scaled by this in the loop
+  constexpr int kTileBytes = kGqaRows * (kFp8 ? 128 : 256);      // one tensor's tile
+  constexpr int kStagedDepth = Shape::kRingBytes / (2 * kTileBytes);
+  constexpr int kLiveHeads = 8 * kTeam;
+  static_assert(kThreads % D == 0, "128 threads finish a head");
   static_assert(kMode == kDense || kMode == kIndex || kMode == kSpans,
                 "blocked lists take the one-head-per-block kernel");
-  static_assert(kLiveHeads * (D + kGqaPad) * 4 <= kStagedWarpBytes, "the combine reuses the ring");
+  static_assert(kLiveHeads * kGqaPitch * 4 <= Shape::kRingBytes, "the combine reuses the ring");
 
-  extern __shared__ __align__(128) unsigned char s_ring[];
+  extern __shared__ __align__(1024) unsigned char s_ring[];
   __shared__ int32_t s_idx[kSparse ? kStagedShortList : 1];
   __shared__ __align__(128) unsigned char s_qtile[kGqaHeads * 256];   // Q of the group, swizzled like a row tile
-  __shared__ float s_m[kWarps][kLiveHeads], s_l[kWarps][kLiveHeads];
+  __shared__ float s_m[kTeams][kLiveHeads], s_l[kTeams][kLiveHeads];
   __shared__ typename std::conditional<kMode == kSpans, SpanRuns, int>::type s_runs;
 
   const int chunk_id = blockIdx.x, kvh = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, j = lane & 3;
+  const int team = warp / kTeam, ht = warp % kTeam;     // ht: the eight heads of the group that are this warp's
   const int G = p.kv_group;
-  const int start = chunk_id * p.chunk;
 
   grid_dependency_wait();
   if (p.early_release) grid_launch_dependents();
+  const int start = chunk_id * p.chunk;
 
   // One round trip for everything that does not depend on the list length: the first kStagedShortList list
   // entries of the chunk (within the host's bound, so inside the caller's row) and the group's query rows.
@@ -160,7 +229,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   {
     const int row = tid >> 3, c0 = (tid & 7) * 2;     // 16 rows x 8 threads; further threads have no part
     if (row < G) {
-      const T* src = reinterpret_cast<const T*>(p.q) + (int64_t)b * p.q_sb + (int64_t)(kvh * G + row) * p.q_sh + 8 * c0;
+      const TQ* src = reinterpret_cast<const TQ*>(p.q) + (int64_t)b * p.q_sb + (int64_t)(kvh * G + row) * p.q_sh + 8 * c0;
       q_lo = ld_stream_16B(src);
       q_hi = ld_stream_16B(src + 8);
     }
@@ -220,7 +289,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       s_idx[i] = checked(row ? __ldg(row + i) : start + w0 + i);
   };
   // a list chunk of up to kStagedShortList entries is one window (no meeting in mid-chunk); longer ones go by 512
-  const int window = kSparse ? (cnt <= kStagedShortList ? kStagedShortList : kStagedWindow) : kStagedDenseWindow;
+  const int window = kSparse ? (cnt <= kStagedShortList ? kStagedShortList : kStagedWindow) : Shape::kDenseWindow;
   if (kSparse) stage_window(0, min(cnt, window));
   // the group's query rows -> shared memory (rows of heads that do not exist are zero)
   if (tid < kGqaHeads * 8) {
@@ -228,29 +297,56 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0)) = q_lo;
     *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0 + 1)) = q_hi;
   }
-  __syncthreads();
-  // A fragments of Q for the eight k-steps: registers for the whole block's life
-  uint32_t qa[8][4];
-  {
-    const int m = lane >> 3, r = lane & 7;
-    const uint32_t base = smem_u32(s_qtile);
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) ldmatrix_x4(qa[ks], base + tile_offset((m & 1) * 8 + r, 2 * ks + (m >> 1)));
-  }
+  if (kSparse) __syncthreads();                        // the first window is staged
   uint64_t policy;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
   const char* kbase = reinterpret_cast<const char*>(
       reinterpret_cast<const T*>(p.k) + (int64_t)b * p.k_sb + (int64_t)kvh * p.k_sh);
   const char* vbase = reinterpret_cast<const char*>(
       reinterpret_cast<const T*>(p.v) + (int64_t)b * p.v_sb + (int64_t)kvh * p.v_sh);
-  const uint32_t ring = smem_u32(s_ring) + warp * kStagedWarpBytes;
+  const uint32_t ring = smem_u32(s_ring) + team * Shape::kRingBytes;
+  // this lane's part in copying a tile: its 16 bytes of every row, and where they go in the first row it copies
+  constexpr int kRowBytes = kFp8 ? 128 : 256, kChunks = kRowBytes / 16, kRowsPerCopy = 32 / kChunks;
+  const char* kcol = kbase + (lane % kChunks) * 16;
+  const char* vcol = vbase + (lane % kChunks) * 16;
+  const int copy_row = ht * (kGqaRows / kTeam) + lane / kChunks;
+  const uint32_t copy_k = kFp8 ? tile8_offset_k(copy_row, lane % kChunks) : tile_offset(copy_row, lane % kChunks);
+  const uint32_t copy_v = kFp8 ? tile8_offset_v(copy_row, lane % kChunks) : tile_offset(copy_row, lane % kChunks);
+  // this lane's part in reading one: fragment addresses are these, XOR-ed with a multiple of 32 (or 64) bytes
+  const uint32_t read_k = kFp8 ? tile8_offset_k(g, j) : tile_offset(lane & 15, lane >> 4);
+  const uint32_t read_v = kFp8 ? tile8_offset_v(2 * j, g) : tile_offset((lane >> 4) * 8 + (lane & 7), (lane >> 3) & 1);
 
-  // running softmax state of heads g (lo) and g+8 (hi); sums are per lane until the end.
-  // o[nt][e]: dims 8 nt + 2j + (e & 1) of head g (e < 2) or g + 8 (e >= 2)
-  float m_lo = neg_inf(), m_hi = neg_inf(), l_lo = 0.f, l_hi = 0.f;
-  float o[16][4];
+  // Running softmax state of heads 8 ht + 2 j + {0, 1}, the same in all lanes of equal j; the sums are per lane until
+  // the end.  o[t][e]: head 8 ht + 2 j + (e & 1), dim 16 t + g + 8 (e >> 1) (8-bit rows: 16 g + 2 t + (e >> 1)).
+  float m[2] = {neg_inf(), neg_inf()}, l[2] = {0.f, 0.f}, o[8][4];
 #pragma unroll
-  for (int u = 0; u < 16; ++u) { o[u][0] = 0.f; o[u][1] = 0.f; o[u][2] = 0.f; o[u][3] = 0.f; }
+  for (int t = 0; t < 8; ++t) { o[t][0] = 0.f; o[t][1] = 0.f; o[t][2] = 0.f; o[t][3] = 0.f; }
+  // B fragments of Q for the eight k-steps: registers for the whole block's life.  8-bit rows: k-step ks of lane
+  // (g, j) is dims 64 (ks / 4) + 16 j + 4 (ks % 4) + 0..3 of head g, the order its K pieces come in.
+  uint32_t qb[8][2];
+  auto load_q = [&]() {
+    const uint32_t base = smem_u32(s_qtile);
+    if constexpr (kFp8) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint4 w = lds_16B(base + tile_offset(8 * ht + g, 8 * (c >> 1) + 2 * j + (c & 1)));
+        qb[2 * c][0] = w.x; qb[2 * c][1] = w.y;
+        qb[2 * c + 1][0] = w.z; qb[2 * c + 1][1] = w.w;
+      }
+    } else {
+#pragma unroll
+      for (int ks = 0; ks < 8; ks += 2) {
+        uint32_t w[4];
+        ldmatrix_x4(w, base + tile_offset(8 * ht + (lane & 7), 2 * ks + (lane >> 3)));
+        qb[ks][0] = w[0]; qb[ks][1] = w[1];
+        qb[ks + 1][0] = w[2]; qb[ks + 1][1] = w[3];
+      }
+    }
+  };
+  auto team_sync = [&]() {
+    __syncwarp();
+    if constexpr (kTeam > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeam * 32) : "memory");
+  };
 
   for (int w0 = 0; w0 < cnt; w0 += window) {
     const int wn = min(window, cnt - w0);
@@ -258,129 +354,163 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       __syncthreads();                                 // every warp is done with the previous window
       stage_window(w0, wn);
       __syncthreads();
+    } else if (w0 > 0) {
+      team_sync();                                     // the ring is filled anew: no lane still reads the last tiles
     }
-    const int first_row = warp * kGqaRows;
-    const int nk = wn > first_row ? (wn - first_row + kWarps * kGqaRows - 1) / (kWarps * kGqaRows) : 0;
-    // position of row (lane & 15) of this warp's k-th tile, -1 if there is none
+    const int first_row = team * kGqaRows;
+    const int nk = wn > first_row ? (wn - first_row + kTeams * kGqaRows - 1) / (kTeams * kGqaRows) : 0;
+    // position of row (lane & 15) of this team's k-th tile, -1 if there is none
     auto tile_pos = [&](int k) {
-      const int r = first_row + k * (kWarps * kGqaRows) + (lane & 15);
+      const int r = first_row + k * (kTeams * kGqaRows) + (lane & 15);
       return r < wn ? (kSparse ? s_idx[r] : start + w0 + r) : -1;
     };
-    // requests tile k of the window (if it exists) into slot k % depth; always closes a copy group
-    auto request = [&](int k) {
+    // Requests tile k of the window (if it exists) into the slot at `slot`; always closes a copy group.  Returns which
+    // of its sixteen rows exist.
+    auto request = [&](int k, uint32_t slot) -> uint32_t {
+      uint32_t live = 0u;
       if (k < nk) {
         const int my_pos = tile_pos(k);
-        const uint32_t slot = ring + (uint32_t)(k % kStagedDepth) * (2 * kStagedTileBytes);
-        const int chunk = lane & 15;
+        live = __ballot_sync(0xffffffffu, my_pos >= 0) & 0xffffu;
+        const uint32_t dk = slot + copy_k, dv = slot + kTileBytes + copy_v;
+        // (the warps of a team copy the rows in turns; from one copy of a lane to its next, only XOR-ed bits and a constant change in the address)
+        constexpr int kCopies = kGqaRows / kRowsPerCopy / kTeam;
+        auto to_k = [&](int i) { return (kFp8 ? dk : dk ^ ((2 * i & 7) << 4)) + i * (kRowsPerCopy * kRowBytes); };
+        auto to_v = [&](int i) { return (dv ^ ((kRowsPerCopy * i & 7) << 4)) + i * (kRowsPerCopy * kRowBytes); };
+        if (live == 0xffffu) {                         // warp-uniform
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int r = 2 * i + (lane >> 4);
-          const int pos = __shfl_sync(0xffffffffu, my_pos, r);
-          const uint32_t bytes = pos >= 0 ? 16u : 0u;
-          const uint64_t row = pos >= 0 ? (uint64_t)(uint32_t)pos : 0ull;
-          const uint32_t off = tile_offset(r, chunk);
-          cp_async_16(slot + off, kbase + row * p.k_row_bytes + chunk * 16, bytes, policy);
-          cp_async_16(slot + kStagedTileBytes + off, vbase + row * p.v_row_bytes + chunk * 16, bytes, policy);
+          for (int i = 0; i < kCopies; ++i) {
+            const uint32_t pos = __shfl_sync(0xffffffffu, my_pos, kRowsPerCopy * i + copy_row);
+            cp_async_16(to_k(i), kcol + (uint64_t)pos * p.k_row_bytes, policy);
+            cp_async_16(to_v(i), vcol + (uint64_t)pos * p.v_row_bytes, policy);
+          }
+        } else {                                       // rows that do not exist are zero
+#pragma unroll 1
+          for (int i = 0; i < kCopies; ++i) {
+            const int pos = __shfl_sync(0xffffffffu, my_pos, kRowsPerCopy * i + copy_row);
+            const uint64_t row = pos >= 0 ? (uint64_t)(uint32_t)pos : 0ull;
+            cp_async_16_or_zero(to_k(i), kcol + row * p.k_row_bytes, pos >= 0 ? 16u : 0u, policy);
+            cp_async_16_or_zero(to_v(i), vcol + row * p.v_row_bytes, pos >= 0 ? 16u : 0u, policy);
+          }
         }
       }
       cp_async_commit();
+      return live;
     };
+    uint32_t lives[kStagedDepth];                      // rows of tiles k, k + 1, ... (registers: shifted by one per tile)
 #pragma unroll
-    for (int k = 0; k < kStagedDepth - 1; ++k) request(k);
-    for (int k = 0; k < nk; ++k) {
-      __syncwarp();                                    // the slot about to be refilled has been read by every lane
-      request(k + kStagedDepth - 1);
+    for (int k = 0; k < kStagedDepth - 1; ++k) lives[k] = request(k, ring + k * (2 * kTileBytes));
+    if (w0 == 0) {                                     // (the query is not needed before the first tiles are requested)
+      if (!kSparse) __syncthreads();
+      load_q();
+    }
+    constexpr uint32_t kRingBytes = kStagedDepth * 2 * kTileBytes;
+    uint32_t kt = ring, refill = ring + kRingBytes - 2 * kTileBytes;   // slots of tile k and of tile k + depth - 1
+    auto after = [&](uint32_t slot) { return slot + 2 * kTileBytes == ring + kRingBytes ? ring : slot + 2 * kTileBytes; };
+    for (int k = 0; k < nk; ++k, kt = after(kt), refill = after(refill)) {
+      team_sync();                                     // the slot about to be refilled has been read by every lane
+      lives[kStagedDepth - 1] = request(k + kStagedDepth - 1, refill);
       cp_async_wait<kStagedDepth - 1>();               // tile k has landed (for this lane's copies) ...
-      __syncwarp();                                    // ... and for every other lane's
-      const uint32_t live = __ballot_sync(0xffffffffu, tile_pos(k) >= 0) & 0xffffu;
+      team_sync();                                     // ... and for every other lane's
+      const uint32_t live = lives[0];
+#pragma unroll
+      for (int i = 0; i + 1 < kStagedDepth; ++i) lives[i] = lives[i + 1];
       if (live == 0u) continue;                        // warp-uniform: nothing to add
-      const uint32_t kt = ring + (uint32_t)(k % kStagedDepth) * (2 * kStagedTileBytes), vt = kt + kStagedTileBytes;
-      const int mm = lane >> 3, rr = lane & 7;
+      const uint32_t ka = kt + read_k, va = kt + kTileBytes + read_v;
 
-      // S = Q . K^T: two n-tiles of 8 rows
-      float s[2][4];
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) { s[nt][0] = 0.f; s[nt][1] = 0.f; s[nt][2] = 0.f; s[nt][3] = 0.f; }
-#pragma unroll
-      for (int ks = 0; ks < 8; ++ks) {
-        uint32_t kb[4];                                // rows 0-7: k lo, k hi; rows 8-15: k lo, k hi
-        ldmatrix_x4(kb, kt + tile_offset((mm >> 1) * 8 + rr, 2 * ks + (mm & 1)));
-        mma_16816<T>(s[0], qa[ks][0], kHi ? qa[ks][1] : 0u, qa[ks][2], kHi ? qa[ks][3] : 0u, kb[0], kb[1], s[0]);
-        mma_16816<T>(s[1], qa[ks][0], kHi ? qa[ks][1] : 0u, qa[ks][2], kHi ? qa[ks][3] : 0u, kb[2], kb[3], s[1]);
-      }
-      // lane (g, j) holds, for heads g (s[.][0..1]) and g+8 (s[.][2..3]), the rows nt*8 + 2j + {0, 1}
-      float mt_lo = neg_inf(), mt_hi = neg_inf();
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const bool ok = (live >> (nt * 8 + 2 * j + e)) & 1u;
-          s[nt][e] = ok ? s[nt][e] * p.scale_log2 : neg_inf();
-          s[nt][2 + e] = ok ? s[nt][2 + e] * p.scale_log2 : neg_inf();
-          mt_lo = fmaxf(mt_lo, s[nt][e]);
-          mt_hi = fmaxf(mt_hi, s[nt][2 + e]);
-        }
-      mt_lo = fmaxf(mt_lo, __shfl_xor_sync(0xffffffffu, mt_lo, 1));
-      mt_lo = fmaxf(mt_lo, __shfl_xor_sync(0xffffffffu, mt_lo, 2));
-      if (kHi) {
-        mt_hi = fmaxf(mt_hi, __shfl_xor_sync(0xffffffffu, mt_hi, 1));
-        mt_hi = fmaxf(mt_hi, __shfl_xor_sync(0xffffffffu, mt_hi, 2));
-      }
-      const float mn_lo = fmaxf(m_lo, mt_lo), mn_hi = fmaxf(m_hi, mt_hi);
-      if (mn_lo > m_lo) {
-        const float alpha = fast_exp2(m_lo - mn_lo);
-        l_lo *= alpha;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) { o[u][0] *= alpha; o[u][1] *= alpha; }
-        m_lo = mn_lo;
-      }
-      if (kHi && mn_hi > m_hi) {
-        const float alpha = fast_exp2(m_hi - mn_hi);
-        l_hi *= alpha;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) { o[u][2] *= alpha; o[u][3] *= alpha; }
-        m_hi = mn_hi;
-      }
-      // weights, split into a 16-bit value and a 16-bit residual: A fragments of P[16 heads, 16 rows]
-      // (a0: head g, rows 2j..; a1: head g+8, rows 2j..; a2: head g, rows 8+2j..; a3: head g+8, rows 8+2j..)
-      uint32_t pa[4], pr[4];
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const float w0 = fast_exp2(s[nt][0] - m_lo), w1 = fast_exp2(s[nt][1] - m_lo);   // -inf gives 0
-        l_lo += w0 + w1;
-        pa[2 * nt] = pack2<T>(w0, w1);
-        const float2 back = unpack2<T>(pa[2 * nt]);
-        pr[2 * nt] = pack2<T>(w0 - back.x, w1 - back.y);
-        if (kHi) {
-          const float x0 = fast_exp2(s[nt][2] - m_hi), x1 = fast_exp2(s[nt][3] - m_hi);
-          l_hi += x0 + x1;
-          pa[2 * nt + 1] = pack2<T>(x0, x1);
-          const float2 bk = unpack2<T>(pa[2 * nt + 1]);
-          pr[2 * nt + 1] = pack2<T>(x0 - bk.x, x1 - bk.y);
-        } else {
-          pa[2 * nt + 1] = 0u;
-          pr[2 * nt + 1] = 0u;
-        }
-      }
-      // O += P . V, sixteen dims (two n-tiles) per ldmatrix
-#pragma unroll
-      for (int dn = 0; dn < 8; ++dn) {
-        uint32_t vb[4];                                // dims 16dn..+7: rows 0-7, rows 8-15; dims 16dn+8..+15: the same
-        ldmatrix_x4_trans(vb, vt + tile_offset((mm & 1) * 8 + rr, 2 * dn + (mm >> 1)));
+      // S^T = K . Q^T: lane (g, j) gets rows g (s[0..1]) and g + 8 (s[2..3]) of heads 2 j and 2 j + 1
+      // (two sums of four k-steps each: half the length of the dependent chain)
+      float s[4] = {0.f, 0.f, 0.f, 0.f}, s_odd[4] = {0.f, 0.f, 0.f, 0.f};
+      if constexpr (kFp8) {
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
-          const int u = 2 * dn + half;
-          if (kHi) {
-            mma_16816<T>(o[u], pa[0], pa[1], pa[2], pa[3], vb[2 * half], vb[2 * half + 1], o[u]);
-            mma_16816<T>(o[u], pr[0], pr[1], pr[2], pr[3], vb[2 * half], vb[2 * half + 1], o[u]);
-          } else {
-            // rows 8..15 of the M dimension are unused: feed zeros, drop what comes back
-            float acc[4] = {o[u][0], o[u][1], 0.f, 0.f};
-            mma_16816<T>(acc, pa[0], 0u, pa[2], 0u, vb[2 * half], vb[2 * half + 1], acc);
-            mma_16816<T>(acc, pr[0], 0u, pr[2], 0u, vb[2 * half], vb[2 * half + 1], acc);
-            o[u][0] = acc[0];
-            o[u][1] = acc[1];
+          const uint4 lo = lds_16B(ka ^ (half << 6)), hi = lds_16B((ka ^ (half << 6)) + 8 * kRowBytes);
+          const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, c[4] = {hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t a0 = e4m3x2_to_bf162(a[i]), a1 = e4m3x2_to_bf162(c[i]);
+            const uint32_t a2 = e4m3x2_to_bf162(a[i] >> 16), a3 = e4m3x2_to_bf162(c[i] >> 16);
+            float (&sum)[4] = (i & 1) ? s_odd : s;
+            mma_16816<TQ>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
           }
+        }
+      } else {
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks) {
+          uint32_t a[4];
+          ldmatrix_x4(a, ka ^ (ks << 5));
+          float (&sum)[4] = (ks & 1) ? s_odd : s;
+          mma_16816<TQ>(sum, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1], sum);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[e] = (s[e] + s_odd[e]) * p.scale_log2;
+      if (live != 0xffffu) {                           // warp-uniform; a masked row's score is -inf
+        const bool live_lo = (live >> g) & 1u, live_hi = (live >> (g + 8)) & 1u;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          s[e] = live_lo ? s[e] : neg_inf();
+          s[2 + e] = live_hi ? s[2 + e] : neg_inf();
+        }
+      }
+      if (__any_sync(0xffffffffu, fmaxf(s[0], s[2]) > m[0] || fmaxf(s[1], s[3]) > m[1])) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {                  // rare after the first tiles
+          float mt = fmaxf(s[e], s[2 + e]);
+          mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 4));
+          mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 8));
+          mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 16));
+          const float mn = fmaxf(m[e], mt);
+          if (mn > m[e]) {
+            const float alpha = fast_exp2(m[e] - mn);
+            l[e] *= alpha;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) { o[t][e] *= alpha; o[t][2 + e] *= alpha; }
+            m[e] = mn;
+          }
+        }
+      }
+      // weights, split into a 16-bit value and a 16-bit residual, transposed into B fragments of P^T[16 rows, 8 heads]
+      uint32_t pa[2], pr[2];
+      // (a maximum of -inf: no finite score yet, every weight is 0)
+      const float r0 = m[0] > neg_inf() ? m[0] : 0.f, r1 = m[1] > neg_inf() ? m[1] : 0.f;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const float w0 = fast_exp2(s[2 * half] - r0) * kUp, w1 = fast_exp2(s[2 * half + 1] - r1) * kUp;   // -inf gives 0
+        l[0] += w0;
+        l[1] += w1;
+        const uint32_t w = pack2<TP>(w0, w1);
+        const float2 back = unpack2<TP>(w);
+        pa[half] = transpose8x8(w);
+        pr[half] = transpose8x8(pack2<TP>(w0 - back.x, w1 - back.y));
+      }
+      // O^T += V^T . P^T, sixteen dims at a time
+      if constexpr (kFp8) {
+        const uint4 v0 = lds_16B(va), v1 = lds_16B(va + kRowBytes);                          // rows 2 j, 2 j + 1
+        const uint4 v2 = lds_16B(va + 8 * kRowBytes), v3 = lds_16B(va + 9 * kRowBytes);      // rows 2 j + 8, 2 j + 9
+        const uint32_t x0[4] = {v0.x, v0.y, v0.z, v0.w}, x1[4] = {v1.x, v1.y, v1.z, v1.w};
+        const uint32_t x2[4] = {v2.x, v2.y, v2.z, v2.w}, x3[4] = {v3.x, v3.y, v3.z, v3.w};
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          // bytes 2 (t & 1) and 2 (t & 1) + 1 of both rows of a pair, interleaved
+          const uint32_t sel = (t & 1) ? 0x7362u : 0x5140u;
+          const uint32_t lo = __byte_perm(x0[t >> 1], x1[t >> 1], sel), hi = __byte_perm(x2[t >> 1], x3[t >> 1], sel);
+          const uint32_t a0 = e4m3x2_to_half2(lo), a1 = e4m3x2_to_half2(lo >> 16);
+          const uint32_t a2 = e4m3x2_to_half2(hi), a3 = e4m3x2_to_half2(hi >> 16);
+          // (the tile's own sum first, rounded to nearest into the running one: the tensor cores truncate, which over
+          // a long list would cost more than the weights' split)
+          float sum[4] = {0.f, 0.f, 0.f, 0.f};
+          mma_16816<TP>(sum, a0, a1, a2, a3, pr[0], pr[1], sum);
+          mma_16816<TP>(sum, a0, a1, a2, a3, pa[0], pa[1], sum);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) o[t][e] += sum[e];
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          uint32_t a[4];                               // dims 16t..+7, 16t+8..+15 of rows 0-7; the same of rows 8-15
+          ldmatrix_x4_trans(a, va ^ (t << 5));
+          mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pa[0], pa[1], o[t]);
+          mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pr[0], pr[1], o[t]);
         }
       }
     }
@@ -395,44 +525,48 @@ decode_partial_gqa_kernel(const DecodeParams p) {
 
   // per-warp triples -> shared memory (the ring is free now)
   __syncthreads();
-  float (*s_acc)[kLiveHeads][D + kGqaPad] = reinterpret_cast<float (*)[kLiveHeads][D + kGqaPad]>(s_ring);
-  l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1);
-  l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-  if (kHi) {
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
-  }
+  // [kTeams][kLiveHeads][kGqaPitch]
+  float (*s_acc)[kLiveHeads][kGqaPitch] = reinterpret_cast<float (*)[kLiveHeads][kGqaPitch]>(s_ring);
 #pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    *reinterpret_cast<float2*>(&s_acc[warp][g][8 * u + 2 * j]) = make_float2(o[u][0], o[u][1]);
-    if (kHi) *reinterpret_cast<float2*>(&s_acc[warp][g + 8][8 * u + 2 * j]) = make_float2(o[u][2], o[u][3]);
-  }
-  if (j == 0) {
-    s_m[warp][g] = m_lo; s_l[warp][g] = l_lo;
-    if (kHi) { s_m[warp][g + 8] = m_hi; s_l[warp][g + 8] = l_hi; }
+  for (int e = 0; e < 2; ++e) {
+    const int head = 8 * ht + 2 * j + e;
+    float sum = l[e];
+    sum += __shfl_xor_sync(0xffffffffu, sum, 4);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+    if (g == 0) { s_m[team][head] = m[e]; s_l[team][head] = sum / kUp; }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      if constexpr (kFp8) {
+        *reinterpret_cast<float2*>(&s_acc[team][head][gqa_column(16 * g + 2 * t)]) = make_float2(o[t][e] / kUp, o[t][2 + e] / kUp);
+      } else {
+        s_acc[team][head][gqa_column(16 * t + g)] = o[t][e];
+        s_acc[team][head][gqa_column(16 * t + g + 8)] = o[t][2 + e];
+      }
+    }
   }
   __syncthreads();
-  // thread d finishes dim d of every head
-  if (tid >= D) return;
-  for (int i = 0; i < G; ++i) {
+  // 128 threads finish a head: thread d its dim d
+  const int d = tid % D;
+  for (int i = tid / D; i < G; i += kThreads / D) {
     const int h = kvh * G + i;
     float M = neg_inf();
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) M = fmaxf(M, s_m[w][i]);
+    for (int w = 0; w < kTeams; ++w) M = fmaxf(M, s_m[w][i]);
     float L = 0.f, A = 0.f;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
+    for (int w = 0; w < kTeams; ++w) {
       const float wgt = (s_m[w][i] > neg_inf()) ? fast_exp2(s_m[w][i] - M) : 0.f;
       L = fmaf(s_l[w][i], wgt, L);
-      A = fmaf(s_acc[w][i][tid], wgt, A);
+      A = fmaf(s_acc[w][i][gqa_column(d)], wgt, A);
     }
     if (p.n_chunks == 1) {
-      store_out<T>(p, b, h, tid, L > 0.f ? A / L : 0.f);
-      if (tid == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L > 0.f ? (M + log2f(L)) * kLn2 : neg_inf();
+      store_out<TQ>(p, b, h, d, L > 0.f ? A / L : 0.f);
+      if (d == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L > 0.f ? (M + log2f(L)) * kLn2 : neg_inf();
     } else {
       const int64_t slot = ((int64_t)b * p.H + h) * p.n_chunks + chunk_id;
-      p.ws_acc[slot * D + tid] = A;
-      if (tid == 0) p.ws_ml[slot] = make_float2(M, L);
+      p.ws_acc[slot * D + d] = A;
+      if (d == 0) p.ws_ml[slot] = make_float2(M, L);
     }
   }
 }

@@ -115,3 +115,78 @@ def test_descriptor_checks():
     assert ssa.decode_workspace_bytes(desc, 64) > 0
     desc.k_stride_t = 136                                       # 136 bytes: not a multiple of 16
     assert ssa.decode_workspace_bytes(desc, 64) == 0
+
+
+@pytest.mark.parametrize("B,group,T,counts", [
+    (3, 2, 140, [1, 16, 129]),          # list ends around a 16-row tile and around a round of the block's tiles
+    (2, 7, 1100, [1023, 1025]),         # ... and around the staging window; a head tile with one head missing
+    (3, 8, 700, [15, 17, 700]),
+    (3, 9, 700, [127, 128, 0]),         # two head tiles, the second with one head; an empty list
+    (2, 16, 2600, [2600, 513]),
+    (40, 4, 300, None),                 # one unit for most SMs: the large blocks, index and span lists
+])
+def test_grouped_heads_over_an_8_bit_cache(B, group, T, counts):
+    # fp32 output: weights carry 22 bits or an absolute 2^-37, sums are fp32 over at most 2600 rows: 2^-22 per weight
+    # and 2^-24 sqrt(2600) per sum bound the error of an N(0, 1) average by 5e-6; 2e-5 is asserted
+    Hkv, D = 2, 128
+    H = group * Hkv
+    p = Fp8Problem(B, H, Hkv, T, D, seed=100 * group + T)
+    rng = np.random.default_rng(T)
+    ctx = [T] * B
+    counts = counts or [int(x) for x in rng.integers(1, T + 1, size=B)]
+    index = np.full((B, T), -1, np.int32)
+    for b, c in enumerate(counts):
+        index[b, :c] = np.sort(rng.choice(T, c, replace=False))
+    out = torch.full((B, H, D), 7.0, dtype=torch.float32, device=DEV)
+    lse = torch.full((B, H), 7.0, dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    d_ctx = torch.tensor(ctx, dtype=torch.int32, device=DEV)
+    desc = ssa.make_desc(p.q, p.k, p.v, out)
+    ws = torch.empty(ssa.decode_spans_workspace_bytes(desc, T, 4), dtype=torch.uint8, device=DEV)
+    ko, vo = p.oracle_kv()
+
+    def check(ref, ref_lse, what):
+        torch.cuda.synchronize()
+        assert float(np.abs(out.double().cpu().numpy() - ref).max()) <= 2e-5, what
+        ok = np.isfinite(ref_lse)
+        np.testing.assert_allclose(lse.double().cpu().numpy()[ok], ref_lse[ok], rtol=2e-6, atol=2e-6, err_msg=what)
+        assert int(status.item()) == 0
+
+    ssa.decode_attn_sparse(desc, p.q, p.k, p.v, d_ctx, torch.from_numpy(index).to(DEV),
+                           torch.tensor(counts, dtype=torch.int32, device=DEV), T, out, lse, ws, status)
+    check(*O.decode_attn_sparse(p.q_bits, ko, vo, ctx, index, counts, 1 / np.sqrt(D), "bf16/e4m3"), "index lists")
+    ssa.decode_attn_dense(desc, p.q, p.k, p.v, d_ctx, out, lse, ws, status)
+    dense = O.decode_attn_dense(p.q_bits, ko, vo, ctx, 1 / np.sqrt(D), "bf16/e4m3")
+    check(*dense, "full context")
+    flat = torch.tensor([[0, T // 2], [T // 2, T]] * B, dtype=torch.int32, device=DEV)
+    offs = torch.arange(0, 2 * B + 1, 2, dtype=torch.int32, device=DEV)
+    ssa.decode_attn_spans(desc, p.q, p.k, p.v, d_ctx, offs, flat, 4, T, out, lse, None, None, ws, status)
+    check(*dense, "span lists")
+
+
+@pytest.mark.parametrize("group", [4, 12])
+def test_grouped_heads_read_every_e4m3_pattern_exactly(group):
+    """One selected row per K/V head: every head of the group returns that V row, exactly; a NaN in K or V shows."""
+    B, Hkv, T, D = 1, 2, 32, 128
+    H = group * Hkv
+    p = Fp8Problem(B, H, Hkv, T, D, seed=3)
+    pats = np.array([x for x in range(256) if x not in (0x7F, 0xFF)], np.uint8)
+    v = p.v_bits.copy()
+    v[0, 0, 5], v[0, 1, 5] = pats[:128], pats[126:254]
+    out = torch.zeros((B, H, D), dtype=torch.float32, device=DEV)
+    desc = ssa.make_desc(p.q, p.k, p.v, out)
+    ws = torch.empty(ssa.decode_workspace_bytes(desc, 32), dtype=torch.uint8, device=DEV)
+    idx = torch.full((1, 32), 5, dtype=torch.int32, device=DEV)
+    one, ctx = (torch.tensor([x], dtype=torch.int32, device=DEV) for x in (1, T))
+
+    def run(v_bits):
+        pv = torch.from_numpy(v_bits).view(torch.float8_e4m3fn).to(DEV)
+        ssa.decode_attn_sparse(desc, p.q, p.k, pv, ctx, idx, one, 32, out, None, ws, None)
+        torch.cuda.synchronize()
+        return out.double().cpu().numpy()[0]
+
+    want = np.repeat(O.decode_e4m3(v[0, :, 5]), group, axis=0)
+    assert np.array_equal(run(v), want)
+    v[0, 0, 5, 77] = 0x7F
+    got = run(v)
+    assert np.isnan(got[:group, 77]).all() and np.isfinite(np.delete(got, 77, axis=1)).all()
