@@ -528,8 +528,8 @@ int32_t ssa_decode_step(const ssa_attn_desc* desc, const ssa_step* step, void* s
  *
  * Same arguments and results as ssa_decode_attn_sparse, minus the workspace.
  * Differences:
- *  - a request whose scratch need (what ssa_decode_workspace_bytes reports
- *    for desc and max_selected) exceeds SSA_STATIC_SCRATCH_BYTES is rejected
+ *  - a request whose scratch need (at most what ssa_decode_workspace_bytes
+ *    reports for desc and max_selected) exceeds SSA_STATIC_SCRATCH_BYTES is rejected
  *    with SSA_ERR_WORKSPACE and nothing is launched;
  *  - the first call on each device looks up the array's device address (the
  *    device must be current); make that first call outside any stream

@@ -79,6 +79,8 @@ struct DecodeParams {
   int32_t H, max_ctx, index_stride, max_selected, chunk, n_chunks, out_f32, early_release;
   int32_t kv_group;         // query heads per K/V head (1: multi-head attention)
   int32_t gqa_wide;         // row-sharing kernel, one large block per SM
+  int32_t even_blocks;      // row-sharing kernel over full contexts: blocks that share the rows evenly (0: fixed chunks)
+  int32_t B;
   // paged cache (page_table != nullptr): logical position t of request b is row
   // page_table[b * page_table_stride + (t >> page_shift)] << page_shift | (t & page_mask) of the pool
   const int32_t* page_table;
@@ -540,7 +542,8 @@ namespace ssa {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool wide; };   // wide: one large row-sharing block per SM
+// wide: one large row-sharing block per SM; even_blocks: that many blocks with even shares of the rows (0: chunks)
+struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool wide; int even_blocks; };
 
 // Grouped query heads go to the kernel that reads a K/V row once for the whole group.
 static bool shares_rows(const ssa_attn_desc* d) {
@@ -574,12 +577,14 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
     // them fit an SM: about one block per resident slot, i.e. as few chunks as keep the SMs busy (measured,
     // B*H_kv = 64..256, context 8192: within 3 % of the best split for groups of 4, 8 and 16 heads).  Ragged batches
     // would rather have shorter chunks (17 requests of 1001..8190 rows, 16 heads: 62 instead of 73 us with chunks of
-    // 1024), batches of like lengths pay for them (all 8190: 102 instead of 90 us), and the host knows no lengths.
+    // 1024), batches of like lengths pay for them (all 8190: 102 instead of 90 us), and the host knows no lengths;
+    // full contexts are therefore cut on the device (make_even), lists keep this split.
     const long long target = sms * 2;
     long long n = target / units;                              // rounded down: never one block over a full wave
     n = std::max<long long>(1, std::min<long long>(n, (max_selected + 255) / 256));
     chunk = (int)(((max_selected + n - 1) / n + 63) / 64 * 64);
   }
+  pl->even_blocks = 0;
   int n_chunks = (max_selected + chunk - 1) / chunk;
   if (n_chunks == 1) chunk = (max_selected + 31) / 32 * 32;
   pl->chunk = chunk;
@@ -589,6 +594,29 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
   return true;
 }
 
+// Full contexts read by the row-sharing kernel: even shares over one block per resident slot, if the lengths of all
+// requests fit a block's scan and the workspace, which callers may have sized by an index list's bound, holds them.
+static size_t even_bytes(const ssa_attn_desc* d, int blocks, size_t* acc_bytes) {
+  const size_t triples = (size_t)2 * blocks * (d->H / d->H_kv);
+  *acc_bytes = (triples * d->D * sizeof(float) + 255) / 256 * 256;
+  return *acc_bytes + (triples * sizeof(float2) + 255) / 256 * 256;
+}
+
+static int even_blocks_wanted(const ssa_attn_desc* d, const Plan& pl) {
+  if (!shares_rows(d) || pl.wide || d->B > kEvenMaxBatch || d->max_ctx <= kEvenMinPieces * kEvenRows) return 0;
+  const long long units = (long long)d->B * d->H_kv, pieces = ((long long)d->max_ctx + kEvenRows - 1) / kEvenRows;
+  if (units * pieces > 0xffffffll) return 0;                         // rows and pieces stay far inside 32 bits
+  return (int)std::min<long long>(2ll * sm_count(), units * ((pieces + kEvenMinPieces - 1) / kEvenMinPieces));
+}
+
+static void make_even(const ssa_attn_desc* d, size_t ws_bytes, Plan* pl) {
+  const int blocks = even_blocks_wanted(d, *pl);
+  size_t acc = 0;
+  if (blocks == 0 || even_bytes(d, blocks, &acc) > ws_bytes) return;
+  pl->even_blocks = blocks;
+  pl->acc_bytes = acc;
+}
+
 // Blocked lists: a block of the grid expands as many list entries as fit kMaskChunk positions.
 static bool make_plan_blockmask(const ssa_attn_desc* d, int block_size, int max_blocks, Plan* pl) {
   if (!d || d->B <= 0 || d->H <= 0 || max_blocks <= 0) return false;
@@ -596,6 +624,7 @@ static bool make_plan_blockmask(const ssa_attn_desc* d, int block_size, int max_
   if (block_size != 32 && block_size != 64 && block_size != 128 && block_size != 256) return false;
   const long long units = (long long)d->B * d->H;
   pl->wide = false;
+  pl->even_blocks = 0;
   pl->chunk = kMaskChunk / block_size;
   pl->n_chunks = (max_blocks + pl->chunk - 1) / pl->chunk;
   pl->acc_bytes = ((size_t)units * pl->n_chunks * d->D * sizeof(float) + 255) / 256 * 256;
@@ -648,6 +677,12 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
         using Shape = GqaShape<T, kHi, kWide>;
         block_threads = Shape::kWarps * 32;
         dynamic_smem = Shape::kSmemBytes;
+        if constexpr (!kWide) {
+          if (p.even_blocks > 0) {
+            kernel = decode_partial_gqa_kernel<T, kDense, kHi, false, true>;
+            return;
+          }
+        }
         kernel = mode == kIndex   ? decode_partial_gqa_kernel<T, kIndex, kHi, kWide>
                  : mode == kSpans ? decode_partial_gqa_kernel<T, kSpans, kHi, kWide>
                                   : decode_partial_gqa_kernel<T, kDense, kHi, kWide>;
@@ -656,6 +691,7 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
       else p.gqa_wide ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{});
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_smem) != cudaSuccess)
         return SSA_ERR_CUDA;
+      if (p.even_blocks > 0) grid = dim3((unsigned)p.even_blocks);
     }
   }
   if (!share) {
@@ -683,7 +719,11 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
   if (ev_e) cudaEventRecord(ev_e, st);
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   int launches = 1;
-  if (p.n_chunks > 1) {
+  if (share && p.even_blocks > 0) {
+    err = launch_pdl(decode_merge_even_kernel<TQ>, dim3((unsigned)p.H, (unsigned)B), dim3(D), st, p);
+    if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
+    ++launches;
+  } else if (p.n_chunks > 1) {
     DecodeParams pm = p;
     if (mode == kSpans) pm.counts = p.ws_counts;        // the first pass left the list lengths there
     err = launch_pdl(decode_merge_kernel<TQ, D>, dim3((unsigned)p.H, (unsigned)B), dim3(D), st, pm);
@@ -757,6 +797,7 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
     return SSA_ERR_SHAPE;
   }
   if (!ws || ws_bytes < pl.total_bytes + (mode == kSpans ? counts_bytes(d) : 0)) return SSA_ERR_WORKSPACE;
+  if (mode == kDense) make_even(d, ws_bytes, &pl);
 
   if (q_host && !(mode == kIndex && !pg && !dense_paged && pl.n_chunks == 1 && !shares_rows(d) &&
                   d->kv_dtype != SSA_FP8_E4M3 && aligned16(q_host)))
@@ -799,11 +840,14 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   p.index_stride = index_stride; p.max_selected = max_selected;
   p.chunk = pl.chunk; p.n_chunks = pl.n_chunks;
   p.gqa_wide = pl.wide ? 1 : 0;
+  p.even_blocks = pl.even_blocks;
+  p.B = d->B;
   p.out_f32 = d->out_dtype == SSA_F32;
   // A grid of a few waves releases the next kernel at once (its blocks wait on
   // chip instead of being launched after the drain); a long grid does so only
   // as its blocks finish, so that waiting blocks do not crowd out its own.
-  p.early_release = (long long)d->B * d->H * pl.n_chunks <= (long long)sm_count() * SSA_MIN_BLOCKS * 6;
+  p.early_release = pl.even_blocks == 0 &&
+                    (long long)d->B * d->H * pl.n_chunks <= (long long)sm_count() * SSA_MIN_BLOCKS * 6;
   const float scale = d->scale > 0.f ? d->scale : 1.0f / sqrtf((float)d->D);
   p.scale_log2 = scale * kLog2e;
 
@@ -1014,7 +1058,9 @@ int32_t ssa_decode_attn_blockmask(const ssa_attn_desc* desc, const void* q, cons
 size_t ssa_decode_workspace_bytes(const ssa_attn_desc* desc, int32_t max_selected) {
   ssa::Plan pl;
   if (!desc || ssa::check_desc(desc) != SSA_OK || !ssa::make_plan(desc, max_selected, &pl)) return 0;
-  return pl.total_bytes;
+  if (max_selected < desc->max_ctx) return pl.total_bytes;
+  size_t acc = 0;                                        // the bound of a full context: room for even shares as well
+  return std::max(pl.total_bytes, ssa::even_bytes(desc, ssa::even_blocks_wanted(desc, pl), &acc));
 }
 
 int32_t ssa_decode_attn_sparse(const ssa_attn_desc* desc, const void* q, const void* k_cache,

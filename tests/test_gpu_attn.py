@@ -448,6 +448,55 @@ def test_grouped_heads_chunks_longer_than_the_staging_area(B, H, Hkv, T):
     assert_parity(out_d[sample], ref_d[sample], False, "long chunks, dense")
 
 
+@pytest.mark.parametrize("B,H,Hkv,T,dtype,lens", [
+    (1, 4, 2, 8000, "bf16", [7937]),                            # two units, each in many shares
+    (5, 8, 2, 3000, "f16", [2999, 0, 1, 64, 65]),               # shares of the smallest size; a request without rows
+    (4, 32, 2, 3000, "bf16", [3000, 257, 2049, 63]),            # sixteen heads: two warps per tile
+    (60, 16, 8, 700, "bf16", None),                             # more units than blocks: several whole ones per share
+    (301, 4, 2, 300, "f16", None),
+    (1024, 2, 1, 260, "bf16", None), (1025, 2, 1, 260, "bf16", None),   # either side of the batch limit
+])
+def test_even_shares_of_ragged_full_contexts(B, H, Hkv, T, dtype, lens):
+    D = 128
+    p = Problem(B, Hkv, T, D, dtype, seed=B + T)
+    rng = np.random.default_rng(B)
+    p.q_bits = random_bits(rng, (B, H, D), dtype)
+    p.H = H
+    p.upload()
+    ctx = lens or [int(x) for x in rng.integers(0, T + 1, size=B)]
+    if not lens:
+        ctx[:3], ctx[-1] = [T, 0, 1], T
+    seqs = list(range(B)) if B <= 60 else sorted({0, 1, 2, 3, B // 2, B - 2, B - 1})
+    k_rep, v_rep = (np.repeat(x[seqs], H // Hkv, axis=1) for x in (p.k_bits, p.v_bits))
+    ref, ref_lse = O.decode_attn_dense(p.q_bits[seqs], k_rep, v_rep, [ctx[b] for b in seqs], scale_of(D), dtype)
+    some = np.isfinite(ref_lse)
+
+    def check(out, lse, what):
+        # fp32 output: the weights' split (2^-17) and fp32 sums of at most 8000 rows (2^-24 sqrt(8000)): below 2e-5
+        assert np.abs(out[seqs] - ref).max() <= 2e-5, what
+        np.testing.assert_allclose(lse[seqs][some], ref_lse[some], rtol=2e-6, atol=2e-6, err_msg=what)
+        assert np.all(np.isneginf(lse[seqs][~some])), what
+
+    out, lse, status = p.dense(ctx)
+    assert status == 0
+    check(out, lse, "even shares")
+    again, lse2, _ = p.dense(ctx)
+    assert np.array_equal(out, again) and np.array_equal(lse, lse2)
+    over = [n if n < T else T + 99 for n in ctx]                # a length above the cache is clamped and flagged
+    out, lse, status = p.dense(over)
+    assert status == (ssa.DEV_BAD_COUNT if over != ctx else 0)
+    check(out, lse, "lengths above the cache")
+    # a workspace of the size that fixed chunks need (one triple per chunk and head; H / Hkv per block) is still taken
+    o = torch.full((B, H, D), 7.0, dtype=torch.float32, device=DEV)
+    ls = torch.full((B, H), 7.0, dtype=torch.float32, device=DEV)
+    desc = ssa.make_desc(p.q, p.k, p.v, o)
+    chunks = -(-T // 256)
+    ws = torch.empty(min(ssa.decode_workspace_bytes(desc, T), B * H * chunks * (4 * D + 8) + 512), dtype=torch.uint8, device=DEV)
+    ssa.decode_attn_dense(desc, p.q, p.k, p.v, torch.tensor(ctx, dtype=torch.int32, device=DEV), o, ls, ws, None)
+    torch.cuda.synchronize()
+    check(o.double().cpu().numpy(), ls.double().cpu().numpy(), "the workspace of fixed chunks")
+
+
 def test_mixed_batch_of_full_context_and_restricted_requests():
     # requests at a "determine span" step attend to everything, the others to their spans, in one launch
     wl = inputs.make_config(2, B=6, H=4)
