@@ -603,8 +603,11 @@ static size_t even_bytes(const ssa_attn_desc* d, int blocks, size_t* acc_bytes) 
 }
 
 static int even_blocks_wanted(const ssa_attn_desc* d, const Plan& pl) {
-  if (!shares_rows(d) || pl.wide || d->B > kEvenMaxBatch || d->max_ctx <= kEvenMinPieces * kEvenRows) return 0;
+  if (!shares_rows(d) || pl.wide || pl.n_chunks == 1 || d->B > kEvenMaxBatch) return 0;
   const long long units = (long long)d->B * d->H_kv, pieces = ((long long)d->max_ctx + kEvenRows - 1) / kEvenRows;
+  // Only where the fixed plan has a second pass too (about 3 us), and shares are long enough to pay for the scan of the
+  // lengths in front of the first rows: 1024 rows, a third of what the measured launch has.
+  if (units * d->max_ctx < 2ll * sm_count() * 1024) return 0;
   if (units * pieces > 0xffffffll) return 0;                         // rows and pieces stay far inside 32 bits
   return (int)std::min<long long>(2ll * sm_count(), units * ((pieces + kEvenMinPieces - 1) / kEvenMinPieces));
 }
