@@ -111,6 +111,14 @@ __device__ __forceinline__ void store_out(const DecodeParams& p, int b, int h, i
   else reinterpret_cast<T*>(p.out)[o] = from_float<T>(val);
 }
 
+// Element d of a finished row and, with d = 0, its lse.  No attended row (L is exactly 0): zeros and -inf.  A NaN among
+// the scores has made L a NaN, which must reach both.
+template <typename T>
+__device__ __forceinline__ void store_row_value(const DecodeParams& p, int b, int h, int d, float M, float L, float A) {
+  store_out<T>(p, b, h, d, L == 0.f ? 0.f : A / L);
+  if (d == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L == 0.f ? neg_inf() : (M + log2f(L)) * kLn2;
+}
+
 // A lane's piece of a cache row: 16 values as eight pairs.  16-bit storage: 32 bytes, a pair per word; 8-bit
 // storage: 16 bytes in w[0..3], two pairs per word.
 struct Piece { uint32_t w[8]; };
@@ -440,6 +448,9 @@ decode_partial_kernel(const DecodeParams p) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) acc[i] = fma2(pw2, piece_pair<T>(vr[u], i), acc[i]);
       }
+    } else {                                            // every score so far is -inf (masked) or NaN, which has to show
+#pragma unroll
+      for (int u = 0; u < kU; ++u) l = s[u] == s[u] ? l : s[u];
     }
   }
 
@@ -467,8 +478,7 @@ decode_partial_kernel(const DecodeParams p) {
       A = fmaf(s_acc[i][tid], w, A);
     }
     if (p.n_chunks == 1) {
-      store_out<TQ>(p, b, h, tid, L > 0.f ? A / L : 0.f);
-      if (tid == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L > 0.f ? (M + log2f(L)) * kLn2 : neg_inf();
+      store_row_value<TQ>(p, b, h, tid, M, L, A);
     } else {
       const int64_t slot = ((int64_t)b * p.H + h) * p.n_chunks + chunk_id;
       p.ws_acc[slot * D + tid] = A;
@@ -529,8 +539,7 @@ decode_merge_kernel(const DecodeParams p) {
       }
     }
   }
-  store_out<T>(p, b, h, d, L > 0.f ? A / L : 0.f);
-  if (d == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L > 0.f ? (M + log2f(L)) * kLn2 : neg_inf();
+  store_row_value<T>(p, b, h, d, M, L, A);
 }
 
 }  // namespace ssa

@@ -647,8 +647,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       A = fmaf(s_acc[w][i][gqa_column(d)], wgt, A);
     }
     if (kEven ? taken == unit_pieces : p.n_chunks == 1) {
-      store_out<TQ>(p, b, h, d, L > 0.f ? A / L : 0.f);
-      if (d == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L > 0.f ? (M + log2f(L)) * kLn2 : neg_inf();
+      store_row_value<TQ>(p, b, h, d, M, L, A);
     } else {
       const int64_t slot = kEven ? (int64_t)(2 * chunk_id + (start == 0 ? 1 : 0)) * G + i
                                  : ((int64_t)b * p.H + h) * p.n_chunks + chunk_id;
@@ -717,8 +716,7 @@ decode_merge_even_kernel(const DecodeParams p) {
       A = fmaf(row[k], w, A);
     }
   }
-  store_out<TQ>(p, b, h, d, L > 0.f ? A / L : 0.f);
-  if (d == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L > 0.f ? (M + log2f(L)) * kLn2 : neg_inf();
+  store_row_value<TQ>(p, b, h, d, M, L, A);
 }
 
 }  // namespace ssa

@@ -496,6 +496,67 @@ def test_even_shares_of_ragged_full_contexts(B, H, Hkv, T, dtype, lens):
     check(o.double().cpu().numpy(), ls.double().cpu().numpy(), "the workspace of fixed chunks")
 
 
+@pytest.mark.parametrize("how", ["sparse", "dense", "spans", "blockmask"])
+@pytest.mark.parametrize("B,H,Hkv,T,D,dtype,sel", [
+    (2, 2, 2, 300, 128, "bf16", 1),           # the one selected row holds the NaN: nothing else gives the row a maximum
+    (2, 2, 2, 300, 64, "f16", 5),             # ... one of five, alone in its group of lanes
+    (2, 3, 3, 1200, 128, "fp8", 1100),        # several chunks and the second pass
+    (2, 8, 2, 300, 128, "bf16", 1), (2, 8, 2, 1200, 128, "f16", 1100),      # rows shared by four heads
+    (40, 24, 2, 300, 128, "bf16", 200), (40, 24, 2, 300, 128, "fp8", 200),  # ... by twelve, large blocks
+    (3, 8, 2, 51000, 128, "bf16", 1100), (2, 24, 2, 1200, 128, "fp8", 1),   # even shares of the full context
+])
+def test_a_nan_in_a_selected_key_shows_and_in_another_does_not(B, H, Hkv, T, D, dtype, sel, how):
+    """softmax over scores with a NaN is NaN: rows and lse of the heads that read the key, of no others."""
+    if how == "blockmask" and T > 2000:
+        pytest.skip("blocked lists take the one-head kernel at every size")
+    kv = {"bf16": torch.bfloat16, "f16": torch.float16, "fp8": torch.float8_e4m3fn}[dtype]
+    gen = torch.Generator().manual_seed(T + sel)
+    k, v = (torch.randn((B, Hkv, T, D), generator=gen).to(kv) for _ in range(2))
+    q = torch.randn((B, H, D), generator=gen).to(torch.bfloat16 if dtype == "fp8" else kv)
+    rng = np.random.default_rng(sel)
+    rows = np.sort(rng.choice(T - 1, sel, replace=False))       # position T - 1 is not in the lists
+    index = np.full((B, (sel + 31) // 32 * 32), -1, np.int32)
+    index[:, :sel] = rows
+    other = T - 1 if how != "dense" else None                   # a key nobody attends to: never read
+    for t, x in ((int(rows[sel // 2]), 0), (other, 1)):
+        if t is not None:
+            k[B - 1, x, t, 3] = float("nan")
+    q, k, v = q.to(DEV), k.to(DEV), v.to(DEV)
+    out = torch.full((B, H, D), 7.0, dtype=torch.float32, device=DEV)
+    lse = torch.full((B, H), 7.0, dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    ctx = torch.full((B,), T, dtype=torch.int32, device=DEV)
+    desc = ssa.make_desc(q, k, v, out)
+    ws_for = lambda n: torch.empty(max(n, 16), dtype=torch.uint8, device=DEV)
+    if how == "sparse":
+        ssa.decode_attn_sparse(desc, q, k, v, ctx, torch.from_numpy(index).to(DEV),
+                               torch.full((B,), sel, dtype=torch.int32, device=DEV), sel, out, lse,
+                               ws_for(ssa.decode_workspace_bytes(desc, sel)), status)
+    elif how == "dense":
+        ssa.decode_attn_dense(desc, q, k, v, ctx, out, lse, ws_for(ssa.decode_workspace_bytes(desc, T)), status)
+    else:
+        spans = torch.from_numpy(np.tile(np.stack([rows, rows + 1], 1).astype(np.int32), (B, 1))).to(DEV)
+        offs = torch.arange(0, B * sel + 1, sel, dtype=torch.int32, device=DEV)
+        if how == "spans":
+            ssa.decode_attn_spans(desc, q, k, v, ctx, offs, spans, sel, sel, out, lse, None, None,
+                                  ws_for(ssa.decode_spans_workspace_bytes(desc, sel, sel)), status)
+        else:
+            bs, n = 64, (T + 63) // 64
+            idx = torch.full((B, n), -1, dtype=torch.int32, device=DEV)
+            mask = torch.zeros((B, n, bs // 32), dtype=torch.int32, device=DEV)
+            cnt = torch.zeros(B, dtype=torch.int32, device=DEV)
+            ssa.spans_to_blockmask(offs, spans, ctx, bs, idx, mask, cnt, status)
+            ssa.decode_attn_blockmask(desc, q, k, v, ctx, idx, mask, cnt, bs, n, out, lse,
+                                      ws_for(ssa.decode_blockmask_workspace_bytes(desc, bs, n)), status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    hit = np.zeros((B, H), bool)
+    hit[B - 1, :H // Hkv] = True                                # the query heads of cache head 0
+    assert np.array_equal(np.isnan(lse.cpu().numpy()), hit)
+    got = out.cpu().numpy()
+    assert np.isnan(got[hit]).all() and np.isfinite(got[~hit]).all()
+
+
 def test_mixed_batch_of_full_context_and_restricted_requests():
     # requests at a "determine span" step attend to everything, the others to their spans, in one launch
     wl = inputs.make_config(2, B=6, H=4)
