@@ -87,8 +87,12 @@ typedef enum { SSA_F16 = 0, SSA_BF16 = 1, SSA_F32 = 2, SSA_FP8_E4M3 = 3 } ssa_dt
  * infinities), one byte per element, read as they are - a caller that keeps a
  * scale with the cache folds K's into `scale` and applies V's to the output;
  * q is then BF16 and out_dtype BF16 or F32.  Such a cache halves the bytes per
- * selected row; grouped query heads over it are served one head per thread
- * block (each head re-reads the rows, mostly from L2).
+ * selected row.  Grouped query heads over it share the rows they read (D = 128
+ * and 2 to 16 heads per K/V head), as over a 16-bit cache: the scores and the
+ * sums are fp32, the softmax weights enter the second contraction as a pair of
+ * fp16 values (22 bits).  Small launches, other groups, D = 64 and the blocked
+ * lists take one head per thread block, fp32 throughout (each head re-reads the
+ * rows, mostly from L2).
  */
 typedef struct {
   int32_t B, H, H_kv, D;
@@ -140,7 +144,11 @@ int32_t ssa_spans_to_index(const int32_t* span_offsets, const int32_t* spans,
  * the per-split partial results (running max, running sum, fp32 accumulator)
  * of the split-KV pass (the paper's kernel runs one thread block per head and
  * request and has no such step); its contents need no initialisation and are
- * dead after the call's work has run.
+ * dead after the call's work has run.  The size has room for the fastest plan
+ * of the call; a call given less takes a slower one if that one's results fit,
+ * and refuses otherwise (SSA_ERR_WORKSPACE).  Full contexts of grouped query
+ * heads are among those: their rows are only cut by the lengths themselves in a
+ * workspace asked for with desc->max_ctx.
  */
 size_t ssa_decode_workspace_bytes(const ssa_attn_desc* desc, int32_t max_selected);
 
@@ -154,7 +162,8 @@ size_t ssa_decode_workspace_bytes(const ssa_attn_desc* desc, int32_t max_selecte
  * read.  The list is index[b*index_stride .. + counts[b]); entries need not be
  * sorted; a duplicated entry is counted twice; an entry outside
  * [0, ctx_lens[b]) is skipped (SSA_DEV_BAD_INDEX).  counts[b] == 0 gives a
- * zero output row and lse = -inf.  `max_selected` is a host-side upper bound
+ * zero output row and lse = -inf; a NaN in a selected key, or in a query, makes
+ * the row and lse of the heads it enters NaN.  `max_selected` is a host-side upper bound
  * on every counts[b] (1 <= max_selected <= index_stride); a larger count is
  * clamped to it (SSA_DEV_BAD_COUNT).
  *

@@ -78,6 +78,7 @@ struct DecodeParams {
   uint32_t k_row_bytes, v_row_bytes;   // token stride of the cache in bytes
   int32_t H, max_ctx, index_stride, max_selected, chunk, n_chunks, out_f32, early_release;
   int32_t kv_group;         // query heads per K/V head (1: multi-head attention)
+  int32_t share_rows;       // row-sharing kernel (otherwise one query head per block)
   int32_t gqa_wide;         // row-sharing kernel, one large block per SM
   int32_t even_blocks;      // row-sharing kernel over full contexts: blocks that share the rows evenly (0: fixed chunks)
   int32_t B;
@@ -551,21 +552,21 @@ namespace ssa {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-// wide: one large row-sharing block per SM; even_blocks: that many blocks with even shares of the rows (0: chunks)
-struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool wide; int even_blocks; };
+// share: row-sharing kernel; wide: one large row-sharing block per SM; even_blocks: that many blocks with even shares of
+// the rows (0: chunks)
+struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool share, wide; int even_blocks; };
 
-// Grouped query heads go to the kernel that reads a K/V row once for the whole group.
-static bool shares_rows(const ssa_attn_desc* d) {
+// Grouped query heads that the kernel which reads a K/V row once for the whole group can serve.
+static bool can_share_rows(const ssa_attn_desc* d) {
   const int group = d->H_kv > 0 ? d->H / d->H_kv : 1;
   return d->D == 128 && group >= 2 && group <= kGqaHeads;
 }
 
-static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
+static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan* pl) {
   if (!d || d->B <= 0 || d->H <= 0 || max_selected <= 0) return false;
   if (d->D != 64 && d->D != 128) return false;
   const long long out_units = (long long)d->B * d->H;                  // triples per chunk
-  const long long units = shares_rows(d) ? (long long)d->B * d->H_kv   // blocks per chunk
-                                         : out_units;
+  const long long units = share ? (long long)d->B * d->H_kv : out_units;   // blocks per chunk
   // The second pass costs about as much as two rounds of a block, so a request is split only when that buys
   // parallelism: one chunk whenever the list fits a block's staging area and either every SM gets a block or
   // the list is short anyway; otherwise 256-entry chunks, halved while the grid has under two blocks per SM.
@@ -574,14 +575,15 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
   int chunk = 256;
   if (max_selected <= kMaxChunk && (units >= sms || max_selected <= 256)) chunk = kMaxChunk;
   else while (chunk > 64 && units * ((max_selected + chunk - 1) / chunk) < want) chunk >>= 1;
+  pl->share = share;
   pl->wide = false;
-  if (shares_rows(d) && 2 * units > sms && units <= sms && max_selected <= 2048) {
+  if (share && 2 * units > sms && units <= sms && max_selected <= 2048) {
     // One unit for most SMs and a short list: the whole list is one large block's work, and the second pass
     // (about 3 us in the stream) is not needed (32 query heads over 4 K/V heads, 32 requests, 819 rows: 15.2 vs
     // 18.0 us).  With fewer units (2 K/V heads: 64) too many SMs would idle: 15.2 vs 14.4 us with four chunks.
     pl->wide = true;
     chunk = (max_selected + 63) / 64 * 64;
-  } else if (shares_rows(d)) {
+  } else if (share) {
     // The row-sharing kernel leaves G triples per chunk, its blocks stream (a ring of tiles per warp) and two of
     // them fit an SM: about one block per resident slot, i.e. as few chunks as keep the SMs busy (measured,
     // B*H_kv = 64..256, context 8192: within 3 % of the best split for groups of 4, 8 and 16 heads).  Ragged batches
@@ -603,6 +605,49 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
   return true;
 }
 
+// The plan every workspace holds: grouped heads share rows.
+static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
+  return make_plan(d, max_selected, d && can_share_rows(d), pl);
+}
+
+// Small launches over an 8-bit cache, grouped heads: a row-sharing block starts up slower (ring, Q fragments), combines G
+// heads one after the other and converts every row; with few rows per block that outweighs reading them G times (from
+// L2).  The lines below were measured over groups of 2, 4, 8, 12 and 16, 8..1600 query heads in all, lists of 40..8000
+// rows and full contexts, by the product of heads and rows (us with one head per block / row-sharing): 1 request, 32
+// heads over 2, 40 rows 2.6 / 5.0; 32 over 8: 160 rows 4.3 / 4.7, 820 rows 7.2 / 7.0; 8 requests of 32 over 4, 160 rows
+// 4.9 / 5.6, 500 rows 8.0 / 8.9, 37 such requests 20.6 / 8.8; 8 of 32 over 2, 500 rows 7.7 / 11.7.  Never where only
+// sharing saves the second pass, nor beyond one wave of blocks - except in groups of two, which then take two waves either
+// way (48 requests of 16 over 8, 40 rows 6.7 / 7.5).
+static bool one_head_blocks_pay(const ssa_attn_desc* d, int max_selected, const Plan& shared, const Plan& single) {
+  if (d->kv_dtype != SSA_FP8_E4M3 || (shared.n_chunks == 1 && single.n_chunks > 1)) return false;
+  const int group = d->H / d->H_kv;
+  const long long heads = (long long)d->B * d->H, rows = heads * max_selected, sms = sm_count();
+  if (group == 2 && single.n_chunks == 1 && heads > SSA_MIN_BLOCKS * sms) return rows <= 100000;
+  if (heads * single.n_chunks > SSA_MIN_BLOCKS * sms) return false;
+  if (single.n_chunks > 1) return rows <= (group <= 4 ? 20000 : group <= 8 ? 70000 : 130000);
+  if (group > 8) return rows <= 160000;
+  if (group <= 4) return rows <= 40000;
+  return rows <= (shared.n_chunks > 1 ? 135000 : heads <= 2 * sms ? 75000 : 48000);
+}
+
+// The plan of a call with a workspace of ws_bytes: one head per block where that pays and the workspace, which callers may
+// have sized by another bound, holds its partial results; otherwise the plan above.
+static bool choose_plan(const ssa_attn_desc* d, int max_selected, size_t ws_bytes, Plan* pl) {
+  if (!make_plan(d, max_selected, pl)) return false;
+  Plan single;
+  if (pl->share && make_plan(d, max_selected, false, &single) && single.total_bytes <= ws_bytes &&
+      one_head_blocks_pay(d, max_selected, *pl, single))
+    *pl = single;
+  return true;
+}
+
+// Workspace with which choose_plan has its choice.
+static size_t plan_bytes(const ssa_attn_desc* d, int max_selected) {
+  Plan pl, chosen;
+  if (!make_plan(d, max_selected, &pl) || !choose_plan(d, max_selected, SIZE_MAX, &chosen)) return 0;
+  return std::max(pl.total_bytes, chosen.total_bytes);
+}
+
 // Full contexts read by the row-sharing kernel: even shares over one block per resident slot, if the lengths of all
 // requests fit a block's scan and the workspace, which callers may have sized by an index list's bound, holds them.
 static size_t even_bytes(const ssa_attn_desc* d, int blocks, size_t* acc_bytes) {
@@ -612,7 +657,7 @@ static size_t even_bytes(const ssa_attn_desc* d, int blocks, size_t* acc_bytes) 
 }
 
 static int even_blocks_wanted(const ssa_attn_desc* d, const Plan& pl) {
-  if (!shares_rows(d) || pl.wide || pl.n_chunks == 1 || d->B > kEvenMaxBatch) return 0;
+  if (!pl.share || pl.wide || pl.n_chunks == 1 || d->B > kEvenMaxBatch) return 0;
   const long long units = (long long)d->B * d->H_kv, pieces = ((long long)d->max_ctx + kEvenRows - 1) / kEvenRows;
   // Only where the fixed plan has a second pass too (about 3 us), and shares are long enough to pay for the scan of the
   // lengths in front of the first rows: 1024 rows, a third of what the measured launch has.
@@ -635,7 +680,7 @@ static bool make_plan_blockmask(const ssa_attn_desc* d, int block_size, int max_
   if (d->D != 64 && d->D != 128) return false;
   if (block_size != 32 && block_size != 64 && block_size != 128 && block_size != 256) return false;
   const long long units = (long long)d->B * d->H;
-  pl->wide = false;
+  pl->share = pl->wide = false;
   pl->even_blocks = 0;
   pl->chunk = kMaskChunk / block_size;
   pl->n_chunks = (max_blocks + pl->chunk - 1) / pl->chunk;
@@ -678,9 +723,8 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
   constexpr bool kFp8 = kIsFp8<T>;
   size_t dynamic_smem = 0;
   unsigned block_threads = kThreads;
-  bool share = false;
+  const bool share = p.share_rows;
   if constexpr (D == 128) {
-    share = p.kv_group >= 2 && p.kv_group <= kGqaHeads && mode != kBlockMask;
     if (share) {
       grid.y = (unsigned)(p.H / p.kv_group);            // one block per K/V head
       const bool hi = p.kv_group > 8;
@@ -801,17 +845,18 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   }
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned16(ws)) return SSA_ERR_ALIGN;
   Plan pl;
+  const size_t list_bytes = mode == kSpans ? counts_bytes(d) : 0;
   if (mode == kBlockMask) {
     if (bl->block_size != 32 && bl->block_size != 64 && bl->block_size != 128 && bl->block_size != 256)
       return SSA_ERR_UNSUPPORTED;
     if (!make_plan_blockmask(d, bl->block_size, max_selected, &pl)) return SSA_ERR_SHAPE;
-  } else if (!make_plan(d, max_selected, &pl)) {
+  } else if (!choose_plan(d, max_selected, ws_bytes - std::min(ws_bytes, list_bytes), &pl)) {
     return SSA_ERR_SHAPE;
   }
-  if (!ws || ws_bytes < pl.total_bytes + (mode == kSpans ? counts_bytes(d) : 0)) return SSA_ERR_WORKSPACE;
+  if (!ws || ws_bytes < pl.total_bytes + list_bytes) return SSA_ERR_WORKSPACE;
   if (mode == kDense) make_even(d, ws_bytes, &pl);
 
-  if (q_host && !(mode == kIndex && !pg && !dense_paged && pl.n_chunks == 1 && !shares_rows(d) &&
+  if (q_host && !(mode == kIndex && !pg && !dense_paged && pl.n_chunks == 1 && !pl.share &&
                   d->kv_dtype != SSA_FP8_E4M3 && aligned16(q_host)))
     return SSA_ERR_UNSUPPORTED;
   DecodeParams p;
@@ -851,6 +896,7 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   p.H = d->H; p.max_ctx = d->max_ctx;
   p.index_stride = index_stride; p.max_selected = max_selected;
   p.chunk = pl.chunk; p.n_chunks = pl.n_chunks;
+  p.share_rows = pl.share ? 1 : 0;
   p.gqa_wide = pl.wide ? 1 : 0;
   p.even_blocks = pl.even_blocks;
   p.B = d->B;
@@ -895,7 +941,7 @@ int32_t decode_attn_sparse_host_queries(const ssa_attn_desc* desc, void* q, cons
 bool host_queries_pay(const ssa_attn_desc* d, int32_t max_selected) {
   Plan pl;
   if (!d || check_desc(d) != SSA_OK || !make_plan(d, max_selected, &pl)) return false;
-  return pl.n_chunks == 1 && !shares_rows(d) && d->kv_dtype != SSA_FP8_E4M3;
+  return pl.n_chunks == 1 && !pl.share && d->kv_dtype != SSA_FP8_E4M3;
 }
 
 // Every block of the span-list kernel repeats the merge of its request's spans (about a microsecond per wave
@@ -903,10 +949,10 @@ bool host_queries_pay(const ssa_attn_desc* d, int32_t max_selected) {
 // own (about 3 us exposed): one kernel up to three waves of blocks.
 bool one_kernel_step_pays(const ssa_attn_desc* d, int32_t max_selected, int32_t max_spans, size_t ws_bytes) {
   Plan pl;
-  if (max_spans <= 0 || max_spans > 32 || !d || check_desc(d) != SSA_OK || !make_plan(d, max_selected, &pl))
-    return false;
+  if (max_spans <= 0 || max_spans > 32 || !d || check_desc(d) != SSA_OK) return false;
+  if (!choose_plan(d, max_selected, ws_bytes - std::min(ws_bytes, counts_bytes(d)), &pl)) return false;
   if (ws_bytes < pl.total_bytes + counts_bytes(d)) return false;
-  const long long units = shares_rows(d) ? (long long)d->B * d->H_kv : (long long)d->B * d->H;
+  const long long units = pl.share ? (long long)d->B * d->H_kv : (long long)d->B * d->H;
   return units * pl.n_chunks <= 3ll * SSA_MIN_BLOCKS * sm_count();
 }
 
@@ -960,10 +1006,10 @@ int32_t ssa_decode_attn_sparse_noalloc(const ssa_attn_desc* desc, const void* q,
 static size_t spans_index_pitch(int32_t max_selected) { return ((size_t)max_selected + 31) / 32 * 32; }
 
 size_t ssa_decode_spans_workspace_bytes(const ssa_attn_desc* desc, int32_t max_selected, int32_t max_spans) {
-  ssa::Plan pl;
-  if (!desc || max_spans <= 0 || ssa::check_desc(desc) != SSA_OK || !ssa::make_plan(desc, max_selected, &pl))
-    return 0;
-  size_t need = pl.total_bytes + ssa::counts_bytes(desc);
+  if (!desc || max_spans <= 0 || ssa::check_desc(desc) != SSA_OK) return 0;
+  size_t need = ssa::plan_bytes(desc, max_selected);
+  if (need == 0) return 0;
+  need += ssa::counts_bytes(desc);
   if (max_spans > ssa::kDirectSpans) need += (size_t)desc->B * spans_index_pitch(max_selected) * sizeof(int32_t);
   return need;
 }
@@ -989,19 +1035,20 @@ int32_t ssa_decode_attn_spans(const ssa_attn_desc* desc, const void* q, const vo
   ssa::Plan pl;
   if (max_selected <= 0 || (index_out && max_selected > index_stride)) return SSA_ERR_CAPACITY;
   if (!ssa::make_plan(desc, max_selected, &pl)) return SSA_ERR_SHAPE;
-  if (!workspace || workspace_bytes < ssa_decode_spans_workspace_bytes(desc, max_selected, max_spans))
-    return SSA_ERR_WORKSPACE;
+  const size_t list_bytes = ssa::counts_bytes(desc) + (size_t)desc->B * spans_index_pitch(max_selected) * sizeof(int32_t);
+  if (!workspace || workspace_bytes < pl.total_bytes + list_bytes) return SSA_ERR_WORKSPACE;
   if (!ssa::aligned16(workspace)) return SSA_ERR_ALIGN;
+  const size_t partial_bytes = (workspace_bytes - list_bytes) / 256 * 256;
   char* ws = static_cast<char*>(workspace);
-  int32_t* counts = counts_out ? counts_out : reinterpret_cast<int32_t*>(ws + pl.total_bytes);
-  int32_t* index = index_out ? index_out : reinterpret_cast<int32_t*>(ws + pl.total_bytes + ssa::counts_bytes(desc));
+  int32_t* counts = counts_out ? counts_out : reinterpret_cast<int32_t*>(ws + partial_bytes);
+  int32_t* index = index_out ? index_out : reinterpret_cast<int32_t*>(ws + partial_bytes + ssa::counts_bytes(desc));
   const int32_t pitch = index_out ? index_stride : (int32_t)spans_index_pitch(max_selected);
   const int32_t cap = max_spans < SSA_MAX_SPANS_PER_SEQ ? max_spans : SSA_MAX_SPANS_PER_SEQ;
   const int32_t rc2 = ssa::spans_to_index_capped(span_offsets, spans, ctx_lens, desc->B, index, pitch, max_selected,
                                                  cap, counts, dev_status, (cudaStream_t)stream);
   if (rc2 != SSA_OK) return rc2;
   return ssa::run(desc, q, k_cache, v_cache, ctx_lens, index, pitch, counts, max_selected, out, lse, workspace,
-                  pl.total_bytes, dev_status, stream, ssa::kIndex);
+                  partial_bytes, dev_status, stream, ssa::kIndex);
 }
 
 // Several query tokens per head: (head, token) pairs become the heads of a wider descriptor over the same cache
@@ -1070,9 +1117,10 @@ int32_t ssa_decode_attn_blockmask(const ssa_attn_desc* desc, const void* q, cons
 size_t ssa_decode_workspace_bytes(const ssa_attn_desc* desc, int32_t max_selected) {
   ssa::Plan pl;
   if (!desc || ssa::check_desc(desc) != SSA_OK || !ssa::make_plan(desc, max_selected, &pl)) return 0;
-  if (max_selected < desc->max_ctx) return pl.total_bytes;
+  const size_t need = ssa::plan_bytes(desc, max_selected);
+  if (max_selected < desc->max_ctx) return need;
   size_t acc = 0;                                        // the bound of a full context: room for even shares as well
-  return std::max(pl.total_bytes, ssa::even_bytes(desc, ssa::even_blocks_wanted(desc, pl), &acc));
+  return std::max(need, ssa::even_bytes(desc, ssa::even_blocks_wanted(desc, pl), &acc));
 }
 
 int32_t ssa_decode_attn_sparse(const ssa_attn_desc* desc, const void* q, const void* k_cache,

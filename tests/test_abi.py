@@ -60,6 +60,21 @@ def test_workspace_query():
     assert ssa.decode_workspace_bytes(d, 0) == 0
 
 
+def test_small_grouped_launches_over_an_8_bit_cache_are_planned_one_head_per_block():
+    """Partial results (one row of D floats and a pair per chunk and head) show the plan: 820 rows, 32 query heads over 2
+    cache heads are 13 chunks per head, shared rows would be 4; over 8 cache heads sharing pays already; a 16-bit cache
+    always shares."""
+    def triples(H_kv, kv_dtype, sel=820):
+        d = good_desc()
+        d.B, d.H, d.H_kv, d.max_ctx, d.kv_dtype, d.out_dtype = 1, 32, H_kv, 8192, kv_dtype, ssa.F32
+        return ssa.decode_workspace_bytes(d, sel) // (4 * 128 + 8)
+
+    assert triples(2, ssa.FP8_E4M3) == 32 * 13
+    assert triples(8, ssa.FP8_E4M3) == 32 * 4
+    assert triples(2, ssa.BF16) == triples(8, ssa.BF16) == 32 * 4
+    assert triples(2, ssa.FP8_E4M3, 40) == triples(2, ssa.BF16, 40) == 32
+
+
 P = C.c_void_p(0x1000)      # never dereferenced: validation fails first
 NUL = None
 
