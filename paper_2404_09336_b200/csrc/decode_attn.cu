@@ -81,6 +81,7 @@ struct DecodeParams {
   int32_t share_rows;       // row-sharing kernel (otherwise one query head per block)
   int32_t gqa_wide;         // row-sharing kernel, one large block per SM
   int32_t even_blocks;      // row-sharing kernel over full contexts: blocks that share the rows evenly (0: fixed chunks)
+  int32_t even_factor;      // ... unless the lengths make slices of `chunk` rows the better cut (even_by_slices)
   int32_t B;
   // paged cache (page_table != nullptr): logical position t of request b is row
   // page_table[b * page_table_stride + (t >> page_shift)] << page_shift | (t & page_mask) of the pool
@@ -648,8 +649,8 @@ static size_t plan_bytes(const ssa_attn_desc* d, int max_selected) {
   return std::max(pl.total_bytes, chosen.total_bytes);
 }
 
-// Full contexts read by the row-sharing kernel: even shares over one block per resident slot, if the lengths of all
-// requests fit a block's scan and the workspace, which callers may have sized by an index list's bound, holds them.
+// Full contexts read by the row-sharing kernel: cut on the device over one block per resident slot, if the lengths of all
+// requests fit a block's scan and the workspace, which callers may have sized by an index list's bound, holds the results.
 static size_t even_bytes(const ssa_attn_desc* d, int blocks, size_t* acc_bytes) {
   const size_t triples = (size_t)2 * blocks * (d->H / d->H_kv);
   *acc_bytes = (triples * d->D * sizeof(float) + 255) / 256 * 256;
@@ -657,13 +658,20 @@ static size_t even_bytes(const ssa_attn_desc* d, int blocks, size_t* acc_bytes) 
 }
 
 static int even_blocks_wanted(const ssa_attn_desc* d, const Plan& pl) {
+  // Only where the fixed plan has a second pass too (about 3 us): one unit per SM at most, hence few requests.
   if (!pl.share || pl.wide || pl.n_chunks == 1 || d->B > kEvenMaxBatch) return 0;
   const long long units = (long long)d->B * d->H_kv, pieces = ((long long)d->max_ctx + kEvenRows - 1) / kEvenRows;
-  // Only where the fixed plan has a second pass too (about 3 us), and shares are long enough to pay for the scan of the
-  // lengths in front of the first rows: 1024 rows, a third of what the measured launch has.
-  if (units * d->max_ctx < 2ll * sm_count() * 1024) return 0;
   if (units * pieces > 0xffffffll) return 0;                         // rows and pieces stay far inside 32 bits
-  return (int)std::min<long long>(2ll * sm_count(), units * ((pieces + kEvenMinPieces - 1) / kEvenMinPieces));
+  const long long blocks = 2ll * sm_count(), share = units * d->max_ctx / blocks;
+  // Below 1024 rows per share, were all contexts as long as the cache, there is nothing to win against the scan of the
+  // lengths in front of the first rows (the lengths themselves may be shorter: even_by_slices).
+  if (share < 1024) return 0;
+  // Nine and more heads over 16-bit rows (two-warp teams) start up dearer: where two slices per unit fill the chip anyway,
+  // shares have to be longer.  16 heads, 136 units, us with fixed slices / equal shares: caches of 4096 rows, all full 52.9
+  // / 60.4, 1024..4096 rows 42.2 / 41.1, 0..4096 rows 41.9 / 47.9; of 8190 rows 91.3 / 99.0, 2047..8190 rows 77.1 / 65.7.
+  if (d->H / d->H_kv > 8 && d->kv_dtype != SSA_FP8_E4M3 && share < 2304 && pl.n_chunks == 2 && 16 * units > 7 * blocks)
+    return 0;
+  return (int)blocks;
 }
 
 static void make_even(const ssa_attn_desc* d, size_t ws_bytes, Plan* pl) {
@@ -776,7 +784,9 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   int launches = 1;
   if (share && p.even_blocks > 0) {
-    err = launch_pdl(decode_merge_even_kernel<TQ>, dim3((unsigned)p.H, (unsigned)B), dim3(D), st, p);
+    const int heads = std::min(p.kv_group, kEvenMergeHeads), splits = (p.kv_group + kEvenMergeHeads - 1) / kEvenMergeHeads;
+    err = launch_pdl(decode_merge_even_kernel<TQ>, dim3((unsigned)(p.H / p.kv_group * splits), (unsigned)B),
+                     dim3((unsigned)(D * heads)), st, p);
     if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
     ++launches;
   } else if (p.n_chunks > 1) {
@@ -899,6 +909,7 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   p.share_rows = pl.share ? 1 : 0;
   p.gqa_wide = pl.wide ? 1 : 0;
   p.even_blocks = pl.even_blocks;
+  p.even_factor = d->kv_dtype == SSA_FP8_E4M3 ? 5 : 6;
   p.B = d->B;
   p.out_f32 = d->out_dtype == SSA_F32;
   // A grid of a few waves releases the next kernel at once (its blocks wait on

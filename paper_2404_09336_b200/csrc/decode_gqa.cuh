@@ -174,18 +174,21 @@ __device__ __forceinline__ uint32_t tile_offset(int row, int chunk) {
   return (uint32_t)(row * 256 + ((chunk ^ (row & 7)) << 4));
 }
 
-// ---- even shares of ragged full contexts ----
+// ---- full contexts cut on the device ----
 // A full-context launch whose blocks each own a fixed slice of one request lasts as long as its longest slice, and the
 // host, which sizes the slices, knows only the longest context the cache can hold.  Here the device cuts the work: the
 // rows of all units (request x K/V head, in that order), in pieces of kEvenRows, form one line, block i of the launch
 // takes the i-th of equal shares of it, whatever units these belong to, and a unit that one share holds whole is
 // finished on the spot; the others leave a partial result per share for decode_merge_even_kernel.  A block has at most
-// two of those: slot 2 i for a unit that began in an earlier share, 2 i + 1 for one that begins in its own.
-// What bounded fixed slices was their last blocks: 17 requests of 1001..8190 rows, 16 query heads on each of 8 K/V
-// heads: 73.3 us with two slices per unit, 62.3 us with even shares (344 MB: 5.5 TB/s).
+// two of those: slot 2 i for a unit that began in an earlier share, 2 i + 1 for one that begins in its own.  Lengths that
+// gain nothing from that are read in the host's slices, by the same kernel (even_by_slices).
+// What bounded fixed slices was their last blocks.  Microseconds, fixed slices / as the device decides (equal shares
+// alone), caches of 8190 rows: 17 requests, 4 heads on each of 8 K/V heads: 2047..8190 rows 62.8 / 58.3, all 8190 rows
+// 85.3 / 86.5 (87.0), 511..585 rows 14.2 / 14.2; 68 requests, 16 heads on each of 2 K/V heads: 77.1 / 65.7, 91.3 / 94.8
+// (99.0), 18.1 / 20.8 (22.0).
 constexpr int kEvenRows = 64;
 constexpr int kEvenMinPieces = 4;                        // no share below 256 rows: block start-up would outweigh it
-constexpr int kEvenMaxBatch = 1024;                      // requests whose lengths a block scans in shared memory
+constexpr int kEvenMaxBatch = 256;                       // requests whose lengths a block scans in shared memory
 
 __device__ __forceinline__ int even_rows(const DecodeParams& p, int n) { return max(0, min(n, p.max_ctx)); }
 // a request without rows still has a piece: its output is written as zeros
@@ -193,20 +196,32 @@ __device__ __forceinline__ int even_pieces(int rows) { return max(1, (rows + kEv
 __device__ __forceinline__ int even_share(const DecodeParams& p, int total) {
   return max(kEvenMinPieces, (total + p.even_blocks - 1) / p.even_blocks);
 }
+// Whether the host's slices (p.chunk rows, p.n_chunks per unit, one per block) serve these lengths better: a share that
+// ends one unit and begins the next starts up and combines twice, which pays only where the longest slice is longer than
+// a share by more than that costs, and over 16-bit rows, where memory bounds the blocks that are left as well, by more
+// than a fifth.  Fitted to both cuts measured over 1184 launches: groups of 2..16, 40..148 units, caches of 3000..16000
+// rows, lengths alike, ragged and far below the cache; the better cut is missed by 0.5 % on average (16-bit), 0.3 % (8-bit).
+__device__ __forceinline__ bool even_by_slices(const DecodeParams& p, int total, int longest) {
+  return 5 * min(p.chunk / kEvenRows, longest) <= p.even_factor * even_share(p, total) + 25;
+}
 
 // Lengths of the requests and, over all before each, the pieces of one K/V head.
-struct EvenLine { int32_t rows[kEvenMaxBatch], before[kEvenMaxBatch + 1], warp_sum[32]; };
+struct EvenLine { int32_t rows[kEvenMaxBatch], before[kEvenMaxBatch + 1], warp_sum[32], warp_most[32]; };
 
+// The lengths -> line.rows, and their sum and maximum in pieces of one K/V head.  Thread t looks after requests
+// [t per, (t + 1) per); returns the pieces in front of those.
 template <int kThreads>
-__device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParams& p, uint32_t& flags) {
+__device__ __forceinline__ int sum_even_line(EvenLine& line, const DecodeParams& p, uint32_t& flags, int& total, int& longest) {
+  constexpr int kWarps = kThreads / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per = (p.B + kThreads - 1) / kThreads, first = tid * per;
-  int own = 0;
+  int own = 0, most = 0;
   for (int b = first; b < min(first + per, p.B); ++b) {
     const int n = __ldg(p.ctx_lens + b), rows = even_rows(p, n);
     if (n > p.max_ctx) flags |= SSA_DEV_BAD_COUNT;
     line.rows[b] = rows;
     own += even_pieces(rows);
+    most = max(most, even_pieces(rows));
   }
   int sum = own;
 #pragma unroll
@@ -214,14 +229,27 @@ __device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParam
     const int up = __shfl_up_sync(0xffffffffu, sum, o);
     if (lane >= o) sum += up;
   }
-  if (lane == 31) line.warp_sum[warp] = sum;
+  most = __reduce_max_sync(0xffffffffu, most);
+  if (lane == 31) { line.warp_sum[warp] = sum; line.warp_most[warp] = most; }
   __syncthreads();
   int at = sum - own;
-  for (int w = 0; w < warp; ++w) at += line.warp_sum[w];
+  total = longest = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    const int s = line.warp_sum[w];
+    if (w < warp) at += s;
+    total += s;
+    longest = max(longest, line.warp_most[w]);
+  }
+  return at;
+}
+
+template <int kThreads>
+__device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParams& p, int at) {
+  const int per = (p.B + kThreads - 1) / kThreads, first = threadIdx.x * per;
   for (int b = first; b < min(first + per, p.B); ++b) {
     line.before[b] = at;
     at += even_pieces(line.rows[b]);
-    if (b == p.B - 1) line.before[p.B] = at;
   }
   __syncthreads();
 }
@@ -269,17 +297,31 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   int kvh = blockIdx.y, b = blockIdx.z, start = chunk_id * p.chunk;
   int piece = 0, piece_end = 0;                        // kEven: what is left of this block's share
   if constexpr (kEven) {
-    scan_even_line<kThreads>(s_line, p, flags);
-    const int kv_heads = p.H / G, total = s_line.before[p.B] * kv_heads, share = even_share(p, total);
-    if ((int64_t)chunk_id * share >= total) return;
-    piece = chunk_id * share;
-    piece_end = min(total - piece, share) + piece;
-    b = 0;                                             // the last request that begins at or before the share
-    for (int step = kEvenMaxBatch / 2; step > 0; step >>= 1)
-      if (b + step < p.B && s_line.before[b + step] * kv_heads <= piece) b += step;
-    const int in_request = piece - s_line.before[b] * kv_heads, of_unit = s_line.before[b + 1] - s_line.before[b];
-    kvh = in_request / of_unit;
-    start = (in_request - kvh * of_unit) * kEvenRows;
+    const int kv_heads = p.H / G;
+    int total, longest;
+    const int at = sum_even_line<kThreads>(s_line, p, flags, total, longest);
+    total *= kv_heads;
+    if (even_by_slices(p, total, longest)) {
+      const int unit = chunk_id / p.n_chunks, slice = chunk_id - unit * p.n_chunks;
+      if (unit >= p.B * kv_heads) return;
+      b = unit / kv_heads;
+      kvh = unit - b * kv_heads;
+      start = slice * p.chunk;
+      piece_end = min(p.chunk / kEvenRows, even_pieces(s_line.rows[b]) - start / kEvenRows);
+      if (piece_end <= 0) return;
+    } else {
+      const int share = even_share(p, total);
+      if ((int64_t)chunk_id * share >= total) return;
+      piece = chunk_id * share;
+      piece_end = min(total - piece, share) + piece;
+      scan_even_line<kThreads>(s_line, p, at);
+      b = 0;                                           // the last request that begins at or before the share
+      for (int step = kEvenMaxBatch / 2; step > 0; step >>= 1)
+        if (b + step < p.B && s_line.before[b + step] * kv_heads <= piece) b += step;
+      const int in_request = piece - s_line.before[b] * kv_heads, of_unit = even_pieces(s_line.rows[b]);
+      kvh = in_request / of_unit;
+      start = (in_request - kvh * of_unit) * kEvenRows;
+    }
   }
 
   while (true) {                                       // kEven: once per unit of the share; else once
@@ -462,8 +504,9 @@ decode_partial_gqa_kernel(const DecodeParams p) {
           }
         } else {
           // rows that do not exist are zero.  (Most tiles of a short list are such tiles: rolled, launches of 40..2500 rows
-          // were 0.7 % slower on average and those of one request up to 9 %.  Two-warp teams, at their register limit, lose.)
-#pragma unroll (kHi ? 1 : kCopies)
+          // were 0.7 % slower on average and those of one request up to 9 %.  Where registers are at their limit - two-warp
+          // teams, 8-bit rows cut on the device: 3 % - unrolling loses.)
+#pragma unroll (kHi || (kFp8 && kEven) ? 1 : kCopies)
           for (int i = 0; i < kCopies; ++i) {
             const int pos = __shfl_sync(0xffffffffu, my_pos, kRowsPerCopy * i + copy_row);
             const uint64_t row = pos >= 0 ? (uint64_t)(uint32_t)pos : 0ull;
@@ -606,7 +649,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   // pieces of this unit that the share ends with or goes on behind
   int unit_pieces = 0, taken = 0;
   if constexpr (kEven) {
-    unit_pieces = s_line.before[b + 1] - s_line.before[b];
+    unit_pieces = even_pieces(s_line.rows[b]);
     taken = min(unit_pieces - start / kEvenRows, piece_end - piece);
   }
   if (!p.early_release && (!kEven || piece + taken == piece_end)) grid_launch_dependents();
@@ -666,33 +709,53 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   }
 }
 
-// Pass 2 of even shares: a unit that lies in more than one share, one query head.  What depends on the lengths alone is
-// worked out before the wait: the launch this grid waits for has itself waited for whatever wrote them.
+// Pass 2 of full contexts cut on the device: the query heads of a unit that more than one block read, kEvenMergeHeads per
+// block: one per block works the cut out twice as often, four leave fewer and larger blocks to squeeze in behind the first
+// pass (17..68 requests, groups of 4..16: 1 % of the whole call slower on average).  What depends on the lengths alone is
+// worked out before the wait: the launch this grid waits for has itself waited for whatever wrote them.  (A note of each
+// unit's blocks left by the first pass instead: 0.6 % faster for groups above eight, 1.7 % slower for the others.)
+constexpr int kEvenMergeHeads = 2;
 template <typename TQ>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128 * kEvenMergeHeads)
 decode_merge_even_kernel(const DecodeParams p) {
   constexpr int D = 128;
-  __shared__ int s_before[4], s_total[4];
-  const int h = blockIdx.x, b = blockIdx.y, d = threadIdx.x;
-  int before = 0, total = 0, own = 0;
-  for (int i = d; i < p.B; i += D) {
-    const int pieces = even_pieces(even_rows(p, __ldcg(p.ctx_lens + i)));
+  __shared__ int s_before[4 * kEvenMergeHeads], s_total[4 * kEvenMergeHeads], s_longest[4 * kEvenMergeHeads];
+  const int G = p.kv_group, kv_heads = p.H / G, splits = (G + kEvenMergeHeads - 1) / kEvenMergeHeads;
+  const int kvh = blockIdx.x / splits, b = blockIdx.y, tid = threadIdx.x, d = tid % D;
+  const int i = (blockIdx.x - kvh * splits) * kEvenMergeHeads + tid / D;     // head of the group
+  int before = 0, total = 0, longest = 0;
+  const int own = even_pieces(even_rows(p, __ldcg(p.ctx_lens + b)));
+  for (int k = tid; k < p.B; k += blockDim.x) {
+    const int pieces = even_pieces(even_rows(p, __ldcg(p.ctx_lens + k)));
     total += pieces;
-    if (i < b) before += pieces;
+    longest = max(longest, pieces);
+    if (k < b) before += pieces;
   }
-  own = even_pieces(even_rows(p, __ldcg(p.ctx_lens + b)));
   before = __reduce_add_sync(0xffffffffu, before);
   total = __reduce_add_sync(0xffffffffu, total);
-  if ((d & 31) == 0) { s_before[d >> 5] = before; s_total[d >> 5] = total; }
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  if ((tid & 31) == 0) { s_before[tid >> 5] = before; s_total[tid >> 5] = total; s_longest[tid >> 5] = longest; }
   __syncthreads();
-  const int G = p.kv_group, kv_heads = p.H / G, kvh = h / G, i = h - kvh * G;
-  before = s_before[0] + s_before[1] + s_before[2] + s_before[3];
-  total = s_total[0] + s_total[1] + s_total[2] + s_total[3];
-  const int share = even_share(p, total * kv_heads), at = before * kv_heads + kvh * own;
-  const int first = at / share, last = (at + own - 1) / share;
+  before = total = longest = 0;
+  for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+    before += s_before[w];
+    total += s_total[w];
+    longest = max(longest, s_longest[w]);
+  }
+  total *= kv_heads;
+  int first, last;
+  if (even_by_slices(p, total, longest)) {
+    first = (b * kv_heads + kvh) * p.n_chunks;
+    last = first + (own - 1) / (p.chunk / kEvenRows);
+  } else {
+    const int share = even_share(p, total), at = before * kv_heads + kvh * own;
+    first = at / share;
+    last = (at + own - 1) / share;
+  }
   grid_dependency_wait();
   grid_launch_dependents();
-  if (first == last) return;                           // the block of that share has stored it
+  if (first == last || i >= G) return;                 // (the block that read it has stored it)
+  const int h = kvh * G + i;
   float M = neg_inf(), L = 0.f, A = 0.f;
   for (int k0 = first; k0 <= last; k0 += kMergeAhead) {
     float2 ml[kMergeAhead];

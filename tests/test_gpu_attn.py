@@ -13,6 +13,10 @@ from parity import assert_parity
 pytestmark = pytest.mark.gpu
 
 
+def ssa_sms():
+    return torch.cuda.get_device_properties(DEV).multi_processor_count
+
+
 def scale_of(D):
     return 1.0 / np.sqrt(D)
 
@@ -448,15 +452,49 @@ def test_grouped_heads_chunks_longer_than_the_staging_area(B, H, Hkv, T):
     assert_parity(out_d[sample], ref_d[sample], False, "long chunks, dense")
 
 
+def full_context_plan(B, H, Hkv, T, blocks):
+    """(pieces per slice, slices per unit) of the host's plan for full contexts of grouped heads over 16-bit rows, and
+    whether the device may cut them by their lengths: the rules beside the code, restated."""
+    units = B * Hkv
+    n = max(1, min(blocks // units, -(-T // 256)))
+    chunk = (-(-T // n) + 63) // 64
+    n = -(-T // (64 * chunk))
+    share = units * T // blocks
+    return chunk, n, n > 1 and share >= 1024 and (H // Hkv <= 8 or share >= 2304 or n != 2 or 16 * units <= 7 * blocks)
+
+
+def even_cut(lens, T, H, Hkv, blocks):
+    """Slots of partial results that a full-context launch cut on the device fills: equal shares of the units' 64-row
+    pieces, or the host's slices where the lengths suit them.  A block's slot 2 i holds a unit begun in an earlier block,
+    2 i + 1 one that begins in its own."""
+    chunk, n, _ = full_context_plan(len(lens), H, Hkv, T, blocks)
+    pieces = [max(1, -(-min(max(x, 0), T) // 64)) for x in lens for _ in range(Hkv)]
+    share = max(4, -(-sum(pieces) // blocks))
+    slots, at = set(), 0
+    slices = 5 * min(chunk, max(pieces)) <= 6 * share + 25
+    for u, k in enumerate(pieces):
+        if slices:
+            parts = range(u * n, u * n + -(-k // chunk))
+        else:
+            parts = range(at // share, (at + k - 1) // share + 1)
+        if len(parts) > 1:
+            slots |= {2 * i + (i == parts[0]) for i in parts}
+        at += k
+    return slots, slices
+
+
 @pytest.mark.parametrize("B,H,Hkv,T,dtype,lens", [
     (3, 8, 2, 51000, "bf16", [50999, 0, 64]),                   # units in many shares; a request without rows, one piece
     (2, 8, 4, 40000, "f16", [37889, 65]),
     (17, 64, 8, 2300, "bf16", None),                            # several whole units per share
     (19, 64, 4, 4100, "f16", None),                             # sixteen heads: two warps per tile
-    (60, 16, 8, 700, "bf16", None), (5, 8, 2, 3000, "f16", [2999, 0, 1, 64, 65]),   # fixed slices: many units, short
+    (17, 64, 8, 2300, "bf16", [2300] * 16 + [2237]), (19, 64, 4, 4100, "f16", [4100] * 19),     # slices: like lengths ...
+    (17, 64, 8, 2300, "bf16", [100 + 9 * b for b in range(17)]), (19, 64, 4, 4100, "f16", [0] * 18 + [65]),     # ... short
+    (60, 16, 8, 700, "bf16", None), (5, 8, 2, 3000, "f16", [2999, 0, 1, 64, 65]),   # fixed slices: many units, short,
+    (37, 64, 4, 2100, "bf16", None),                            # ... sixteen heads where two slices per unit fill the chip
 ])
 def test_even_shares_of_ragged_full_contexts(B, H, Hkv, T, dtype, lens):
-    D = 128
+    D, G = 128, H // Hkv
     p = Problem(B, Hkv, T, D, dtype, seed=B + T)
     rng = np.random.default_rng(B)
     p.q_bits = random_bits(rng, (B, H, D), dtype)
@@ -465,8 +503,8 @@ def test_even_shares_of_ragged_full_contexts(B, H, Hkv, T, dtype, lens):
     ctx = lens or [int(x) for x in rng.integers(0, T + 1, size=B)]
     if not lens:
         ctx[:3], ctx[-1] = [T, 0, 1], T
-    seqs = list(range(B)) if B <= 60 else sorted({0, 1, 2, 3, B // 2, B - 2, B - 1})
-    k_rep, v_rep = (np.repeat(x[seqs], H // Hkv, axis=1) for x in (p.k_bits, p.v_bits))
+    seqs = sorted({0, 1, 2, 3, B // 2, B - 2, B - 1} & set(range(B))) if B > 20 else list(range(B))
+    k_rep, v_rep = (np.repeat(x[seqs], G, axis=1) for x in (p.k_bits, p.v_bits))
     ref, ref_lse = O.decode_attn_dense(p.q_bits[seqs], k_rep, v_rep, [ctx[b] for b in seqs], scale_of(D), dtype)
     some = np.isfinite(ref_lse)
 
@@ -485,15 +523,36 @@ def test_even_shares_of_ragged_full_contexts(B, H, Hkv, T, dtype, lens):
     out, lse, status = p.dense(over)
     assert status == (ssa.DEV_BAD_COUNT if over != ctx else 0)
     check(out, lse, "lengths above the cache")
-    # a workspace of the size that fixed chunks need (one triple per chunk and head; H / Hkv per block) is still taken
+
+    # which cut ran shows in the workspace; one sized for fixed slices alone (a bound below the full context asks for no
+    # more) is taken as well, and nothing is written behind either
     o = torch.full((B, H, D), 7.0, dtype=torch.float32, device=DEV)
     ls = torch.full((B, H), 7.0, dtype=torch.float32, device=DEV)
     desc = ssa.make_desc(p.q, p.k, p.v, o)
-    chunks = -(-T // 256)
-    ws = torch.empty(min(ssa.decode_workspace_bytes(desc, T), B * H * chunks * (4 * D + 8) + 512), dtype=torch.uint8, device=DEV)
-    ssa.decode_attn_dense(desc, p.q, p.k, p.v, torch.tensor(ctx, dtype=torch.int32, device=DEV), o, ls, ws, None)
-    torch.cuda.synchronize()
-    check(o.double().cpu().numpy(), ls.double().cpu().numpy(), "the workspace of fixed chunks")
+    d_ctx = torch.tensor(ctx, dtype=torch.int32, device=DEV)
+    full, fixed = ssa.decode_workspace_bytes(desc, T), ssa.decode_workspace_bytes(desc, T - 1)
+    blocks = 2 * ssa_sms()
+    even = full_context_plan(B, H, Hkv, T, blocks)[2]
+    assert (full > fixed) == even and full >= fixed
+
+    def call(nbytes, **kw):
+        ws = torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device=DEV)
+        o.fill_(7.0)
+        rc = ssa.decode_attn_dense(desc, p.q, p.k, p.v, d_ctx, o, ls, ws[:nbytes], None, **kw)
+        torch.cuda.synchronize()
+        assert bool((ws[nbytes:] == 0xA5).all())
+        return rc, ws[:nbytes].cpu().numpy()
+
+    for nbytes, what in ((full, "the workspace of the full context"), (fixed, "the workspace of fixed slices")):
+        _, ws = call(nbytes)
+        check(o.double().cpu().numpy(), ls.double().cpu().numpy(), what)
+        if even and nbytes == full:
+            acc = (2 * blocks * G * D * 4 + 255) // 256 * 256
+            ml = ws[acc:acc + 2 * blocks * G * 8].reshape(2 * blocks, -1)
+            slots, slices = even_cut(ctx, T, H, Hkv, blocks)
+            assert {int(i) for i in np.flatnonzero((ml != 0xA5).any(axis=1))} == slots
+            assert slices == (lens is not None and B > 10)
+    assert call(fixed - 1, check=False)[0] == ssa.ERR_WORKSPACE
 
 
 @pytest.mark.parametrize("how", ["sparse", "dense", "spans", "blockmask"])
