@@ -431,10 +431,10 @@ decode_partial_kernel(const DecodeParams p) {
 #pragma unroll
       for (int o = kLanesPerRow / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
       s[u] = checked ? d + s[u] : d;                  // -inf stays -inf
-      mt = fmaxf(mt, s[u]);
+      mt = max_or_nan(mt, s[u]);
     }
-    const float m_new = fmaxf(m, mt);
-    if (m_new > neg_inf()) {
+    const float m_new = max_or_nan(m, mt);
+    if (m_new != neg_inf()) {                           // (a NaN among the scores: m stays, the weights become NaN)
       if (m_new > m) {                                // rare after the first tiles
         const float alpha = fast_exp2(m - m_new);     // m = -inf gives 0
         l *= alpha;
@@ -450,9 +450,6 @@ decode_partial_kernel(const DecodeParams p) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) acc[i] = fma2(pw2, piece_pair<T>(vr[u], i), acc[i]);
       }
-    } else {                                            // every score so far is -inf (masked) or NaN, which has to show
-#pragma unroll
-      for (int u = 0; u < kU; ++u) l = s[u] == s[u] ? l : s[u];
     }
   }
 

@@ -120,4 +120,11 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+// The larger of two values, NaN if one of them is.
+__device__ __forceinline__ float max_or_nan(float a, float b) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+
 }  // namespace ssa
