@@ -22,18 +22,19 @@
 // which dimension is free as long as Q (for K) and the output (for V) follow,
 // so a lane takes whole 16-byte pieces of a row.
 // The rows travel global -> shared memory by asynchronous 16-byte copies
-// (cp.async, evict-first in L2) into a ring of tiles that every warp keeps for
-// itself, and the fragments come out of that ring with ldmatrix.  The bytes in
-// flight are set by the ring (three tiles of 16 rows x (K + V) = 24 KB per
-// warp, 96 KB per block, two blocks per SM), not by fragment registers, and a
-// warp works on one tile while its next two are on their way; no block
-// barrier inside the tile loop.  (An earlier version loaded the fragments
-// straight from global memory into registers, one tile in flight per warp:
-// 5-15 % slower on long lists.)
+// (cp.async, evict-first in L2) into a ring of tiles that every team of warps
+// (one warp per head tile, GqaShape) keeps for itself, and the fragments come
+// out of that ring.  The bytes in flight are set by the ring (three tiles of
+// 16 rows x (K + V), 24 KB per team; 8-bit rows with up to eight heads: twice
+// the teams with 12 KB; 96 KB per block, two blocks per SM), not by fragment
+// registers, and a team works on one tile while its next two are on their way;
+// a team waits for itself, no block barrier sits inside the tile loop.  (An
+// earlier version loaded the fragments straight from global memory into
+// registers, one tile in flight per warp: 5-15 % slower on long lists.)
 //
 // Shared-memory tiles are [16 rows][256 bytes] with the 16-byte chunk index
 // XOR-ed with (row & 7), so that the eight row addresses of an ldmatrix hit
-// eight different bank groups.
+// eight different bank groups; [16 rows][128 bytes] for 8-bit rows (below).
 // The softmax weights are the fp32 accumulators of S; they enter the second
 // contraction as a 16-bit value plus a 16-bit residual (two mma passes), so
 // the result keeps fp32-level accuracy instead of the 2^-9 of a bf16 weight.
@@ -81,7 +82,7 @@ __device__ __forceinline__ void mma_16816<__half>(float (&d)[4], uint32_t a0, ui
 }
 
 constexpr int kGqaRows = 16;            // rows per warp per iteration
-constexpr int kGqaHeads = 16;           // M of the mma: most query heads one block serves
+constexpr int kGqaHeads = 16;           // two head tiles of the mma's N = 8: most query heads one block serves
 // floats per head row of the block-level combine, dim d at d + 2 (d / 16): lanes that hold dims 16 apart (8-bit rows)
 // or one apart (16-bit rows) and heads two apart store to different banks
 constexpr int kGqaPitch = 148;
@@ -111,10 +112,11 @@ constexpr int kStagedShortList = 1024;                   // ... unless the whole
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// 16-byte asynchronous copy global -> shared, not kept in L1, evict-first in L2; src_bytes = 0 writes zeros.
+// 16-byte asynchronous copy global -> shared, not kept in L1, evict-first in L2.
 __device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, uint64_t policy) {
   asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
 }
+// The same; src_bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async_16_or_zero(uint32_t dst, const void* src, uint32_t src_bytes, uint64_t policy) {
   asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;"
                ::"r"(dst), "l"(src), "r"(src_bytes), "l"(policy)
@@ -211,7 +213,8 @@ struct EvenLine { int32_t rows[kEvenMaxBatch], before[kEvenMaxBatch + 1], warp_s
 // The lengths -> line.rows, and their sum and maximum in pieces of one K/V head.  Thread t looks after requests
 // [t per, (t + 1) per); returns the pieces in front of those.
 template <int kThreads>
-__device__ __forceinline__ int sum_even_line(EvenLine& line, const DecodeParams& p, uint32_t& flags, int& total, int& longest) {
+__device__ __forceinline__ int sum_even_line(EvenLine& line, const DecodeParams& p, uint32_t& flags, int& total,
+                                             int& longest) {
   constexpr int kWarps = kThreads / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per = (p.B + kThreads - 1) / kThreads, first = tid * per;
@@ -325,387 +328,389 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   }
 
   while (true) {                                       // kEven: once per unit of the share; else once
-  // One round trip for everything that does not depend on the list length: the first kStagedShortList list
-  // entries of the chunk (within the host's bound, so inside the caller's row) and the group's query rows.
-  constexpr int kAhead = kStagedShortList / kThreads;
-  int32_t ahead[kAhead];
-  const bool listed = kMode == kIndex && p.index != nullptr;
-  if (listed) {
-    const int32_t* row = p.index + (int64_t)b * p.index_stride + start;
-#pragma unroll
-    for (int jj = 0; jj < kAhead; ++jj) {
-      const int i = tid + jj * kThreads;
-      ahead[jj] = (i < p.chunk && start + i < p.max_selected) ? __ldg(row + i) : -1;
-    }
-  }
-  uint4 q_lo = make_uint4(0u, 0u, 0u, 0u), q_hi = make_uint4(0u, 0u, 0u, 0u);
-  {
-    const int row = tid >> 3, c0 = (tid & 7) * 2;     // 16 rows x 8 threads; further threads have no part
-    if (row < G) {
-      const TQ* src = reinterpret_cast<const TQ*>(p.q) + (int64_t)b * p.q_sb + (int64_t)(kvh * G + row) * p.q_sh + 8 * c0;
-      q_lo = ld_stream_16B(src);
-      q_hi = ld_stream_16B(src + 8);
-    }
-  }
-  int n, c;
-  if constexpr (kEven) n = c = s_line.rows[b];
-  else request_sizes(p, b, n, c, flags);
-  if constexpr (kMode == kSpans) {
-    const int first = p.span_offsets ? __ldg(p.span_offsets + b) : b * p.span_cap;
-    const int S = p.span_offsets ? __ldg(p.span_offsets + b + 1) - first : p.span_cap;
-    const int total = merge_spans_block<kThreads>(s_runs, p.spans + first, S, p.span_cap, n);
-    c = min(total, p.max_selected);
-    if (total > p.max_selected) flags |= SSA_DEV_OVERFLOW;
-    if (tid == 0) flags |= s_runs.flags;
-    if (chunk_id == 0 && kvh == 0 && tid == 0) {
-      if (p.counts_out) p.counts_out[b] = c;
-      if (p.ws_counts) p.ws_counts[b] = c;
-    }
-  }
-  if (!kEven && start >= c && chunk_id > 0) return;
-  const int most = kEven ? min(piece_end - piece, (c + kEvenRows - 1) / kEvenRows) * kEvenRows : p.chunk;
-  const int cnt = max(0, min(most, c - start));
-
-  auto stage_window = [&](int w0, int wn) {
-    if constexpr (kMode == kSpans) {
-      int32_t* out = (kvh == 0 && p.index_out) ? p.index_out + (int64_t)b * p.index_stride + start + w0 : nullptr;
-      for (int i = tid; i < wn; i += kThreads) {
-        const int v = span_position(s_runs, start + w0 + i);
-        s_idx[i] = v;
-        if (out) out[i] = v;
-      }
-      return;
-    }
-    // position -> what the tile loop uses: -1 for an entry outside the context, the pool row for a paged cache
-    auto checked = [&](int v) {
-      if (v < 0 || v >= n) {
-        flags |= SSA_DEV_BAD_INDEX;
-        return -1;
-      }
-      if (p.page_table) {
-        const int page = __ldg(p.page_table + (int64_t)b * p.page_table_stride + (v >> p.page_shift));
-        if ((unsigned)page < (unsigned)p.n_pages) return (page << p.page_shift) | (v & p.page_mask);
-        flags |= SSA_DEV_BAD_INDEX;
-        return -1;
-      }
-      return v;
-    };
-    if (listed && w0 == 0) {                             // the entries requested ahead cover any first window
+    // One round trip for everything that does not depend on the list length: the first kStagedShortList list
+    // entries of the chunk (within the host's bound, so inside the caller's row) and the group's query rows.
+    constexpr int kAhead = kStagedShortList / kThreads;
+    int32_t ahead[kAhead];
+    const bool listed = kMode == kIndex && p.index != nullptr;
+    if (listed) {
+      const int32_t* row = p.index + (int64_t)b * p.index_stride + start;
 #pragma unroll
       for (int jj = 0; jj < kAhead; ++jj) {
         const int i = tid + jj * kThreads;
-        if (i < wn) s_idx[i] = checked(ahead[jj]);
+        ahead[jj] = (i < p.chunk && start + i < p.max_selected) ? __ldg(row + i) : -1;
       }
-      return;
     }
-    const int32_t* row = listed ? p.index + (int64_t)b * p.index_stride + start + w0 : nullptr;
-    for (int i = tid; i < wn; i += kThreads)             // no list: the position itself (a paged full context)
-      s_idx[i] = checked(row ? __ldg(row + i) : start + w0 + i);
-  };
-  // a list chunk of up to kStagedShortList entries is one window (no meeting in mid-chunk); longer ones go by 512
-  const int window = kSparse ? (cnt <= kStagedShortList ? kStagedShortList : kStagedWindow) : Shape::kDenseWindow;
-  if (kSparse) stage_window(0, min(cnt, window));
-  // the group's query rows -> shared memory (rows of heads that do not exist are zero)
-  auto store_q = [&]() {
-    if (tid < kGqaHeads * 8) {
-      const int row = tid >> 3, c0 = (tid & 7) * 2;
-      *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0)) = q_lo;
-      *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0 + 1)) = q_hi;
+    uint4 q_lo = make_uint4(0u, 0u, 0u, 0u), q_hi = make_uint4(0u, 0u, 0u, 0u);
+    {
+      const int row = tid >> 3, c0 = (tid & 7) * 2;     // 16 rows x 8 threads; further threads have no part
+      if (row < G) {
+        const TQ* src = reinterpret_cast<const TQ*>(p.q) + (int64_t)b * p.q_sb + (int64_t)(kvh * G + row) * p.q_sh + 8 * c0;
+        q_lo = ld_stream_16B(src);
+        q_hi = ld_stream_16B(src + 8);
+      }
     }
-  };
-  if (kSparse) {
-    store_q();
-    __syncthreads();                                   // the first window is staged
-  }
-  uint64_t policy;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-  const char* kbase = reinterpret_cast<const char*>(
-      reinterpret_cast<const T*>(p.k) + (int64_t)b * p.k_sb + (int64_t)kvh * p.k_sh);
-  const char* vbase = reinterpret_cast<const char*>(
-      reinterpret_cast<const T*>(p.v) + (int64_t)b * p.v_sb + (int64_t)kvh * p.v_sh);
-  const uint32_t ring = smem_u32(s_ring) + team * Shape::kRingBytes;
-  // this lane's part in copying a tile: its 16 bytes of every row, and where they go in the first row it copies
-  constexpr int kRowBytes = kFp8 ? 128 : 256, kChunks = kRowBytes / 16, kRowsPerCopy = 32 / kChunks;
-  const char* kcol = kbase + (lane % kChunks) * 16;
-  const char* vcol = vbase + (lane % kChunks) * 16;
-  const int copy_row = ht * (kGqaRows / kTeam) + lane / kChunks;
-  const uint32_t copy_k = kFp8 ? tile8_offset_k(copy_row, lane % kChunks) : tile_offset(copy_row, lane % kChunks);
-  const uint32_t copy_v = kFp8 ? tile8_offset_v(copy_row, lane % kChunks) : tile_offset(copy_row, lane % kChunks);
-  // this lane's part in reading one: fragment addresses are these, XOR-ed with a multiple of 32 (or 64) bytes
-  const uint32_t read_k = kFp8 ? tile8_offset_k(g, j) : tile_offset(lane & 15, lane >> 4);
-  const uint32_t read_v = kFp8 ? tile8_offset_v(2 * j, g) : tile_offset((lane >> 4) * 8 + (lane & 7), (lane >> 3) & 1);
+    int n, c;
+    if constexpr (kEven) n = c = s_line.rows[b];
+    else request_sizes(p, b, n, c, flags);
+    if constexpr (kMode == kSpans) {
+      const int first = p.span_offsets ? __ldg(p.span_offsets + b) : b * p.span_cap;
+      const int S = p.span_offsets ? __ldg(p.span_offsets + b + 1) - first : p.span_cap;
+      const int total = merge_spans_block<kThreads>(s_runs, p.spans + first, S, p.span_cap, n);
+      c = min(total, p.max_selected);
+      if (total > p.max_selected) flags |= SSA_DEV_OVERFLOW;
+      if (tid == 0) flags |= s_runs.flags;
+      if (chunk_id == 0 && kvh == 0 && tid == 0) {
+        if (p.counts_out) p.counts_out[b] = c;
+        if (p.ws_counts) p.ws_counts[b] = c;
+      }
+    }
+    if (!kEven && start >= c && chunk_id > 0) return;
+    const int most = kEven ? min(piece_end - piece, (c + kEvenRows - 1) / kEvenRows) * kEvenRows : p.chunk;
+    const int cnt = max(0, min(most, c - start));
 
-  // Running softmax state of heads 8 ht + 2 j + {0, 1}, the same in all lanes of equal j; the sums are per lane until
-  // the end.  o[t][e]: head 8 ht + 2 j + (e & 1), dim 16 t + g + 8 (e >> 1) (8-bit rows: 16 g + 2 t + (e >> 1)).
-  float m[2] = {neg_inf(), neg_inf()}, l[2] = {0.f, 0.f}, o[8][4];
-#pragma unroll
-  for (int t = 0; t < 8; ++t) { o[t][0] = 0.f; o[t][1] = 0.f; o[t][2] = 0.f; o[t][3] = 0.f; }
-  // B fragments of Q for the eight k-steps: registers for the whole block's life.  8-bit rows: k-step ks of lane
-  // (g, j) is dims 64 (ks / 4) + 16 j + 4 (ks % 4) + 0..3 of head g, the order its K pieces come in.
-  uint32_t qb[8][2];
-  auto load_q = [&]() {
-    const uint32_t base = smem_u32(s_qtile);
-    if constexpr (kFp8) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const uint4 w = lds_16B(base + tile_offset(8 * ht + g, 8 * (c >> 1) + 2 * j + (c & 1)));
-        qb[2 * c][0] = w.x; qb[2 * c][1] = w.y;
-        qb[2 * c + 1][0] = w.z; qb[2 * c + 1][1] = w.w;
+    auto stage_window = [&](int w0, int wn) {
+      if constexpr (kMode == kSpans) {
+        int32_t* out = (kvh == 0 && p.index_out) ? p.index_out + (int64_t)b * p.index_stride + start + w0 : nullptr;
+        for (int i = tid; i < wn; i += kThreads) {
+          const int v = span_position(s_runs, start + w0 + i);
+          s_idx[i] = v;
+          if (out) out[i] = v;
+        }
+        return;
       }
-    } else {
+      // position -> what the tile loop uses: -1 for an entry outside the context, the pool row for a paged cache
+      auto checked = [&](int v) {
+        if (v < 0 || v >= n) {
+          flags |= SSA_DEV_BAD_INDEX;
+          return -1;
+        }
+        if (p.page_table) {
+          const int page = __ldg(p.page_table + (int64_t)b * p.page_table_stride + (v >> p.page_shift));
+          if ((unsigned)page < (unsigned)p.n_pages) return (page << p.page_shift) | (v & p.page_mask);
+          flags |= SSA_DEV_BAD_INDEX;
+          return -1;
+        }
+        return v;
+      };
+      if (listed && w0 == 0) {                             // the entries requested ahead cover any first window
 #pragma unroll
-      for (int ks = 0; ks < 8; ks += 2) {
-        uint32_t w[4];
-        ldmatrix_x4(w, base + tile_offset(8 * ht + (lane & 7), 2 * ks + (lane >> 3)));
-        qb[ks][0] = w[0]; qb[ks][1] = w[1];
-        qb[ks + 1][0] = w[2]; qb[ks + 1][1] = w[3];
+        for (int jj = 0; jj < kAhead; ++jj) {
+          const int i = tid + jj * kThreads;
+          if (i < wn) s_idx[i] = checked(ahead[jj]);
+        }
+        return;
       }
-    }
-  };
-  auto team_sync = [&]() {
-    __syncwarp();
-    if constexpr (kTeam > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeam * 32) : "memory");
-  };
-
-  for (int w0 = 0; w0 < cnt; w0 += window) {
-    const int wn = min(window, cnt - w0);
-    if (kSparse && w0 > 0) {
-      __syncthreads();                                 // every warp is done with the previous window
-      stage_window(w0, wn);
-      __syncthreads();
-    } else if (w0 > 0) {
-      team_sync();                                     // the ring is filled anew: no lane still reads the last tiles
-    }
-    const int first_row = team * kGqaRows;
-    const int nk = wn > first_row ? (wn - first_row + kTeams * kGqaRows - 1) / (kTeams * kGqaRows) : 0;
-    // position of row (lane & 15) of this team's k-th tile, -1 if there is none
-    auto tile_pos = [&](int k) {
-      const int r = first_row + k * (kTeams * kGqaRows) + (lane & 15);
-      return r < wn ? (kSparse ? s_idx[r] : start + w0 + r) : -1;
+      const int32_t* row = listed ? p.index + (int64_t)b * p.index_stride + start + w0 : nullptr;
+      for (int i = tid; i < wn; i += kThreads)             // no list: the position itself (a paged full context)
+        s_idx[i] = checked(row ? __ldg(row + i) : start + w0 + i);
     };
-    // Requests tile k of the window (if it exists) into the slot at `slot`; always closes a copy group.  Returns which
-    // of its sixteen rows exist.
-    auto request = [&](int k, uint32_t slot) -> uint32_t {
-      uint32_t live = 0u;
-      if (k < nk) {
-        const int my_pos = tile_pos(k);
-        live = __ballot_sync(0xffffffffu, my_pos >= 0) & 0xffffu;
-        const uint32_t dk = slot + copy_k, dv = slot + kTileBytes + copy_v;
-        // (the warps of a team copy the rows in turns; from one copy of a lane to its next, only XOR-ed bits and a constant change in the address)
-        constexpr int kCopies = kGqaRows / kRowsPerCopy / kTeam;
-        auto to_k = [&](int i) { return (kFp8 ? dk : dk ^ ((2 * i & 7) << 4)) + i * (kRowsPerCopy * kRowBytes); };
-        auto to_v = [&](int i) { return (dv ^ ((kRowsPerCopy * i & 7) << 4)) + i * (kRowsPerCopy * kRowBytes); };
-        if (live == 0xffffu) {                         // warp-uniform
+    // a list chunk of up to kStagedShortList entries is one window (no meeting in mid-chunk); longer ones go by 512
+    const int window = kSparse ? (cnt <= kStagedShortList ? kStagedShortList : kStagedWindow) : Shape::kDenseWindow;
+    if (kSparse) stage_window(0, min(cnt, window));
+    // the group's query rows -> shared memory (rows of heads that do not exist are zero)
+    auto store_q = [&]() {
+      if (tid < kGqaHeads * 8) {
+        const int row = tid >> 3, c0 = (tid & 7) * 2;
+        *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0)) = q_lo;
+        *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0 + 1)) = q_hi;
+      }
+    };
+    if (kSparse) {
+      store_q();
+      __syncthreads();                                   // the first window is staged
+    }
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    const char* kbase = reinterpret_cast<const char*>(
+        reinterpret_cast<const T*>(p.k) + (int64_t)b * p.k_sb + (int64_t)kvh * p.k_sh);
+    const char* vbase = reinterpret_cast<const char*>(
+        reinterpret_cast<const T*>(p.v) + (int64_t)b * p.v_sb + (int64_t)kvh * p.v_sh);
+    const uint32_t ring = smem_u32(s_ring) + team * Shape::kRingBytes;
+    // this lane's part in copying a tile: its 16 bytes of every row, and where they go in the first row it copies
+    constexpr int kRowBytes = kFp8 ? 128 : 256, kChunks = kRowBytes / 16, kRowsPerCopy = 32 / kChunks;
+    const char* kcol = kbase + (lane % kChunks) * 16;
+    const char* vcol = vbase + (lane % kChunks) * 16;
+    const int copy_row = ht * (kGqaRows / kTeam) + lane / kChunks;
+    const uint32_t copy_k = kFp8 ? tile8_offset_k(copy_row, lane % kChunks) : tile_offset(copy_row, lane % kChunks);
+    const uint32_t copy_v = kFp8 ? tile8_offset_v(copy_row, lane % kChunks) : tile_offset(copy_row, lane % kChunks);
+    // this lane's part in reading one: fragment addresses are these, XOR-ed with a multiple of 32 (or 64) bytes
+    const uint32_t read_k = kFp8 ? tile8_offset_k(g, j) : tile_offset(lane & 15, lane >> 4);
+    const uint32_t read_v = kFp8 ? tile8_offset_v(2 * j, g) : tile_offset((lane >> 4) * 8 + (lane & 7), (lane >> 3) & 1);
+
+    // Running softmax state of heads 8 ht + 2 j + {0, 1}, the same in all lanes of equal j; the sums are per lane until
+    // the end.  o[t][e]: head 8 ht + 2 j + (e & 1), dim 16 t + g + 8 (e >> 1) (8-bit rows: 16 g + 2 t + (e >> 1)).
+    float m[2] = {neg_inf(), neg_inf()}, l[2] = {0.f, 0.f}, o[8][4];
 #pragma unroll
-          for (int i = 0; i < kCopies; ++i) {
-            const uint32_t pos = __shfl_sync(0xffffffffu, my_pos, kRowsPerCopy * i + copy_row);
-            cp_async_16(to_k(i), kcol + (uint64_t)pos * p.k_row_bytes, policy);
-            cp_async_16(to_v(i), vcol + (uint64_t)pos * p.v_row_bytes, policy);
+    for (int t = 0; t < 8; ++t) { o[t][0] = 0.f; o[t][1] = 0.f; o[t][2] = 0.f; o[t][3] = 0.f; }
+    // B fragments of Q for the eight k-steps: registers for the whole block's life.  8-bit rows: k-step ks of lane
+    // (g, j) is dims 64 (ks / 4) + 16 j + 4 (ks % 4) + 0..3 of head g, the order its K pieces come in.
+    uint32_t qb[8][2];
+    auto load_q = [&]() {
+      const uint32_t base = smem_u32(s_qtile);
+      if constexpr (kFp8) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint4 w = lds_16B(base + tile_offset(8 * ht + g, 8 * (c >> 1) + 2 * j + (c & 1)));
+          qb[2 * c][0] = w.x; qb[2 * c][1] = w.y;
+          qb[2 * c + 1][0] = w.z; qb[2 * c + 1][1] = w.w;
+        }
+      } else {
+#pragma unroll
+        for (int ks = 0; ks < 8; ks += 2) {
+          uint32_t w[4];
+          ldmatrix_x4(w, base + tile_offset(8 * ht + (lane & 7), 2 * ks + (lane >> 3)));
+          qb[ks][0] = w[0]; qb[ks][1] = w[1];
+          qb[ks + 1][0] = w[2]; qb[ks + 1][1] = w[3];
+        }
+      }
+    };
+    auto team_sync = [&]() {
+      __syncwarp();
+      if constexpr (kTeam > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeam * 32) : "memory");
+    };
+
+    for (int w0 = 0; w0 < cnt; w0 += window) {
+      const int wn = min(window, cnt - w0);
+      if (kSparse && w0 > 0) {
+        __syncthreads();                                 // every warp is done with the previous window
+        stage_window(w0, wn);
+        __syncthreads();
+      } else if (w0 > 0) {
+        team_sync();                                     // the ring is filled anew: no lane still reads the last tiles
+      }
+      const int first_row = team * kGqaRows;
+      const int nk = wn > first_row ? (wn - first_row + kTeams * kGqaRows - 1) / (kTeams * kGqaRows) : 0;
+      // position of row (lane & 15) of this team's k-th tile, -1 if there is none
+      auto tile_pos = [&](int k) {
+        const int r = first_row + k * (kTeams * kGqaRows) + (lane & 15);
+        return r < wn ? (kSparse ? s_idx[r] : start + w0 + r) : -1;
+      };
+      // Requests tile k of the window (if it exists) into the slot at `slot`; always closes a copy group.  Returns which
+      // of its sixteen rows exist.
+      auto request = [&](int k, uint32_t slot) -> uint32_t {
+        uint32_t live = 0u;
+        if (k < nk) {
+          const int my_pos = tile_pos(k);
+          live = __ballot_sync(0xffffffffu, my_pos >= 0) & 0xffffu;
+          const uint32_t dk = slot + copy_k, dv = slot + kTileBytes + copy_v;
+          // (the warps of a team copy the rows in turns; from one copy of a lane to its next only XOR-ed bits and a
+          // constant change in the address)
+          constexpr int kCopies = kGqaRows / kRowsPerCopy / kTeam;
+          auto to_k = [&](int i) { return (kFp8 ? dk : dk ^ ((2 * i & 7) << 4)) + i * (kRowsPerCopy * kRowBytes); };
+          auto to_v = [&](int i) { return (dv ^ ((kRowsPerCopy * i & 7) << 4)) + i * (kRowsPerCopy * kRowBytes); };
+          if (live == 0xffffu) {                         // warp-uniform
+#pragma unroll
+            for (int i = 0; i < kCopies; ++i) {
+              const uint32_t pos = __shfl_sync(0xffffffffu, my_pos, kRowsPerCopy * i + copy_row);
+              cp_async_16(to_k(i), kcol + (uint64_t)pos * p.k_row_bytes, policy);
+              cp_async_16(to_v(i), vcol + (uint64_t)pos * p.v_row_bytes, policy);
+            }
+          } else {
+            // rows that do not exist are zero.  (Most tiles of a short list are such tiles: rolled, launches of 40..2500
+            // rows were 0.7 % slower on average and those of one request up to 9 %.  Where registers are at their limit -
+            // two-warp teams, 8-bit rows cut on the device: 3 % - unrolling loses.)
+#pragma unroll (kHi || (kFp8 && kEven) ? 1 : kCopies)
+            for (int i = 0; i < kCopies; ++i) {
+              const int pos = __shfl_sync(0xffffffffu, my_pos, kRowsPerCopy * i + copy_row);
+              const uint64_t row = pos >= 0 ? (uint64_t)(uint32_t)pos : 0ull;
+              cp_async_16_or_zero(to_k(i), kcol + row * p.k_row_bytes, pos >= 0 ? 16u : 0u, policy);
+              cp_async_16_or_zero(to_v(i), vcol + row * p.v_row_bytes, pos >= 0 ? 16u : 0u, policy);
+            }
+          }
+        }
+        cp_async_commit();
+        return live;
+      };
+      uint32_t lives[kStagedDepth];                      // rows of tiles k, k + 1, ... (registers: shifted by one per tile)
+#pragma unroll
+      for (int k = 0; k < kStagedDepth - 1; ++k) lives[k] = request(k, ring + k * (2 * kTileBytes));
+      if (w0 == 0) {                                     // (the query is not needed before the first tiles are requested)
+        if (!kSparse) {
+          store_q();
+          __syncthreads();
+        }
+        load_q();
+      }
+      constexpr uint32_t kRingBytes = kStagedDepth * 2 * kTileBytes;
+      uint32_t kt = ring, refill = ring + kRingBytes - 2 * kTileBytes;   // slots of tile k and of tile k + depth - 1
+      auto after = [&](uint32_t slot) { return slot + 2 * kTileBytes == ring + kRingBytes ? ring : slot + 2 * kTileBytes; };
+      for (int k = 0; k < nk; ++k, kt = after(kt), refill = after(refill)) {
+        team_sync();                                     // the slot about to be refilled has been read by every lane
+        lives[kStagedDepth - 1] = request(k + kStagedDepth - 1, refill);
+        cp_async_wait<kStagedDepth - 1>();               // tile k has landed (for this lane's copies) ...
+        team_sync();                                     // ... and for every other lane's
+        const uint32_t live = lives[0];
+#pragma unroll
+        for (int i = 0; i + 1 < kStagedDepth; ++i) lives[i] = lives[i + 1];
+        if (live == 0u) continue;                        // warp-uniform: nothing to add
+        const uint32_t ka = kt + read_k, va = kt + kTileBytes + read_v;
+
+        // S^T = K . Q^T: lane (g, j) gets rows g (s[0..1]) and g + 8 (s[2..3]) of heads 2 j and 2 j + 1
+        // (two sums of four k-steps each: half the length of the dependent chain)
+        float s[4] = {0.f, 0.f, 0.f, 0.f}, s_odd[4] = {0.f, 0.f, 0.f, 0.f};
+        if constexpr (kFp8) {
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const uint4 lo = lds_16B(ka ^ (half << 6)), hi = lds_16B((ka ^ (half << 6)) + 8 * kRowBytes);
+            const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, c[4] = {hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const uint32_t a0 = e4m3x2_to_bf162(a[i]), a1 = e4m3x2_to_bf162(c[i]);
+              const uint32_t a2 = e4m3x2_to_bf162(a[i] >> 16), a3 = e4m3x2_to_bf162(c[i] >> 16);
+              float (&sum)[4] = (i & 1) ? s_odd : s;
+              mma_16816<TQ>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
+            }
           }
         } else {
-          // rows that do not exist are zero.  (Most tiles of a short list are such tiles: rolled, launches of 40..2500 rows
-          // were 0.7 % slower on average and those of one request up to 9 %.  Where registers are at their limit - two-warp
-          // teams, 8-bit rows cut on the device: 3 % - unrolling loses.)
-#pragma unroll (kHi || (kFp8 && kEven) ? 1 : kCopies)
-          for (int i = 0; i < kCopies; ++i) {
-            const int pos = __shfl_sync(0xffffffffu, my_pos, kRowsPerCopy * i + copy_row);
-            const uint64_t row = pos >= 0 ? (uint64_t)(uint32_t)pos : 0ull;
-            cp_async_16_or_zero(to_k(i), kcol + row * p.k_row_bytes, pos >= 0 ? 16u : 0u, policy);
-            cp_async_16_or_zero(to_v(i), vcol + row * p.v_row_bytes, pos >= 0 ? 16u : 0u, policy);
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks) {
+            uint32_t a[4];
+            ldmatrix_x4(a, ka ^ (ks << 5));
+            float (&sum)[4] = (ks & 1) ? s_odd : s;
+            mma_16816<TQ>(sum, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1], sum);
           }
         }
-      }
-      cp_async_commit();
-      return live;
-    };
-    uint32_t lives[kStagedDepth];                      // rows of tiles k, k + 1, ... (registers: shifted by one per tile)
 #pragma unroll
-    for (int k = 0; k < kStagedDepth - 1; ++k) lives[k] = request(k, ring + k * (2 * kTileBytes));
-    if (w0 == 0) {                                     // (the query is not needed before the first tiles are requested)
-      if (!kSparse) {
-        store_q();
-        __syncthreads();
-      }
-      load_q();
-    }
-    constexpr uint32_t kRingBytes = kStagedDepth * 2 * kTileBytes;
-    uint32_t kt = ring, refill = ring + kRingBytes - 2 * kTileBytes;   // slots of tile k and of tile k + depth - 1
-    auto after = [&](uint32_t slot) { return slot + 2 * kTileBytes == ring + kRingBytes ? ring : slot + 2 * kTileBytes; };
-    for (int k = 0; k < nk; ++k, kt = after(kt), refill = after(refill)) {
-      team_sync();                                     // the slot about to be refilled has been read by every lane
-      lives[kStagedDepth - 1] = request(k + kStagedDepth - 1, refill);
-      cp_async_wait<kStagedDepth - 1>();               // tile k has landed (for this lane's copies) ...
-      team_sync();                                     // ... and for every other lane's
-      const uint32_t live = lives[0];
+        for (int e = 0; e < 4; ++e) s[e] = (s[e] + s_odd[e]) * p.scale_log2;
+        if (live != 0xffffu) {                           // warp-uniform; a masked row's score is -inf
+          const bool live_lo = (live >> g) & 1u, live_hi = (live >> (g + 8)) & 1u;
 #pragma unroll
-      for (int i = 0; i + 1 < kStagedDepth; ++i) lives[i] = lives[i + 1];
-      if (live == 0u) continue;                        // warp-uniform: nothing to add
-      const uint32_t ka = kt + read_k, va = kt + kTileBytes + read_v;
-
-      // S^T = K . Q^T: lane (g, j) gets rows g (s[0..1]) and g + 8 (s[2..3]) of heads 2 j and 2 j + 1
-      // (two sums of four k-steps each: half the length of the dependent chain)
-      float s[4] = {0.f, 0.f, 0.f, 0.f}, s_odd[4] = {0.f, 0.f, 0.f, 0.f};
-      if constexpr (kFp8) {
+          for (int e = 0; e < 2; ++e) {
+            s[e] = live_lo ? s[e] : neg_inf();
+            s[2 + e] = live_hi ? s[2 + e] : neg_inf();
+          }
+        }
+        if (__any_sync(0xffffffffu, fmaxf(s[0], s[2]) > m[0] || fmaxf(s[1], s[3]) > m[1])) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {                  // rare after the first tiles
+            float mt = fmaxf(s[e], s[2 + e]);
+            mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 4));
+            mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 8));
+            mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 16));
+            const float mn = fmaxf(m[e], mt);
+            if (mn > m[e]) {
+              const float alpha = fast_exp2(m[e] - mn);
+              l[e] *= alpha;
+#pragma unroll
+              for (int t = 0; t < 8; ++t) { o[t][e] *= alpha; o[t][2 + e] *= alpha; }
+              m[e] = mn;
+            }
+          }
+        }
+        // weights, split into a 16-bit value and a 16-bit residual, transposed into B fragments of P^T[16 rows, 8 heads]
+        uint32_t pa[2], pr[2];
+        // (a maximum of -inf: no finite score yet, every weight is 0)
+        const float r0 = m[0] > neg_inf() ? m[0] : 0.f, r1 = m[1] > neg_inf() ? m[1] : 0.f;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
-          const uint4 lo = lds_16B(ka ^ (half << 6)), hi = lds_16B((ka ^ (half << 6)) + 8 * kRowBytes);
-          const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, c[4] = {hi.x, hi.y, hi.z, hi.w};
+          const float w0 = fast_exp2(s[2 * half] - r0) * kUp, w1 = fast_exp2(s[2 * half + 1] - r1) * kUp;   // -inf gives 0
+          l[0] += w0;
+          l[1] += w1;
+          const uint32_t w = pack2<TP>(w0, w1);
+          const float2 back = unpack2<TP>(w);
+          pa[half] = transpose8x8(w);
+          pr[half] = transpose8x8(pack2<TP>(w0 - back.x, w1 - back.y));
+        }
+        // O^T += V^T . P^T, sixteen dims at a time
+        if constexpr (kFp8) {
+          const uint4 v0 = lds_16B(va), v1 = lds_16B(va + kRowBytes);                          // rows 2 j, 2 j + 1
+          const uint4 v2 = lds_16B(va + 8 * kRowBytes), v3 = lds_16B(va + 9 * kRowBytes);      // rows 2 j + 8, 2 j + 9
+          const uint32_t x0[4] = {v0.x, v0.y, v0.z, v0.w}, x1[4] = {v1.x, v1.y, v1.z, v1.w};
+          const uint32_t x2[4] = {v2.x, v2.y, v2.z, v2.w}, x3[4] = {v3.x, v3.y, v3.z, v3.w};
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const uint32_t a0 = e4m3x2_to_bf162(a[i]), a1 = e4m3x2_to_bf162(c[i]);
-            const uint32_t a2 = e4m3x2_to_bf162(a[i] >> 16), a3 = e4m3x2_to_bf162(c[i] >> 16);
-            float (&sum)[4] = (i & 1) ? s_odd : s;
-            mma_16816<TQ>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
+          for (int t = 0; t < 8; ++t) {
+            // bytes 2 (t & 1) and 2 (t & 1) + 1 of both rows of a pair, interleaved
+            const uint32_t sel = (t & 1) ? 0x7362u : 0x5140u;
+            const uint32_t lo = __byte_perm(x0[t >> 1], x1[t >> 1], sel), hi = __byte_perm(x2[t >> 1], x3[t >> 1], sel);
+            const uint32_t a0 = e4m3x2_to_half2(lo), a1 = e4m3x2_to_half2(lo >> 16);
+            const uint32_t a2 = e4m3x2_to_half2(hi), a3 = e4m3x2_to_half2(hi >> 16);
+            // (the tile's own sum first, rounded to nearest into the running one: the tensor cores truncate, which over
+            // a long list would cost more than the weights' split)
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_16816<TP>(sum, a0, a1, a2, a3, pr[0], pr[1], sum);
+            mma_16816<TP>(sum, a0, a1, a2, a3, pa[0], pa[1], sum);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[t][e] += sum[e];
           }
-        }
-      } else {
+        } else {
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-          uint32_t a[4];
-          ldmatrix_x4(a, ka ^ (ks << 5));
-          float (&sum)[4] = (ks & 1) ? s_odd : s;
-          mma_16816<TQ>(sum, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1], sum);
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) s[e] = (s[e] + s_odd[e]) * p.scale_log2;
-      if (live != 0xffffu) {                           // warp-uniform; a masked row's score is -inf
-        const bool live_lo = (live >> g) & 1u, live_hi = (live >> (g + 8)) & 1u;
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          s[e] = live_lo ? s[e] : neg_inf();
-          s[2 + e] = live_hi ? s[2 + e] : neg_inf();
-        }
-      }
-      if (__any_sync(0xffffffffu, fmaxf(s[0], s[2]) > m[0] || fmaxf(s[1], s[3]) > m[1])) {
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {                  // rare after the first tiles
-          float mt = fmaxf(s[e], s[2 + e]);
-          mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 4));
-          mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 8));
-          mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, 16));
-          const float mn = fmaxf(m[e], mt);
-          if (mn > m[e]) {
-            const float alpha = fast_exp2(m[e] - mn);
-            l[e] *= alpha;
-#pragma unroll
-            for (int t = 0; t < 8; ++t) { o[t][e] *= alpha; o[t][2 + e] *= alpha; }
-            m[e] = mn;
+          for (int t = 0; t < 8; ++t) {
+            uint32_t a[4];                               // dims 16t..+7, 16t+8..+15 of rows 0-7; the same of rows 8-15
+            ldmatrix_x4_trans(a, va ^ (t << 5));
+            mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pa[0], pa[1], o[t]);
+            mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pr[0], pr[1], o[t]);
           }
         }
       }
-      // weights, split into a 16-bit value and a 16-bit residual, transposed into B fragments of P^T[16 rows, 8 heads]
-      uint32_t pa[2], pr[2];
-      // (a maximum of -inf: no finite score yet, every weight is 0)
-      const float r0 = m[0] > neg_inf() ? m[0] : 0.f, r1 = m[1] > neg_inf() ? m[1] : 0.f;
+      cp_async_wait<0>();                                // only empty groups can be pending here
+    }
+    if (p.dev_status && kvh == 0) {
+      const uint32_t f = ((kEven || tid == 0) && chunk_id == 0) ? flags : (flags & SSA_DEV_BAD_INDEX);
+      if (f) atomicOr(p.dev_status, f);
+    }
+
+    // pieces of this unit that the share ends with or goes on behind
+    int unit_pieces = 0, taken = 0;
+    if constexpr (kEven) {
+      unit_pieces = even_pieces(s_line.rows[b]);
+      taken = min(unit_pieces - start / kEvenRows, piece_end - piece);
+    }
+    if (!p.early_release && (!kEven || piece + taken == piece_end)) grid_launch_dependents();
+
+    // per-warp triples -> shared memory (the ring is free now)
+    __syncthreads();
+    // [kTeams][kLiveHeads][kGqaPitch]
+    float (*s_acc)[kLiveHeads][kGqaPitch] = reinterpret_cast<float (*)[kLiveHeads][kGqaPitch]>(s_ring);
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const float w0 = fast_exp2(s[2 * half] - r0) * kUp, w1 = fast_exp2(s[2 * half + 1] - r1) * kUp;   // -inf gives 0
-        l[0] += w0;
-        l[1] += w1;
-        const uint32_t w = pack2<TP>(w0, w1);
-        const float2 back = unpack2<TP>(w);
-        pa[half] = transpose8x8(w);
-        pr[half] = transpose8x8(pack2<TP>(w0 - back.x, w1 - back.y));
-      }
-      // O^T += V^T . P^T, sixteen dims at a time
-      if constexpr (kFp8) {
-        const uint4 v0 = lds_16B(va), v1 = lds_16B(va + kRowBytes);                          // rows 2 j, 2 j + 1
-        const uint4 v2 = lds_16B(va + 8 * kRowBytes), v3 = lds_16B(va + 9 * kRowBytes);      // rows 2 j + 8, 2 j + 9
-        const uint32_t x0[4] = {v0.x, v0.y, v0.z, v0.w}, x1[4] = {v1.x, v1.y, v1.z, v1.w};
-        const uint32_t x2[4] = {v2.x, v2.y, v2.z, v2.w}, x3[4] = {v3.x, v3.y, v3.z, v3.w};
+    for (int e = 0; e < 2; ++e) {
+      const int head = 8 * ht + 2 * j + e;
+      float sum = l[e];
+      sum += __shfl_xor_sync(0xffffffffu, sum, 4);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+      if (g == 0) { s_m[team][head] = m[e]; s_l[team][head] = sum / kUp; }
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          // bytes 2 (t & 1) and 2 (t & 1) + 1 of both rows of a pair, interleaved
-          const uint32_t sel = (t & 1) ? 0x7362u : 0x5140u;
-          const uint32_t lo = __byte_perm(x0[t >> 1], x1[t >> 1], sel), hi = __byte_perm(x2[t >> 1], x3[t >> 1], sel);
-          const uint32_t a0 = e4m3x2_to_half2(lo), a1 = e4m3x2_to_half2(lo >> 16);
-          const uint32_t a2 = e4m3x2_to_half2(hi), a3 = e4m3x2_to_half2(hi >> 16);
-          // (the tile's own sum first, rounded to nearest into the running one: the tensor cores truncate, which over
-          // a long list would cost more than the weights' split)
-          float sum[4] = {0.f, 0.f, 0.f, 0.f};
-          mma_16816<TP>(sum, a0, a1, a2, a3, pr[0], pr[1], sum);
-          mma_16816<TP>(sum, a0, a1, a2, a3, pa[0], pa[1], sum);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) o[t][e] += sum[e];
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          uint32_t a[4];                               // dims 16t..+7, 16t+8..+15 of rows 0-7; the same of rows 8-15
-          ldmatrix_x4_trans(a, va ^ (t << 5));
-          mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pa[0], pa[1], o[t]);
-          mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pr[0], pr[1], o[t]);
+      for (int t = 0; t < 8; ++t) {
+        if constexpr (kFp8) {
+          *reinterpret_cast<float2*>(&s_acc[team][head][gqa_column(16 * g + 2 * t)]) =
+              make_float2(o[t][e] / kUp, o[t][2 + e] / kUp);
+        } else {
+          s_acc[team][head][gqa_column(16 * t + g)] = o[t][e];
+          s_acc[team][head][gqa_column(16 * t + g + 8)] = o[t][2 + e];
         }
       }
     }
-    cp_async_wait<0>();                                // only empty groups can be pending here
-  }
-  if (p.dev_status && kvh == 0) {
-    const uint32_t f = ((kEven || tid == 0) && chunk_id == 0) ? flags : (flags & SSA_DEV_BAD_INDEX);
-    if (f) atomicOr(p.dev_status, f);
-  }
-
-  // pieces of this unit that the share ends with or goes on behind
-  int unit_pieces = 0, taken = 0;
-  if constexpr (kEven) {
-    unit_pieces = even_pieces(s_line.rows[b]);
-    taken = min(unit_pieces - start / kEvenRows, piece_end - piece);
-  }
-  if (!p.early_release && (!kEven || piece + taken == piece_end)) grid_launch_dependents();
-
-  // per-warp triples -> shared memory (the ring is free now)
-  __syncthreads();
-  // [kTeams][kLiveHeads][kGqaPitch]
-  float (*s_acc)[kLiveHeads][kGqaPitch] = reinterpret_cast<float (*)[kLiveHeads][kGqaPitch]>(s_ring);
+    __syncthreads();
+    // 128 threads finish a head: thread d its dim d
+    const int d = tid % D;
+    for (int i = tid / D; i < G; i += kThreads / D) {
+      const int h = kvh * G + i;
+      float M = neg_inf();
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const int head = 8 * ht + 2 * j + e;
-    float sum = l[e];
-    sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-    sum += __shfl_xor_sync(0xffffffffu, sum, 8);
-    sum += __shfl_xor_sync(0xffffffffu, sum, 16);
-    if (g == 0) { s_m[team][head] = m[e]; s_l[team][head] = sum / kUp; }
+      for (int w = 0; w < kTeams; ++w) M = fmaxf(M, s_m[w][i]);
+      float L = 0.f, A = 0.f;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      if constexpr (kFp8) {
-        *reinterpret_cast<float2*>(&s_acc[team][head][gqa_column(16 * g + 2 * t)]) = make_float2(o[t][e] / kUp, o[t][2 + e] / kUp);
+      for (int w = 0; w < kTeams; ++w) {
+        const float wgt = (s_m[w][i] > neg_inf()) ? fast_exp2(s_m[w][i] - M) : 0.f;
+        L = fmaf(s_l[w][i], wgt, L);
+        A = fmaf(s_acc[w][i][gqa_column(d)], wgt, A);
+      }
+      if (kEven ? taken == unit_pieces : p.n_chunks == 1) {
+        store_row_value<TQ>(p, b, h, d, M, L, A);
       } else {
-        s_acc[team][head][gqa_column(16 * t + g)] = o[t][e];
-        s_acc[team][head][gqa_column(16 * t + g + 8)] = o[t][2 + e];
+        const int64_t slot = kEven ? (int64_t)(2 * chunk_id + (start == 0 ? 1 : 0)) * G + i
+                                   : ((int64_t)b * p.H + h) * p.n_chunks + chunk_id;
+        p.ws_acc[slot * D + d] = A;
+        if (d == 0) p.ws_ml[slot] = make_float2(M, L);
       }
     }
-  }
-  __syncthreads();
-  // 128 threads finish a head: thread d its dim d
-  const int d = tid % D;
-  for (int i = tid / D; i < G; i += kThreads / D) {
-    const int h = kvh * G + i;
-    float M = neg_inf();
-#pragma unroll
-    for (int w = 0; w < kTeams; ++w) M = fmaxf(M, s_m[w][i]);
-    float L = 0.f, A = 0.f;
-#pragma unroll
-    for (int w = 0; w < kTeams; ++w) {
-      const float wgt = (s_m[w][i] > neg_inf()) ? fast_exp2(s_m[w][i] - M) : 0.f;
-      L = fmaf(s_l[w][i], wgt, L);
-      A = fmaf(s_acc[w][i][gqa_column(d)], wgt, A);
-    }
-    if (kEven ? taken == unit_pieces : p.n_chunks == 1) {
-      store_row_value<TQ>(p, b, h, d, M, L, A);
-    } else {
-      const int64_t slot = kEven ? (int64_t)(2 * chunk_id + (start == 0 ? 1 : 0)) * G + i
-                                 : ((int64_t)b * p.H + h) * p.n_chunks + chunk_id;
-      p.ws_acc[slot * D + d] = A;
-      if (d == 0) p.ws_ml[slot] = make_float2(M, L);
-    }
-  }
-  if constexpr (!kEven) break;
-  piece += taken;
-  if (piece >= piece_end) break;
-  start = 0;                                           // the next unit of the line
-  if (++kvh == p.H / G) { kvh = 0; ++b; }
-  __syncthreads();                                     // ring, query rows and triples are free again
+    if constexpr (!kEven) break;
+    piece += taken;
+    if (piece >= piece_end) break;
+    start = 0;                                           // the next unit of the line
+    if (++kvh == p.H / G) { kvh = 0; ++b; }
+    __syncthreads();                                     // ring, query rows and triples are free again
   }
 }
 
