@@ -291,6 +291,18 @@ def test_small_grouped_launches_one_head_per_block_or_in_the_workspace_of_shared
         assert bool((ws[nbytes:] == 0xA5).all())
         assert float(np.linalg.norm(out.double().cpu().numpy() - ref)) <= 1e-6 * float(np.linalg.norm(ref))
         np.testing.assert_allclose(lse.double().cpu().numpy(), ref_lse, rtol=2e-6, atol=2e-6)
+    # the same rows as one-token spans, more than a block merges on chip: lists and partial results share the workspace
+    spans = np.concatenate([np.stack([r, r + 1], 1)[:c] for r, c in zip(index, counts)]).astype(np.int32)
+    offs = torch.from_numpy(np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)).to(DEV)
+    nbytes = ssa.decode_spans_workspace_bytes(desc, sel, sel)
+    ws2 = torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device=DEV)
+    listed = out.clone()
+    ssa.decode_attn_sparse(desc, p.q, p.k, p.v, d_ctx, torch.from_numpy(index).to(DEV), d_cnt, sel, listed, lse,
+                           torch.empty(ssa.decode_workspace_bytes(desc, sel), dtype=torch.uint8, device=DEV), None)
+    ssa.decode_attn_spans(desc, p.q, p.k, p.v, d_ctx, offs, torch.from_numpy(spans).to(DEV), sel, sel, out, lse, None, None,
+                          ws2[:nbytes], None)
+    torch.cuda.synchronize()
+    assert torch.equal(out, listed) and bool((ws2[nbytes:] == 0xA5).all())
     before = ssa.launch_count()                                 # one head per block needs no second pass up to 512 rows
     ssa.decode_attn_sparse(desc, p.q, p.k, p.v, d_ctx, torch.from_numpy(index).to(DEV), d_cnt, sel, out, lse, ws, None)
     assert ssa.launch_count() - before == (2 if sel > 512 else 1)
