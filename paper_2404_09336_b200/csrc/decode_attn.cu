@@ -79,6 +79,8 @@ struct DecodeParams {
   int32_t H, max_ctx, index_stride, max_selected, chunk, n_chunks, out_f32, early_release;
   int32_t kv_group;         // query heads per K/V head (1: multi-head attention)
   int32_t share_rows;       // row-sharing kernel (otherwise one query head per block)
+  int32_t head_splits;      // row-sharing kernel: blocks that share the heads of a group, heads_per_block each
+  int32_t heads_per_block;
   int32_t gqa_wide;         // row-sharing kernel, one large block per SM
   int32_t even_blocks;      // row-sharing kernel over full contexts: blocks that share the rows evenly (0: fixed chunks)
   int32_t even_factor;      // ... unless the lengths make slices of `chunk` rows the better cut (even_by_slices)
@@ -554,17 +556,23 @@ namespace ssa {
 // the rows (0: chunks)
 struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool share, wide; int even_blocks; };
 
-// Grouped query heads that the kernel which reads a K/V row once for the whole group can serve.
+// Grouped query heads that the kernel which reads a K/V row once for many heads can serve.
 static bool can_share_rows(const ssa_attn_desc* d) {
   const int group = d->H_kv > 0 ? d->H / d->H_kv : 1;
-  return d->D == 128 && group >= 2 && group <= kGqaHeads;
+  return d->D == 128 && group >= 2;
 }
+
+// A row-sharing block serves up to kGqaHeads heads; larger groups (several query tokens per head) take several blocks per
+// chunk, side by side in the grid, so that all but the first find the rows in L2.  One head per block instead reads every
+// row from L2 once per head (us, one head per block / row-sharing, 32 heads on each of 4 K/V heads, bf16): 3 requests of
+// 12897 rows 201 / 33, 8 of 2000 listed rows 63.7 / 18.4, 24 of 40 15.5 / 6.7.  (Small launches: one_head_blocks_pay.)
+static int head_splits(const ssa_attn_desc* d) { return (d->H / d->H_kv + kGqaHeads - 1) / kGqaHeads; }
 
 static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan* pl) {
   if (!d || d->B <= 0 || d->H <= 0 || max_selected <= 0) return false;
   if (d->D != 64 && d->D != 128) return false;
   const long long out_units = (long long)d->B * d->H;                  // triples per chunk
-  const long long units = share ? (long long)d->B * d->H_kv : out_units;   // blocks per chunk
+  const long long units = share ? (long long)d->B * d->H_kv * head_splits(d) : out_units;   // blocks per chunk
   // The second pass costs about as much as two rounds of a block, so a request is split only when that buys
   // parallelism: one chunk whenever the list fits a block's staging area and either every SM gets a block or
   // the list is short anyway; otherwise 256-entry chunks, halved while the grid has under two blocks per SM.
@@ -615,9 +623,11 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
 // heads over 2, 40 rows 2.6 / 5.0; 32 over 8: 160 rows 4.3 / 4.7, 820 rows 7.2 / 7.0; 8 requests of 32 over 4, 160 rows
 // 4.9 / 5.6, 500 rows 8.0 / 8.9, 37 such requests 20.6 / 8.8; 8 of 32 over 2, 500 rows 7.7 / 11.7.  Never where only
 // sharing saves the second pass, nor beyond one wave of blocks - except in groups of two, which then take two waves either
-// way (48 requests of 16 over 8, 40 rows 6.7 / 7.5).
+// way (48 requests of 16 over 8, 40 rows 6.7 / 7.5).  Groups of more than kGqaHeads over 16-bit rows follow the lines of the
+// large groups: 1 request, 20 heads over 1, 3000 rows 8.3 / 9.4, 12000 rows 17.9 / 12.0; 2 requests of 96 over 4, 300 rows
+// 6.9 / 8.0, 2000 rows 20.6 / 11.7.
 static bool one_head_blocks_pay(const ssa_attn_desc* d, int max_selected, const Plan& shared, const Plan& single) {
-  if (d->kv_dtype != SSA_FP8_E4M3 || (shared.n_chunks == 1 && single.n_chunks > 1)) return false;
+  if ((d->kv_dtype != SSA_FP8_E4M3 && head_splits(d) == 1) || (shared.n_chunks == 1 && single.n_chunks > 1)) return false;
   const int group = d->H / d->H_kv;
   const long long heads = (long long)d->B * d->H, rows = heads * max_selected, sms = sm_count();
   if (group == 2 && single.n_chunks == 1 && heads > SSA_MIN_BLOCKS * sms) return rows <= 100000;
@@ -629,12 +639,13 @@ static bool one_head_blocks_pay(const ssa_attn_desc* d, int max_selected, const 
 }
 
 // The plan of a call with a workspace of ws_bytes: one head per block where that pays and the workspace, which callers may
-// have sized by another bound, holds its partial results; otherwise the plan above.
+// have sized by another bound, holds its partial results; otherwise the plan above.  (Above kGqaHeads heads per K/V head
+// that is also the plan for a workspace too small for the one above.)
 static bool choose_plan(const ssa_attn_desc* d, int max_selected, size_t ws_bytes, Plan* pl) {
   if (!make_plan(d, max_selected, pl)) return false;
   Plan single;
   if (pl->share && make_plan(d, max_selected, false, &single) && single.total_bytes <= ws_bytes &&
-      one_head_blocks_pay(d, max_selected, *pl, single))
+      (one_head_blocks_pay(d, max_selected, *pl, single) || (head_splits(d) > 1 && pl->total_bytes > ws_bytes)))
     *pl = single;
   return true;
 }
@@ -659,7 +670,7 @@ static int even_blocks_wanted(const ssa_attn_desc* d, const Plan& pl) {
   if (!pl.share || pl.wide || pl.n_chunks == 1 || d->B > kEvenMaxBatch) return 0;
   const long long units = (long long)d->B * d->H_kv, pieces = ((long long)d->max_ctx + kEvenRows - 1) / kEvenRows;
   if (units * pieces > 0xffffffll) return 0;                         // rows and pieces stay far inside 32 bits
-  const long long blocks = 2ll * sm_count(), share = units * d->max_ctx / blocks;
+  const long long blocks = 2ll * sm_count() / head_splits(d), share = units * d->max_ctx / blocks;
   // Below 1024 rows per share, were all contexts as long as the cache, there is nothing to win against the scan of the
   // lengths in front of the first rows (the lengths themselves may be shorter: even_by_slices).
   if (share < 1024) return 0;
@@ -731,28 +742,32 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
   const bool share = p.share_rows;
   if constexpr (D == 128) {
     if (share) {
-      grid.y = (unsigned)(p.H / p.kv_group);            // one block per K/V head
-      const bool hi = p.kv_group > 8;
-      auto pick = [&](auto hi_tag, auto wide_tag) {
-        constexpr bool kHi = decltype(hi_tag)::value, kWide = decltype(wide_tag)::value;
+      grid.x *= (unsigned)p.head_splits;
+      grid.y = (unsigned)(p.H / p.kv_group);            // one block, or head_splits, per K/V head
+      auto pick = [&](auto hi_tag, auto wide_tag, auto fine_tag) {
+        constexpr bool kHi = decltype(hi_tag)::value, kWide = decltype(wide_tag)::value, kFine = decltype(fine_tag)::value;
         using Shape = GqaShape<T, kHi, kWide>;
         block_threads = Shape::kWarps * 32;
         dynamic_smem = Shape::kSmemBytes;
         if constexpr (!kWide) {
           if (p.even_blocks > 0) {
-            kernel = decode_partial_gqa_kernel<T, kDense, kHi, false, true>;
+            kernel = decode_partial_gqa_kernel<T, kDense, kHi, false, true, kFine>;
             return;
           }
         }
-        kernel = mode == kIndex   ? decode_partial_gqa_kernel<T, kIndex, kHi, kWide>
-                 : mode == kSpans ? decode_partial_gqa_kernel<T, kSpans, kHi, kWide>
-                                  : decode_partial_gqa_kernel<T, kDense, kHi, kWide>;
+        kernel = mode == kIndex   ? decode_partial_gqa_kernel<T, kIndex, kHi, kWide, false, kFine>
+                 : mode == kSpans ? decode_partial_gqa_kernel<T, kSpans, kHi, kWide, false, kFine>
+                                  : decode_partial_gqa_kernel<T, kDense, kHi, kWide, false, kFine>;
       };
-      if (hi) p.gqa_wide ? pick(std::true_type{}, std::true_type{}) : pick(std::true_type{}, std::false_type{});
-      else p.gqa_wide ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{});
+      constexpr std::true_type yes;
+      constexpr std::false_type no;
+      constexpr std::bool_constant<!kFp8> fine;         // (8-bit rows have it anyway)
+      if (p.head_splits > 1) p.gqa_wide ? pick(yes, yes, fine) : pick(yes, no, fine);   // nine heads a block at least
+      else if (p.heads_per_block > 8) p.gqa_wide ? pick(yes, yes, no) : pick(yes, no, no);
+      else p.gqa_wide ? pick(no, yes, no) : pick(no, no, no);
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_smem) != cudaSuccess)
         return SSA_ERR_CUDA;
-      if (p.even_blocks > 0) grid = dim3((unsigned)p.even_blocks);
+      if (p.even_blocks > 0) grid = dim3((unsigned)(p.even_blocks * p.head_splits));
     }
   }
   if (!share) {
@@ -904,6 +919,8 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   p.index_stride = index_stride; p.max_selected = max_selected;
   p.chunk = pl.chunk; p.n_chunks = pl.n_chunks;
   p.share_rows = pl.share ? 1 : 0;
+  p.head_splits = pl.share ? head_splits(d) : 1;
+  p.heads_per_block = (p.kv_group + p.head_splits - 1) / p.head_splits;
   p.gqa_wide = pl.wide ? 1 : 0;
   p.even_blocks = pl.even_blocks;
   p.even_factor = d->kv_dtype == SSA_FP8_E4M3 ? 5 : 6;
@@ -960,7 +977,7 @@ bool one_kernel_step_pays(const ssa_attn_desc* d, int32_t max_selected, int32_t 
   if (max_spans <= 0 || max_spans > 32 || !d || check_desc(d) != SSA_OK) return false;
   if (!choose_plan(d, max_selected, ws_bytes - std::min(ws_bytes, counts_bytes(d)), &pl)) return false;
   if (ws_bytes < pl.total_bytes + counts_bytes(d)) return false;
-  const long long units = pl.share ? (long long)d->B * d->H_kv : (long long)d->B * d->H;
+  const long long units = pl.share ? (long long)d->B * d->H_kv * head_splits(d) : (long long)d->B * d->H;
   return units * pl.n_chunks <= 3ll * SSA_MIN_BLOCKS * sm_count();
 }
 
@@ -1000,7 +1017,9 @@ int32_t ssa_decode_attn_sparse_noalloc(const ssa_attn_desc* desc, const void* q,
   if (!ssa::aligned16(q) || !ssa::aligned16(k_cache) || !ssa::aligned16(v_cache) || !ssa::aligned16(out))
     return SSA_ERR_ALIGN;
   ssa::Plan pl;
-  if (!ssa::make_plan(desc, max_selected, &pl)) return SSA_ERR_SHAPE;
+  // (groups above kGqaHeads are taken as far as their one-head-per-block plan fits, like multi-head calls)
+  const bool share = ssa::can_share_rows(desc) && ssa::head_splits(desc) == 1;
+  if (!ssa::make_plan(desc, max_selected, share, &pl)) return SSA_ERR_SHAPE;
   if (pl.total_bytes > SSA_STATIC_SCRATCH_BYTES) return SSA_ERR_WORKSPACE;   // beyond the built-in scratch
   void* scratch = ssa::static_scratch_address();
   if (!scratch) return SSA_ERR_CUDA;

@@ -1,7 +1,8 @@
-// Pass 1 of the decode attention for grouped query heads (G = H / H_kv query
-// heads share one K/V head, 2 <= G <= 16, D = 128; also several query tokens
-// per head, which are served the same way): one block per (chunk, K/V head,
-// request) reads every selected row ONCE and serves all G heads.
+// Pass 1 of the decode attention for grouped query heads (G = H / H_kv >= 2
+// query heads share one K/V head, D = 128; also several query tokens per
+// head, which are served the same way): one block per (chunk, K/V head,
+// request) reads every selected row ONCE and serves all G heads; above
+// sixteen heads (kGqaHeads) several blocks share them.
 //
 // With G heads per row the work per byte is G times that of multi-head
 // attention and the packed-FMA path of decode_partial_kernel runs out of issue
@@ -259,8 +260,11 @@ __device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParam
 
 // kWide serves launches with at most one unit (request x K/V head) per SM and short lists: a whole list is then one
 // block's work, no second pass.
-// kEven (full contexts): even shares, see above; the grid is (even_blocks, 1, 1).
-template <typename T, int kMode, bool kHi, bool kWide, bool kEven = false>
+// kEven (full contexts): even shares, see above; the grid is (even_blocks * head_splits, 1, 1).
+// kFine (16-bit rows): weights to 22 bits and more, and tiles summed on their own, as 8-bit rows have it anyway: error of a
+// row against 64 bits 1.5e-7 instead of 1.4..3.2e-6.  For groups of more than kGqaHeads heads, which one head per block
+// served with 1.4..2.5e-7.  It costs them a tenth to a fifth (24 requests, 128 heads over 4, 2000 rows: 40.8 -> 48.6 us).
+template <typename T, int kMode, bool kHi, bool kWide, bool kEven = false, bool kFine = false>
 __global__ void __launch_bounds__(GqaShape<T, kHi, kWide>::kWarps * 32, kWide ? 1 : 2)
 decode_partial_gqa_kernel(const DecodeParams p) {
   using Shape = GqaShape<T, kHi, kWide>;
@@ -271,7 +275,8 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   constexpr bool kFp8 = kIsFp8<T>;
   using TQ = typename Storage<T>::Query;                // type of the query rows and of a stored output
   using TP = typename std::conditional<kFp8, __half, T>::type;   // type of the weights in the second contraction
-  constexpr float kUp = kFp8 ? 8192.f : 1.f;            // weights (and all they enter) are scaled by this in the loop
+  constexpr bool kHalfWeights = std::is_same<TP, __half>::value;
+  constexpr float kUp = kFp8 || (kFine && kHalfWeights) ? 8192.f : 1.f;   // weights (and all they enter) are scaled by this in the loop
   constexpr int kTileBytes = kGqaRows * (kFp8 ? 128 : 256);      // one tensor's tile
   constexpr int kStagedDepth = Shape::kRingBytes / (2 * kTileBytes);
   constexpr int kLiveHeads = 8 * kTeam;
@@ -288,11 +293,16 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   __shared__ typename std::conditional<kMode == kSpans, SpanRuns, int>::type s_runs;
   __shared__ typename std::conditional<kEven, EvenLine, int>::type s_line;
 
-  const int chunk_id = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, j = lane & 3;
-  const int team = warp / kTeam, ht = warp % kTeam;     // ht: the eight heads of the group that are this warp's
+  const int team = warp / kTeam, ht = warp % kTeam;     // ht: the eight heads of the block's that are this warp's
   const int G = p.kv_group;
+  int chunk_id = blockIdx.x, part = 0;                 // the block serves the part-th heads_per_block heads of the group
+  if (p.head_splits > 1) {
+    chunk_id = blockIdx.x / p.head_splits;
+    part = blockIdx.x - chunk_id * p.head_splits;
+  }
+  const int h0 = part * p.heads_per_block, heads = min(p.heads_per_block, G - h0);
 
   grid_dependency_wait();
   if (p.early_release) grid_launch_dependents();
@@ -344,8 +354,9 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     uint4 q_lo = make_uint4(0u, 0u, 0u, 0u), q_hi = make_uint4(0u, 0u, 0u, 0u);
     {
       const int row = tid >> 3, c0 = (tid & 7) * 2;     // 16 rows x 8 threads; further threads have no part
-      if (row < G) {
-        const TQ* src = reinterpret_cast<const TQ*>(p.q) + (int64_t)b * p.q_sb + (int64_t)(kvh * G + row) * p.q_sh + 8 * c0;
+      if (row < heads) {
+        const TQ* src =
+            reinterpret_cast<const TQ*>(p.q) + (int64_t)b * p.q_sb + (int64_t)(kvh * G + h0 + row) * p.q_sh + 8 * c0;
         q_lo = ld_stream_16B(src);
         q_hi = ld_stream_16B(src + 8);
       }
@@ -360,7 +371,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       c = min(total, p.max_selected);
       if (total > p.max_selected) flags |= SSA_DEV_OVERFLOW;
       if (tid == 0) flags |= s_runs.flags;
-      if (chunk_id == 0 && kvh == 0 && tid == 0) {
+      if (chunk_id == 0 && kvh == 0 && part == 0 && tid == 0) {
         if (p.counts_out) p.counts_out[b] = c;
         if (p.ws_counts) p.ws_counts[b] = c;
       }
@@ -371,7 +382,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
 
     auto stage_window = [&](int w0, int wn) {
       if constexpr (kMode == kSpans) {
-        int32_t* out = (kvh == 0 && p.index_out) ? p.index_out + (int64_t)b * p.index_stride + start + w0 : nullptr;
+        int32_t* out = (kvh == 0 && part == 0 && p.index_out) ? p.index_out + (int64_t)b * p.index_stride + start + w0 : nullptr;
         for (int i = tid; i < wn; i += kThreads) {
           const int v = span_position(s_runs, start + w0 + i);
           s_idx[i] = v;
@@ -599,7 +610,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
           }
         }
         // weights, split into a 16-bit value and a 16-bit residual, transposed into B fragments of P^T[16 rows, 8 heads]
-        uint32_t pa[2], pr[2];
+        uint32_t pa[2], pr[2], pl[2];                    // pl: what is left of a bf16 weight behind two bf16 terms (kFine)
         // (a maximum of -inf: no finite score yet, every weight is 0)
         const float r0 = m[0] > neg_inf() ? m[0] : 0.f, r1 = m[1] > neg_inf() ? m[1] : 0.f;
 #pragma unroll
@@ -610,7 +621,12 @@ decode_partial_gqa_kernel(const DecodeParams p) {
           const uint32_t w = pack2<TP>(w0, w1);
           const float2 back = unpack2<TP>(w);
           pa[half] = transpose8x8(w);
-          pr[half] = transpose8x8(pack2<TP>(w0 - back.x, w1 - back.y));
+          const uint32_t rest = pack2<TP>(w0 - back.x, w1 - back.y);
+          pr[half] = transpose8x8(rest);
+          if constexpr (kFine && !kHalfWeights) {
+            const float2 mid = unpack2<TP>(rest);
+            pl[half] = transpose8x8(pack2<TP>((w0 - back.x) - mid.x, (w1 - back.y) - mid.y));
+          }
         }
         // O^T += V^T . P^T, sixteen dims at a time
         if constexpr (kFp8) {
@@ -638,14 +654,23 @@ decode_partial_gqa_kernel(const DecodeParams p) {
           for (int t = 0; t < 8; ++t) {
             uint32_t a[4];                               // dims 16t..+7, 16t+8..+15 of rows 0-7; the same of rows 8-15
             ldmatrix_x4_trans(a, va ^ (t << 5));
-            mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pa[0], pa[1], o[t]);
-            mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pr[0], pr[1], o[t]);
+            if constexpr (kFine) {
+              float sum[4] = {0.f, 0.f, 0.f, 0.f};
+              if constexpr (!kHalfWeights) mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pl[0], pl[1], sum);
+              mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pr[0], pr[1], sum);
+              mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pa[0], pa[1], sum);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) o[t][e] += sum[e];
+            } else {
+              mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pa[0], pa[1], o[t]);
+              mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pr[0], pr[1], o[t]);
+            }
           }
         }
       }
       cp_async_wait<0>();                                // only empty groups can be pending here
     }
-    if (p.dev_status && kvh == 0) {
+    if (p.dev_status && kvh == 0 && part == 0) {
       const uint32_t f = ((kEven || tid == 0) && chunk_id == 0) ? flags : (flags & SSA_DEV_BAD_INDEX);
       if (f) atomicOr(p.dev_status, f);
     }
@@ -676,16 +701,16 @@ decode_partial_gqa_kernel(const DecodeParams p) {
           *reinterpret_cast<float2*>(&s_acc[team][head][gqa_column(16 * g + 2 * t)]) =
               make_float2(o[t][e] / kUp, o[t][2 + e] / kUp);
         } else {
-          s_acc[team][head][gqa_column(16 * t + g)] = o[t][e];
-          s_acc[team][head][gqa_column(16 * t + g + 8)] = o[t][2 + e];
+          s_acc[team][head][gqa_column(16 * t + g)] = o[t][e] / kUp;
+          s_acc[team][head][gqa_column(16 * t + g + 8)] = o[t][2 + e] / kUp;
         }
       }
     }
     __syncthreads();
     // 128 threads finish a head: thread d its dim d
     const int d = tid % D;
-    for (int i = tid / D; i < G; i += kThreads / D) {
-      const int h = kvh * G + i;
+    for (int i = tid / D; i < heads; i += kThreads / D) {
+      const int h = kvh * G + h0 + i;
       float M = neg_inf();
 #pragma unroll
       for (int w = 0; w < kTeams; ++w) M = fmaxf(M, s_m[w][i]);
@@ -699,7 +724,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       if (kEven ? taken == unit_pieces : p.n_chunks == 1) {
         store_row_value<TQ>(p, b, h, d, M, L, A);
       } else {
-        const int64_t slot = kEven ? (int64_t)(2 * chunk_id + (start == 0 ? 1 : 0)) * G + i
+        const int64_t slot = kEven ? (int64_t)(2 * chunk_id + (start == 0 ? 1 : 0)) * G + h0 + i
                                    : ((int64_t)b * p.H + h) * p.n_chunks + chunk_id;
         p.ws_acc[slot * D + d] = A;
         if (d == 0) p.ws_ml[slot] = make_float2(M, L);
