@@ -1,4 +1,4 @@
-"""Compile libssa.so (sm_100a) in-tree with nvcc.
+"""Compile libssa.so (sm_100a) in-tree with nvcc, and the Python calls into it (_ssa_call.so) with gcc.
 
     python -m paper_2404_09336_b200.build [-o OUT] [-DNAME=VALUE ...]
 """
@@ -9,6 +9,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -16,6 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libssa.so")
 PROBE_SRC = os.path.join(HERE, "probe", "gather_probe.cu")
 PROBE_LIB = os.path.join(HERE, "libssa_probe.so")
+BINDING_SRC = os.path.join(HERE, "binding", "ssa_call.c")
+BINDING = os.path.join(HERE, "_ssa_call.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -67,9 +70,28 @@ def build_probe(force: bool = False) -> str:
     return PROBE_LIB
 
 
+def build_binding(force: bool = False) -> str:
+    """The extension module that hands the arguments of Python calls to libssa."""
+    header = os.path.join(ROOT, "include", "ssa.h")
+    if not force and not _stale(BINDING, [BINDING_SRC, header]):
+        return BINDING
+    gcc = shutil.which("gcc") or shutil.which("cc")
+    if gcc is None:
+        raise RuntimeError("gcc not found: _ssa_call.so cannot be built")
+    tmp = BINDING + f".tmp{os.getpid()}"
+    cmd = [gcc, "-shared", "-fPIC", "-O2", "-Wall", "-I", sysconfig.get_paths()["include"], "-I", os.path.dirname(header),
+           "-o", tmp, BINDING_SRC]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("gcc failed:\n" + res.stdout + res.stderr)
+    os.replace(tmp, BINDING)
+    return BINDING
+
+
 if __name__ == "__main__":
     args = sys.argv[1:]
     out = args[args.index("-o") + 1] if "-o" in args else LIB
     build_library(force=True, defines=[a for a in args if a.startswith("-D")], out=out, verbose=True)
     if "-o" not in args:
+        build_binding(force=True)
         build_probe(force=True)

@@ -1,9 +1,10 @@
-"""ctypes binding of libssa (include/ssa.h): argument marshalling only.
+"""Binding of libssa (include/ssa.h): argument marshalling only.
 
 Every function takes torch CUDA tensors (used purely as device memory) and
 hands their addresses, sizes and strides to the C entry point of the same
-name.  Nothing is computed here, and there is no fallback: if the shared
-library cannot be loaded the import fails.
+name; the calls of a decode step do so in binding/ssa_call.c, the rest through
+ctypes.  Nothing is computed here, and there is no fallback: if the shared
+library or the binding cannot be loaded the import fails.
 """
 from __future__ import annotations
 
@@ -130,6 +131,14 @@ def _load():
 
 lib = _load()
 LIBRARY_PATH = lib._name
+_build.build_binding()              # no-op when the in-tree binding is current
+from . import _ssa_call as _call    # noqa: E402
+_call.bind({name: C.cast(getattr(lib, name), C.c_void_p).value
+            for name in ("ssa_spans_to_index", "ssa_decode_attn_sparse", "ssa_decode_attn_spans",
+                         "ssa_decode_attn_sparse_multiq", "ssa_decode_attn_dense_multiq", "ssa_spans_to_blockmask",
+                         "ssa_decode_attn_blockmask", "ssa_decode_attn_sparse_paged", "ssa_decode_attn_dense_paged",
+                         "ssa_refs_to_index", "ssa_refs_to_spans", "ssa_decode_step", "ssa_decode_attn_sparse_noalloc",
+                         "ssa_decode_attn_dense")})
 
 
 def status_string(code: int) -> str:
@@ -144,14 +153,17 @@ def launch_count() -> int:
     return int(lib.ssa_launch_count())
 
 
-def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+# torch.cuda.current_stream() makes a Stream object per call (1 us); its address alone is a tenth of that
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None and _device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device())
         stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _row_stride(index):
@@ -188,9 +200,7 @@ def make_desc(q, k_cache, v_cache, out, max_ctx=None, scale: float = 0.0) -> Att
 
 def spans_to_index(span_offsets, spans, ctx_lens, index, counts, dev_status=None, stream=None, check=True):
     """ssa_spans_to_index: index[B, index_stride] and counts[B] are written."""
-    rc = lib.ssa_spans_to_index(_ptr(span_offsets), _ptr(spans), _ptr(ctx_lens), int(ctx_lens.numel()),
-                                _ptr(index), _row_stride(index), _ptr(counts), _ptr(dev_status),
-                                _stream(stream))
+    rc = _call.spans_to_index(span_offsets, spans, ctx_lens, index, counts, dev_status, _stream(stream))
     return _check("ssa_spans_to_index", rc, check)
 
 
@@ -201,11 +211,8 @@ def decode_workspace_bytes(desc: AttnDesc, max_selected: int) -> int:
 def decode_attn_sparse(desc, q, k_cache, v_cache, ctx_lens, index, counts, max_selected, out, lse=None,
                        workspace=None, dev_status=None, stream=None, check=True):
     """ssa_decode_attn_sparse: out (and lse) are written."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_sparse(C.byref(desc), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens),
-                                    _ptr(index), _row_stride(index) if index is not None else 0,
-                                    _ptr(counts), int(max_selected), _ptr(out), _ptr(lse), _ptr(workspace),
-                                    ws_bytes, _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_sparse(desc, q, k_cache, v_cache, ctx_lens, index, counts, max_selected, out, lse,
+                                  workspace, dev_status, _stream(stream))
     return _check("ssa_decode_attn_sparse", rc, check)
 
 
@@ -219,11 +226,8 @@ def decode_spans_workspace_bytes(desc: AttnDesc, max_selected: int, max_spans: i
 def decode_attn_spans(desc, q, k_cache, v_cache, ctx_lens, span_offsets, spans, max_spans, max_selected, out, lse=None,
                       index_out=None, counts_out=None, workspace=None, dev_status=None, stream=None, check=True):
     """ssa_decode_attn_spans: span lists -> attention output in one call; index_out / counts_out optional."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_spans(C.byref(desc), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens),
-                                   _ptr(span_offsets), _ptr(spans), int(max_spans), int(max_selected), _ptr(out),
-                                   _ptr(lse), _ptr(index_out), _row_stride(index_out) if index_out is not None else 0,
-                                   _ptr(counts_out), _ptr(workspace), ws_bytes, _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_spans(desc, q, k_cache, v_cache, ctx_lens, span_offsets, spans, max_spans, max_selected, out,
+                                 lse, index_out, counts_out, workspace, dev_status, _stream(stream))
     return _check("ssa_decode_attn_spans", rc, check)
 
 
@@ -241,22 +245,16 @@ def decode_multiq_workspace_bytes(desc: AttnDesc, n_q: int, max_selected: int) -
 def decode_attn_sparse_multiq(desc, n_q, q_stride_t, o_stride_t, q, k_cache, v_cache, ctx_lens, index, counts,
                               max_selected, out, lse=None, workspace=None, dev_status=None, stream=None, check=True):
     """ssa_decode_attn_sparse_multiq: n_q query rows per head over one selected set; out / lse are written."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_sparse_multiq(C.byref(desc), int(n_q), int(q_stride_t), int(o_stride_t), _ptr(q),
-                                           _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens), _ptr(index),
-                                           _row_stride(index) if index is not None else 0, _ptr(counts),
-                                           int(max_selected), _ptr(out), _ptr(lse), _ptr(workspace), ws_bytes,
-                                           _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_sparse_multiq(desc, n_q, q_stride_t, o_stride_t, q, k_cache, v_cache, ctx_lens, index, counts,
+                                         max_selected, out, lse, workspace, dev_status, _stream(stream))
     return _check("ssa_decode_attn_sparse_multiq", rc, check)
 
 
 def decode_attn_dense_multiq(desc, n_q, q_stride_t, o_stride_t, q, k_cache, v_cache, ctx_lens, out, lse=None,
                              workspace=None, dev_status=None, stream=None, check=True):
     """ssa_decode_attn_dense_multiq: n_q query rows per head over the full context."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_dense_multiq(C.byref(desc), int(n_q), int(q_stride_t), int(o_stride_t), _ptr(q),
-                                          _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens), _ptr(out), _ptr(lse),
-                                          _ptr(workspace), ws_bytes, _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_dense_multiq(desc, n_q, q_stride_t, o_stride_t, q, k_cache, v_cache, ctx_lens, out, lse,
+                                        workspace, dev_status, _stream(stream))
     return _check("ssa_decode_attn_dense_multiq", rc, check)
 
 
@@ -264,9 +262,8 @@ def spans_to_blockmask(span_offsets, spans, ctx_lens, block_size, block_idx, blo
                        dev_status=None, stream=None, check=True):
     """ssa_spans_to_blockmask: block_idx[B, stride], block_mask[B, stride, block_size/32] and
     block_counts[B] are written."""
-    rc = lib.ssa_spans_to_blockmask(_ptr(span_offsets), _ptr(spans), _ptr(ctx_lens), int(ctx_lens.numel()),
-                                    int(block_size), _ptr(block_idx), _ptr(block_mask), _row_stride(block_idx),
-                                    _ptr(block_counts), _ptr(dev_status), _stream(stream))
+    rc = _call.spans_to_blockmask(span_offsets, spans, ctx_lens, block_size, block_idx, block_mask, block_counts,
+                                  dev_status, _stream(stream))
     return _check("ssa_spans_to_blockmask", rc, check)
 
 
@@ -277,12 +274,8 @@ def decode_blockmask_workspace_bytes(desc: AttnDesc, block_size: int, max_blocks
 def decode_attn_blockmask(desc, q, k_cache, v_cache, ctx_lens, block_idx, block_mask, block_counts, block_size,
                           max_blocks, out, lse=None, workspace=None, dev_status=None, stream=None, check=True):
     """ssa_decode_attn_blockmask: out (and lse) are written."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_blockmask(C.byref(desc), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens),
-                                       _ptr(block_idx), _ptr(block_mask),
-                                       _row_stride(block_idx) if block_idx is not None else 0, _ptr(block_counts),
-                                       int(block_size), int(max_blocks), _ptr(out), _ptr(lse), _ptr(workspace),
-                                       ws_bytes, _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_blockmask(desc, q, k_cache, v_cache, ctx_lens, block_idx, block_mask, block_counts,
+                                     block_size, max_blocks, out, lse, workspace, dev_status, _stream(stream))
     return _check("ssa_decode_attn_blockmask", rc, check)
 
 
@@ -318,52 +311,32 @@ def make_paging(page_table, page_size: int, n_pages: int) -> Paging:
 def decode_attn_sparse_paged(desc, q, k_pool, v_pool, paging, ctx_lens, index, counts, max_selected, out, lse=None,
                              workspace=None, dev_status=None, stream=None, check=True):
     """ssa_decode_attn_sparse_paged: as decode_attn_sparse over a paged cache."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_sparse_paged(C.byref(desc), _ptr(q), _ptr(k_pool), _ptr(v_pool),
-                                          C.byref(paging) if paging is not None else None, _ptr(ctx_lens),
-                                          _ptr(index), _row_stride(index) if index is not None else 0, _ptr(counts),
-                                          int(max_selected), _ptr(out), _ptr(lse), _ptr(workspace), ws_bytes,
-                                          _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_sparse_paged(desc, q, k_pool, v_pool, paging, ctx_lens, index, counts, max_selected, out, lse,
+                                        workspace, dev_status, _stream(stream))
     return _check("ssa_decode_attn_sparse_paged", rc, check)
 
 
 def decode_attn_dense_paged(desc, q, k_pool, v_pool, paging, ctx_lens, out, lse=None, workspace=None,
                             dev_status=None, stream=None, check=True):
     """ssa_decode_attn_dense_paged: full-context attention over a paged cache."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_dense_paged(C.byref(desc), _ptr(q), _ptr(k_pool), _ptr(v_pool),
-                                         C.byref(paging) if paging is not None else None, _ptr(ctx_lens), _ptr(out),
-                                         _ptr(lse), _ptr(workspace), ws_bytes, _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_dense_paged(desc, q, k_pool, v_pool, paging, ctx_lens, out, lse, workspace, dev_status,
+                                       _stream(stream))
     return _check("ssa_decode_attn_dense_paged", rc, check)
-
-
-def _anchor_tables(line_offsets, lines, anchor_offsets, anchor_line, ref_offsets, refs, prefix_len, line_start,
-                   ctx_lens) -> AnchorTables:
-    t = AnchorTables()
-    for name, ten in (("line_offsets", line_offsets), ("lines", lines), ("anchor_offsets", anchor_offsets),
-                      ("anchor_line", anchor_line), ("ref_offsets", ref_offsets), ("refs", refs),
-                      ("prefix_len", prefix_len), ("line_start", line_start), ("ctx_lens", ctx_lens)):
-        setattr(t, name, None if ten is None else ten.data_ptr())
-    return t
 
 
 def refs_to_index(line_offsets, lines, anchor_offsets, anchor_line, ref_offsets, refs, prefix_len, line_start,
                   ctx_lens, index, counts, dev_status=None, stream=None, check=True):
     """ssa_refs_to_index: references -> index[B, index_stride] and counts[B] in one launch."""
-    t = _anchor_tables(line_offsets, lines, anchor_offsets, anchor_line, ref_offsets, refs, prefix_len, line_start,
-                       ctx_lens)
-    rc = lib.ssa_refs_to_index(C.byref(t), int(ctx_lens.numel()), _ptr(index), _row_stride(index), _ptr(counts),
-                               _ptr(dev_status), _stream(stream))
+    rc = _call.refs_to_index(line_offsets, lines, anchor_offsets, anchor_line, ref_offsets, refs, prefix_len, line_start,
+                             ctx_lens, index, counts, dev_status, _stream(stream))
     return _check("ssa_refs_to_index", rc, check)
 
 
 def refs_to_spans(line_offsets, lines, anchor_offsets, anchor_line, ref_offsets, refs, prefix_len, line_start,
                   ctx_lens, span_offsets_out, spans_out, dev_status=None, stream=None, check=True):
     """ssa_refs_to_spans: spans_out[B, span_stride, 2] and span_offsets_out[B+1] are written."""
-    t = _anchor_tables(line_offsets, lines, anchor_offsets, anchor_line, ref_offsets, refs, prefix_len, line_start,
-                       ctx_lens)
-    rc = lib.ssa_refs_to_spans(C.byref(t), int(ctx_lens.numel()), _ptr(span_offsets_out), _ptr(spans_out),
-                               int(spans_out.shape[1]), _ptr(dev_status), _stream(stream))
+    rc = _call.refs_to_spans(line_offsets, lines, anchor_offsets, anchor_line, ref_offsets, refs, prefix_len, line_start,
+                             ctx_lens, span_offsets_out, spans_out, spans_out.shape[1], dev_status, _stream(stream))
     return _check("ssa_refs_to_spans", rc, check)
 
 
@@ -392,7 +365,7 @@ def make_step(span_offsets, spans, ctx_lens, index, counts, q, k_cache, v_cache,
 
 def decode_step(desc: AttnDesc, step: Step, stream=None, check=True):
     """ssa_decode_step: [copy in] -> span lists to index lists and attention (one kernel or two) -> [copy out]."""
-    return _check("ssa_decode_step", lib.ssa_decode_step(C.byref(desc), C.byref(step), _stream(stream)), check)
+    return _check("ssa_decode_step", _call.decode_step(desc, step, _stream(stream)), check)
 
 
 STATIC_SCRATCH_BYTES = 8 << 20
@@ -403,20 +376,15 @@ def decode_attn_sparse_noalloc(desc, q, k_cache, v_cache, ctx_lens, index, count
     """ssa_decode_attn_sparse_noalloc: as decode_attn_sparse, with the scratch
     memory taken from the library's built-in array instead of a workspace
     tensor (for callers that must not allocate; see include/ssa.h)."""
-    rc = lib.ssa_decode_attn_sparse_noalloc(C.byref(desc), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens),
-                                            _ptr(index), _row_stride(index) if index is not None else 0,
-                                            _ptr(counts), int(max_selected), _ptr(out), _ptr(lse),
-                                            _ptr(dev_status), _stream(stream))
+    rc = _call.decode_attn_sparse_noalloc(desc, q, k_cache, v_cache, ctx_lens, index, counts, max_selected, out, lse,
+                                          dev_status, _stream(stream))
     return _check("ssa_decode_attn_sparse_noalloc", rc, check)
 
 
 def decode_attn_dense(desc, q, k_cache, v_cache, ctx_lens, out, lse=None, workspace=None, dev_status=None,
                       stream=None, check=True):
     """ssa_decode_attn_dense: out (and lse) are written."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = lib.ssa_decode_attn_dense(C.byref(desc), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens),
-                                   _ptr(out), _ptr(lse), _ptr(workspace), ws_bytes, _ptr(dev_status),
-                                   _stream(stream))
+    rc = _call.decode_attn_dense(desc, q, k_cache, v_cache, ctx_lens, out, lse, workspace, dev_status, _stream(stream))
     return _check("ssa_decode_attn_dense", rc, check)
 
 
