@@ -43,11 +43,10 @@ namespace ssa {
 #define SSA_MIN_BLOCKS 4
 #endif
 
-constexpr int kWarps = SSA_WARPS;      // warps per block in pass 1
-constexpr int kThreads = kWarps * 32;
-constexpr int kU = SSA_U;              // 32-byte loads in flight per lane, per tensor
+constexpr int kSmallBlock = SSA_WARPS; // warps per block in pass 1, where blocks are many; see block_warps for larger ones
+constexpr int kWarpSlots = SSA_WARPS * SSA_MIN_BLOCKS;   // warps of an SM
 constexpr int kMaxChunk = 512;         // index entries staged per block
-constexpr int kIdxPerThread = kMaxChunk / kThreads;
+constexpr int kMaxWideChunk = 1024;    // ... of more than kSmallBlock warps
 constexpr int kMaskChunk = 512;        // positions a block expands from bitmasks
 enum { kDense = 0, kIndex = 1, kBlockMask = 2, kSpans = 3 };
 
@@ -78,6 +77,7 @@ struct DecodeParams {
   uint32_t k_row_bytes, v_row_bytes;   // token stride of the cache in bytes
   int32_t H, max_ctx, index_stride, max_selected, chunk, n_chunks, out_f32, early_release;
   int32_t kv_group;         // query heads per K/V head (1: multi-head attention)
+  int32_t warps;            // warps of a one-head block
   int32_t share_rows;       // row-sharing kernel (otherwise one query head per block)
   int32_t head_splits;      // row-sharing kernel: blocks that share the heads of a group, heads_per_block each
   int32_t heads_per_block;
@@ -161,30 +161,58 @@ __device__ __forceinline__ void zero_piece(Piece& r) {
   for (int i = 0; i < 8; ++i) r.w[i] = 0u;
 }
 
+// Over the lanes of a warp that hold the same dims (lane groups of kLanesPerRow): largest value, sum.
+template <int kLanesPerRow>
+__device__ __forceinline__ float lane_groups_max(float v) {
+#pragma unroll
+  for (int o = kLanesPerRow; o < 32; o <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+template <int kLanesPerRow>
+__device__ __forceinline__ float lane_groups_sum(float v) {
+#pragma unroll
+  for (int o = kLanesPerRow; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// Lanes kBit apart hold 2 N pairs of the same dims: the sums of the first N to the lane without that bit, of the last to the other.
+template <int kBit, int N>
+__device__ __forceinline__ void halve_between(float2 (&out)[N], const float2 (&in)[2 * N], int lane) {
+  const bool upper = lane & kBit;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float2 keep = upper ? in[i + N] : in[i], give = upper ? in[i] : in[i + N];
+    out[i].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, kBit);
+    out[i].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, kBit);
+  }
+}
+
 // kPaged (index lists only): positions are translated through the page table while they are staged, and a
 // missing list stands for 0, 1, 2, ...; kept out of the unpaged instantiations so that they stay as they are.
 // kHostQ (index lists, one chunk per request): the query rows are still in page-locked host memory.  Each block
 // asks for its row (D/8 threads, 16 bytes each) before anything else, so that the trip across the bus overlaps
 // the block's start-up, shares it through shared memory and writes the device copy the caller expects at q.
-template <typename T, int D, int kMode, bool kAligned32, bool kPaged = false, bool kHostQ = false>
-__global__ void __launch_bounds__(kThreads, SSA_MIN_BLOCKS)
+// kWarps: see block_warps.
+template <typename T, int D, int kMode, bool kAligned32, bool kPaged = false, bool kHostQ = false, int kWarps = kSmallBlock>
+__global__ void __launch_bounds__(kWarps * 32, kWarpSlots / kWarps)
 decode_partial_kernel(const DecodeParams p) {
+  constexpr int kThreads = kWarps * 32, kStage = kWarps > kSmallBlock ? kMaxWideChunk : kMaxChunk;
+  constexpr int kIdxPerThread = kStage / kThreads;
+  constexpr bool kWide = kWarps > kSmallBlock;
   static_assert(!kPaged || kMode == kIndex, "a paged cache is read through staged positions");
   static_assert(!kHostQ || (kMode == kIndex && !kPaged), "host-resident queries: plain index lists only");
   using TQ = typename Storage<T>::Query;              // type of the query rows and of a stored output
   constexpr bool kFp8 = kIsFp8<T>;
-  constexpr int kU = kFp8 ? 2 * SSA_U : SSA_U;        // 8-bit pieces are half as large: twice as many in flight
+  constexpr int kU = kFp8 ? 2 * SSA_U : SSA_U;        // pieces in flight per lane and tensor; 8-bit ones are half as large
   constexpr bool kSparse = kMode != kDense;           // positions come from shared memory
   constexpr int kLanesPerRow = D / 16;                // 32-byte pieces per row
   constexpr int kRowsPerLoad = 32 / kLanesPerRow;     // rows one warp-wide load covers
   constexpr int kTileRows = kRowsPerLoad * kU;        // rows per warp per iteration
-  constexpr int kGroups = kWarps * kRowsPerLoad;      // independent softmax streams
+  constexpr int kGroups = kWide ? kWarps : kWarps * kRowsPerLoad;   // triples the block combines
   static_assert(kThreads >= D, "the epilogue uses one thread per output element");
-  static_assert(kMaxChunk == kIdxPerThread * kThreads && (32 * kIdxPerThread) % kTileRows == 0,
-                "a warp stages whole tiles");
-  static_assert(kMaskChunk / 32 <= 32, "a lane per word of the bitmasks");
+  static_assert(kStage == kIdxPerThread * kThreads && (32 * kIdxPerThread) % kTileRows == 0, "a warp stages whole tiles");
+  static_assert(kMaskChunk / 32 <= 32 && kMaskChunk / 32 >= kWarps, "a lane per word of the bitmasks");
 
-  __shared__ int32_t s_idx[kSparse ? kMaxChunk : 1];
+  __shared__ int32_t s_idx[kSparse ? kStage : 1];
   __shared__ __align__(16) float s_acc[kGroups][D];
   __shared__ float s_m[kGroups], s_l[kGroups];
   __shared__ typename std::conditional<kMode == kSpans, SpanRuns, int>::type s_runs;
@@ -474,12 +502,33 @@ decode_partial_kernel(const DecodeParams p) {
   if (!p.early_release) grid_launch_dependents();
 
   // combine the lane groups of the block
-  const int g = warp * kRowsPerLoad + sub;
+  if constexpr (kWide) {
+    // first those of a warp, each lane ending up with its share of the warp's sum
+    const float top = lane_groups_max<kLanesPerRow>(m);
+    const float w = (m > neg_inf()) ? fast_exp2(m - top) : 0.f;
+    l = lane_groups_sum<kLanesPerRow>(l * w);
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    *reinterpret_cast<float4*>(&s_acc[g][col * 16 + 4 * i]) =
-        make_float4(acc[2 * i].x, acc[2 * i].y, acc[2 * i + 1].x, acc[2 * i + 1].y);
-  if (col == 0) { s_m[g] = m; s_l[g] = l; }
+    for (int i = 0; i < 8; ++i) { acc[i].x *= w; acc[i].y *= w; }
+    float2 part4[4], part2[2];
+    halve_between<16>(part4, acc, lane);
+    halve_between<8>(part2, part4, lane);
+    const int d = col * 16 + ((lane & 16) ? 8 : 0) + ((lane & 8) ? 4 : 0);
+    if constexpr (kLanesPerRow == 8) {
+      *reinterpret_cast<float4*>(&s_acc[warp][d]) = make_float4(part2[0].x, part2[0].y, part2[1].x, part2[1].y);
+    } else {
+      float2 part1[1];
+      halve_between<4>(part1, part2, lane);
+      *reinterpret_cast<float2*>(&s_acc[warp][d + ((lane & 4) ? 2 : 0)]) = part1[0];
+    }
+    if (lane == 0) { s_m[warp] = top; s_l[warp] = l; }
+  } else {
+    const int g = warp * kRowsPerLoad + sub;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<float4*>(&s_acc[g][col * 16 + 4 * i]) =
+          make_float4(acc[2 * i].x, acc[2 * i].y, acc[2 * i + 1].x, acc[2 * i + 1].y);
+    if (col == 0) { s_m[g] = m; s_l[g] = l; }
+  }
   __syncthreads();
   if (tid < D) {
     float M = neg_inf();
@@ -568,7 +617,8 @@ namespace ssa {
 // ---------------------------------------------------------------------------
 // share: row-sharing kernel; wide: one large row-sharing block per SM; even_blocks: that many blocks with even shares of
 // the rows (0: chunks)
-struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool share, wide; int even_blocks; };
+// warps: of a one-head block
+struct Plan { int chunk, n_chunks; size_t acc_bytes, total_bytes; bool share, wide; int even_blocks, warps; };
 
 // Grouped query heads that the kernel which reads a K/V row once for many heads can serve.
 static bool can_share_rows(const ssa_attn_desc* d) {
@@ -582,6 +632,18 @@ static bool can_share_rows(const ssa_attn_desc* d) {
 // 12897 rows 201 / 33, 8 of 2000 listed rows 63.7 / 18.4, 24 of 40 15.5 / 6.7.  (Small launches: one_head_blocks_pay.)
 static int head_splits(const ssa_attn_desc* d) { return (d->H / d->H_kv + kGqaHeads - 1) / kGqaHeads; }
 
+// Warps of a one-head block that takes up to `rows` rows, in a launch of `blocks`.  A warp has sixteen rows of 128 16-bit
+// values on their way at a time (as many bytes of others) and takes about 1.1 us a turn, however few other warps there are.
+// A launch that leaves the SMs room therefore gets blocks of two or four times the warps, as far as the rows give each of
+// them a turn.  Four warps / this, us, 16-bit rows of 128 in index lists: 32 heads x 80 rows 4.1 / 3.1, x 256 rows 6.4 / 4.2;
+// 148 heads x 200 rows 6.8 / 5.1, x 512 rows 11.7 / 7.9; 296 heads x 200 rows 8.1 / 7.3, x 512 rows 14.1 / 12.3.
+static int block_warps(const ssa_attn_desc* d, long long blocks, int rows) {
+  const int turn = 16 * (128 / d->D) * (d->kv_dtype == SSA_FP8_E4M3 ? 2 : 1);
+  int warps = kSmallBlock;
+  while (warps < kWarpSlots && rows > warps * turn && blocks * 2 * warps <= (long long)kWarpSlots * sm_count()) warps *= 2;
+  return warps;
+}
+
 static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan* pl) {
   if (!d || d->B <= 0 || d->H <= 0 || max_selected <= 0) return false;
   if (d->D != 64 && d->D != 128) return false;
@@ -590,10 +652,17 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   // The second pass costs about as much as two rounds of a block, so a request is split only when that buys
   // parallelism: one chunk whenever the list fits a block's staging area and either every SM gets a block or
   // the list is short anyway; otherwise 256-entry chunks, halved while the grid has under two blocks per SM.
+  // Large blocks (block_warps) stage up to 1024 entries, and taking a list of 513..1024 whole is better from a fifth of a
+  // block per SM on (us, chunks / whole: 32 heads x 820 rows 7.7 / 7.3, 148 x 820 12.8 / 10.8, 296 x 820 21.0 / 17.8, but 8 x 820
+  // 5.7 / 6.7); over an 8-bit cache, whose rows are fewer turns, not where a second block would leave most SMs idle
+  // (160 x 1024 12.2 / 13.5), nor for grouped heads, whose lines (one_head_blocks_pay) were measured with chunks.
   const long long sms = sm_count();
   const long long want = sms * 2;
   int chunk = 256;
   if (max_selected <= kMaxChunk && (units >= sms || max_selected <= 256)) chunk = kMaxChunk;
+  else if (!share && max_selected <= kMaxWideChunk && units <= want && 5 * units >= sms &&
+           (d->kv_dtype != SSA_FP8_E4M3 || (d->H == d->H_kv && (units <= sms || 5 * units >= 7 * sms))))
+    chunk = kMaxWideChunk;                             // (at most two blocks per SM, over 512 rows: large blocks)
   else while (chunk > 64 && units * ((max_selected + chunk - 1) / chunk) < want) chunk >>= 1;
   pl->share = share;
   pl->wide = false;
@@ -618,6 +687,7 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   pl->even_blocks = 0;
   int n_chunks = (max_selected + chunk - 1) / chunk;
   if (n_chunks == 1) chunk = (max_selected + 31) / 32 * 32;
+  pl->warps = block_warps(d, units * n_chunks, chunk);
   pl->chunk = chunk;
   pl->n_chunks = n_chunks;
   pl->acc_bytes = ((size_t)out_units * n_chunks * d->D * sizeof(float) + 255) / 256 * 256;
@@ -714,6 +784,7 @@ static bool make_plan_blockmask(const ssa_attn_desc* d, int block_size, int max_
   pl->even_blocks = 0;
   pl->chunk = kMaskChunk / block_size;
   pl->n_chunks = (max_blocks + pl->chunk - 1) / pl->chunk;
+  pl->warps = block_warps(d, units * pl->n_chunks, kMaskChunk);
   pl->acc_bytes = ((size_t)units * pl->n_chunks * d->D * sizeof(float) + 255) / 256 * 256;
   pl->total_bytes = pl->acc_bytes + ((size_t)units * pl->n_chunks * sizeof(float2) + 255) / 256 * 256;
   return true;
@@ -752,7 +823,7 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
   using TQ = typename Storage<T>::Query;
   constexpr bool kFp8 = kIsFp8<T>;
   size_t dynamic_smem = 0;
-  unsigned block_threads = kThreads;
+  unsigned block_threads = 0;
   const bool share = p.share_rows;
   if constexpr (D == 128) {
     if (share) {
@@ -785,24 +856,30 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
     }
   }
   if (!share) {
-    constexpr bool kWide = !kFp8;                       // 8-bit rows are read in 16-byte pieces: one instantiation
-    const bool a32 = kWide && aligned32;
-    if constexpr (!kFp8) {
-      if (p.q_host)                                     // run() has checked: index lists, one chunk, no paging
-        kernel = a32 ? decode_partial_kernel<T, D, kIndex, true, false, true>
-                     : decode_partial_kernel<T, D, kIndex, false, false, true>;
-    }
-    if (p.q_host) {
-    } else if (mode == kIndex && p.page_table)
-      kernel = a32 ? decode_partial_kernel<T, D, kIndex, kWide, true> : decode_partial_kernel<T, D, kIndex, false, true>;
-    else if (mode == kIndex)
-      kernel = a32 ? decode_partial_kernel<T, D, kIndex, kWide> : decode_partial_kernel<T, D, kIndex, false>;
-    else if (mode == kBlockMask)
-      kernel = a32 ? decode_partial_kernel<T, D, kBlockMask, kWide> : decode_partial_kernel<T, D, kBlockMask, false>;
-    else if (mode == kSpans)
-      kernel = a32 ? decode_partial_kernel<T, D, kSpans, kWide> : decode_partial_kernel<T, D, kSpans, false>;
-    else
-      kernel = a32 ? decode_partial_kernel<T, D, kDense, kWide> : decode_partial_kernel<T, D, kDense, false>;
+    auto pick = [&](auto aligned_tag, auto warps_tag) {
+      constexpr bool kA = decltype(aligned_tag)::value;
+      constexpr int kW = decltype(warps_tag)::value;
+      block_threads = kW * 32;
+      if constexpr (!kFp8) {
+        if (p.q_host) {                                 // run() has checked: index lists, one chunk, no paging
+          kernel = decode_partial_kernel<T, D, kIndex, kA, false, true, kW>;
+          return;
+        }
+      }
+      kernel = mode == kIndex ? (p.page_table ? decode_partial_kernel<T, D, kIndex, kA, true, false, kW>
+                                              : decode_partial_kernel<T, D, kIndex, kA, false, false, kW>)
+               : mode == kBlockMask ? decode_partial_kernel<T, D, kBlockMask, kA, false, false, kW>
+               : mode == kSpans     ? decode_partial_kernel<T, D, kSpans, kA, false, false, kW>
+                                    : decode_partial_kernel<T, D, kDense, kA, false, false, kW>;
+    };
+    auto by_warps = [&](auto aligned_tag) {
+      if (p.warps == kWarpSlots) pick(aligned_tag, std::integral_constant<int, kWarpSlots>{});
+      else if (p.warps > kSmallBlock) pick(aligned_tag, std::integral_constant<int, 2 * kSmallBlock>{});
+      else pick(aligned_tag, std::integral_constant<int, kSmallBlock>{});
+    };
+    // (8-bit rows are read in 16-byte pieces: one instantiation)
+    if (!kFp8 && aligned32) by_warps(std::bool_constant<!kFp8>{});
+    else by_warps(std::false_type{});
   }
   if (ev_b) cudaEventRecord(ev_b, st);
   cudaError_t err = launch_pdl_smem(kernel, grid, dim3(block_threads), dynamic_smem, st, p);
@@ -933,6 +1010,7 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   p.index_stride = index_stride; p.max_selected = max_selected;
   p.chunk = pl.chunk; p.n_chunks = pl.n_chunks;
   p.share_rows = pl.share ? 1 : 0;
+  p.warps = pl.warps;
   p.head_splits = pl.share ? head_splits(d) : 1;
   p.heads_per_block = (p.kv_group + p.head_splits - 1) / p.head_splits;
   p.gqa_wide = pl.wide ? 1 : 0;

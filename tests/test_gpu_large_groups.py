@@ -73,7 +73,8 @@ def test_large_groups_against_the_oracle(dtype, B, Hkv, G, T, counts):
     pages = [x.transpose(1, 2).reshape(B * T, 1, Hkv, D).contiguous() for x in (k.view(torch.uint8), v.view(torch.uint8))] \
         if dtype == "fp8" else [x.transpose(1, 2).reshape(B * T, 1, Hkv, D).contiguous() for x in (k, v)]
     kp, vp = (x.view(k.dtype) for x in pages)
-    paging = ssa.make_paging(torch.arange(B * T, dtype=torch.int32, device=DEV).view(B, T), 1, B * T)
+    table = torch.arange(B * T, dtype=torch.int32, device=DEV).view(B, T)
+    paging = ssa.make_paging(table, 1, B * T)
     ssa.decode_attn_sparse_paged(ssa.make_desc_paged(q, kp, vp, out, T), q, kp, vp, paging, d_ctx, d_idx, d_cnt, T, out, lse,
                                  ws[:need], status)
     check(*listed, "a paged cache")

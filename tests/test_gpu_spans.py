@@ -330,3 +330,50 @@ def test_argument_checks_launch_nothing():
     assert call(ws=None) == ssa.ERR_WORKSPACE
     assert ssa.launch_count() == before
     assert call() == ssa.OK
+
+
+@pytest.mark.parametrize("B,H,D,dtype,T", [
+    (1, 8, 128, "bf16", 64), (1, 8, 128, "bf16", 65), (2, 16, 128, "f16", 129), (1, 8, 128, "bf16", 256),    # 4, 8, 16 warps
+    (1, 8, 128, "bf16", 257), (1, 32, 128, "bf16", 513), (4, 37, 128, "f16", 1024), (1, 32, 128, "bf16", 1025),   # whole lists / chunks
+    (37, 4, 128, "bf16", 300), (149, 1, 128, "f16", 257), (74, 4, 128, "bf16", 1024), (297, 1, 128, "f16", 129),   # 8 warps / 4
+    (1, 32, 64, "bf16", 257), (4, 40, 64, "f16", 1000),
+])
+def test_blocks_of_more_warps_where_a_launch_leaves_room(B, H, D, dtype, T):
+    """Index lists, span lists, a paged cache and full contexts at the sizes where a block's warps or its chunk change.  fp32
+    output and at most 1025 rows: the sums' roundings stay below 2^-24 sqrt(1025) of the result; four times that is asserted."""
+    rng = np.random.default_rng(T + B)
+    p = Problem(B, H, T, D, dtype, seed=T + H)
+    lists = []
+    for b in range(B):
+        n = T if b == 0 else int(rng.integers(0, T + 1))       # one full list, the others ragged, possibly empty
+        cut = sorted(rng.integers(0, T - n + 1, size=2).tolist())
+        lists.append([(cut[0], cut[0] + n // 2), (cut[1] + n // 2, cut[1] + n)])
+    ctx = [T] * B
+    index, counts, _ = O.spans_to_index_batch(np.arange(0, 2 * B + 1, 2), np.asarray(lists, np.int32).reshape(-1, 2), ctx, T)
+    seqs = sorted({0, 1, B // 2, B - 1} & set(range(B)))
+    ref, ref_lse = O.decode_attn_sparse(p.q_bits, p.k_bits, p.v_bits, ctx, index, counts, 1 / np.sqrt(D), dtype, seqs=seqs)
+    ok = np.isfinite(ref_lse[seqs])
+
+    def check(out, lse, what, ref=ref, ref_lse=ref_lse, ok=ok):
+        assert float(np.linalg.norm((out - ref)[seqs])) <= 8e-6 * float(np.linalg.norm(ref[seqs])), what
+        np.testing.assert_allclose(lse[seqs][ok], ref_lse[seqs][ok], rtol=2e-6, atol=2e-6, err_msg=what)
+        assert np.all(np.isneginf(lse[seqs][~ok])), what
+
+    out, lse, status, _ = p.sparse(ctx, index, counts.tolist(), max_selected=T)
+    assert status == 0
+    check(out, lse, "index lists")
+    spans, span_lse = run_spans(p, lists, ctx, T)[:2]
+    assert np.array_equal(spans, out) and np.array_equal(span_lse, lse)
+    k, v = (x.transpose(1, 2).reshape(B * T, 1, H, D).contiguous() for x in (p.k, p.v))
+    o, ls = torch.zeros((B, H, D), device=DEV), torch.zeros((B, H), device=DEV)
+    desc = ssa.make_desc_paged(p.q, k, v, o, T)
+    ws = torch.empty(ssa.decode_workspace_bytes(desc, T), dtype=torch.uint8, device=DEV)
+    table = torch.arange(B * T, dtype=torch.int32, device=DEV).view(B, T)
+    ssa.decode_attn_sparse_paged(desc, p.q, k, v, ssa.make_paging(table, 1, B * T),
+                                 *(torch.from_numpy(np.ascontiguousarray(x, dtype=np.int32)).to(DEV) for x in (ctx, index, counts)),
+                                 T, o, ls, ws)
+    torch.cuda.synchronize()
+    assert np.array_equal(o.double().cpu().numpy(), out) and np.array_equal(ls.double().cpu().numpy(), lse)
+    dense, dense_lse, _ = p.dense(counts.tolist())
+    want, want_lse = O.decode_attn_dense(p.q_bits, p.k_bits, p.v_bits, counts, 1 / np.sqrt(D), dtype, seqs=seqs)
+    check(dense, dense_lse, "full contexts", want, want_lse)
