@@ -6,24 +6,51 @@
 
 namespace ssa {
 
-// Called by all 32 lanes of one warp for request b.  Span 0 is the
+// Where request b's tables begin and how long they are, and its first two spans: one trip to memory.
+struct RefTables {
+  int l0, n_lines, a0, n_anchors, r0, n_refs;
+  int2 prefix, current;                     // the instruction prefix and the line being generated
+};
+__device__ __forceinline__ RefTables locate_refs(const ssa_anchor_tables& t, int b) {
+  RefTables r;
+  r.l0 = t.line_offsets[b];
+  r.a0 = t.anchor_offsets[b];
+  r.r0 = t.ref_offsets[b];
+  r.n_lines = max(t.line_offsets[b + 1] - r.l0, 0);
+  r.n_anchors = max(t.anchor_offsets[b + 1] - r.a0, 0);
+  r.n_refs = max(t.ref_offsets[b + 1] - r.r0, 0);
+  r.prefix = make_int2(0, t.prefix_len[b]);
+  r.current = make_int2(t.line_start[b], t.ctx_lens[b]);
+  return r;
+}
+
+// The tables as they lie in global memory.
+struct RefsInMemory {
+  const int2 *lines, *refs;
+  const int32_t* anchors;
+  __device__ __forceinline__ RefsInMemory(const ssa_anchor_tables& t, const RefTables& r)
+      : lines(reinterpret_cast<const int2*>(t.lines) + r.l0), refs(reinterpret_cast<const int2*>(t.refs) + r.r0),
+        anchors(t.anchor_line + r.a0) {}
+  __device__ __forceinline__ int2 line(int i) const { return __ldg(lines + i); }
+  __device__ __forceinline__ int2 ref(int i) const { return __ldg(refs + i); }
+  __device__ __forceinline__ int anchor(int i) const { return __ldg(anchors + i); }
+};
+
+// Called by all 32 lanes of one warp for one request.  Span 0 is the
 // instruction prefix, span 1 the line being generated; then the lanes take the
 // references 32 at a time: each lane resolves one (lo, hi) pair to a first
 // line and a count of lines, a shuffle prefix sum turns the counts into output
 // positions, and the lane hands its spans to put(position, span).  Returns the
 // number of spans the request resolves to (put decides what to do with
-// positions beyond its capacity).
-template <typename Put>
-__device__ __forceinline__ int resolve_refs_warp(const ssa_anchor_tables& t, int b, int lane, uint32_t& flags,
+// positions beyond its capacity).  `tables`: RefsInMemory, or a copy of what
+// that shows.
+template <typename Tables, typename Put>
+__device__ __forceinline__ int resolve_refs_warp(const RefTables& r, const Tables& tables, int lane, uint32_t& flags,
                                                  Put put) {
-  const int l0 = t.line_offsets[b], n_lines = max(t.line_offsets[b + 1] - l0, 0);
-  const int a0 = t.anchor_offsets[b], n_anchors = max(t.anchor_offsets[b + 1] - a0, 0);
-  const int r0 = t.ref_offsets[b], n_refs = max(t.ref_offsets[b + 1] - r0, 0);
-  const int2* lines = reinterpret_cast<const int2*>(t.lines) + l0;
-  const int2* refs = reinterpret_cast<const int2*>(t.refs) + r0;
+  const int n_lines = r.n_lines, n_anchors = r.n_anchors, n_refs = r.n_refs;
   if (lane == 0) {
-    put(0, make_int2(0, t.prefix_len[b]));
-    put(1, make_int2(t.line_start[b], t.ctx_lens[b]));
+    put(0, r.prefix);
+    put(1, r.current);
   }
   int written = 2;
   for (int base = 0; base < n_refs; base += 32) {
@@ -31,7 +58,7 @@ __device__ __forceinline__ int resolve_refs_warp(const ssa_anchor_tables& t, int
     int first = 0, count = 0;
     bool by_anchor = false;
     if (base + lane < n_refs) {
-      const int2 ref = refs[base + lane];
+      const int2 ref = tables.ref(base + lane);
       if (ref.x == ref.y && ref.x < 0) {
         if (n_lines + ref.x >= 0) { first = n_lines + ref.x; count = 1; }
         else flags |= SSA_DEV_BAD_REF;
@@ -55,7 +82,7 @@ __device__ __forceinline__ int resolve_refs_warp(const ssa_anchor_tables& t, int
         int li[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          li[k] = (a + k < first + count && a + k < n_anchors) ? __ldg(t.anchor_line + a0 + a + k) : -1;
+          li[k] = (a + k < first + count && a + k < n_anchors) ? tables.anchor(a + k) : -1;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           if (a + k >= first + count) break;
@@ -78,16 +105,16 @@ __device__ __forceinline__ int resolve_refs_warp(const ssa_anchor_tables& t, int
         int2 span[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          li[k] = (a + k < first + count && a + k < n_anchors) ? __ldg(t.anchor_line + a0 + a + k) : -1;
+          li[k] = (a + k < first + count && a + k < n_anchors) ? tables.anchor(a + k) : -1;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          span[k] = (li[k] >= 0 && li[k] < n_lines) ? __ldg(lines + li[k]) : make_int2(0, 0);
+          span[k] = (li[k] >= 0 && li[k] < n_lines) ? tables.line(li[k]) : make_int2(0, 0);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           if (li[k] >= 0 && li[k] < n_lines) put(at++, span[k]);
       }
     } else if (count == 1) {
-      put(at, lines[first]);
+      put(at, tables.line(first));
     }
     written += __shfl_sync(0xffffffffu, incl, 31);
   }

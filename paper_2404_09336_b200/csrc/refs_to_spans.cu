@@ -22,7 +22,8 @@ refs_to_spans_kernel(const ssa_anchor_tables t, int32_t B, int32_t* __restrict__
   uint32_t flags = 0;
   if (lane == 0) span_offsets_out[b] = b * span_stride;
   // spans beyond the row are counted, not stored (overflow)
-  const int written = resolve_refs_warp(t, b, lane, flags, [&](int at, int2 span) {
+  const RefTables r = locate_refs(t, b);
+  const int written = resolve_refs_warp(r, RefsInMemory(t, r), lane, flags, [&](int at, int2 span) {
     if (at < span_stride) row[at] = span;
   });
   if (written > span_stride) flags |= SSA_DEV_OVERFLOW;

@@ -120,3 +120,14 @@ def test_invariance_to_order_and_splitting():
     assert np.array_equal(counts, counts2)
     for b in range(wl.B):
         assert np.array_equal(base[b, :counts[b]], again[b, :counts[b]])
+
+
+@pytest.mark.parametrize("n", [31, 32, 33, 127, 128, 129, 255, 256, 257])
+def test_span_counts_where_the_sort_changes(n):
+    """Equal starts, nested, empty, reversed and clipped spans among n; few requests (short slices) and many."""
+    rnd = random.Random(n)
+    spans = [(s, s + rnd.randint(-3, 40)) for s in (rnd.randint(-5, 1500) for _ in range(n))]
+    spans[::5] = [spans[0]] * len(spans[::5])
+    for B in (1, 3, 160):
+        lists = [spans[b % 3:] + spans[:b % 3] if b % 4 else spans[:b % n] for b in range(B)]
+        compare(lists, [1400 + b % 9 for b in range(B)], 1536)

@@ -267,3 +267,21 @@ def test_generation_loop_with_growing_context():
         ref, _ = O.decode_attn_sparse(p.q_bits, p.k_bits, p.v_bits, ctx_l, want_idx, want_cnt, 1 / np.sqrt(D), "bf16")
         assert_parity(out.double().cpu().numpy(), ref, False, f"step {step}")
         ctx += 1                                                               # the next token's row is appended
+
+
+@pytest.mark.parametrize("n_spans", [1, 32, 33, 128, 129, 256, 257, 700])
+@pytest.mark.parametrize("n_lines", [512, 513])
+def test_one_launch_where_the_sort_or_the_table_copy_changes(n_spans, n_lines):
+    """Span counts on both sides of every way to sort them (equal starts, empty and reversed spans among them), tables that
+    just fit and just do not fit shared memory, and one long list next to an empty request: bit-exact lists."""
+    rnd = random.Random(n_spans + n_lines)
+    lines = [(s, s + rnd.randint(-2, 9)) for s in (rnd.randint(0, 3 * n_lines) for _ in range(n_lines))]
+    lines[1::7] = [lines[0]] * len(lines[1::7])
+    anchors = [rnd.randrange(n_lines) for _ in range(n_lines)]
+    some = dict(lines=lines, anchors=anchors, prefix=0, start=3 * n_lines, ctx=3 * n_lines + 3)
+    one_each = dict(some, refs=[(i % n_lines, i % n_lines) for i in range(max(n_spans - 2, 0))])
+    in_ranges = dict(some, refs=[(-n_lines, -n_lines), (0, max(0, min(n_lines - 1, n_spans - 4)))])
+    empty = dict(lines=[], anchors=[], refs=[], prefix=0, start=0, ctx=0)
+    for stride in (40, 3 * n_lines + 3):
+        compare_index([one_each, empty, in_ranges], stride)
+        compare_index([in_ranges] * 80 + [one_each], stride)
