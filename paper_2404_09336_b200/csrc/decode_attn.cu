@@ -829,25 +829,24 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
     if (share) {
       grid.x *= (unsigned)p.head_splits;
       grid.y = (unsigned)(p.H / p.kv_group);            // one block, or head_splits, per K/V head
-      auto pick = [&](auto hi_tag, auto wide_tag, auto fine_tag) {
-        constexpr bool kHi = decltype(hi_tag)::value, kWide = decltype(wide_tag)::value, kFine = decltype(fine_tag)::value;
+      auto pick = [&](auto hi_tag, auto wide_tag, auto split_tag) {
+        constexpr bool kHi = decltype(hi_tag)::value, kWide = decltype(wide_tag)::value, kSplit = decltype(split_tag)::value;
         using Shape = GqaShape<T, kHi, kWide>;
         block_threads = Shape::kWarps * 32;
         dynamic_smem = Shape::kSmemBytes;
         if constexpr (!kWide) {
           if (p.even_blocks > 0) {
-            kernel = decode_partial_gqa_kernel<T, kDense, kHi, false, true, kFine>;
+            kernel = decode_partial_gqa_kernel<T, kDense, kHi, false, true, kSplit>;
             return;
           }
         }
-        kernel = mode == kIndex   ? decode_partial_gqa_kernel<T, kIndex, kHi, kWide, false, kFine>
-                 : mode == kSpans ? decode_partial_gqa_kernel<T, kSpans, kHi, kWide, false, kFine>
-                                  : decode_partial_gqa_kernel<T, kDense, kHi, kWide, false, kFine>;
+        kernel = mode == kIndex   ? decode_partial_gqa_kernel<T, kIndex, kHi, kWide, false, kSplit>
+                 : mode == kSpans ? decode_partial_gqa_kernel<T, kSpans, kHi, kWide, false, kSplit>
+                                  : decode_partial_gqa_kernel<T, kDense, kHi, kWide, false, kSplit>;
       };
       constexpr std::true_type yes;
       constexpr std::false_type no;
-      constexpr std::bool_constant<!kFp8> fine;         // (8-bit rows have it anyway)
-      if (p.head_splits > 1) p.gqa_wide ? pick(yes, yes, fine) : pick(yes, no, fine);   // nine heads a block at least
+      if (p.head_splits > 1) p.gqa_wide ? pick(yes, yes, yes) : pick(yes, no, yes);   // nine heads a block at least
       else if (p.heads_per_block > 8) p.gqa_wide ? pick(yes, yes, no) : pick(yes, no, no);
       else p.gqa_wide ? pick(no, yes, no) : pick(no, no, no);
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_smem) != cudaSuccess)

@@ -261,10 +261,11 @@ __device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParam
 // kWide serves launches with at most one unit (request x K/V head) per SM and short lists: a whole list is then one
 // block's work, no second pass.
 // kEven (full contexts): even shares, see above; the grid is (even_blocks * head_splits, 1, 1).
-// kFine (16-bit rows): weights to 22 bits and more, and tiles summed on their own, as 8-bit rows have it anyway: error of a
-// row against 64 bits 1.5e-7 instead of 1.4..3.2e-6.  For groups of more than kGqaHeads heads, which one head per block
-// served with 1.4..2.5e-7.  It costs them a tenth to a fifth (24 requests, 128 heads over 4, 2000 rows: 40.8 -> 48.6 us).
-template <typename T, int kMode, bool kHi, bool kWide, bool kEven = false, bool kFine = false>
+// kSplit: groups of more than kGqaHeads heads; head_splits blocks, side by side, serve heads_per_block of them each.  Over
+// 16-bit rows their weights enter to 22 bits and more, and tiles are summed on their own, as 8-bit rows have it anyway: error
+// of a row against 64 bits 1.5e-7 instead of 1.4..3.2e-6, since one head per block, which served them before, has 1.4..2.5e-7.
+// It costs them a tenth to a fifth (24 requests, 128 heads over 4, 2000 rows: 40.8 -> 48.6 us).
+template <typename T, int kMode, bool kHi, bool kWide, bool kEven = false, bool kSplit = false>
 __global__ void __launch_bounds__(GqaShape<T, kHi, kWide>::kWarps * 32, kWide ? 1 : 2)
 decode_partial_gqa_kernel(const DecodeParams p) {
   using Shape = GqaShape<T, kHi, kWide>;
@@ -275,6 +276,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   constexpr bool kFp8 = kIsFp8<T>;
   using TQ = typename Storage<T>::Query;                // type of the query rows and of a stored output
   using TP = typename std::conditional<kFp8, __half, T>::type;   // type of the weights in the second contraction
+  constexpr bool kFine = kSplit && !kFp8;
   constexpr bool kHalfWeights = std::is_same<TP, __half>::value;
   constexpr float kUp = kFp8 || (kFine && kHalfWeights) ? 8192.f : 1.f;   // weights (and all they enter) are scaled by this in the loop
   constexpr int kTileBytes = kGqaRows * (kFp8 ? 128 : 256);      // one tensor's tile
@@ -291,18 +293,16 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   __shared__ __align__(128) unsigned char s_qtile[kGqaHeads * 256];   // Q of the group, swizzled like a row tile
   __shared__ float s_m[kTeams][kLiveHeads], s_l[kTeams][kLiveHeads];
   __shared__ typename std::conditional<kMode == kSpans, SpanRuns, int>::type s_runs;
+  __shared__ typename std::conditional<kMode == kSpans, WarpRuns, int>::type s_wruns[kMode == kSpans ? kWarps : 1];
   __shared__ typename std::conditional<kEven, EvenLine, int>::type s_line;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, j = lane & 3;
   const int team = warp / kTeam, ht = warp % kTeam;     // ht: the eight heads of the block's that are this warp's
   const int G = p.kv_group;
-  int chunk_id = blockIdx.x, part = 0;                 // the block serves the part-th heads_per_block heads of the group
-  if (p.head_splits > 1) {
-    chunk_id = blockIdx.x / p.head_splits;
-    part = blockIdx.x - chunk_id * p.head_splits;
-  }
-  const int h0 = part * p.heads_per_block, heads = min(p.heads_per_block, G - h0);
+  // the block serves the part-th heads_per_block heads of the group
+  const int chunk_id = kSplit ? blockIdx.x / p.head_splits : blockIdx.x, part = kSplit ? blockIdx.x - chunk_id * p.head_splits : 0;
+  const int h0 = kSplit ? part * p.heads_per_block : 0, heads = kSplit ? min(p.heads_per_block, G - h0) : G;
 
   grid_dependency_wait();
   if (p.early_release) grid_launch_dependents();
@@ -361,16 +361,33 @@ decode_partial_gqa_kernel(const DecodeParams p) {
         q_hi = ld_stream_16B(src + 8);
       }
     }
+    // span lists: up to 32 spans are merged by every warp for itself, which needs no barrier (one warp for the block, us: 32
+    // requests of 819 rows, four heads on each of 8 K/V heads over an 8-bit cache 17.75 -> 16.98, 20 requests of 5199 or 316
+    // rows over a 16-bit one 79.4 -> 72.2); a lane asks for "its" span right away
+    int span_first = 0, span_n = 0, runs = 1;           // runs: span_cap rounded up to a power of two
+    int2 my_span = make_int2(0, 0);
+    const bool warp_merge = kMode == kSpans && p.span_cap <= 32;
+    if constexpr (kMode == kSpans) {
+      span_first = p.span_offsets ? __ldg(p.span_offsets + b) : b * p.span_cap;
+      span_n = p.span_offsets ? __ldg(p.span_offsets + b + 1) - span_first : p.span_cap;
+      if (warp_merge && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
+      while (warp_merge && runs < p.span_cap) runs <<= 1;
+    }
     int n, c;
     if constexpr (kEven) n = c = s_line.rows[b];
     else request_sizes(p, b, n, c, flags);
     if constexpr (kMode == kSpans) {
-      const int first = p.span_offsets ? __ldg(p.span_offsets + b) : b * p.span_cap;
-      const int S = p.span_offsets ? __ldg(p.span_offsets + b + 1) - first : p.span_cap;
-      const int total = merge_spans_block<kThreads>(s_runs, p.spans + first, S, p.span_cap, n);
+      int total;
+      if (warp_merge) {
+        int S = max(span_n, 0);
+        if (S > p.span_cap) { S = p.span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
+        total = merge_spans_warp(s_wruns[warp], my_span, S, runs, n, flags);
+      } else {
+        total = merge_spans_block<kThreads>(s_runs, p.spans + span_first, span_n, p.span_cap, n);
+        if (tid == 0) flags |= s_runs.flags;
+      }
       c = min(total, p.max_selected);
       if (total > p.max_selected) flags |= SSA_DEV_OVERFLOW;
-      if (tid == 0) flags |= s_runs.flags;
       if (chunk_id == 0 && kvh == 0 && part == 0 && tid == 0) {
         if (p.counts_out) p.counts_out[b] = c;
         if (p.ws_counts) p.ws_counts[b] = c;
@@ -384,7 +401,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       if constexpr (kMode == kSpans) {
         int32_t* out = (kvh == 0 && part == 0 && p.index_out) ? p.index_out + (int64_t)b * p.index_stride + start + w0 : nullptr;
         for (int i = tid; i < wn; i += kThreads) {
-          const int v = span_position(s_runs, start + w0 + i);
+          const int v = warp_merge ? span_position(s_wruns[warp], runs, start + w0 + i) : span_position(s_runs, start + w0 + i);
           s_idx[i] = v;
           if (out) out[i] = v;
         }
