@@ -18,8 +18,9 @@
 // the heads in the M dimension instead, a group of up to eight heads paid for
 // sixteen, twice the matrix instructions.
 // 16-bit tiles come out of shared memory with ldmatrix (.trans for V).  8-bit
-// rows (e4m3) are read with plain 16-byte loads and converted in registers,
-// exactly: K to bf16 (the type of its queries), V to fp16; which lane holds
+// rows (e4m3) are read with plain 16-byte loads and converted to fp16 in
+// registers, exactly, one instruction per pair; their bf16 query rows become
+// fp16 times a power of two of their own (scaled_query).  Which lane holds
 // which dimension is free as long as Q (for K) and the output (for V) follow,
 // so a lane takes whole 16-byte pieces of a row.
 // The rows travel global -> shared memory by asynchronous 16-byte copies
@@ -151,15 +152,37 @@ __device__ __forceinline__ uint4 lds_16B(uint32_t addr) {
   return r;
 }
 
-// Two e4m3 values (low 16 bits) -> two fp16 or two bf16 (both exact).
+// Two e4m3 values (low 16 bits) -> two fp16 (exact).
 __device__ __forceinline__ uint32_t e4m3x2_to_half2(uint32_t pair) {
   uint32_t h2;
   asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((unsigned short)pair));
   return h2;
 }
-__device__ __forceinline__ uint32_t e4m3x2_to_bf162(uint32_t pair) {
-  const float2 f = e4m3x2_to_float2(pair);
-  return pack2<__nv_bfloat16>(f.x, f.y);
+// A query row over an 8-bit cache: sixteen bf16 values of each of eight neighbouring lanes -> fp16 values times 2^k, the
+// largest in [2^14, 2^15); returns 2^-k.  Exact for values down to 2^-32 of the row's largest and off by less than 2^-39 of
+// that below, far under the scores' own rounding.  (With bf16 queries the rows of K had to become bf16, by way of two fp32
+// values: four instructions per pair instead of one.  us, four heads on each of 8 K/V heads: 32 requests of
+// 819 rows 16.98 -> 16.30, 17 full contexts of 8190 rows 57.2 -> 52.2.  The powers of two cancel: same bits.)
+__device__ __forceinline__ float scaled_query(uint4& lo, uint4& hi) {
+  uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  uint32_t most = 0u;                                   // largest finite magnitude, as the bits of a bf16 value
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t a = w[i] & 0x7fffu, b = (w[i] >> 16) & 0x7fffu;
+    most = max(most, max(a < 0x7f80u ? a : 0u, b < 0x7f80u ? b : 0u));
+  }
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+  const int up = min(max(268 - (int)(most >> 7), 1), 253);   // biased exponents of 2^k and, below, of 2^-k
+  const float scale = __int_as_float(up << 23);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float2 f = unpack2<__nv_bfloat16>(w[i]);
+    w[i] = pack2<__half>(f.x * scale, f.y * scale);
+  }
+  lo = make_uint4(w[0], w[1], w[2], w[3]);
+  hi = make_uint4(w[4], w[5], w[6], w[7]);
+  return __int_as_float((254 - up) << 23);
 }
 
 // 8-bit tiles, [16 rows][128 B]: 16-byte chunk `chunk` of a row.  The XOR keeps the eight lanes that a 16-byte
@@ -292,6 +315,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   __shared__ int32_t s_idx[kSparse ? kStagedShortList : 1];
   __shared__ __align__(128) unsigned char s_qtile[kGqaHeads * 256];   // Q of the group, swizzled like a row tile
   __shared__ float s_m[kTeams][kLiveHeads], s_l[kTeams][kLiveHeads];
+  __shared__ float s_back[kFp8 ? kGqaHeads : 1];         // 8-bit rows: what undoes the scaling of a head's query row
   __shared__ typename std::conditional<kMode == kSpans, SpanRuns, int>::type s_runs;
   __shared__ typename std::conditional<kMode == kSpans, WarpRuns, int>::type s_wruns[kMode == kSpans ? kWarps : 1];
   __shared__ typename std::conditional<kEven, EvenLine, int>::type s_line;
@@ -440,6 +464,10 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     auto store_q = [&]() {
       if (tid < kGqaHeads * 8) {
         const int row = tid >> 3, c0 = (tid & 7) * 2;
+        if constexpr (kFp8) {
+          const float back = scaled_query(q_lo, q_hi);
+          if (c0 == 0) s_back[row] = back;
+        }
         *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0)) = q_lo;
         *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0 + 1)) = q_hi;
       }
@@ -474,9 +502,12 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     // B fragments of Q for the eight k-steps: registers for the whole block's life.  8-bit rows: k-step ks of lane
     // (g, j) is dims 64 (ks / 4) + 16 j + 4 (ks % 4) + 0..3 of head g, the order its K pieces come in.
     uint32_t qb[8][2];
+    float score_scale[2] = {p.scale_log2, p.scale_log2};   // of heads 8 ht + 2 j + {0, 1}
     auto load_q = [&]() {
       const uint32_t base = smem_u32(s_qtile);
       if constexpr (kFp8) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) score_scale[e] = p.scale_log2 * s_back[8 * ht + 2 * j + e];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const uint4 w = lds_16B(base + tile_offset(8 * ht + g, 8 * (c >> 1) + 2 * j + (c & 1)));
@@ -584,10 +615,10 @@ decode_partial_gqa_kernel(const DecodeParams p) {
             const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, c[4] = {hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              const uint32_t a0 = e4m3x2_to_bf162(a[i]), a1 = e4m3x2_to_bf162(c[i]);
-              const uint32_t a2 = e4m3x2_to_bf162(a[i] >> 16), a3 = e4m3x2_to_bf162(c[i] >> 16);
+              const uint32_t a0 = e4m3x2_to_half2(a[i]), a1 = e4m3x2_to_half2(c[i]);
+              const uint32_t a2 = e4m3x2_to_half2(a[i] >> 16), a3 = e4m3x2_to_half2(c[i] >> 16);
               float (&sum)[4] = (i & 1) ? s_odd : s;
-              mma_16816<TQ>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
+              mma_16816<__half>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
             }
           }
         } else {
@@ -600,7 +631,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
           }
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[e] = (s[e] + s_odd[e]) * p.scale_log2;
+        for (int e = 0; e < 4; ++e) s[e] = (s[e] + s_odd[e]) * score_scale[e & 1];
         if (live != 0xffffu) {                           // warp-uniform; a masked row's score is -inf
           const bool live_lo = (live >> g) & 1u, live_hi = (live >> (g + 8)) & 1u;
 #pragma unroll

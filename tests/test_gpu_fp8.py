@@ -307,3 +307,42 @@ def test_small_grouped_launches_one_head_per_block_or_in_the_workspace_of_shared
     ssa.decode_attn_sparse(desc, p.q, p.k, p.v, d_ctx, torch.from_numpy(index).to(DEV), d_cnt, sel, out, lse, ws, None)
     assert ssa.launch_count() - before == (2 if sel > 512 else 1)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("group", [2, 8, 12, 20])
+@pytest.mark.parametrize("kind", ["wide", "tiny", "huge", "spread", "not finite"])
+def test_shared_rows_over_an_8_bit_cache_whatever_the_magnitude_of_the_queries(group, kind):
+    """The row-sharing kernel scales query rows by powers of two.  Rows near the ends of the bf16 range (with a softmax scale
+    that brings the scores back), rows whose elements span 2^40, and rows with an infinity or a NaN next to ordinary ones.
+    Bound: scores of up to 8 sqrt(128) |k| carry 2^-24 sqrt(128) relative each; 4e-6 in the 2-norm is asserted (measured at
+    most 6.4e-7, the same with unscaled queries)."""
+    B, Hkv, T, D = 2, 2, 8000, 128
+    H = group * Hkv
+    p = Fp8Problem(B, H, Hkv, T, D, seed=group)
+    rng = np.random.default_rng(group)
+    q = rng.standard_normal((B, H, D)).astype(np.float32)
+    scale = 1 / np.sqrt(D)
+    if kind == "wide":
+        q *= 8
+    elif kind in ("tiny", "huge"):
+        q *= np.float32(2.0 ** (-124 if kind == "tiny" else 120))
+        scale = 2.0 ** (120 if kind == "tiny" else -122)
+    elif kind == "spread":
+        q *= np.exp2(-40 * rng.random((B, H, D))).astype(np.float32)
+    else:
+        q[0, 1, 5], q[1, H - 1, 127] = np.inf, np.nan
+    q_bits = round_to_storage(q, "bf16")
+    d_q = torch.from_numpy(q_bits.view(np.int16)).view(torch.bfloat16).to(DEV)
+    out, lse = torch.zeros((B, H, D), device=DEV), torch.zeros((B, H), device=DEV)
+    desc = ssa.make_desc(d_q, p.k, p.v, out, scale=scale)
+    ws = torch.empty(ssa.decode_workspace_bytes(desc, T), dtype=torch.uint8, device=DEV)
+    ctx = [T, 4321]
+    ssa.decode_attn_dense(desc, d_q, p.k, p.v, torch.tensor(ctx, dtype=torch.int32, device=DEV), out, lse, ws)
+    torch.cuda.synchronize()
+    got, got_lse = out.double().cpu().numpy(), lse.double().cpu().numpy()
+    bad = ~np.isfinite(q).all(axis=-1)
+    assert np.isnan(got[bad]).all() and np.isnan(got_lse[bad]).all()
+    q_bits[bad] = 0
+    ref, ref_lse = O.decode_attn_dense(q_bits, *p.oracle_kv(), ctx, scale, "bf16/e4m3")
+    assert float(np.linalg.norm((got - ref)[~bad])) <= 4e-6 * float(np.linalg.norm(ref[~bad]))
+    np.testing.assert_allclose(got_lse[~bad], ref_lse[~bad], rtol=2e-6, atol=2e-6)
