@@ -88,7 +88,7 @@ typedef enum { SSA_F16 = 0, SSA_BF16 = 1, SSA_F32 = 2, SSA_FP8_E4M3 = 3 } ssa_dt
  * scale with the cache folds K's into `scale` and applies V's to the output;
  * q is then BF16 and out_dtype BF16 or F32.  Such a cache halves the bytes per
  * selected row.  Grouped query heads over it share the rows they read (D = 128
- * and 2 to 16 heads per K/V head), as over a 16-bit cache: the scores and the
+ * and two or more heads per K/V head), as over a 16-bit cache: the scores and the
  * sums are fp32, the softmax weights enter the second contraction as a pair of
  * fp16 values (22 bits).  Small launches, other groups, D = 64 and the blocked
  * lists take one head per thread block, fp32 throughout (each head re-reads the
