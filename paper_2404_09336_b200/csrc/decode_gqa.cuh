@@ -20,7 +20,8 @@
 // 16-bit tiles come out of shared memory with ldmatrix (.trans for V).  8-bit
 // rows (e4m3) are read with plain 16-byte loads and converted to fp16 in
 // registers, exactly, one instruction per pair; their bf16 query rows become
-// fp16 times a power of two of their own (scaled_query).  Which lane holds
+// fp16 times a power of two of their own (scaled_query), or, where that would
+// lose a bit, stay bf16 against rows of K in bf16.  Which lane holds
 // which dimension is free as long as Q (for K) and the output (for V) follow,
 // so a lane takes whole 16-byte pieces of a row.
 // The rows travel global -> shared memory by asynchronous 16-byte copies
@@ -152,18 +153,27 @@ __device__ __forceinline__ uint4 lds_16B(uint32_t addr) {
   return r;
 }
 
-// Two e4m3 values (low 16 bits) -> two fp16 (exact).
-__device__ __forceinline__ uint32_t e4m3x2_to_half2(uint32_t pair) {
+// Two e4m3 values (low 16 bits) -> two fp16 or two bf16 (both exact).
+template <typename T>
+__device__ __forceinline__ uint32_t e4m3x2_to_16bit(uint32_t pair);
+template <>
+__device__ __forceinline__ uint32_t e4m3x2_to_16bit<__half>(uint32_t pair) {
   uint32_t h2;
   asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((unsigned short)pair));
   return h2;
 }
+template <>
+__device__ __forceinline__ uint32_t e4m3x2_to_16bit<__nv_bfloat16>(uint32_t pair) {
+  const float2 f = e4m3x2_to_float2(pair);
+  return pack2<__nv_bfloat16>(f.x, f.y);
+}
 // A query row over an 8-bit cache: sixteen bf16 values of each of eight neighbouring lanes -> fp16 values times 2^k, the
-// largest in [2^14, 2^15); returns 2^-k.  Exact for values down to 2^-32 of the row's largest and off by less than 2^-39 of
-// that below, far under the scores' own rounding.  (With bf16 queries the rows of K had to become bf16, by way of two fp32
-// values: four instructions per pair instead of one.  us, four heads on each of 8 K/V heads: 32 requests of
-// 819 rows 16.98 -> 16.30, 17 full contexts of 8190 rows 57.2 -> 52.2.  The powers of two cancel: same bits.)
-__device__ __forceinline__ float scaled_query(uint4& lo, uint4& hi) {
+// largest in [2^14, 2^15).  Returns what turns its scores into log2 units, scale_log2 2^-k, or 0 where that is no normal
+// number or a value is not an fp16 number times 2^-k: such a row (elements that differ by 2^31 and more) is for bf16 scores.
+// (With bf16 queries the rows of K have to become bf16, by way of two fp32 values: four instructions per pair instead of
+// one.  us, four heads on each of 8 K/V heads: 32 requests of 819 rows 16.98 -> 16.30, 17 full contexts of 8190 rows 57.2 ->
+// 52.2.  The values are the same and the powers of two cancel: same bits.)
+__device__ __forceinline__ float scaled_query(uint4& lo, uint4& hi, float scale_log2) {
   uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
   uint32_t most = 0u;                                   // largest finite magnitude, as the bits of a bf16 value
 #pragma unroll
@@ -173,16 +183,24 @@ __device__ __forceinline__ float scaled_query(uint4& lo, uint4& hi) {
   }
 #pragma unroll
   for (int o = 1; o < 8; o <<= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
-  const int up = min(max(268 - (int)(most >> 7), 1), 253);   // biased exponents of 2^k and, below, of 2^-k
+  const int up = most == 0u ? 127 : min(268 - (int)(most >> 7), 253);   // biased exponents of 2^k and, below, of 2^-k
   const float scale = __int_as_float(up << 23);
+  bool lost = false;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const float2 f = unpack2<__nv_bfloat16>(w[i]);
-    w[i] = pack2<__half>(f.x * scale, f.y * scale);
+    float2 f = unpack2<__nv_bfloat16>(w[i]);
+    f.x *= scale;
+    f.y *= scale;
+    w[i] = pack2<__half>(f.x, f.y);
+    const float2 back = unpack2<__half>(w[i]);
+    lost |= (back.x != f.x && f.x == f.x) || (back.y != f.y && f.y == f.y);   // (a NaN stays one)
   }
   lo = make_uint4(w[0], w[1], w[2], w[3]);
   hi = make_uint4(w[4], w[5], w[6], w[7]);
-  return __int_as_float((254 - up) << 23);
+  const float unit = scale_log2 * __int_as_float((254 - up) << 23);
+  lost |= !(unit >= 1.17549435e-38f && unit <= 3.40282347e38f);
+  const uint32_t row_lost = __ballot_sync(0xffffffffu, lost) >> (threadIdx.x & 24) & 0xffu;
+  return row_lost ? 0.f : unit;
 }
 
 // 8-bit tiles, [16 rows][128 B]: 16-byte chunk `chunk` of a row.  The XOR keeps the eight lanes that a 16-byte
@@ -315,7 +333,7 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   __shared__ int32_t s_idx[kSparse ? kStagedShortList : 1];
   __shared__ __align__(128) unsigned char s_qtile[kGqaHeads * 256];   // Q of the group, swizzled like a row tile
   __shared__ float s_m[kTeams][kLiveHeads], s_l[kTeams][kLiveHeads];
-  __shared__ float s_back[kFp8 ? kGqaHeads : 1];         // 8-bit rows: what undoes the scaling of a head's query row
+  __shared__ float s_unit[kFp8 ? kGqaHeads : 1];         // 8-bit rows: of a head's scaled query row (scaled_query)
   __shared__ typename std::conditional<kMode == kSpans, SpanRuns, int>::type s_runs;
   __shared__ typename std::conditional<kMode == kSpans, WarpRuns, int>::type s_wruns[kMode == kSpans ? kWarps : 1];
   __shared__ typename std::conditional<kEven, EvenLine, int>::type s_line;
@@ -465,8 +483,8 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       if (tid < kGqaHeads * 8) {
         const int row = tid >> 3, c0 = (tid & 7) * 2;
         if constexpr (kFp8) {
-          const float back = scaled_query(q_lo, q_hi);
-          if (c0 == 0) s_back[row] = back;
+          const float unit = scaled_query(q_lo, q_hi, p.scale_log2);
+          if (c0 == 0) s_unit[row] = unit;
         }
         *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0)) = q_lo;
         *reinterpret_cast<uint4*>(s_qtile + tile_offset(row, c0 + 1)) = q_hi;
@@ -503,14 +521,23 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     // (g, j) is dims 64 (ks / 4) + 16 j + 4 (ks % 4) + 0..3 of head g, the order its K pieces come in.
     uint32_t qb[8][2];
     float score_scale[2] = {p.scale_log2, p.scale_log2};   // of heads 8 ht + 2 j + {0, 1}
+    bool bf16_scores = false;                              // 8-bit rows: a query row of this warp is not for fp16
     auto load_q = [&]() {
       const uint32_t base = smem_u32(s_qtile);
       if constexpr (kFp8) {
+        bf16_scores = __any_sync(0xffffffffu, s_unit[8 * ht + (lane & 7)] == 0.f) != 0;
+        if (!bf16_scores) {
 #pragma unroll
-        for (int e = 0; e < 2; ++e) score_scale[e] = p.scale_log2 * s_back[8 * ht + 2 * j + e];
+          for (int e = 0; e < 2; ++e) score_scale[e] = s_unit[8 * ht + 2 * j + e];
+        }
+        const int head = 8 * ht + g;
+        const TQ* const row = reinterpret_cast<const TQ*>(p.q) + (int64_t)b * p.q_sb + (int64_t)(kvh * G + h0 + head) * p.q_sh;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const uint4 w = lds_16B(base + tile_offset(8 * ht + g, 8 * (c >> 1) + 2 * j + (c & 1)));
+          const int chunk = 8 * (c >> 1) + 2 * j + (c & 1);
+          uint4 w;
+          if (!bf16_scores) w = lds_16B(base + tile_offset(head, chunk));
+          else w = head < heads ? ld_stream_16B(row + 8 * chunk) : make_uint4(0u, 0u, 0u, 0u);
           qb[2 * c][0] = w.x; qb[2 * c][1] = w.y;
           qb[2 * c + 1][0] = w.z; qb[2 * c + 1][1] = w.w;
         }
@@ -609,18 +636,23 @@ decode_partial_gqa_kernel(const DecodeParams p) {
         // (two sums of four k-steps each: half the length of the dependent chain)
         float s[4] = {0.f, 0.f, 0.f, 0.f}, s_odd[4] = {0.f, 0.f, 0.f, 0.f};
         if constexpr (kFp8) {
+          auto scores = [&](auto type) {
+            using TS = decltype(type);
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            const uint4 lo = lds_16B(ka ^ (half << 6)), hi = lds_16B((ka ^ (half << 6)) + 8 * kRowBytes);
-            const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, c[4] = {hi.x, hi.y, hi.z, hi.w};
+            for (int half = 0; half < 2; ++half) {
+              const uint4 lo = lds_16B(ka ^ (half << 6)), hi = lds_16B((ka ^ (half << 6)) + 8 * kRowBytes);
+              const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, c[4] = {hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint32_t a0 = e4m3x2_to_half2(a[i]), a1 = e4m3x2_to_half2(c[i]);
-              const uint32_t a2 = e4m3x2_to_half2(a[i] >> 16), a3 = e4m3x2_to_half2(c[i] >> 16);
-              float (&sum)[4] = (i & 1) ? s_odd : s;
-              mma_16816<__half>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
+              for (int i = 0; i < 4; ++i) {
+                const uint32_t a0 = e4m3x2_to_16bit<TS>(a[i]), a1 = e4m3x2_to_16bit<TS>(c[i]);
+                const uint32_t a2 = e4m3x2_to_16bit<TS>(a[i] >> 16), a3 = e4m3x2_to_16bit<TS>(c[i] >> 16);
+                float (&sum)[4] = (i & 1) ? s_odd : s;
+                mma_16816<TS>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
+              }
             }
-          }
+          };
+          if (bf16_scores) scores(__nv_bfloat16());      // warp-uniform
+          else scores(__half());
         } else {
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks) {
@@ -687,8 +719,8 @@ decode_partial_gqa_kernel(const DecodeParams p) {
             // bytes 2 (t & 1) and 2 (t & 1) + 1 of both rows of a pair, interleaved
             const uint32_t sel = (t & 1) ? 0x7362u : 0x5140u;
             const uint32_t lo = __byte_perm(x0[t >> 1], x1[t >> 1], sel), hi = __byte_perm(x2[t >> 1], x3[t >> 1], sel);
-            const uint32_t a0 = e4m3x2_to_half2(lo), a1 = e4m3x2_to_half2(lo >> 16);
-            const uint32_t a2 = e4m3x2_to_half2(hi), a3 = e4m3x2_to_half2(hi >> 16);
+            const uint32_t a0 = e4m3x2_to_16bit<__half>(lo), a1 = e4m3x2_to_16bit<__half>(lo >> 16);
+            const uint32_t a2 = e4m3x2_to_16bit<__half>(hi), a3 = e4m3x2_to_16bit<__half>(hi >> 16);
             // (the tile's own sum first, rounded to nearest into the running one: the tensor cores truncate, which over
             // a long list would cost more than the weights' split)
             float sum[4] = {0.f, 0.f, 0.f, 0.f};

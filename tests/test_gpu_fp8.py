@@ -346,3 +346,40 @@ def test_shared_rows_over_an_8_bit_cache_whatever_the_magnitude_of_the_queries(g
     ref, ref_lse = O.decode_attn_dense(q_bits, *p.oracle_kv(), ctx, scale, "bf16/e4m3")
     assert float(np.linalg.norm((got - ref)[~bad])) <= 4e-6 * float(np.linalg.norm(ref[~bad]))
     np.testing.assert_allclose(got_lse[~bad], ref_lse[~bad], rtol=2e-6, atol=2e-6)
+
+
+@pytest.mark.parametrize("group,T,top", [
+    (2, 8000, 31), (8, 8000, 60), (12, 8000, 36), (20, 8000, 31), (33, 8000, 60), (8, 76000, 36), (20, 38000, 36)])
+def test_shared_rows_over_an_8_bit_cache_with_keys_of_zero_where_the_query_is_largest(group, T, top):
+    """A head dimension that K does not use (zeros: a narrower head padded to 128) leaves q free there: its size must not
+    cost the other dimensions anything.  Every third query row has elements near 2^top there and a zero weight in every score;
+    the others are ordinary.  The products left are those of ordinary rows, so the bound is theirs: scores of N(0, 1) carry
+    2^-24 sqrt(128) relative, the rows at most four times that, 3e-6 in the 2-norm."""
+    B, Hkv, D = 2, 2, 128
+    H = group * Hkv
+    p = Fp8Problem(B, H, Hkv, T, D, seed=group + top)
+    rng = np.random.default_rng(top)
+    p.k_bits[..., 96:] = 0
+    p.k = torch.from_numpy(p.k_bits).view(torch.float8_e4m3fn).to(DEV)
+    q = rng.standard_normal((B, H, D)).astype(np.float32)
+    q[:, ::3, 96:] *= np.float32(2.0 ** top)
+    q_bits = round_to_storage(q, "bf16")
+    d_q = torch.from_numpy(q_bits.view(np.int16)).view(torch.bfloat16).to(DEV)
+    out, lse = torch.zeros((B, H, D), device=DEV), torch.zeros((B, H), device=DEV)
+    desc = ssa.make_desc(d_q, p.k, p.v, out)
+    ws = torch.empty(max(ssa.decode_workspace_bytes(desc, T), ssa.decode_spans_workspace_bytes(desc, T, 2)),
+                     dtype=torch.uint8, device=DEV)
+    ctx = [T, 4321]
+    d_ctx = torch.tensor(ctx, dtype=torch.int32, device=DEV)
+    ref, ref_lse = O.decode_attn_dense(q_bits, *p.oracle_kv(), ctx, 1 / np.sqrt(D), "bf16/e4m3")
+    index = torch.arange(T, dtype=torch.int32, device=DEV).expand(B, T).contiguous()
+    spans = torch.tensor([[0, 100], [100, T]] * B, dtype=torch.int32, device=DEV)
+    offs = torch.tensor([0, 2, 4], dtype=torch.int32, device=DEV)
+    for call in (lambda: ssa.decode_attn_dense(desc, d_q, p.k, p.v, d_ctx, out, lse, ws),
+                 lambda: ssa.decode_attn_sparse(desc, d_q, p.k, p.v, d_ctx, index, d_ctx, T, out, lse, ws),
+                 lambda: ssa.decode_attn_spans(desc, d_q, p.k, p.v, d_ctx, offs, spans, 2, T, out, lse, None, None, ws)):
+        call()
+        torch.cuda.synchronize()
+        assert float(np.linalg.norm(out.double().cpu().numpy() - ref)) <= 3e-6 * float(np.linalg.norm(ref))
+        np.testing.assert_allclose(lse.double().cpu().numpy(), ref_lse, rtol=2e-6, atol=2e-6)
+        out.zero_()
