@@ -90,9 +90,10 @@ typedef enum { SSA_F16 = 0, SSA_BF16 = 1, SSA_F32 = 2, SSA_FP8_E4M3 = 3 } ssa_dt
  * selected row.  Grouped query heads over it share the rows they read (D = 128
  * and two or more heads per K/V head), as over a 16-bit cache: the scores and the
  * sums are fp32, the softmax weights enter the second contraction as a pair of
- * fp16 values (22 bits).  Small launches, other groups, D = 64 and the blocked
- * lists take one head per thread block, fp32 throughout (each head re-reads the
- * rows, mostly from L2).
+ * fp16 values (22 bits; weights far below the largest to an absolute 2^-37 of
+ * it, or as many terms as they need above sixteen heads per K/V head).  Small
+ * launches, other groups, D = 64 and the blocked lists take one head per thread
+ * block, fp32 throughout (each head re-reads the rows, mostly from L2).
  */
 typedef struct {
   int32_t B, H, H_kv, D;

@@ -43,7 +43,7 @@
 // the result keeps fp32-level accuracy instead of the 2^-9 of a bf16 weight.
 // Over an 8-bit cache they are fp16 pairs of 2^13 times the weight: 22 bits
 // for the large ones and an absolute error below 2^-37 of the largest for the
-// rest.
+// rest; above sixteen heads (kSplit) further terms hold the rest as well.
 // Included by decode_attn.cu after DecodeParams and its helpers.
 #pragma once
 
@@ -302,10 +302,16 @@ __device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParam
 // kWide serves launches with at most one unit (request x K/V head) per SM and short lists: a whole list is then one
 // block's work, no second pass.
 // kEven (full contexts): even shares, see above; the grid is (even_blocks * head_splits, 1, 1).
-// kSplit: groups of more than kGqaHeads heads; head_splits blocks, side by side, serve heads_per_block of them each.  Over
-// 16-bit rows their weights enter to 22 bits and more, and tiles are summed on their own, as 8-bit rows have it anyway: error
-// of a row against 64 bits 1.5e-7 instead of 1.4..3.2e-6, since one head per block, which served them before, has 1.4..2.5e-7.
-// It costs them a tenth to a fifth (24 requests, 128 heads over 4, 2000 rows: 40.8 -> 48.6 us).
+// kSplit: groups of more than kGqaHeads heads; head_splits blocks, side by side, serve heads_per_block of them each.  One
+// head per block, which served them before, has fp32 weights and an error of a row against 64 bits of 1.5..2.6e-7; smaller
+// groups have 1.4..3.2e-6.  So here tiles are summed on their own, as 8-bit rows have it anyway; bf16 weights enter whole, in
+// three terms; fp16 ones in two (2^-23 of a weight; their exponential itself is good to 2^-22) and, far below the largest
+// one, as many more as they have bits; and the k-steps of fp16 scores are added outside the tensor cores.  Errors then, over
+// N(0, 1) in fp16 / bf16 / 8 bits: 16 x 4096 rows 2.0 / 2.0 / 1.8e-7 (one head per block 2.1 / 2.0 / 2.0e-7), 24 x 2000
+// 2.0 / 2.0 / 1.8e-7 (2.0 / 2.0 / 1.9), 24 x 40 1.2 / 1.2 / 1.1e-7 (1.5); only past some 6000 rows per block the running
+// sums, each of one team, show: 2.7 / 2.7 / 2.6e-7 over 17 x 8 K/V heads of 8190 rows (2.2e-7).  Time, us: 24 requests, 128
+// heads over 4, 2000 rows 48.0 / 50.5 / 52.6; with queries twice and six times as large, whose many small weights take the
+// further terms, 57.9 and 79.0 in fp16, 65.7 and 95.6 over 8 bits; one head per block 258 / 253 / 231.
 template <typename T, int kMode, bool kHi, bool kWide, bool kEven = false, bool kSplit = false>
 __global__ void __launch_bounds__(GqaShape<T, kHi, kWide>::kWarps * 32, kWide ? 1 : 2)
 decode_partial_gqa_kernel(const DecodeParams p) {
@@ -317,9 +323,8 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   constexpr bool kFp8 = kIsFp8<T>;
   using TQ = typename Storage<T>::Query;                // type of the query rows and of a stored output
   using TP = typename std::conditional<kFp8, __half, T>::type;   // type of the weights in the second contraction
-  constexpr bool kFine = kSplit && !kFp8;
   constexpr bool kHalfWeights = std::is_same<TP, __half>::value;
-  constexpr float kUp = kFp8 || (kFine && kHalfWeights) ? 8192.f : 1.f;   // weights (and all they enter) are scaled by this in the loop
+  constexpr float kUp = kFp8 || (kSplit && kHalfWeights) ? 8192.f : 1.f;   // weights (and all they enter) are scaled by this in the loop
   constexpr int kTileBytes = kGqaRows * (kFp8 ? 128 : 256);      // one tensor's tile
   constexpr int kStagedDepth = Shape::kRingBytes / (2 * kTileBytes);
   constexpr int kLiveHeads = 8 * kTeam;
@@ -659,7 +664,15 @@ decode_partial_gqa_kernel(const DecodeParams p) {
             uint32_t a[4];
             ldmatrix_x4(a, ka ^ (ks << 5));
             float (&sum)[4] = (ks & 1) ? s_odd : s;
-            mma_16816<TQ>(sum, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1], sum);
+            if constexpr (kSplit && kHalfWeights) {
+              // (products of fp16 values fill the sum's 24 bits and the tensor cores truncate: k-steps are added here)
+              float step[4] = {0.f, 0.f, 0.f, 0.f};
+              mma_16816<TQ>(step, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1], step);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) sum[e] += step[e];
+            } else {
+              mma_16816<TQ>(sum, a[0], a[1], a[2], a[3], qb[ks][0], qb[ks][1], sum);
+            }
           }
         }
 #pragma unroll
@@ -689,8 +702,10 @@ decode_partial_gqa_kernel(const DecodeParams p) {
             }
           }
         }
-        // weights, split into a 16-bit value and a 16-bit residual, transposed into B fragments of P^T[16 rows, 8 heads]
-        uint32_t pa[2], pr[2], pl[2];                    // pl: what is left of a bf16 weight behind two bf16 terms (kFine)
+        // weights, split into a 16-bit value and a 16-bit residual (kSplit: bf16 into three terms, with which nothing of them
+        // is left), transposed into B fragments of P^T[16 rows, 8 heads]
+        uint32_t pa[2], pr[2], pl[2];
+        bool small = false;                              // kSplit: a weight whose fp16 terms have less than 23 bits
         // (a maximum of -inf: no finite score yet, every weight is 0)
         const float r0 = m[0] > neg_inf() ? m[0] : 0.f, r1 = m[1] > neg_inf() ? m[1] : 0.f;
 #pragma unroll
@@ -703,50 +718,93 @@ decode_partial_gqa_kernel(const DecodeParams p) {
           pa[half] = transpose8x8(w);
           const uint32_t rest = pack2<TP>(w0 - back.x, w1 - back.y);
           pr[half] = transpose8x8(rest);
-          if constexpr (kFine && !kHalfWeights) {
+          if constexpr (kSplit && !kHalfWeights) {
             const float2 mid = unpack2<TP>(rest);
             pl[half] = transpose8x8(pack2<TP>((w0 - back.x) - mid.x, (w1 - back.y) - mid.y));
           }
+          if constexpr (kSplit && kHalfWeights)          // 0 < weight < 1/4 (and not a NaN), by the bits
+            small |= __float_as_uint(w0) - 1u < 0x3e7fffffu || __float_as_uint(w1) - 1u < 0x3e7fffffu;
         }
-        // O^T += V^T . P^T, sixteen dims at a time
-        if constexpr (kFp8) {
-          const uint4 v0 = lds_16B(va), v1 = lds_16B(va + kRowBytes);                          // rows 2 j, 2 j + 1
-          const uint4 v2 = lds_16B(va + 8 * kRowBytes), v3 = lds_16B(va + 9 * kRowBytes);      // rows 2 j + 8, 2 j + 9
-          const uint32_t x0[4] = {v0.x, v0.y, v0.z, v0.w}, x1[4] = {v1.x, v1.y, v1.z, v1.w};
-          const uint32_t x2[4] = {v2.x, v2.y, v2.z, v2.w}, x3[4] = {v3.x, v3.y, v3.z, v3.w};
+        // fragments of V^T, sixteen dims at a time
+        auto for_dims = [&](auto use) {
+          if constexpr (kFp8) {
+            const uint4 v0 = lds_16B(va), v1 = lds_16B(va + kRowBytes);                          // rows 2 j, 2 j + 1
+            const uint4 v2 = lds_16B(va + 8 * kRowBytes), v3 = lds_16B(va + 9 * kRowBytes);      // rows 2 j + 8, 2 j + 9
+            const uint32_t x0[4] = {v0.x, v0.y, v0.z, v0.w}, x1[4] = {v1.x, v1.y, v1.z, v1.w};
+            const uint32_t x2[4] = {v2.x, v2.y, v2.z, v2.w}, x3[4] = {v3.x, v3.y, v3.z, v3.w};
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            // bytes 2 (t & 1) and 2 (t & 1) + 1 of both rows of a pair, interleaved
-            const uint32_t sel = (t & 1) ? 0x7362u : 0x5140u;
-            const uint32_t lo = __byte_perm(x0[t >> 1], x1[t >> 1], sel), hi = __byte_perm(x2[t >> 1], x3[t >> 1], sel);
-            const uint32_t a0 = e4m3x2_to_16bit<__half>(lo), a1 = e4m3x2_to_16bit<__half>(lo >> 16);
-            const uint32_t a2 = e4m3x2_to_16bit<__half>(hi), a3 = e4m3x2_to_16bit<__half>(hi >> 16);
-            // (the tile's own sum first, rounded to nearest into the running one: the tensor cores truncate, which over
-            // a long list would cost more than the weights' split)
-            float sum[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_16816<TP>(sum, a0, a1, a2, a3, pr[0], pr[1], sum);
-            mma_16816<TP>(sum, a0, a1, a2, a3, pa[0], pa[1], sum);
+            for (int t = 0; t < 8; ++t) {
+              // bytes 2 (t & 1) and 2 (t & 1) + 1 of both rows of a pair, interleaved
+              const uint32_t sel = (t & 1) ? 0x7362u : 0x5140u;
+              const uint32_t lo = __byte_perm(x0[t >> 1], x1[t >> 1], sel), hi = __byte_perm(x2[t >> 1], x3[t >> 1], sel);
+              const uint32_t a[4] = {e4m3x2_to_16bit<__half>(lo), e4m3x2_to_16bit<__half>(lo >> 16),
+                                     e4m3x2_to_16bit<__half>(hi), e4m3x2_to_16bit<__half>(hi >> 16)};
+              use(t, a);
+            }
+          } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) o[t][e] += sum[e];
+            for (int t = 0; t < 8; ++t) {
+              uint32_t a[4];                             // dims 16t..+7, 16t+8..+15 of rows 0-7; the same of rows 8-15
+              ldmatrix_x4_trans(a, va ^ (t << 5));
+              use(t, a);
+            }
           }
-        } else {
+        };
+        if constexpr (kSplit && kHalfWeights) {
+          // Weights below 2^-15 of the largest, of which the terms hold less, down to nothing at 2^-38: further terms, the
+          // first 2^24 up and each next 2^11, until nothing is left (nine reach the last bit of the smallest normal one).
+          if (__any_sync(0xffffffffu, small)) {          // warp-uniform; costs a tile of such rows about half a tile per term
+            float left[4];
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            uint32_t a[4];                               // dims 16t..+7, 16t+8..+15 of rows 0-7; the same of rows 8-15
-            ldmatrix_x4_trans(a, va ^ (t << 5));
-            if constexpr (kFine) {
-              float sum[4] = {0.f, 0.f, 0.f, 0.f};
-              if constexpr (!kHalfWeights) mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pl[0], pl[1], sum);
-              mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pr[0], pr[1], sum);
-              mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pa[0], pa[1], sum);
+            for (int e = 0; e < 4; e += 2) {
+              const float w0 = fast_exp2(s[e] - r0) * kUp, w1 = fast_exp2(s[e + 1] - r1) * kUp;
+              const float2 first = unpack2<TP>(pack2<TP>(w0, w1));
+              const float2 second = unpack2<TP>(pack2<TP>(w0 - first.x, w1 - first.y));
+              left[e] = (w0 - first.x) - second.x;
+              left[e + 1] = (w1 - first.y) - second.y;
+            }
+            float up = 16777216.f, unit = 1.f;
+#pragma unroll 1
+            for (int term = 0; term < 9; ++term) {
+              const bool some = fabsf(left[0]) > 0.f || fabsf(left[1]) > 0.f || fabsf(left[2]) > 0.f || fabsf(left[3]) > 0.f;
+              if (!__any_sync(0xffffffffu, some)) break;
+              unit /= up;
+              uint32_t more[2];
 #pragma unroll
-              for (int e = 0; e < 4; ++e) o[t][e] += sum[e];
-            } else {
-              mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pa[0], pa[1], o[t]);
-              mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pr[0], pr[1], o[t]);
+              for (int half = 0; half < 2; ++half) {
+                const float w0 = left[2 * half] * up, w1 = left[2 * half + 1] * up;
+                const uint32_t w = pack2<TP>(w0, w1);
+                const float2 back = unpack2<TP>(w);
+                more[half] = transpose8x8(w);
+                left[2 * half] = w0 - back.x;
+                left[2 * half + 1] = w1 - back.y;
+              }
+              for_dims([&](int t, const uint32_t (&a)[4]) {
+                float sum[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_16816<TP>(sum, a[0], a[1], a[2], a[3], more[0], more[1], sum);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) o[t][e] = fmaf(sum[e], unit, o[t][e]);
+              });
+              up = 2048.f;
             }
           }
         }
+        // O^T += V^T . P^T
+        for_dims([&](int t, const uint32_t (&a)[4]) {
+          if constexpr (kFp8 || kSplit) {
+            // (the tile's own sum first, rounded to nearest into the running one: the tensor cores truncate, which over
+            // a long list would cost more than the weights' split)
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+            if constexpr (kSplit && !kHalfWeights) mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pl[0], pl[1], sum);
+            mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pr[0], pr[1], sum);
+            mma_16816<TP>(sum, a[0], a[1], a[2], a[3], pa[0], pa[1], sum);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[t][e] += sum[e];
+          } else {
+            mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pa[0], pa[1], o[t]);
+            mma_16816<TP>(o[t], a[0], a[1], a[2], a[3], pr[0], pr[1], o[t]);
+          }
+        });
       }
       cp_async_wait<0>();                                // only empty groups can be pending here
     }

@@ -6,10 +6,11 @@ import torch
 
 from oracle import ssa_oracle as O
 from paper_2404_09336_b200 import ssa
+from paper_2404_09336_b200.inputs import round_to_storage
 from paper_2404_09336_b200.runner import bits_to_tensor
 
 from gpu_util import DEV, random_bits
-from test_gpu_fp8 import Fp8Problem
+from test_gpu_fp8 import Fp8Problem, to_e4m3_bits
 
 pytestmark = pytest.mark.gpu
 
@@ -23,6 +24,13 @@ def problem(dtype, B, H, Hkv, T, seed):
     return (*(bits_to_tensor(x, dtype).to(DEV) for x in bits), *bits, dtype)
 
 
+def upload(dtype, q_bits, k_bits, v_bits):
+    if dtype != "fp8":
+        return tuple(bits_to_tensor(x, dtype).to(DEV) for x in (q_bits, k_bits, v_bits))
+    return (bits_to_tensor(q_bits, "bf16").to(DEV),
+            *(torch.from_numpy(x).view(torch.float8_e4m3fn).to(DEV) for x in (k_bits, v_bits)))
+
+
 @pytest.mark.parametrize("dtype,B,Hkv,G,T,counts", [
     ("bf16", 1, 1, 17, 300, [129]),                             # small: one head per block
     ("bf16", 3, 3, 17, 1300, [1300, 0, 17]),                    # 9 + 8 heads, several chunks; an empty list
@@ -34,9 +42,9 @@ def problem(dtype, B, H, Hkv, T, seed):
     ("fp8", 2, 2, 32, 38000, [129, 1000]),
 ])
 def test_large_groups_against_the_oracle(dtype, B, Hkv, G, T, counts):
-    """fp32 output.  Weights carry 22 bits or more (or an absolute 2^-37), a tile's products are summed on their own, sums
-    are fp32: independent errors of 2^-22 per weight or product stay below 2.4e-7 of the result in the 2-norm (measured:
-    1.0e-7..1.9e-7; one head per block 1.4e-7..2.5e-7); four times that is asserted."""
+    """fp32 output.  Weights carry 23 bits or more, a tile's products are summed on their own, sums are fp32: independent errors
+    of 2^-22 per weight or product stay below 2.4e-7 of the result in the 2-norm (measured: 1.0e-7..1.9e-7; one head per block
+    1.4e-7..2.5e-7); four times that is asserted."""
     H, D = G * Hkv, 128
     q, k, v, qb, kb, vb, name = problem(dtype, B, H, Hkv, T, seed=G + T)
     rng = np.random.default_rng(T)
@@ -111,3 +119,74 @@ def test_large_group_in_the_workspace_of_one_head_per_block():
         assert bool((ws[nbytes:] == 0xA5).all())
     ssa.decode_attn_sparse_noalloc(desc, q, k, v, d_ctx, idx, d_cnt, T, out, None, None)
     check()
+
+
+# dtype, B, Hkv, G, T: lists (one large block per SM, several chunks, one block) and full contexts, those of the last two cut
+# on the device
+SHAPES = [("bf16", 30, 2, 32, 300), ("f16", 2, 4, 24, 1100), ("fp8", 2, 2, 33, 2500), ("f16", 150, 1, 20, 70),
+          ("f16", 1, 1, 20, 76000), ("bf16", 1, 2, 17, 76000), ("fp8", 1, 2, 32, 38000)]
+
+
+class _PerHead:
+    """A cache of K/V heads, looked up by query head."""
+
+    def __init__(self, bits, group):
+        self.bits, self.group = bits, group
+
+    def __getitem__(self, at):
+        return self.bits[at[0], at[1] // self.group]
+
+
+def reference(q_bits, k_bits, v_bits, B, T, G, scale, name):
+    """Full contexts of the first, the middle and the last request, first and last heads of the first and the last K/V head."""
+    H = q_bits.shape[1]
+    kv = (_PerHead(x, G) for x in (k_bits, v_bits))
+    return O.decode_attn_dense(q_bits, *kv, [T] * B, scale, name, heads=sorted({0, G - 1, H - G, H - 1}),
+                               seqs=sorted({0, B // 2, B - 1}))
+
+
+def all_calls(desc, q, k, v, T, out, lse):
+    """Index lists, a paged cache, span lists (by every warp and by one) and full contexts of all T rows."""
+    B, Hkv, D = q.shape[0], k.shape[1], q.shape[2]
+    need = max(ssa.decode_spans_workspace_bytes(desc, T, 40), ssa.decode_workspace_bytes(desc, T))
+    ws = torch.empty(need, dtype=torch.uint8, device=DEV)
+    ctx = torch.full((B,), T, dtype=torch.int32, device=DEV)
+    index = torch.arange(T, dtype=torch.int32, device=DEV).expand(B, T).contiguous()
+    raw = (lambda x: x.view(torch.uint8)) if k.element_size() == 1 else (lambda x: x)
+    kp, vp = (raw(x).transpose(1, 2).reshape(B * T, 1, Hkv, D).contiguous().view(x.dtype) for x in (k, v))
+    table = torch.arange(B * T, dtype=torch.int32, device=DEV).view(B, T)
+    paging, paged = ssa.make_paging(table, 1, B * T), ssa.make_desc_paged(q, kp, vp, out, T, scale=desc.scale)
+    few = torch.tensor([[0, T // 2], [T // 2, T]] * B, dtype=torch.int32, device=DEV)
+    many = torch.tensor([[0, T // 2]] * 38 + [[T // 2, T], [5, 9]], dtype=torch.int32, device=DEV).repeat(B, 1)
+    step = lambda n: torch.arange(0, n * B + 1, n, dtype=torch.int32, device=DEV)
+    yield "index lists", lambda: ssa.decode_attn_sparse(desc, q, k, v, ctx, index, ctx, T, out, lse, ws)
+    yield "a paged cache", lambda: ssa.decode_attn_sparse_paged(paged, q, kp, vp, paging, ctx, index, ctx, T, out, lse, ws)
+    yield "full contexts", lambda: ssa.decode_attn_dense(desc, q, k, v, ctx, out, lse, ws)
+    yield "few spans", lambda: ssa.decode_attn_spans(desc, q, k, v, ctx, step(2), few, 2, T, out, lse, None, None, ws)
+    yield "many spans", lambda: ssa.decode_attn_spans(desc, q, k, v, ctx, step(40), many, 40, T, out, lse, None, None, ws)
+
+
+@pytest.mark.parametrize("dtype,B,Hkv,G,T", SHAPES)
+def test_rows_far_below_the_largest_weight_of_a_large_group(dtype, B, Hkv, G, T):
+    """Every seventh row has a score 20 above the others' (every 21st, 40) and a V row of zeros, so the output is what the
+    light rows add: their weights, 2^-29 and 2^-58 of the largest, must be fp32 values like all others and not be cut off.
+    Bound: scores of 40 are 58 in log2 units, where fp32 values lie 2^-18 apart: 2.7e-6 of a weight; 1e-5 is asserted."""
+    H, D = G * Hkv, 128
+    q, k, v, qb, kb, vb, name = problem(dtype, B, H, Hkv, T, seed=T)
+    bits = lambda x, what: (to_e4m3_bits if what == "fp8" else lambda y: round_to_storage(y, what))(np.full(1, x, np.float32))[0]
+    qb[..., 0], kb[..., 0] = bits(8, "bf16" if dtype == "fp8" else dtype), 0
+    heavy = np.arange(0, T, 7)
+    kb[:, :, heavy, 0], kb[:, :, heavy[::3], 0], vb[:, :, heavy] = bits(20, dtype), bits(40, dtype), 0
+    q, k, v = upload(dtype, qb, kb, vb)
+    out, lse = torch.zeros((B, H, D), device=DEV), torch.zeros((B, H), device=DEV)
+    desc = ssa.make_desc(q, k, v, out, scale=0.125)
+    ref, ref_lse = reference(qb, kb, vb, B, T, G, 0.125, name)
+    some = ~np.isnan(ref_lse)
+    assert 0 < np.abs(ref[some]).max() < 2.0 ** -50
+    for what, call in all_calls(desc, q, k, v, T, out, lse):
+        call()
+        torch.cuda.synchronize()
+        got = out.double().cpu().numpy()[some]
+        assert float(np.linalg.norm(got - ref[some])) <= 1e-5 * float(np.linalg.norm(ref[some])), what
+        np.testing.assert_allclose(lse.double().cpu().numpy()[some], ref_lse[some], rtol=2e-6, atol=2e-6, err_msg=what)
+        out.fill_(7.0)
