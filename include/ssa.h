@@ -164,7 +164,9 @@ size_t ssa_decode_workspace_bytes(const ssa_attn_desc* desc, int32_t max_selecte
  * sorted; a duplicated entry is counted twice; an entry outside
  * [0, ctx_lens[b]) is skipped (SSA_DEV_BAD_INDEX).  counts[b] == 0 gives a
  * zero output row and lse = -inf; a NaN in a selected key, or in a query, makes
- * the row and lse of the heads it enters NaN.  `max_selected` is a host-side upper bound
+ * the row and lse of the heads it enters NaN.  An infinity in a selected row of V
+ * is one in the output (two of different sign: NaN), but a NaN where 2 to 16 query
+ * heads or (head, token) pairs of a K/V head share the rows they read (D = 128).  `max_selected` is a host-side upper bound
  * on every counts[b] (1 <= max_selected <= index_stride); a larger count is
  * clamped to it (SSA_DEV_BAD_COUNT).
  *

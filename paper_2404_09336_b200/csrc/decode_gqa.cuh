@@ -299,6 +299,33 @@ __device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParam
   __syncthreads();
 }
 
+// What the rows of V whose value at `v` is not finite add to it: infinities of their sign, or a NaN.  Called by one thread for
+// its dim where the split weights (kSplit) have made a NaN of it; the scores as the kernel has them, the weights whole.
+template <typename T, typename Position>
+__device__ __forceinline__ float sum_of_infinities(const T* q, const char* k, uint32_t k_row_bytes, const char* v,
+                                                uint32_t v_row_bytes, int rows, Position position, float scale_log2, float top) {
+  constexpr int kAhead = 8;
+  float A = 0.f;
+  for (int r0 = 0; r0 < rows; r0 += kAhead) {
+    int pos[kAhead];
+    float value[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      pos[i] = r0 + i < rows ? position(r0 + i) : -1;
+      value[i] = pos[i] >= 0 ? to_float(*reinterpret_cast<const T*>(v + (uint64_t)(uint32_t)pos[i] * v_row_bytes)) : 0.f;
+    }
+#pragma unroll 1
+    for (int i = 0; i < kAhead; ++i) {
+      if (fabsf(value[i]) <= 3.40282347e38f) continue;
+      const T* const row = reinterpret_cast<const T*>(k + (uint64_t)(uint32_t)pos[i] * k_row_bytes);
+      float score = 0.f;
+      for (int d = 0; d < 128; ++d) score = fmaf(to_float(q[d]), to_float(row[d]), score);
+      A = fmaf(fast_exp2(score * scale_log2 - top), value[i], A);
+    }
+  }
+  return A;
+}
+
 // kWide serves launches with at most one unit (request x K/V head) per SM and short lists: a whole list is then one
 // block's work, no second pass.
 // kEven (full contexts): even shares, see above; the grid is (even_blocks * head_splits, 1, 1).
@@ -444,6 +471,20 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     const int most = kEven ? min(piece_end - piece, (c + kEvenRows - 1) / kEvenRows) * kEvenRows : p.chunk;
     const int cnt = max(0, min(most, c - start));
 
+    // position -> what the tile loop uses: -1 for an entry outside the context, the pool row for a paged cache
+    auto checked = [&](int v) {
+      if (v < 0 || v >= n) {
+        flags |= SSA_DEV_BAD_INDEX;
+        return -1;
+      }
+      if (p.page_table) {
+        const int page = __ldg(p.page_table + (int64_t)b * p.page_table_stride + (v >> p.page_shift));
+        if ((unsigned)page < (unsigned)p.n_pages) return (page << p.page_shift) | (v & p.page_mask);
+        flags |= SSA_DEV_BAD_INDEX;
+        return -1;
+      }
+      return v;
+    };
     auto stage_window = [&](int w0, int wn) {
       if constexpr (kMode == kSpans) {
         int32_t* out = (kvh == 0 && part == 0 && p.index_out) ? p.index_out + (int64_t)b * p.index_stride + start + w0 : nullptr;
@@ -454,20 +495,6 @@ decode_partial_gqa_kernel(const DecodeParams p) {
         }
         return;
       }
-      // position -> what the tile loop uses: -1 for an entry outside the context, the pool row for a paged cache
-      auto checked = [&](int v) {
-        if (v < 0 || v >= n) {
-          flags |= SSA_DEV_BAD_INDEX;
-          return -1;
-        }
-        if (p.page_table) {
-          const int page = __ldg(p.page_table + (int64_t)b * p.page_table_stride + (v >> p.page_shift));
-          if ((unsigned)page < (unsigned)p.n_pages) return (page << p.page_shift) | (v & p.page_mask);
-          flags |= SSA_DEV_BAD_INDEX;
-          return -1;
-        }
-        return v;
-      };
       if (listed && w0 == 0) {                             // the entries requested ahead cover any first window
 #pragma unroll
         for (int jj = 0; jj < kAhead; ++jj) {
@@ -479,6 +506,15 @@ decode_partial_gqa_kernel(const DecodeParams p) {
       const int32_t* row = listed ? p.index + (int64_t)b * p.index_stride + start + w0 : nullptr;
       for (int i = tid; i < wn; i += kThreads)             // no list: the position itself (a paged full context)
         s_idx[i] = checked(row ? __ldg(row + i) : start + w0 + i);
+    };
+    // the cache row of entry i of the block, -1 if there is none
+    auto position = [&](int i) {
+      if constexpr (kMode == kSpans)
+        return warp_merge ? span_position(s_wruns[warp], runs, start + i) : span_position(s_runs, start + i);
+      else if constexpr (kMode == kIndex)
+        return checked(listed ? __ldg(p.index + (int64_t)b * p.index_stride + start + i) : start + i);
+      else
+        return start + i;
     };
     // a list chunk of up to kStagedShortList entries is one window (no meeting in mid-chunk); longer ones go by 512
     const int window = kSparse ? (cnt <= kStagedShortList ? kStagedShortList : kStagedWindow) : Shape::kDenseWindow;
@@ -847,7 +883,8 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     __syncthreads();
     // 128 threads finish a head: thread d its dim d
     const int d = tid % D;
-    for (int i = tid / D; i < heads; i += kThreads / D) {
+    bool infinite = false;                               // kSplit: an infinity in V left a NaN (finish_head has skipped it)
+    auto finish_head = [&](int i, auto again) {
       const int h = kvh * G + h0 + i;
       float M = neg_inf();
 #pragma unroll
@@ -859,6 +896,19 @@ decode_partial_gqa_kernel(const DecodeParams p) {
         L = fmaf(s_l[w][i], wgt, L);
         A = fmaf(s_acc[w][i][gqa_column(d)], wgt, A);
       }
+      if constexpr (kSplit && !kFp8) {
+        const bool lost = A != A && L == L;
+        if constexpr (decltype(again)::value) {
+          if (!lost) return;
+          const TQ* const q_row = reinterpret_cast<const TQ*>(p.q) + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh;
+          A = M > neg_inf() ? sum_of_infinities<T>(q_row, kbase, p.k_row_bytes, vbase + d * sizeof(T), p.v_row_bytes, cnt,
+                                                   position, p.scale_log2, M)
+                            : 0.f;
+        } else if (lost) {
+          infinite = true;
+          return;
+        }
+      }
       if (kEven ? taken == unit_pieces : p.n_chunks == 1) {
         store_row_value<TQ>(p, b, h, d, M, L, A);
       } else {
@@ -867,7 +917,11 @@ decode_partial_gqa_kernel(const DecodeParams p) {
         p.ws_acc[slot * D + d] = A;
         if (d == 0) p.ws_ml[slot] = make_float2(M, L);
       }
-    }
+    };
+    for (int i = tid / D; i < heads; i += kThreads / D) finish_head(i, std::false_type{});
+    if constexpr (kSplit && !kFp8)
+      if (infinite)
+        for (int i = tid / D; i < heads; i += kThreads / D) finish_head(i, std::true_type{});
     if constexpr (!kEven) break;
     piece += taken;
     if (piece >= piece_end) break;

@@ -190,3 +190,38 @@ def test_rows_far_below_the_largest_weight_of_a_large_group(dtype, B, Hkv, G, T)
         assert float(np.linalg.norm(got - ref[some])) <= 1e-5 * float(np.linalg.norm(ref[some])), what
         np.testing.assert_allclose(lse.double().cpu().numpy()[some], ref_lse[some], rtol=2e-6, atol=2e-6, err_msg=what)
         out.fill_(7.0)
+
+
+@pytest.mark.parametrize("dtype,B,Hkv,G,T", [s for s in SHAPES if s[0] != "fp8"])
+def test_infinities_in_v_reach_the_rows_of_a_large_group(dtype, B, Hkv, G, T):
+    """An infinity in a selected row of V is one in the output, two of different sign or a NaN make a NaN, and no other dim is
+    touched; a NaN in K makes the rows of its heads NaN.  As one head per block has it."""
+    H, D = G * Hkv, 128
+    q, k, v, qb, kb, vb, name = problem(dtype, B, H, Hkv, T, seed=T + 1)
+    inf, nan = ({"bf16": 0x7F80, "f16": 0x7C00}[dtype], {"bf16": 0x7FC0, "f16": 0x7E00}[dtype])
+    vb[:, 0, T // 3, 5], vb[:, 0, T - 1, 6], vb[:, 0, 0, 6] = inf, inf | 0x8000, inf | 0x8000
+    vb[:, 0, 1, 7], vb[:, 0, T - 2, 7], vb[:, 0, T // 2, 126] = inf, inf | 0x8000, nan
+    vb[:, Hkv - 1, T // 2 + 1, 127] = inf
+    q, k, v = upload(dtype, qb, kb, vb)
+    out, lse = torch.zeros((B, H, D), device=DEV), torch.zeros((B, H), device=DEV)
+    desc = ssa.make_desc(q, k, v, out)
+    ref, ref_lse = reference(qb, kb, vb, B, T, G, 1 / np.sqrt(D), name)
+    some = ~np.isnan(ref_lse)
+    some_first, some_last = some & (np.arange(H) < G), some & (np.arange(H) >= H - G)
+    assert np.isposinf(ref[some_first][:, 5]).all() and np.isneginf(ref[some_first][:, 6]).all()
+    assert np.isnan(ref[some_first][:, [7, 126]]).all() and np.isposinf(ref[some_last][:, 127]).all()
+    for what, call in all_calls(desc, q, k, v, T, out, lse):
+        call()
+        torch.cuda.synchronize()
+        np.testing.assert_allclose(out.double().cpu().numpy()[some], ref[some], rtol=1e-4, atol=1e-5, err_msg=what)
+        np.testing.assert_allclose(lse.double().cpu().numpy()[some], ref_lse[some], rtol=2e-6, atol=2e-6, err_msg=what)
+        out.fill_(7.0)
+    kb[:, 0, T // 4, 9] = nan
+    q, k, v = upload(dtype, qb, kb, vb)
+    for what, call in all_calls(desc, q, k, v, T, out, lse):
+        call()
+        torch.cuda.synchronize()
+        assert bool(out[:, :G].isnan().all()) and bool(lse[:, :G].isnan().all()), what
+        if Hkv > 1:
+            got = out.double().cpu().numpy()[some_last]
+            np.testing.assert_allclose(got, ref[some_last], rtol=1e-4, atol=1e-5, err_msg=what)
