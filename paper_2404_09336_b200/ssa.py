@@ -133,7 +133,8 @@ lib = _load()
 LIBRARY_PATH = lib._name
 _build.build_binding()              # no-op when the in-tree binding is current
 from . import _ssa_call as _call    # noqa: E402
-_call.bind({name: C.cast(getattr(lib, name), C.c_void_p).value
+_call.bind({"ssa_attn_desc": AttnDesc, "ssa_step": Step, "ssa_paging": Paging} |
+           {name: C.cast(getattr(lib, name), C.c_void_p).value
             for name in ("ssa_spans_to_index", "ssa_decode_attn_sparse", "ssa_decode_attn_spans",
                          "ssa_decode_attn_sparse_multiq", "ssa_decode_attn_dense_multiq", "ssa_spans_to_blockmask",
                          "ssa_decode_attn_blockmask", "ssa_decode_attn_sparse_paged", "ssa_decode_attn_dense_paged",

@@ -107,3 +107,32 @@ def test_wrong_arguments_raise_before_the_entry_point():
     assert not got
     # another library's binding in the same process is its own
     assert ssa.decode_attn_dense(d["desc"], None, None, None, None, None, stream=0, check=False) == ssa.ERR_NULL
+
+
+class _Longer(ssa.AttnDesc):
+    _fields_ = [("note", C.c_int64)]
+
+
+def test_only_the_descriptor_s_own_class_is_taken():
+    """Null tensors: a call that gets past its descriptor is refused by the library, not by the binding."""
+    tail = (None,) * 8 + (0,)
+    big = type("Big", (C.Structure,), {"_fields_": [("x", C.c_char * 400)]})()
+    for wrong in (ssa.Step(), ssa.Paging(), big, bytes(400), bytearray(112), np.zeros(14, np.int64), None, 5):
+        with pytest.raises(TypeError, match="ssa_attn_desc"):
+            ssa._call.decode_attn_dense(wrong, *tail)
+        if wrong is not None:
+            with pytest.raises(TypeError, match="ssa_paging"):
+                if isinstance(wrong, ssa.Paging):
+                    wrong = ssa.AttnDesc()
+                ssa._call.decode_attn_dense_paged(ssa.AttnDesc(), None, None, None, wrong, *tail[3:])
+    for wrong in (ssa.AttnDesc(), bytes(400), big):
+        with pytest.raises(TypeError, match="ssa_step"):
+            ssa._call.decode_step(ssa.AttnDesc(), wrong, 0)
+    for right in (ssa.AttnDesc(), _Longer()):
+        assert ssa._call.decode_attn_dense(right, *tail) == ssa.ERR_NULL
+    # bound without classes: a buffer of the exact size
+    module, got, _ = bound()
+    for wrong in (ssa.Step(), bytes(C.sizeof(ssa.AttnDesc) + 1)):
+        with pytest.raises(TypeError):
+            module.decode_attn_dense(wrong, *tail)
+    assert not got and module.decode_attn_dense(ssa.AttnDesc(), *tail) == 3
