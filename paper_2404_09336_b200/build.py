@@ -1,4 +1,4 @@
-"""Compile libssa.so (sm_100a) in-tree with nvcc, and the Python calls into it (_ssa_call.so) with gcc.
+"""Compile libssa.so (sm_100a) in-tree with nvcc, and the Python calls into it (_ssa_call.*.so) with gcc.
 
     python -m paper_2404_09336_b200.build [-o OUT] [-DNAME=VALUE ...]
 """
@@ -18,7 +18,8 @@ LIB = os.path.join(HERE, "libssa.so")
 PROBE_SRC = os.path.join(HERE, "probe", "gather_probe.cu")
 PROBE_LIB = os.path.join(HERE, "libssa_probe.so")
 BINDING_SRC = os.path.join(HERE, "binding", "ssa_call.c")
-BINDING = os.path.join(HERE, "_ssa_call.so")
+# (the suffix names the interpreter whose C interface it was compiled for: another one builds its own)
+BINDING = os.path.join(HERE, "_ssa_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -77,7 +78,7 @@ def build_binding(force: bool = False) -> str:
         return BINDING
     gcc = shutil.which("gcc") or shutil.which("cc")
     if gcc is None:
-        raise RuntimeError("gcc not found: _ssa_call.so cannot be built")
+        raise RuntimeError("gcc not found: _ssa_call cannot be built")
     tmp = BINDING + f".tmp{os.getpid()}"
     cmd = [gcc, "-shared", "-fPIC", "-O2", "-Wall", "-I", sysconfig.get_paths()["include"], "-I", os.path.dirname(header),
            "-o", tmp, BINDING_SRC]

@@ -2,14 +2,18 @@
 
 Every function takes torch CUDA tensors (used purely as device memory) and
 hands their addresses, sizes and strides to the C entry point of the same
-name; the calls of a decode step do so in binding/ssa_call.c, the rest through
-ctypes.  Nothing is computed here, and there is no fallback: if the shared
-library or the binding cannot be loaded the import fails.
+name; the calls of a decode step do so in binding/ssa_call.c (through ctypes, with
+a warning, where that cannot be compiled), the rest through ctypes.  Nothing is
+computed here, and there is no fallback: if the shared library cannot be loaded
+the import fails.
 """
 from __future__ import annotations
 
 import ctypes as C
+import functools
+import importlib.util
 import os
+import warnings
 
 import torch
 
@@ -131,15 +135,74 @@ def _load():
 
 lib = _load()
 LIBRARY_PATH = lib._name
-_build.build_binding()              # no-op when the in-tree binding is current
-from . import _ssa_call as _call    # noqa: E402
-_call.bind({"ssa_attn_desc": AttnDesc, "ssa_step": Step, "ssa_paging": Paging} |
-           {name: C.cast(getattr(lib, name), C.c_void_p).value
-            for name in ("ssa_spans_to_index", "ssa_decode_attn_sparse", "ssa_decode_attn_spans",
-                         "ssa_decode_attn_sparse_multiq", "ssa_decode_attn_dense_multiq", "ssa_spans_to_blockmask",
-                         "ssa_decode_attn_blockmask", "ssa_decode_attn_sparse_paged", "ssa_decode_attn_dense_paged",
-                         "ssa_refs_to_index", "ssa_refs_to_spans", "ssa_decode_step", "ssa_decode_attn_sparse_noalloc",
-                         "ssa_decode_attn_dense")})
+
+# The calls of a decode step and their arguments, as binding/ssa_call.c reads them: D, S, P structure (P: or None), i integer,
+# t tensor or None, r the same and its row stride (R: behind the next tensor), w and its bytes, n and its number of elements.
+_CALLS = {
+    "spans_to_index": "ttnrtti",
+    "decode_attn_sparse": "Dttttrtittwti",
+    "decode_attn_spans": "Dttttttiittrtwti",
+    "decode_attn_sparse_multiq": "Diiittttrtittwti",
+    "decode_attn_dense_multiq": "Diiittttttwti",
+    "spans_to_blockmask": "ttniRttti",
+    "decode_attn_blockmask": "DttttRttiittwti",
+    "decode_attn_sparse_paged": "DtttPtrtittwti",
+    "decode_attn_dense_paged": "DtttPtttwti",
+    "refs_to_index": "ttttttttnrtti",
+    "refs_to_spans": "ttttttttnttiti",
+    "decode_step": "DSi",
+    "decode_attn_sparse_noalloc": "Dttttrtittti",
+    "decode_attn_dense": "Dttttttwti",
+}
+
+
+class _CtypesCalls:
+    """The calls of binding/ssa_call.c through ctypes (some 7 us slower each), where it cannot be compiled."""
+
+    def __init__(self, library):
+        for name in _CALLS:
+            setattr(self, name, functools.partial(self._call, name, getattr(library, "ssa_" + name)))
+
+    @staticmethod
+    def _call(name, entry, *args):
+        kinds, given, behind = _CALLS[name], [], []
+        if len(args) != len(kinds):
+            raise TypeError(f"{name}: {len(args)} arguments, {len(kinds)} wanted")
+        for kind, a in zip(kinds, args):
+            if kind == "i":
+                given.append(int(a))
+            elif kind in "DSP":
+                given.append(None if kind == "P" and a is None else C.byref(a))
+            else:
+                given.append(None if a is None else C.c_void_p(a.data_ptr()))
+                given += behind
+                behind = [0 if a is None else _row_stride(a)] if kind == "R" else []
+                if kind == "n":
+                    given.append(a.numel())
+                elif kind == "r":
+                    given.append(0 if a is None else _row_stride(a))
+                elif kind == "w":
+                    given.append(0 if a is None else a.numel() * a.element_size())
+        if name.startswith("refs"):
+            given[:9] = [C.byref(AnchorTables(*given[:9]))]
+        return entry(*given)
+
+
+def _load_calls():
+    try:
+        path = _build.build_binding()   # no-op when the in-tree binding is current
+    except RuntimeError as e:           # a finished library on a machine without a C compiler or Python's headers
+        warnings.warn(f"calls go through ctypes, some 7 us slower each: {e}", RuntimeWarning, stacklevel=2)
+        return _CtypesCalls(lib)
+    spec = importlib.util.spec_from_file_location(__package__ + "._ssa_call", path)
+    calls = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(calls)
+    calls.bind({"ssa_attn_desc": AttnDesc, "ssa_step": Step, "ssa_paging": Paging} |
+               {"ssa_" + name: C.cast(getattr(lib, "ssa_" + name), C.c_void_p).value for name in _CALLS})
+    return calls
+
+
+_call = _load_calls()
 
 
 def status_string(code: int) -> str:

@@ -2,6 +2,8 @@
 entry points are Python callbacks with the C signatures, so nothing here needs a GPU."""
 import ctypes as C
 import importlib.util
+import sysconfig
+import types
 
 import numpy as np
 import pytest
@@ -136,3 +138,31 @@ def test_only_the_descriptor_s_own_class_is_taken():
         with pytest.raises(TypeError):
             module.decode_attn_dense(wrong, *tail)
     assert not got and module.decode_attn_dense(ssa.AttnDesc(), *tail) == 3
+
+
+def test_each_interpreter_has_a_binding_of_its_own():
+    assert build.BINDING.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and ssa._call.__file__ == build.BINDING
+
+
+def test_calls_go_through_ctypes_where_the_binding_cannot_be_built(monkeypatch):
+    """A finished library, no compiler: the import warns, and every argument arrives as through the binding."""
+    def no_compiler():
+        raise RuntimeError("gcc not found")
+    monkeypatch.setattr(build, "build_binding", no_compiler)
+    with pytest.warns(RuntimeWarning, match="gcc not found"):
+        calls = ssa._load_calls()
+    assert calls.decode_attn_dense(ssa.AttnDesc(), *(None,) * 8, 0) == ssa.ERR_NULL
+    with pytest.raises((TypeError, C.ArgumentError)):
+        calls.decode_attn_dense(ssa.Step(), *(None,) * 8, 0)
+    monkeypatch.undo()
+    module, got, keep = bound()
+    through = ssa._CtypesCalls(types.SimpleNamespace(**{"ssa_" + name: f for name, f in zip(CALLS, keep)}))
+    optional = {"lse", "ws", "status", "paging"}
+    for rows in (1, 3):
+        d = values(rows)
+        for name, (args, _) in CALLS.items():
+            for absent in (set(), optional | ({"idx"} if "attn" in name else set())):
+                given = [None if w in absent else d[w] if w in d else int(w) for w in args.split()]
+                assert getattr(module, name)(*given) == 3
+                want = got.pop(name)
+                assert getattr(through, name)(*given) == 3 and got.pop(name) == want, name
