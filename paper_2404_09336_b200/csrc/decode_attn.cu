@@ -644,6 +644,12 @@ static int block_warps(const ssa_attn_desc* d, long long blocks, int rows) {
   return warps;
 }
 
+// Bytes of the partial results (accumulator row, maximum and sum) of `triples` (row, chunk) pairs, and of the accumulators.
+static size_t triples_bytes(const ssa_attn_desc* d, size_t triples, size_t* acc_bytes) {
+  *acc_bytes = (triples * d->D * sizeof(float) + 255) / 256 * 256;
+  return *acc_bytes + (triples * sizeof(float2) + 255) / 256 * 256;
+}
+
 static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan* pl) {
   if (!d || d->B <= 0 || d->H <= 0 || max_selected <= 0) return false;
   if (d->D != 64 && d->D != 128) return false;
@@ -690,8 +696,7 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   pl->warps = block_warps(d, units * n_chunks, chunk);
   pl->chunk = chunk;
   pl->n_chunks = n_chunks;
-  pl->acc_bytes = ((size_t)out_units * n_chunks * d->D * sizeof(float) + 255) / 256 * 256;
-  pl->total_bytes = pl->acc_bytes + ((size_t)out_units * n_chunks * sizeof(float2) + 255) / 256 * 256;
+  pl->total_bytes = triples_bytes(d, (size_t)out_units * n_chunks, &pl->acc_bytes);
   return true;
 }
 
@@ -734,19 +739,31 @@ static bool choose_plan(const ssa_attn_desc* d, int max_selected, size_t ws_byte
   return true;
 }
 
-// Workspace with which choose_plan has its choice.
+// Workspace with which choose_plan has its choice, here and for fewer requests and shorter lists: those are cut into more
+// chunks, up to the blocks that fill the SMs.  One head per block: chunks of 256 (this launch may take its lists whole), and,
+// as halving ends once there are two blocks per SM, fewer than four per SM of 64 rows or more; row-sharing blocks: two per SM
+// at most, of 256 rows or more.  (Whether a smaller call then has its choice of the two is another matter: choose_plan.)
 static size_t plan_bytes(const ssa_attn_desc* d, int max_selected) {
   Plan pl, chosen;
   if (!make_plan(d, max_selected, &pl) || !choose_plan(d, max_selected, SIZE_MAX, &chosen)) return 0;
-  return std::max(pl.total_bytes, chosen.total_bytes);
+  const long long rows = (long long)d->B * d->H, sms = sm_count();
+  auto cut = [&](int chunk) { return rows * ((max_selected + chunk - 1) / chunk); };
+  long long triples = rows;
+  if (pl.share) {
+    const long long per_block = (d->H / d->H_kv + head_splits(d) - 1) / head_splits(d);
+    triples = std::max(triples, std::min(2 * sms * per_block, cut(256)));
+  } else {
+    if (max_selected > kMaxChunk) triples = cut(256);
+    if (max_selected > 256) triples = std::max(triples, std::min(4 * sms, cut(64)));
+  }
+  size_t acc = 0;
+  return std::max({pl.total_bytes, chosen.total_bytes, triples_bytes(d, (size_t)triples, &acc)});
 }
 
 // Full contexts read by the row-sharing kernel: cut on the device over one block per resident slot, if the lengths of all
 // requests fit a block's scan and the workspace, which callers may have sized by an index list's bound, holds the results.
 static size_t even_bytes(const ssa_attn_desc* d, int blocks, size_t* acc_bytes) {
-  const size_t triples = (size_t)2 * blocks * (d->H / d->H_kv);
-  *acc_bytes = (triples * d->D * sizeof(float) + 255) / 256 * 256;
-  return *acc_bytes + (triples * sizeof(float2) + 255) / 256 * 256;
+  return triples_bytes(d, (size_t)2 * blocks * (d->H / d->H_kv), acc_bytes);
 }
 
 static int even_blocks_wanted(const ssa_attn_desc* d, const Plan& pl) {
@@ -785,8 +802,7 @@ static bool make_plan_blockmask(const ssa_attn_desc* d, int block_size, int max_
   pl->chunk = kMaskChunk / block_size;
   pl->n_chunks = (max_blocks + pl->chunk - 1) / pl->chunk;
   pl->warps = block_warps(d, units * pl->n_chunks, kMaskChunk);
-  pl->acc_bytes = ((size_t)units * pl->n_chunks * d->D * sizeof(float) + 255) / 256 * 256;
-  pl->total_bytes = pl->acc_bytes + ((size_t)units * pl->n_chunks * sizeof(float2) + 255) / 256 * 256;
+  pl->total_bytes = triples_bytes(d, (size_t)units * pl->n_chunks, &pl->acc_bytes);
   return true;
 }
 

@@ -210,3 +210,34 @@ def test_struct_layouts_of_the_binding_match_the_header(tmp_path):
     want = [C.sizeof(ssa.AttnDesc), C.sizeof(ssa.Step), C.sizeof(ssa.AnchorTables), C.sizeof(ssa.Paging),
             ssa.AttnDesc.scale.offset, ssa.Step.flags.offset, ssa.Step.host_in.offset, ssa.Paging.n_pages.offset]
     assert got == want
+
+
+def test_workspace_of_a_larger_batch_serves_smaller_ones():
+    """A size asked for once, for the largest batch and the longest lists, holds what any smaller call needs: its partial
+    results (a row of D floats and a pair per head and chunk) with one head per block, where that is the only plan and the
+    size is the need; with shared rows, two blocks per SM at most, of 256 rows or more (148 SMs, also where there is none)."""
+    rows = [1, 64, 65, 128, 200, 256, 257, 300, 400, 512, 513, 700, 768, 820, 1000, 1024, 1025, 1500, 2048, 2049, 4000, 16000]
+    batches = [1, 2, 3, 4, 5, 6, 7, 9, 10, 12, 14, 16, 18, 20, 24, 28, 32, 37, 40, 48, 64, 148, 149, 200, 296, 297]
+    up = lambda n, to: -(-n // to) * to
+
+    def needed(d, r):
+        G = d.H // d.H_kv
+        if G == 1 or d.D == 64:
+            return ssa.decode_workspace_bytes(d, r)
+        units, n = d.B * d.H_kv * -(-G // 16), 1
+        if not (148 < 2 * units and units <= 148 and r <= 2048):
+            n = max(1, min(296 // units, -(-r // 256)))
+            n = -(-r // up(-(-r // n), 64))
+        return up(d.B * d.H * n * 4 * d.D, 256) + up(d.B * d.H * n * 8, 256)
+
+    # (groups of 2 to 16 are older and go by their own need)
+    for H, H_kv in ((8, 8), (32, 32), (10, 10), (1, 1), (128, 8), (136, 8), (96, 4), (24, 1), (17, 1), (200, 10)):
+        for D in (64, 128):
+            for kv in (ssa.F16, ssa.FP8_E4M3):
+                most = [0] * len(rows)                  # needed by the batches so far, with up to rows[i] rows
+                for B in batches:
+                    for i, r in enumerate(rows):
+                        d = good_desc()
+                        d.B, d.H, d.H_kv, d.D, d.max_ctx, d.kv_dtype, d.out_dtype = B, H, H_kv, D, 20000, kv, ssa.F32
+                        most[i] = max(most[i], most[max(i - 1, 0)], needed(d, r))
+                        assert ssa.decode_workspace_bytes(d, r) >= most[i], (H, H_kv, D, kv, B, r)

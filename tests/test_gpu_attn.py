@@ -969,3 +969,27 @@ def test_host_driven_step_wherever_the_query_rows_sit_in_the_input_arena(order):
     assert ds.counts.cpu().numpy().tolist() == counts.tolist()
     ref, _ = O.decode_attn_sparse(wl.q_bits(), *wl.kv_bits(), wl.ctx_lens, index, counts, scale_of(D), wl.dtype)
     assert_parity(ds.out_f64(), ref, False, order)
+
+
+@pytest.mark.parametrize("H,D", [(8, 128), (5, 64)])
+def test_smaller_batches_run_in_the_workspace_of_the_largest(H, D):
+    """One allocation for the largest batch: smaller ones, whose lists are cut into more chunks, give what they give with a
+    size of their own, to the bit, and nothing is written behind the size."""
+    p = Problem(4, H, 1100, D, seed=D)
+    out = torch.zeros((4, H, D), dtype=torch.float32, device=DEV)
+    index = torch.arange(1024, dtype=torch.int32, device=DEV).expand(4, 1024).contiguous()
+    nbytes = ssa.decode_workspace_bytes(ssa.make_desc(p.q, p.k, p.v, out), 1024)
+    ws = torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device=DEV)
+    for B in (4, 3, 2, 1):
+        q, k, v, o = p.q[:B], p.k[:B], p.v[:B], out[:B]
+        desc = ssa.make_desc(q, k, v, o)
+        for sel in (200, 257, 600, 1024):
+            ctx, cnt = (torch.full((B,), n, dtype=torch.int32, device=DEV) for n in (1100, sel))
+            own = torch.empty(ssa.decode_workspace_bytes(desc, sel), dtype=torch.uint8, device=DEV)
+            ssa.decode_attn_sparse(desc, q, k, v, ctx, index, cnt, sel, o, None, own)
+            want = o.clone()
+            o.fill_(7.0)
+            ssa.decode_attn_sparse(desc, q, k, v, ctx, index, cnt, sel, o, None, ws[:nbytes])
+            torch.cuda.synchronize()
+            assert torch.equal(o, want), (B, sel)
+    assert bool((ws[nbytes:] == 0xA5).all())
