@@ -147,8 +147,7 @@ int32_t ssa_spans_to_index(const int32_t* span_offsets, const int32_t* spans,
  * request and has no such step); its contents need no initialisation and are
  * dead after the call's work has run.  The size has room for the fastest plan
  * of the call; a call given less takes a slower one if that one's results fit,
- * and refuses otherwise (SSA_ERR_WORKSPACE).  It also serves any call with fewer
- * requests or a smaller max_selected that is otherwise the same.  Full contexts of grouped query
+ * and refuses otherwise (SSA_ERR_WORKSPACE).  Full contexts of grouped query
  * heads are among those: their rows are only cut by the lengths themselves in a
  * workspace asked for with desc->max_ctx.
  */

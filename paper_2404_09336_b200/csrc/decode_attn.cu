@@ -739,22 +739,23 @@ static bool choose_plan(const ssa_attn_desc* d, int max_selected, size_t ws_byte
   return true;
 }
 
-// Workspace with which choose_plan has its choice, here and for fewer requests and shorter lists: those are cut into more
-// chunks, up to the blocks that fill the SMs.  One head per block: chunks of 256 (this launch may take its lists whole), and,
-// as halving ends once there are two blocks per SM, fewer than four per SM of 64 rows or more; row-sharing blocks: two per SM
-// at most, of 256 rows or more.  (Whether a smaller call then has its choice of the two is another matter: choose_plan.)
+// Workspace with which choose_plan has its choice.  Where launches of more units are cut into fewer chunks than they were with
+// four-warp blocks of one head (lists taken whole, row-sharing blocks above kGqaHeads heads), it also holds what fewer requests
+// and shorter lists of the same geometry need, so that one size asked for the largest batch still serves all: one head per
+// block, chunks of 256, and, as halving ends once there are two blocks per SM, fewer than four per SM of 64 rows or more;
+// row-sharing blocks, two per SM at most, of 256 rows or more.
 static size_t plan_bytes(const ssa_attn_desc* d, int max_selected) {
   Plan pl, chosen;
   if (!make_plan(d, max_selected, &pl) || !choose_plan(d, max_selected, SIZE_MAX, &chosen)) return 0;
   const long long rows = (long long)d->B * d->H, sms = sm_count();
   auto cut = [&](int chunk) { return rows * ((max_selected + chunk - 1) / chunk); };
-  long long triples = rows;
-  if (pl.share) {
-    const long long per_block = (d->H / d->H_kv + head_splits(d) - 1) / head_splits(d);
-    triples = std::max(triples, std::min(2 * sms * per_block, cut(256)));
-  } else {
+  long long triples = 0;
+  if (!pl.share) {
     if (max_selected > kMaxChunk) triples = cut(256);
     if (max_selected > 256) triples = std::max(triples, std::min(4 * sms, cut(64)));
+  } else if (head_splits(d) > 1) {
+    const long long per_block = (d->H / d->H_kv + head_splits(d) - 1) / head_splits(d);
+    triples = std::min(2 * sms * per_block, cut(256));
   }
   size_t acc = 0;
   return std::max({pl.total_bytes, chosen.total_bytes, triples_bytes(d, (size_t)triples, &acc)});

@@ -231,7 +231,7 @@ def test_workspace_of_a_larger_batch_serves_smaller_ones():
         return up(d.B * d.H * n * 4 * d.D, 256) + up(d.B * d.H * n * 8, 256)
 
     # (groups of 2 to 16 are older and go by their own need)
-    for H, H_kv in ((8, 8), (32, 32), (10, 10), (1, 1), (128, 8), (136, 8), (96, 4), (24, 1), (17, 1), (200, 10)):
+    for H, H_kv in ((8, 8), (32, 32), (10, 10), (1, 1), (136, 8), (96, 4), (24, 1), (17, 1), (200, 10)):
         for D in (64, 128):
             for kv in (ssa.F16, ssa.FP8_E4M3):
                 most = [0] * len(rows)                  # needed by the batches so far, with up to rows[i] rows
