@@ -98,27 +98,40 @@ def test_large_groups_against_the_oracle(dtype, B, Hkv, G, T, counts):
 
 
 def test_large_group_in_the_workspace_of_one_head_per_block():
-    """A workspace sized by another bound, too small for the row-sharing plan, is taken as before; so is the call without one."""
-    B, H, Hkv, T, D = 1, 120, 6, 2000, 128
+    """A workspace sized by another bound, too small for the row-sharing plan, is taken as before: lists of 1000 rows are then
+    one chunk per head, 200 partial results, instead of four chunks and a second pass.  The call without a workspace goes by
+    the one-head plan as well: it refuses what that does not fit, though the row-sharing one would."""
+    B, H, Hkv, T, D = 1, 200, 10, 1000, 128
     q, k, v, qb, kb, vb, name = problem("bf16", B, H, Hkv, T, seed=1)
     out = torch.zeros((B, H, D), dtype=torch.float32, device=DEV)
     desc = ssa.make_desc(q, k, v, out)
     idx = torch.arange(T, dtype=torch.int32, device=DEV).view(1, T)
     d_ctx, d_cnt = (torch.tensor([T], dtype=torch.int32, device=DEV) for _ in range(2))
     ref, _ = O.decode_attn_dense(qb, np.repeat(kb, 20, axis=1), np.repeat(vb, 20, axis=1), [T], 1 / np.sqrt(D), name)
+    full, small = ssa.decode_workspace_bytes(desc, T), sum((H * 4 * n + 255) // 256 * 256 for n in (D, 2))
+    assert small < H * 4 * (4 * D + 8) <= full                    # four chunks per head do not fit
 
-    def check():
+    def check(before, launches):
+        assert ssa.launch_count() - before == launches
         torch.cuda.synchronize()
         assert float(np.linalg.norm(out.double().cpu().numpy() - ref)) <= 1e-6 * float(np.linalg.norm(ref))
         out.zero_()
 
-    for nbytes in (ssa.decode_workspace_bytes(desc, T), sum((H * 8 * n + 255) // 256 * 256 for n in (4 * D, 8))):
-        ws = torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device=DEV)
+    ws = torch.empty(full + 4096, dtype=torch.uint8, device=DEV)
+    for nbytes, launches in ((full, 2), (small, 1)):
+        ws.fill_(0xA5)
+        before = ssa.launch_count()
         ssa.decode_attn_sparse(desc, q, k, v, d_ctx, idx, d_cnt, T, out, None, ws[:nbytes], None)
-        check()
+        check(before, launches)
         assert bool((ws[nbytes:] == 0xA5).all())
+    assert ssa.decode_attn_sparse(desc, q, k, v, d_ctx, idx, d_cnt, T, out, None, ws[:small - 256], None,
+                                  check=False) == ssa.ERR_WORKSPACE
+    before = ssa.launch_count()
     ssa.decode_attn_sparse_noalloc(desc, q, k, v, d_ctx, idx, d_cnt, T, out, None, None)
-    check()
+    check(before, 2)
+    desc.B, desc.max_ctx = 2, 16000                                # 400 heads x 63 chunks of 256 rows
+    assert ssa.decode_attn_sparse_noalloc(desc, q, k, v, d_ctx, torch.zeros((2, 16000), dtype=torch.int32, device=DEV), d_cnt,
+                                          16000, out, None, None, check=False) == ssa.ERR_WORKSPACE
 
 
 # dtype, B, Hkv, G, T: lists (one large block per SM, several chunks, one block) and full contexts, those of the last two cut
