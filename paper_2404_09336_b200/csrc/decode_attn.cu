@@ -1169,8 +1169,8 @@ int32_t ssa_decode_attn_spans(const ssa_attn_desc* desc, const void* q, const vo
   if (rc != SSA_OK) return rc;
   ssa::Plan pl;
   if (max_selected <= 0 || (index_out && max_selected > index_stride)) return SSA_ERR_CAPACITY;
-  if (!ssa::make_plan(desc, max_selected, &pl)) return SSA_ERR_SHAPE;
   const size_t list_bytes = ssa::counts_bytes(desc) + (size_t)desc->B * spans_index_pitch(max_selected) * sizeof(int32_t);
+  if (!ssa::choose_plan(desc, max_selected, workspace_bytes - std::min(workspace_bytes, list_bytes), &pl)) return SSA_ERR_SHAPE;
   if (!workspace || workspace_bytes < pl.total_bytes + list_bytes) return SSA_ERR_WORKSPACE;
   if (!ssa::aligned16(workspace)) return SSA_ERR_ALIGN;
   const size_t partial_bytes = (workspace_bytes - list_bytes) / 256 * 256;

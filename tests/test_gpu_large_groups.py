@@ -126,6 +126,17 @@ def test_large_group_in_the_workspace_of_one_head_per_block():
         assert bool((ws[nbytes:] == 0xA5).all())
     assert ssa.decode_attn_sparse(desc, q, k, v, d_ctx, idx, d_cnt, T, out, None, ws[:small - 256], None,
                                   check=False) == ssa.ERR_WORKSPACE
+    # span lists, few of them and more than a block merges on chip (their index list then shares the workspace)
+    for n, lists in ((2, 256), (T, 256 + 4 * 1024)):
+        spans = torch.tensor([[T * i // n, T * (i + 1) // n] for i in range(n)], dtype=torch.int32, device=DEV)
+        offs, nbytes = torch.tensor([0, n], dtype=torch.int32, device=DEV), small + lists
+        ws.fill_(0xA5)
+        before = ssa.launch_count()
+        ssa.decode_attn_spans(desc, q, k, v, d_ctx, offs, spans, n, T, out, None, None, None, ws[:nbytes], None)
+        check(before, 1 if n == 2 else 2)
+        assert bool((ws[nbytes:] == 0xA5).all())
+        assert ssa.decode_attn_spans(desc, q, k, v, d_ctx, offs, spans, n, T, out, None, None, None, ws[:nbytes - 256], None,
+                                     check=False) == ssa.ERR_WORKSPACE
     before = ssa.launch_count()
     ssa.decode_attn_sparse_noalloc(desc, q, k, v, d_ctx, idx, d_cnt, T, out, None, None)
     check(before, 2)
