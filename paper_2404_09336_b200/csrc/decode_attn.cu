@@ -658,15 +658,19 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   // The second pass costs about as much as two rounds of a block, so a request is split only when that buys
   // parallelism: one chunk whenever the list fits a block's staging area and either every SM gets a block or
   // the list is short anyway; otherwise 256-entry chunks, halved while the grid has under two blocks per SM.
-  // Large blocks (block_warps) stage up to 1024 entries, and taking a list of 513..1024 whole is better from a fifth of a
-  // block per SM on (us, chunks / whole: 32 heads x 820 rows 7.7 / 7.3, 148 x 820 12.8 / 10.8, 296 x 820 21.0 / 17.8, but 8 x 820
-  // 5.7 / 6.7); over an 8-bit cache, whose rows are fewer turns, not where a second block would leave most SMs idle
-  // (160 x 1024 12.2 / 13.5), nor for grouped heads, whose lines (one_head_blocks_pay) were measured with chunks.
+  // Large blocks (block_warps) stage up to 1024 entries, and taking a list of 257..1024 whole is better from a fifth of a
+  // block per SM on, as far as 768 rows of 128 (16-bit ones are three turns of sixteen warps), and from two fifths on beyond
+  // that (us, chunks / whole: 32 heads x 300 rows 4.9 / 4.4, x 700 6.7 / 6.5, but x 820 7.1 / 7.7 and x 1024 8.0 / 8.3; 48 x 820
+  // 7.9 / 8.2, 64 x 820 8.8 / 8.6, 80 x 820 10.7 / 9.2, 296 x 820 24.6 / 21.1, but 8 x 820 5.7 / 6.7; 8-bit rows, 32 x 700 6.6 /
+  // 6.3, x 1024 7.2 / 7.4; 32 x 1024 rows of 64 8.8 / 4.9); over an 8-bit cache, whose rows are fewer turns, not where a second
+  // block would leave most SMs idle (160 x 1024 12.2 / 13.5), nor for grouped heads, whose lines (one_head_blocks_pay) were
+  // measured with chunks.
   const long long sms = sm_count();
   const long long want = sms * 2;
   int chunk = 256;
   if (max_selected <= kMaxChunk && (units >= sms || max_selected <= 256)) chunk = kMaxChunk;
-  else if (!share && max_selected <= kMaxWideChunk && units <= want && 5 * units >= sms &&
+  else if (!share && max_selected <= kMaxWideChunk && units <= want &&
+           5 * units >= (max_selected * d->D <= 768 * 128 ? sms : 2 * sms) &&
            (d->kv_dtype != SSA_FP8_E4M3 || (d->H == d->H_kv && (units <= sms || 5 * units >= 7 * sms))))
     chunk = kMaxWideChunk;                             // (at most two blocks per SM, over 512 rows: large blocks)
   else while (chunk > 64 && units * ((max_selected + chunk - 1) / chunk) < want) chunk >>= 1;

@@ -993,3 +993,21 @@ def test_smaller_batches_run_in_the_workspace_of_the_largest(H, D):
             torch.cuda.synchronize()
             assert torch.equal(o, want), (B, sel)
     assert bool((ws[nbytes:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("H,D,sel,launches", [
+    (32, 128, 768, 1), (32, 128, 769, 2), (59, 128, 1024, 2), (60, 128, 1024, 1), (32, 64, 1024, 1), (29, 128, 700, 2)])
+def test_lists_taken_whole_by_large_blocks(H, D, sel, launches):
+    """Where a list of 257..1024 rows is one block's work (one launch) and where it is cut (148 SMs): lists longer than 768 rows
+    of 128 only from two fifths of a block per SM on."""
+    if ssa_sms() != 148:
+        pytest.skip("lines of a chip with 148 SMs")
+    p = Problem(1, H, 1100, D, seed=sel)
+    index = np.arange(sel, dtype=np.int32)[None]
+    before = ssa.launch_count()
+    out, lse, status, _ = p.sparse([1100], index, [sel])
+    assert ssa.launch_count() - before == launches and status == 0
+    heads = [0, H - 1]
+    ref, ref_lse = O.decode_attn_sparse(p.q_bits, p.k_bits, p.v_bits, [1100], index, [sel], scale_of(D), "bf16", heads=heads)
+    assert_parity(out[:, heads], ref[:, heads], False, "lists taken whole")
+    np.testing.assert_allclose(lse[:, heads], ref_lse[:, heads], rtol=1e-5, atol=1e-5)
