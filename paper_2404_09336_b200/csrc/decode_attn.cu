@@ -47,6 +47,7 @@ constexpr int kSmallBlock = SSA_WARPS; // warps per block in pass 1, where block
 constexpr int kWarpSlots = SSA_WARPS * SSA_MIN_BLOCKS;   // warps of an SM
 constexpr int kMaxChunk = 512;         // index entries staged per block
 constexpr int kMaxWideChunk = 1024;    // ... of more than kSmallBlock warps
+__host__ __device__ constexpr int staged_entries(int warps) { return warps > kSmallBlock ? kMaxWideChunk : kMaxChunk; }
 constexpr int kMaskChunk = 512;        // positions a block expands from bitmasks
 enum { kDense = 0, kIndex = 1, kBlockMask = 2, kSpans = 3 };
 
@@ -195,7 +196,7 @@ __device__ __forceinline__ void halve_between(float2 (&out)[N], const float2 (&i
 template <typename T, int D, int kMode, bool kAligned32, bool kPaged = false, bool kHostQ = false, int kWarps = kSmallBlock>
 __global__ void __launch_bounds__(kWarps * 32, kWarpSlots / kWarps)
 decode_partial_kernel(const DecodeParams p) {
-  constexpr int kThreads = kWarps * 32, kStage = kWarps > kSmallBlock ? kMaxWideChunk : kMaxChunk;
+  constexpr int kThreads = kWarps * 32, kStage = staged_entries(kWarps);
   constexpr int kIdxPerThread = kStage / kThreads;
   constexpr bool kWide = kWarps > kSmallBlock;
   static_assert(!kPaged || kMode == kIndex, "a paged cache is read through staged positions");
@@ -669,10 +670,10 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   const long long want = sms * 2;
   int chunk = 256;
   if (max_selected <= kMaxChunk && (units >= sms || max_selected <= 256)) chunk = kMaxChunk;
-  else if (!share && max_selected <= kMaxWideChunk && units <= want &&
+  else if (!share && max_selected <= staged_entries(block_warps(d, units, max_selected)) && units <= want &&
            5 * units >= (max_selected * d->D <= 768 * 128 ? sms : 2 * sms) &&
            (d->kv_dtype != SSA_FP8_E4M3 || (d->H == d->H_kv && (units <= sms || 5 * units >= 7 * sms))))
-    chunk = kMaxWideChunk;                             // (at most two blocks per SM, over 512 rows: large blocks)
+    chunk = kMaxWideChunk;
   else while (chunk > 64 && units * ((max_selected + chunk - 1) / chunk) < want) chunk >>= 1;
   pl->share = share;
   pl->wide = false;
@@ -876,6 +877,7 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
     }
   }
   if (!share) {
+    if ((mode == kIndex || mode == kSpans) && p.chunk > staged_entries(p.warps)) return SSA_ERR_SHAPE;   // (no plan does)
     auto pick = [&](auto aligned_tag, auto warps_tag) {
       constexpr bool kA = decltype(aligned_tag)::value;
       constexpr int kW = decltype(warps_tag)::value;

@@ -3,10 +3,13 @@ bad arguments on the host before anything is launched (no GPU needed)."""
 import ctypes as C
 import os
 import re
+import shutil
+import subprocess
 
 import pytest
+import torch
 
-from paper_2404_09336_b200 import ssa
+from paper_2404_09336_b200 import build, ssa
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -241,3 +244,29 @@ def test_workspace_of_a_larger_batch_serves_smaller_ones():
                         d.B, d.H, d.H_kv, d.D, d.max_ctx, d.kv_dtype, d.out_dtype = B, H, H_kv, D, 20000, kv, ssa.F32
                         most[i] = max(most[i], most[max(i - 1, 0)], needed(d, r))
                         assert ssa.decode_workspace_bytes(d, r) >= most[i], (H, H_kv, D, kv, B, r)
+
+
+@pytest.mark.skipif(torch.cuda.is_available() or shutil.which("nvcc") is None, reason="enters launches with addresses that are none")
+@pytest.mark.parametrize("defines", [["-DSSA_MIN_BLOCKS=2"], ["-DSSA_WARPS=8", "-DSSA_MIN_BLOCKS=2"]])
+def test_lists_are_taken_whole_only_by_blocks_that_can_stage_them(tmp_path, defines):
+    """Blocks of the smallest size stage 512 entries.  With other block sizes (a build define) a launch of 200 heads may get no
+    larger ones, and then 1000 rows must be cut.  The workspace of one partial result per head shows which: too small, or
+    enough, so that the call goes on to a launch that this machine, without a GPU, refuses."""
+    out = str(tmp_path / "libssa.so")
+    subprocess.run(["nvcc", "-std=c++17", "-O0", "-Xcicc", "-O0", "-Xcompiler", "-fPIC,-O0", "-shared", "--threads", "0",
+                    "-gencode", "arch=compute_100a,code=compute_100a", *defines, "-I", build.ROOT + "/include",
+                    "-I", build.CSRC, "-o", out, *build.sources()], check=True, capture_output=True)
+    lib = C.CDLL(out)
+    f = lib.ssa_decode_attn_sparse
+    f.restype, f.argtypes = C.c_int32, ssa.lib.ssa_decode_attn_sparse.argtypes
+
+    def call(library, H, rows):
+        d = good_desc()
+        d.B, d.H, d.H_kv, d.max_ctx = 1, H, H, 2000
+        one_each = sum((H * 4 * n + 255) // 256 * 256 for n in (128, 2))
+        return library(C.byref(d), P, P, P, P, P, rows, P, rows, P, NUL, P, one_each, NUL, NUL)
+
+    assert call(f, 200, 512) == ssa.ERR_CUDA
+    assert call(f, 200, 1000) == ssa.ERR_WORKSPACE
+    assert call(f, 74, 1000) == ssa.ERR_CUDA              # one block per two SMs: room for large ones
+    assert call(ssa.lib.ssa_decode_attn_sparse, 200, 1000) == ssa.ERR_CUDA
