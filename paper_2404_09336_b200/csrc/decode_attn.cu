@@ -807,7 +807,7 @@ static bool make_plan_blockmask(const ssa_attn_desc* d, int block_size, int max_
   pl->even_blocks = 0;
   pl->chunk = kMaskChunk / block_size;
   pl->n_chunks = (max_blocks + pl->chunk - 1) / pl->chunk;
-  pl->warps = block_warps(d, units * pl->n_chunks, kMaskChunk);
+  pl->warps = block_warps(d, units * pl->n_chunks, std::min(pl->chunk, max_blocks) * block_size);
   pl->total_bytes = triples_bytes(d, (size_t)units * pl->n_chunks, &pl->acc_bytes);
   return true;
 }

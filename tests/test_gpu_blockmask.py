@@ -210,3 +210,27 @@ def test_full_size_workload_through_the_blocked_lists():
     ds.step()
     torch.cuda.synchronize()
     np.testing.assert_allclose(ds.out_f64(), got, rtol=0, atol=4e-3)       # bf16 outputs of the two paths
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("bs,listed", [(32, 1), (32, 2), (64, 1), (32, 5), (128, 1), (64, 3), (256, 1)])
+def test_short_blocked_lists_take_the_blocks_of_index_lists_of_their_length(bs, listed, D):
+    """Warps of a block follow the rows that a launch's lists can hold (block_warps): a few whole blocks are then the same sums
+    in the same order as an index list of their positions, to the bit."""
+    B, H, T = 3, 4, 1024
+    p = Problem(B, H, T, D, seed=bs + listed)
+    blocks = torch.arange(1, 1 + listed, dtype=torch.int32, device=DEV).expand(B, listed).contiguous()
+    mask = torch.full((B, listed, bs // 32), -1, dtype=torch.int32, device=DEV)
+    ctx, few, rows = (torch.full((B,), n, dtype=torch.int32, device=DEV) for n in (T, listed, listed * bs))
+    index = torch.arange(bs, bs + listed * bs, dtype=torch.int32, device=DEV).expand(B, listed * bs).contiguous()
+    out, want = (torch.zeros((B, H, D), dtype=torch.float32, device=DEV) for _ in range(2))
+    desc = ssa.make_desc(p.q, p.k, p.v, out)
+    ws = torch.empty(max(ssa.decode_blockmask_workspace_bytes(desc, bs, listed), ssa.decode_workspace_bytes(desc, bs * listed)),
+                     dtype=torch.uint8, device=DEV)
+    ssa.decode_attn_blockmask(desc, p.q, p.k, p.v, ctx, blocks, mask, few, bs, listed, out, None, ws)
+    ssa.decode_attn_sparse(desc, p.q, p.k, p.v, ctx, index, rows, bs * listed, want, None, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    ref, _ = O.decode_attn_sparse(p.q_bits, p.k_bits, p.v_bits, [T] * B, index.cpu().numpy(), [bs * listed] * B,
+                                  1 / np.sqrt(D), "bf16")
+    assert_parity(out.double().cpu().numpy(), ref, False, "short blocked lists")
