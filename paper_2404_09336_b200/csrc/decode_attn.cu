@@ -1076,10 +1076,11 @@ int32_t decode_attn_sparse_host_queries(const ssa_attn_desc* desc, void* q, cons
              workspace_bytes, dev_status, stream, kIndex, nullptr, nullptr, nullptr, q_host);
 }
 
-// One chunk per request (every row then crosses the bus once), multi-head 16-bit cache.
-bool host_queries_pay(const ssa_attn_desc* d, int32_t max_selected) {
+// One chunk per request (every row then crosses the bus once) and one head per block over a 16-bit cache, by the plan that the
+// call with this workspace will take.
+bool host_queries_pay(const ssa_attn_desc* d, int32_t max_selected, size_t ws_bytes) {
   Plan pl;
-  if (!d || check_desc(d) != SSA_OK || !make_plan(d, max_selected, &pl)) return false;
+  if (!d || check_desc(d) != SSA_OK || !choose_plan(d, max_selected, ws_bytes, &pl)) return false;
   return pl.n_chunks == 1 && !pl.share && d->kv_dtype != SSA_FP8_E4M3;
 }
 

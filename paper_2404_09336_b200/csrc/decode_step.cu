@@ -102,7 +102,8 @@ extern "C" int32_t ssa_decode_step(const ssa_attn_desc* desc, const ssa_step* s,
     const size_t q_bytes = ((size_t)(desc->B - 1) * desc->q_stride_b + (size_t)(desc->H - 1) * desc->q_stride_h +
                             desc->D) * 2;
     size_t skip_head = 0, skip_tail = 0;
-    if (host_twin(s->q) && q_bytes % 16 == 0 && q_bytes <= s->in_bytes && ssa::host_queries_pay(desc, s->max_selected)) {
+    if (host_twin(s->q) && q_bytes % 16 == 0 && q_bytes <= s->in_bytes &&
+        ssa::host_queries_pay(desc, s->max_selected, s->workspace_bytes)) {
       if (q_dev == arena) skip_head = q_bytes;
       else if (q_dev + q_bytes == arena + s->in_bytes) skip_tail = q_bytes;
     }

@@ -28,6 +28,6 @@ int32_t decode_attn_sparse_host_queries(const ssa_attn_desc* desc, void* q, cons
                                         int32_t index_stride, const int32_t* counts, int32_t max_selected, void* out,
                                         float* lse, void* workspace, size_t workspace_bytes, uint32_t* dev_status,
                                         void* stream);
-bool host_queries_pay(const ssa_attn_desc* desc, int32_t max_selected);
+bool host_queries_pay(const ssa_attn_desc* desc, int32_t max_selected, size_t ws_bytes);
 
 }  // namespace ssa

@@ -971,6 +971,49 @@ def test_host_driven_step_wherever_the_query_rows_sit_in_the_input_arena(order):
     assert_parity(ds.out_f64(), ref, False, order)
 
 
+@pytest.mark.parametrize("H,H_kv,fetched", [(4, 4, True), (20, 1, True), (40, 2, True), (16, 1, False), (8, 4, False)])
+def test_who_fetches_the_query_rows_of_a_host_driven_step(H, H_kv, fetched):
+    """Blocks that serve one head each - also those of a small launch of more than sixteen heads per K/V head - fetch their own
+    query rows, blocks that share rows among heads find theirs copied with the arena.  What lies between the rows tells
+    which: it arrives on the device with the arena only."""
+    B, D, T, sel, gap = 2, 128, 512, 200, 8
+    rng = np.random.default_rng(H)
+    q_host = torch.full((B, H, D + gap), 0.25, dtype=torch.bfloat16)
+    q_host[..., :D] = torch.from_numpy(rng.standard_normal((B, H, D)).astype(np.float32)).to(torch.bfloat16)
+    tail = torch.tensor([T] * B + [0, 2, 4, 0] + [0, 100, 300, 400] * B, dtype=torch.int32)   # lengths, offsets, spans
+    q_bytes = (B * H * (D + gap) - gap) * 2
+    rest = (q_bytes + 255) // 256 * 256
+    h_in = torch.zeros(rest + (tail.numel() * 4 + 255) // 256 * 256, dtype=torch.uint8).pin_memory()
+    h_in[:q_bytes] = q_host.view(torch.uint8).flatten()[:q_bytes]
+    h_in[rest:rest + 4 * tail.numel()] = tail.view(torch.uint8)
+    d_in = torch.full(h_in.shape, 0xAB, dtype=torch.uint8, device=DEV)
+    ints = d_in[rest:rest + 4 * tail.numel()].view(torch.int32)
+    ctx, offs, spans = ints[:B], ints[B:B + B + 1], ints[B + 4:].view(-1, 2)
+    q = torch.as_strided(d_in[:q_bytes].view(torch.bfloat16), (B, H, D), (H * (D + gap), D + gap, 1))
+    k, v = (torch.from_numpy(rng.standard_normal((B, H_kv, T, D)).astype(np.float32)).to(torch.bfloat16) for _ in range(2))
+    kd, vd = k.to(DEV), v.to(DEV)
+    out, lse = torch.zeros((B, H, D), device=DEV), torch.zeros((B, H), device=DEV)
+    index = torch.full((B, 256), -1, dtype=torch.int32, device=DEV)
+    d_tail = torch.zeros(512, dtype=torch.uint8, device=DEV)
+    counts, status = d_tail[:4 * B].view(torch.int32), d_tail[256:260].view(torch.int32)
+    h_tail = torch.zeros(512, dtype=torch.uint8).pin_memory()
+    desc = ssa.make_desc(q, kd, vd, out)
+    ws = torch.empty(ssa.decode_workspace_bytes(desc, sel), dtype=torch.uint8, device=DEV)
+    st = ssa.make_step(offs, spans, ctx, index, counts, q, kd, vd, sel, out, lse, ws, status, host_in=h_in, dev_in=d_in,
+                       host_out=h_tail, dev_out=d_tail, copy_by_kernel=True, max_spans=2)
+    ssa.decode_step(desc, st)
+    torch.cuda.synchronize()
+    assert h_tail[:4 * B].view(torch.int32).tolist() == [sel] * B and int(status.item()) == 0
+    between = d_in[2 * D:2 * (D + gap)].cpu()
+    assert torch.equal(between, torch.full_like(between, 0xAB)) == fetched
+    assert torch.equal(q.cpu(), q_host[..., :D])
+    at = list(range(100)) + list(range(300, 400))
+    rows = (x[:, :, at].double().repeat_interleave(H // H_kv, dim=1) for x in (k, v))
+    kr, vr = rows
+    ref = torch.softmax((kr @ q_host[..., :D].double()[..., None])[..., 0] / D ** 0.5, -1)[:, :, None] @ vr
+    assert_parity(out.double().cpu().numpy(), ref[:, :, 0].numpy(), False, "host-driven step")
+
+
 @pytest.mark.parametrize("H,D", [(8, 128), (5, 64)])
 def test_smaller_batches_run_in_the_workspace_of_the_largest(H, D):
     """One allocation for the largest batch: smaller ones, whose lists are cut into more chunks, give what they give with a
