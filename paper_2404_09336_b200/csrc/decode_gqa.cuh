@@ -169,36 +169,34 @@ __device__ __forceinline__ uint32_t e4m3x2_to_16bit<__nv_bfloat16>(uint32_t pair
 }
 // A query row over an 8-bit cache: sixteen bf16 values of each of eight neighbouring lanes -> fp16 values times 2^k, the
 // largest in [2^14, 2^15).  Returns what turns its scores into log2 units, scale_log2 2^-k, or 0 where that is no normal
-// number or a value is not an fp16 number times 2^-k: such a row (elements that differ by 2^31 and more) is for bf16 scores.
-// (With bf16 queries the rows of K have to become bf16, by way of two fp32 values: four instructions per pair instead of
-// one.  us, four heads on each of 8 K/V heads: 32 requests of 819 rows 16.98 -> 16.30, 17 full contexts of 8190 rows 57.2 ->
-// 52.2.  The values are the same and the powers of two cancel: same bits.)
+// number or a bit may be lost (exponents more than 31 apart): such a row is for bf16 scores.  (With bf16 queries the rows of
+// K have to become bf16, by way of two fp32 values: four instructions per pair instead of one.  us, four heads on each of 8
+// K/V heads: 32 requests of 819 rows 16.98 -> 16.38, 17 full contexts of 8190 rows 57.2 -> 52.5.  The values are the same and
+// the powers of two cancel: same bits.)
 __device__ __forceinline__ float scaled_query(uint4& lo, uint4& hi, float scale_log2) {
   uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-  uint32_t most = 0u;                                   // largest finite magnitude, as the bits of a bf16 value
+  uint32_t most = 0u, least = 0xffffffffu;              // largest finite, smallest other than 0 (less 1): bits of bf16 values
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const uint32_t a = w[i] & 0x7fffu, b = (w[i] >> 16) & 0x7fffu;
     most = max(most, max(a < 0x7f80u ? a : 0u, b < 0x7f80u ? b : 0u));
+    least = min(least, min(a - 1u, b - 1u));
   }
 #pragma unroll
   for (int o = 1; o < 8; o <<= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
   const int up = most == 0u ? 127 : min(268 - (int)(most >> 7), 253);   // biased exponents of 2^k and, below, of 2^-k
   const float scale = __int_as_float(up << 23);
-  bool lost = false;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    float2 f = unpack2<__nv_bfloat16>(w[i]);
-    f.x *= scale;
-    f.y *= scale;
-    w[i] = pack2<__half>(f.x, f.y);
-    const float2 back = unpack2<__half>(w[i]);
-    lost |= (back.x != f.x && f.x == f.x) || (back.y != f.y && f.y == f.y);   // (a NaN stays one)
+    const float2 f = unpack2<__nv_bfloat16>(w[i]);
+    w[i] = pack2<__half>(f.x * scale, f.y * scale);
   }
   lo = make_uint4(w[0], w[1], w[2], w[3]);
   hi = make_uint4(w[4], w[5], w[6], w[7]);
   const float unit = scale_log2 * __int_as_float((254 - up) << 23);
-  lost |= !(unit >= 1.17549435e-38f && unit <= 3.40282347e38f);
+  // (the last bit of a value lies 7 below its exponent, that of fp16 numbers at 2^-24, the largest value at 2^14 or above)
+  const bool lost = most != 0u && (int)(most >> 7) - max((int)((least + 1u) >> 7), 1) > 31 ||
+                    !(unit >= 1.17549435e-38f && unit <= 3.40282347e38f);
   const uint32_t row_lost = __ballot_sync(0xffffffffu, lost) >> (threadIdx.x & 24) & 0xffu;
   return row_lost ? 0.f : unit;
 }
@@ -677,9 +675,12 @@ decode_partial_gqa_kernel(const DecodeParams p) {
         // (two sums of four k-steps each: half the length of the dependent chain)
         float s[4] = {0.f, 0.f, 0.f, 0.f}, s_odd[4] = {0.f, 0.f, 0.f, 0.f};
         if constexpr (kFp8) {
+          // (rows of K in bf16 are rare and stay out of the way of the usual loop: rolled for one-warp teams and marked unlikely
+          // over full contexts, where registers are tightest: 32 requests of 820 rows, four heads on each of 8 K/V heads, 14.7 us
+          // unrolled, 13.1 so; two-warp teams would lose a tenth by it)
           auto scores = [&](auto type) {
             using TS = decltype(type);
-#pragma unroll
+#pragma unroll (!kHi && std::is_same<TS, __nv_bfloat16>::value ? 1 : 2)
             for (int half = 0; half < 2; ++half) {
               const uint4 lo = lds_16B(ka ^ (half << 6)), hi = lds_16B((ka ^ (half << 6)) + 8 * kRowBytes);
               const uint32_t a[4] = {lo.x, lo.y, lo.z, lo.w}, c[4] = {hi.x, hi.y, hi.z, hi.w};
@@ -687,12 +688,13 @@ decode_partial_gqa_kernel(const DecodeParams p) {
               for (int i = 0; i < 4; ++i) {
                 const uint32_t a0 = e4m3x2_to_16bit<TS>(a[i]), a1 = e4m3x2_to_16bit<TS>(c[i]);
                 const uint32_t a2 = e4m3x2_to_16bit<TS>(a[i] >> 16), a3 = e4m3x2_to_16bit<TS>(c[i] >> 16);
+                const uint32_t b0 = half == 0 ? qb[i][0] : qb[4 + i][0], b1 = half == 0 ? qb[i][1] : qb[4 + i][1];
                 float (&sum)[4] = (i & 1) ? s_odd : s;
-                mma_16816<TS>(sum, a0, a1, a2, a3, qb[4 * half + i][0], qb[4 * half + i][1], sum);
+                mma_16816<TS>(sum, a0, a1, a2, a3, b0, b1, sum);
               }
             }
           };
-          if (bf16_scores) scores(__nv_bfloat16());      // warp-uniform
+          if (kMode == kDense && !kHi ? __builtin_expect(bf16_scores, false) : bf16_scores) scores(__nv_bfloat16());   // warp-uniform
           else scores(__half());
         } else {
 #pragma unroll
