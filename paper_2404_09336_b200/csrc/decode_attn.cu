@@ -637,7 +637,9 @@ static int head_splits(const ssa_attn_desc* d) { return (d->H / d->H_kv + kGqaHe
 // values on their way at a time (as many bytes of others) and takes about 1.1 us a turn, however few other warps there are.
 // A launch that leaves the SMs room therefore gets blocks of two or four times the warps, as far as the rows give each of
 // them a turn.  Four warps / this, us, 16-bit rows of 128 in index lists: 32 heads x 80 rows 4.1 / 3.1, x 256 rows 6.4 / 4.2;
-// 148 heads x 200 rows 6.8 / 5.1, x 512 rows 11.7 / 7.9; 296 heads x 200 rows 8.1 / 7.3, x 512 rows 14.1 / 12.3.
+// 148 heads x 200 rows 6.8 / 5.1, x 512 rows 11.7 / 7.9; 296 heads x 200 rows 8.1 / 7.3, x 512 rows 14.1 / 12.3.  16-bit rows
+// of 64: 32 x 160 rows 3.2 / 2.7, 148 x 512 7.0 / 5.6, 296 x 512 9.6 / 8.7; 8-bit rows of 128: 32 x 160 3.8 / 3.3, 148 x 512
+// 8.6 / 7.3, 296 x 512 10.9 / 10.0; of 64: 148 x 512 4.7 / 3.8, 296 x 400 6.7 / 6.6.
 static int block_warps(const ssa_attn_desc* d, long long blocks, int rows) {
   const int turn = 16 * (128 / d->D) * (d->kv_dtype == SSA_FP8_E4M3 ? 2 : 1);
   int warps = kSmallBlock;

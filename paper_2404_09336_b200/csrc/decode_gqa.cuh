@@ -341,7 +341,7 @@ template <typename T, int kMode, bool kHi, bool kWide, bool kEven = false, bool 
 __global__ void __launch_bounds__(GqaShape<T, kHi, kWide>::kWarps * 32, kWide ? 1 : 2)
 decode_partial_gqa_kernel(const DecodeParams p) {
   using Shape = GqaShape<T, kHi, kWide>;
-  constexpr int kWarps = Shape::kWarps, kThreads = kWarps * 32;   // hide the library-wide four-warp constants in here
+  constexpr int kWarps = Shape::kWarps, kThreads = kWarps * 32;
   constexpr int kTeam = Shape::kTeam, kTeams = Shape::kTeams;
   constexpr int D = 128;
   constexpr bool kSparse = kMode != kDense;
