@@ -630,7 +630,7 @@ static bool can_share_rows(const ssa_attn_desc* d) {
 // A row-sharing block serves up to kGqaHeads heads; larger groups (several query tokens per head) take several blocks per
 // chunk, side by side in the grid, so that all but the first find the rows in L2.  One head per block instead reads every
 // row from L2 once per head (us, one head per block / row-sharing, 32 heads on each of 4 K/V heads, bf16): 3 requests of
-// 12897 rows 201 / 33, 8 of 2000 listed rows 63.7 / 18.4, 24 of 40 15.5 / 6.7.  (Small launches: one_head_blocks_pay.)
+// 12897 rows 194 / 34, 8 of 2000 listed rows 88 / 20, 24 of 40 14.7 / 6.3.  (Small launches: one_head_blocks_pay.)
 static int head_splits(const ssa_attn_desc* d) { return (d->H / d->H_kv + kGqaHeads - 1) / kGqaHeads; }
 
 // Warps of a one-head block that takes up to `rows` rows, in a launch of `blocks`.  A warp has sixteen rows of 128 16-bit
