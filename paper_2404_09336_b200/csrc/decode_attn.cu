@@ -77,6 +77,7 @@ struct DecodeParams {
   int64_t q_sb, q_sh, k_sb, k_sh, v_sb, v_sh, o_sb, o_sh;
   uint32_t k_row_bytes, v_row_bytes;   // token stride of the cache in bytes
   int32_t H, max_ctx, index_stride, max_selected, chunk, n_chunks, out_f32, early_release;
+  int32_t early_blocks, early_rows, early_warps;   // see plan_early
   int32_t kv_group;         // query heads per K/V head (1: multi-head attention)
   int32_t warps;            // warps of a one-head block
   int32_t share_rows;       // row-sharing kernel (otherwise one query head per block)
@@ -187,6 +188,46 @@ __device__ __forceinline__ void halve_between(float2 (&out)[N], const float2 (&i
   }
 }
 
+// Called before grid_dependency_wait() by each of the first p.early_warps warps of a block: they ask for the first p.early_rows rows of the
+// block in L2, by the lists as they stand.  Neighbouring lanes take the
+// sectors of a row: with a row per lane the requests took four times as long to issue.  (Lists, counts, lengths and page tables are
+// read where the host says they are, and no further; what they name is checked against max_ctx and n_pages.  Span lists are left
+// alone: their offsets, not yet to be trusted, would say where to read.)
+template <typename T, int D, int kMode, bool kPaged>
+__device__ __forceinline__ void prefetch_early(const DecodeParams& p, int b, int kvh, int start, int warp) {
+  constexpr int kSectors = D * (int)sizeof(T) / 32, kRows = 32 / kSectors;   // of a row; rows an instruction covers
+  const int lane = threadIdx.x & 31;
+  const char* const krows =
+      reinterpret_cast<const char*>(reinterpret_cast<const T*>(p.k) + (int64_t)b * p.k_sb + (int64_t)kvh * p.k_sh);
+  const char* const vrows =
+      reinterpret_cast<const char*>(reinterpret_cast<const T*>(p.v) + (int64_t)b * p.v_sb + (int64_t)kvh * p.v_sh);
+  const bool listed = kMode == kIndex && (!kPaged || p.index != nullptr);
+  const int n = min(load_early(p.ctx_lens + b), p.max_ctx);
+  const int c = min(p.counts ? load_early(p.counts + b) : n, p.max_selected);
+  const int rows = min(p.early_rows, min(p.chunk, p.max_selected - start));
+  for (int r0 = 32 * warp; r0 < rows; r0 += 32 * p.early_warps) {
+    const int r = r0 + lane;
+    int pos = -1;
+    if (r < rows) {
+      pos = listed ? load_early(p.index + (int64_t)b * p.index_stride + start + r) : start + r;
+      if (start + r >= c) pos = -1;
+    }
+    if (pos < 0 || pos >= n) pos = -1;
+    if (kPaged && pos >= 0) {
+      const int page = load_early(p.page_table + (int64_t)b * p.page_table_stride + (pos >> p.page_shift));
+      pos = (unsigned)page < (unsigned)p.n_pages ? (page << p.page_shift) | (pos & p.page_mask) : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < 32; i += kRows) {
+      const int row = __shfl_sync(0xffffffffu, pos, i + lane / kSectors);
+      if (row >= 0) {
+        prefetch_sector(krows + (uint64_t)(uint32_t)row * p.k_row_bytes + lane % kSectors * 32);
+        prefetch_sector(vrows + (uint64_t)(uint32_t)row * p.v_row_bytes + lane % kSectors * 32);
+      }
+    }
+  }
+}
+
 // kPaged (index lists only): positions are translated through the page table while they are staged, and a
 // missing list stands for 0, 1, 2, ...; kept out of the unpaged instantiations so that they stay as they are.
 // kHostQ (index lists, one chunk per request): the query rows are still in page-locked host memory.  Each block
@@ -225,6 +266,11 @@ decode_partial_kernel(const DecodeParams p) {
   const int col = lane % kLanesPerRow, sub = lane / kLanesPerRow;
   const int start = chunk_id * p.chunk;
 
+  // (kHostQ: the query row, across the bus, comes first.  Blocked lists have mostly been made by the launch in front, which
+  // leaves no time, and take two trips: 52 requests of 32 heads, six rows each, 14.0 / 16.0 us)
+  if constexpr ((kMode == kIndex || kMode == kDense) && kWarps == kSmallBlock && !kHostQ)
+    if (warp < p.early_warps && blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) < (unsigned)p.early_blocks)
+      prefetch_early<T, D, kMode, kPaged>(p, b, h / p.kv_group, start, warp);
   grid_dependency_wait();
   if (p.early_release) grid_launch_dependents();      // small grid: let the next kernel's blocks move in now
 
@@ -936,6 +982,31 @@ struct SpanLists { const int32_t* span_offsets; const int32_t* spans; int32_t sp
 
 static size_t counts_bytes(const ssa_attn_desc* d) { return ((size_t)d->B * sizeof(int32_t) + 255) / 256 * 256; }
 
+// Which blocks use the time before grid_dependency_wait(), and how (prefetch_early).  Launches follow one another, and the blocks
+// of one move in while the last blocks of the one in front drain, 3..7 us before they may begin; the memory system is half idle
+// then, and altogether so for two microseconds more, until the lists have arrived and name the first rows.  What is asked for in
+// L2 meanwhile should fill that gap and no more, since the blocks in front still wait for their own rows.
+// One head per block: blocks of kSmallBlock warps, five of eight that fit the chip (the others come too late to gain by it), two
+// turns of rows each, by one warp.  us, 64 requests of 32 heads over 141 listed rows: none 28.5, so 27.0; 592 blocks with one
+// turn 26.9, with two 28.3, 370 with four 28.2, all four warps asking 28.1; 16 x 32 heads x 200 rows 12.1 / 10.0, 37 x 32 x 100
+// 15.0 / 13.1, 20 x 32 x 400 28.3 / 27.0.  A launch of a wave or less over lists of one turn has nothing to gain (16 x 32 x 40
+// 4.55 / 4.65; 37 x 32 x 40 9.1 / 8.2), nor have the shortest lists behind an index launch (61 x 32 x 15 14.2 / 14.4) and launches
+// of larger blocks, two per SM at most (7 requests of 8 heads and up to 900 rows 11.7 / 13.2).
+// Row-sharing launches are a wave: three of four blocks, the rows that fill the rings, by four warps, or what these ask for at once
+// where there are fewer blocks than SMs.  us, 32 heads over 8, 32 requests of 820 rows 21.9 / 18.6, of 400 13.6 / 11.2, 8-bit rows
+// 15.6 / 14.1; 4 requests of 820 9.2 / 8.7, of 100 4.9 / 4.9; one warp asking 19.4 for the first of these, for 512 rows 20.3.  (Not
+// groups above sixteen, whose registers are short.)
+static void plan_early(const ssa_attn_desc* d, const Plan& pl, int max_selected, DecodeParams* p) {
+  const int sms = sm_count(), turn = kSmallBlock * 16 * (128 / d->D) * (d->kv_dtype == SSA_FP8_E4M3 ? 2 : 1);
+  p->early_blocks = 0;
+  p->early_warps = pl.share ? 4 : 1;
+  p->early_rows = !pl.share ? 2 * turn : (long long)d->B * d->H_kv * pl.n_chunks < sms ? 128 : 192;
+  if (pl.share) p->early_blocks = sms * 3 / 2;
+  else if (pl.warps == kSmallBlock && (max_selected > turn || (2 * max_selected > turn &&
+                                                               (long long)d->B * d->H * pl.n_chunks > SSA_MIN_BLOCKS * sms)))
+    p->early_blocks = sms * SSA_MIN_BLOCKS * 5 / 8;
+}
+
 // mode kDense: index/counts unused.  kIndex: the index list.  kBlockMask: `counts`
 // are the numbers of listed blocks, `index_stride` the list capacity in blocks,
 // `max_selected` the host bound on listed blocks, `bl` the lists.  kSpans: `sl`
@@ -1047,6 +1118,7 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   // as its blocks finish, so that waiting blocks do not crowd out its own.
   p.early_release = pl.even_blocks == 0 &&
                     (long long)d->B * d->H * pl.n_chunks <= (long long)sm_count() * SSA_MIN_BLOCKS * 6;
+  plan_early(d, pl, max_selected, &p);
   const float scale = d->scale > 0.f ? d->scale : 1.0f / sqrtf((float)d->D);
   p.scale_log2 = scale * kLog2e;
 

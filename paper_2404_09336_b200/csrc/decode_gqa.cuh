@@ -376,6 +376,11 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   const int chunk_id = kSplit ? blockIdx.x / p.head_splits : blockIdx.x, part = kSplit ? blockIdx.x - chunk_id * p.head_splits : 0;
   const int h0 = kSplit ? part * p.heads_per_block : 0, heads = kSplit ? min(p.heads_per_block, G - h0) : G;
 
+  if constexpr (!kEven && !kSplit && kMode != kSpans)
+    if (warp < p.early_warps && blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) < (unsigned)p.early_blocks) {
+      if (kMode == kIndex && p.page_table) prefetch_early<T, D, kIndex, true>(p, blockIdx.z, blockIdx.y, blockIdx.x * p.chunk, warp);
+      else prefetch_early<T, D, kMode, false>(p, blockIdx.z, blockIdx.y, blockIdx.x * p.chunk, warp);
+    }
   grid_dependency_wait();
   if (p.early_release) grid_launch_dependents();
   uint32_t flags = 0;

@@ -26,6 +26,17 @@ int sm_count();   // multiprocessors of the current device (cached; no synchroni
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Before that wait a block may only read, and what it reads may be about to change: an input that the kernel in front is
+// still writing.  It is good for guesses alone: which cache rows to prefetch, or work that is checked against the
+// inputs after the wait.  (relaxed.gpu: from L2, so that no stale line is left in L1.)
+__device__ __forceinline__ int32_t load_early(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// The 32 bytes around p into L2.
+__device__ __forceinline__ void prefetch_sector(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t dynamic_smem,
                                    cudaStream_t stream, Args... args) {
