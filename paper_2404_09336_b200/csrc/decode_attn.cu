@@ -66,6 +66,7 @@ struct DecodeParams {
   const int32_t* span_offsets;  // span lists only: [B+1]
   const int2* spans;            //   (start, end) pairs
   int32_t span_cap;             //   spans taken per request (<= kDirectSpans)
+  int32_t spans_readable;       //   pairs that may be read from `spans` on before their offsets can be trusted (0: none)
   int32_t* index_out;           //   optional copy of the positions, [B, index_stride]
   int32_t* counts_out;          //   optional number of positions per request
   int32_t* ws_counts;           //   the same for the second pass (when n_chunks > 1)
@@ -77,13 +78,14 @@ struct DecodeParams {
   int64_t q_sb, q_sh, k_sb, k_sh, v_sb, v_sh, o_sb, o_sh;
   uint32_t k_row_bytes, v_row_bytes;   // token stride of the cache in bytes
   int32_t H, max_ctx, index_stride, max_selected, chunk, n_chunks, out_f32, early_release;
-  int32_t early_blocks, early_rows, early_warps;   // see plan_early
+  int32_t early_blocks, guess_blocks;   // see plan_early
+  int16_t early_rows, early_warps;
   int32_t kv_group;         // query heads per K/V head (1: multi-head attention)
-  int32_t warps;            // warps of a one-head block
-  int32_t share_rows;       // row-sharing kernel (otherwise one query head per block)
+  int16_t warps;            // warps of a one-head block
+  uint8_t share_rows;       // row-sharing kernel (otherwise one query head per block)
+  uint8_t gqa_wide;         // row-sharing kernel, one large block per SM
   int32_t head_splits;      // row-sharing kernel: blocks that share the heads of a group, heads_per_block each
   int32_t heads_per_block;
-  int32_t gqa_wide;         // row-sharing kernel, one large block per SM
   int32_t even_blocks;      // row-sharing kernel over full contexts: blocks that share the rows evenly (0: fixed chunks)
   int32_t even_factor;      // ... unless the lengths make slices of `chunk` rows the better cut (even_by_slices)
   int32_t B;
@@ -191,10 +193,11 @@ __device__ __forceinline__ void halve_between(float2 (&out)[N], const float2 (&i
 // Called before grid_dependency_wait() by each of the first p.early_warps warps of a block: they ask for the first p.early_rows rows of the
 // block in L2, by the lists as they stand.  Neighbouring lanes take the
 // sectors of a row: with a row per lane the requests took four times as long to issue.  (Lists, counts, lengths and page tables are
-// read where the host says they are, and no further; what they name is checked against max_ctx and n_pages.  Span lists are left
-// alone: their offsets, not yet to be trusted, would say where to read.)
+// read where the host says they are, and no further; what they name is checked against max_ctx and n_pages.)
+// kSpans: the warp has the request's runs in `runs` (runs_p of them, n and c positions).
 template <typename T, int D, int kMode, bool kPaged>
-__device__ __forceinline__ void prefetch_early(const DecodeParams& p, int b, int kvh, int start, int warp) {
+__device__ __forceinline__ void prefetch_early(const DecodeParams& p, int b, int kvh, int start, int warp,
+                                               const WarpRuns* runs = nullptr, int runs_p = 0, int n_of_spans = 0, int c_of_spans = 0) {
   constexpr int kSectors = D * (int)sizeof(T) / 32, kRows = 32 / kSectors;   // of a row; rows an instruction covers
   const int lane = threadIdx.x & 31;
   const char* const krows =
@@ -202,14 +205,15 @@ __device__ __forceinline__ void prefetch_early(const DecodeParams& p, int b, int
   const char* const vrows =
       reinterpret_cast<const char*>(reinterpret_cast<const T*>(p.v) + (int64_t)b * p.v_sb + (int64_t)kvh * p.v_sh);
   const bool listed = kMode == kIndex && (!kPaged || p.index != nullptr);
-  const int n = min(load_early(p.ctx_lens + b), p.max_ctx);
-  const int c = min(p.counts ? load_early(p.counts + b) : n, p.max_selected);
+  const int n = kMode == kSpans ? n_of_spans : min(load_early(p.ctx_lens + b), p.max_ctx);
+  const int c = kMode == kSpans ? c_of_spans : min(p.counts ? load_early(p.counts + b) : n, p.max_selected);
   const int rows = min(p.early_rows, min(p.chunk, p.max_selected - start));
   for (int r0 = 32 * warp; r0 < rows; r0 += 32 * p.early_warps) {
     const int r = r0 + lane;
     int pos = -1;
     if (r < rows) {
-      pos = listed ? load_early(p.index + (int64_t)b * p.index_stride + start + r) : start + r;
+      if constexpr (kMode == kSpans) pos = start + r < c ? span_position(*runs, runs_p, start + r) : -1;
+      else pos = listed ? load_early(p.index + (int64_t)b * p.index_stride + start + r) : start + r;
       if (start + r >= c) pos = -1;
     }
     if (pos < 0 || pos >= n) pos = -1;
@@ -271,6 +275,21 @@ decode_partial_kernel(const DecodeParams p) {
   if constexpr ((kMode == kIndex || kMode == kDense) && kWarps == kSmallBlock && !kHostQ)
     if (warp < p.early_warps && blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) < (unsigned)p.early_blocks)
       prefetch_early<T, D, kMode, kPaged>(p, b, h / p.kv_group, start, warp);
+  // span lists of up to 32: blocks that wait merge them meanwhile, and see afterwards whether that still holds
+  const bool warp_merge = kMode == kSpans && p.span_cap <= 32;
+  int warp_runs = 1;                                  // span_cap rounded up to a power of two
+  while (warp_merge && warp_runs < p.span_cap) warp_runs <<= 1;
+  EarlySpans guess;
+  guess.there = false;
+  if constexpr (kMode == kSpans) {
+    const unsigned block = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+    if (warp_merge && p.spans_readable > 0 && block < (unsigned)p.guess_blocks) {
+      guess = merge_spans_early(s_wruns[warp], p.span_offsets, p.spans, p.spans_readable, p.ctx_lens, p.max_ctx, b, p.span_cap, warp_runs);
+      if (guess.there && warp < p.early_warps && block < (unsigned)p.early_blocks)
+        prefetch_early<T, D, kSpans, false>(p, b, h / p.kv_group, start, warp, &s_wruns[warp], warp_runs, guess.n,
+                                            min(guess.total, p.max_selected));
+    }
+  }
   grid_dependency_wait();
   if (p.early_release) grid_launch_dependents();      // small grid: let the next kernel's blocks move in now
 
@@ -312,8 +331,8 @@ decode_partial_kernel(const DecodeParams p) {
   // fixed-stride table needs no offsets, so the spans then arrive together with the sizes and the query)
   int span_first = 0, span_n = 0;
   int2 my_span = make_int2(0, 0);
-  const bool warp_merge = kMode == kSpans && p.span_cap <= 32;
   if constexpr (kMode == kSpans) {
+    if (guess.there && lane < guess.S) my_span = __ldg(p.spans + guess.first + lane);
     if (p.span_offsets) {
       span_first = __ldg(p.span_offsets + b);
       span_n = __ldg(p.span_offsets + b + 1) - span_first;
@@ -321,7 +340,7 @@ decode_partial_kernel(const DecodeParams p) {
       span_first = b * p.span_cap;
       span_n = p.span_cap;
     }
-    if (warp_merge && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
+    if (warp_merge && !guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
   }
   // blocked lists: every warp takes all words of the block's entries, one per lane (those beyond the list are ignored below)
   int mask_block = -1;
@@ -337,12 +356,14 @@ decode_partial_kernel(const DecodeParams p) {
   uint32_t flags = 0;
   int n, c;
   request_sizes(p, b, n, c, flags);
-  int warp_runs = 1;                                  // span_cap rounded up to a power of two
-  while (warp_merge && warp_runs < p.span_cap) warp_runs <<= 1;
   if constexpr (kMode == kSpans) {
     // the request's spans -> disjoint ascending runs in shared memory (every block of the request repeats this)
     int total;
-    if (warp_merge) {                                 // up to 32 spans: every warp merges them for itself, no barrier
+    if (warp_merge && still_the_spans(guess, span_first, span_n, n, my_span)) {
+      total = guess.total;
+      flags |= guess.flags;
+    } else if (warp_merge) {                          // up to 32 spans: every warp merges them for itself, no barrier
+      if (guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
       int S = max(span_n, 0);
       if (S > p.span_cap) { S = p.span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
       total = merge_spans_warp(s_wruns[warp], my_span, S, warp_runs, n, flags);
@@ -994,17 +1015,29 @@ static size_t counts_bytes(const ssa_attn_desc* d) { return ((size_t)d->B * size
 // of larger blocks, two per SM at most (7 requests of 8 heads and up to 900 rows 11.7 / 13.2).
 // Row-sharing launches are a wave: three of four blocks, the rows that fill the rings, by four warps, or what these ask for at once
 // where there are fewer blocks than SMs.  us, 32 heads over 8, 32 requests of 820 rows 21.9 / 18.6, of 400 13.6 / 11.2, 8-bit rows
-// 15.6 / 14.1; 4 requests of 820 9.2 / 8.7, of 100 4.9 / 4.9; one warp asking 19.4 for the first of these, for 512 rows 20.3.  (Not
+// 15.6 / 14.1; 4 requests of 820 9.2 / 8.7, of 100 4.9 / 4.9; one warp asking 19.4 for the first of these, for 512 rows 20.3; 2 full contexts of 300 rows, 12
+// heads, 7.8 / 7.9: these, and whoever else is few, have no lists to wait for.  (Not
 // groups above sixteen, whose registers are short.)
-static void plan_early(const ssa_attn_desc* d, const Plan& pl, int max_selected, DecodeParams* p) {
+// Span lists of up to 32 are merged before the wait by every block that fits the chip, and by the others as before: checking
+// that the list is still the same takes one trip, reading and merging it two and 0.4 us.  us, one-kernel steps, merged after / before
+// the wait: 16 requests, 32 heads, three spans of 40: 10.9 / 8.9, 48 x 8 heads, 14 of 20: 13.7 / 12.3, 4 x 8, six of 20 5.1 / 4.6.
+// What then is left for row-sharing blocks to prefetch in pays for lists of one chunk that take them longest: 32 heads over 8, 32
+// requests of six spans of 100 15.9 / 13.3, 8-bit rows 12.4 / 11.4; but with a merge launch in front, which is short, 4 requests of
+// 14 spans 10.0 / 11.0, and 16 of three, 8-bit rows, 7.3 / 7.6.
+static void plan_early(const ssa_attn_desc* d, const Plan& pl, int max_selected, int mode, DecodeParams* p) {
   const int sms = sm_count(), turn = kSmallBlock * 16 * (128 / d->D) * (d->kv_dtype == SSA_FP8_E4M3 ? 2 : 1);
+  const bool few = (long long)d->B * d->H_kv * pl.n_chunks < sms;
   p->early_blocks = 0;
   p->early_warps = pl.share ? 4 : 1;
-  p->early_rows = !pl.share ? 2 * turn : (long long)d->B * d->H_kv * pl.n_chunks < sms ? 128 : 192;
-  if (pl.share) p->early_blocks = sms * 3 / 2;
+  p->early_rows = !pl.share ? 2 * turn : few ? 128 : 192;
+  const bool in_time = mode == kSpans ? pl.n_chunks == 1 && max_selected * (d->kv_dtype == SSA_FP8_E4M3 ? 1 : 2) >= 600
+                                      : mode != kDense || !few;
+  if (pl.share) p->early_blocks = in_time ? sms * 3 / 2 : 0;
   else if (pl.warps == kSmallBlock && (max_selected > turn || (2 * max_selected > turn &&
                                                                (long long)d->B * d->H * pl.n_chunks > SSA_MIN_BLOCKS * sms)))
     p->early_blocks = sms * SSA_MIN_BLOCKS * 5 / 8;
+  p->guess_blocks = pl.share ? 2 * sms : kWarpSlots / pl.warps * sms;
+  p->spans_readable = mode == kSpans ? (int)std::min<size_t>(readable_bytes(p->spans) / sizeof(int2), 0x7fffffff) : 0;
 }
 
 // mode kDense: index/counts unused.  kIndex: the index list.  kBlockMask: `counts`
@@ -1118,7 +1151,7 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
   // as its blocks finish, so that waiting blocks do not crowd out its own.
   p.early_release = pl.even_blocks == 0 &&
                     (long long)d->B * d->H * pl.n_chunks <= (long long)sm_count() * SSA_MIN_BLOCKS * 6;
-  plan_early(d, pl, max_selected, &p);
+  plan_early(d, pl, max_selected, mode, &p);
   const float scale = d->scale > 0.f ? d->scale : 1.0f / sqrtf((float)d->D);
   p.scale_log2 = scale * kLog2e;
 

@@ -376,8 +376,21 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   const int chunk_id = kSplit ? blockIdx.x / p.head_splits : blockIdx.x, part = kSplit ? blockIdx.x - chunk_id * p.head_splits : 0;
   const int h0 = kSplit ? part * p.heads_per_block : 0, heads = kSplit ? min(p.heads_per_block, G - h0) : G;
 
-  if constexpr (!kEven && !kSplit && kMode != kSpans)
-    if (warp < p.early_warps && blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) < (unsigned)p.early_blocks) {
+  const unsigned block = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+  const bool warp_merge = kMode == kSpans && p.span_cap <= 32;
+  int runs = 1;                                        // span_cap rounded up to a power of two
+  while (warp_merge && runs < p.span_cap) runs <<= 1;
+  EarlySpans guess;                                    // (see decode_partial_kernel)
+  guess.there = false;
+  if constexpr (kMode == kSpans) {
+    if (warp_merge && p.spans_readable > 0 && block < (unsigned)p.guess_blocks) {
+      guess = merge_spans_early(s_wruns[warp], p.span_offsets, p.spans, p.spans_readable, p.ctx_lens, p.max_ctx, blockIdx.z, p.span_cap, runs);
+      if (!kSplit && guess.there && warp < p.early_warps && block < (unsigned)p.early_blocks)
+        prefetch_early<T, D, kSpans, false>(p, blockIdx.z, blockIdx.y, blockIdx.x * p.chunk, warp, &s_wruns[warp], runs, guess.n,
+                                            min(guess.total, p.max_selected));
+    }
+  } else if constexpr (!kEven && !kSplit)
+    if (warp < p.early_warps && block < (unsigned)p.early_blocks) {
       if (kMode == kIndex && p.page_table) prefetch_early<T, D, kIndex, true>(p, blockIdx.z, blockIdx.y, blockIdx.x * p.chunk, warp);
       else prefetch_early<T, D, kMode, false>(p, blockIdx.z, blockIdx.y, blockIdx.x * p.chunk, warp);
     }
@@ -441,21 +454,24 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     // span lists: up to 32 spans are merged by every warp for itself, which needs no barrier (one warp for the block, us: 32
     // requests of 819 rows, four heads on each of 8 K/V heads over an 8-bit cache 17.75 -> 16.98, 20 requests of 5199 or 316
     // rows over a 16-bit one 79.4 -> 72.2); a lane asks for "its" span right away
-    int span_first = 0, span_n = 0, runs = 1;           // runs: span_cap rounded up to a power of two
+    int span_first = 0, span_n = 0;
     int2 my_span = make_int2(0, 0);
-    const bool warp_merge = kMode == kSpans && p.span_cap <= 32;
     if constexpr (kMode == kSpans) {
+      if (guess.there && lane < guess.S) my_span = __ldg(p.spans + guess.first + lane);
       span_first = p.span_offsets ? __ldg(p.span_offsets + b) : b * p.span_cap;
       span_n = p.span_offsets ? __ldg(p.span_offsets + b + 1) - span_first : p.span_cap;
-      if (warp_merge && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
-      while (warp_merge && runs < p.span_cap) runs <<= 1;
+      if (warp_merge && !guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
     }
     int n, c;
     if constexpr (kEven) n = c = s_line.rows[b];
     else request_sizes(p, b, n, c, flags);
     if constexpr (kMode == kSpans) {
       int total;
-      if (warp_merge) {
+      if (warp_merge && still_the_spans(guess, span_first, span_n, n, my_span)) {
+        total = guess.total;
+        flags |= guess.flags;
+      } else if (warp_merge) {
+        if (guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
         int S = max(span_n, 0);
         if (S > p.span_cap) { S = p.span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
         total = merge_spans_warp(s_wruns[warp], my_span, S, runs, n, flags);

@@ -177,6 +177,39 @@ __device__ __forceinline__ int merge_spans_warp(WarpRuns& w, int2 my_span, int S
   return total;
 }
 
+// A request's spans merged ahead of grid_dependency_wait() (merge_spans_early), for a guess that is checked after it
+// (still_the_spans): the kernel in front may yet write the list.
+struct EarlySpans {
+  bool there;                               // warp-uniform: the list could be read
+  int first, S, n, total;                   // where it was, how long; the context; what merge_spans_warp returned
+  int2 span;                                // lane i < S: span i
+  uint32_t flags;
+};
+
+// `readable`: the pairs that may be read from `spans` on, whatever span_offsets says.
+__device__ __forceinline__ EarlySpans merge_spans_early(WarpRuns& w, const int32_t* span_offsets, const int2* spans, int readable,
+                                                        const int32_t* ctx_lens, int max_ctx, int b, int cap, int P) {
+  EarlySpans e;
+  const int lane = threadIdx.x & 31;
+  e.first = span_offsets ? load_early(span_offsets + b) : b * cap;
+  e.S = span_offsets ? load_early(span_offsets + b + 1) - e.first : cap;
+  e.n = max(min(load_early(ctx_lens + b), max_ctx), 0);
+  e.there = e.first >= 0 && e.S >= 0 && e.S <= cap && e.first <= readable - e.S;
+  e.span = make_int2(0, 0);
+  e.flags = 0;
+  e.total = 0;
+  if (e.there) {
+    if (lane < e.S) e.span = load_early(spans + e.first + lane);
+    e.total = merge_spans_warp(w, e.span, e.S, P, e.n, e.flags);
+  }
+  return e;
+}
+
+// Whether the list is still what was merged: `now` is the span this lane finds where it found e.span.
+__device__ __forceinline__ bool still_the_spans(const EarlySpans& e, int first, int S, int n, int2 now) {
+  return __all_sync(0xffffffffu, e.there && first == e.first && S == e.S && n == e.n && now.x == e.span.x && now.y == e.span.y) != 0;
+}
+
 // The k-th attended position (0 <= k < offs[P]) among P runs.
 __device__ __forceinline__ int span_position(const WarpRuns& w, int P, int k) {
   int lo = 0;

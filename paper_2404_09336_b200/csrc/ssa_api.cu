@@ -2,6 +2,8 @@
 // hook and the launch counter.
 #include <atomic>
 
+#include <cuda.h>
+
 #include "ssa_common.cuh"
 
 namespace ssa {
@@ -24,6 +26,31 @@ int sm_count() {
   }
   cached[dev].store(n, std::memory_order_relaxed);
   return n;
+}
+
+// One driver query, 35 ns.  (Only cudaMalloc's memory, what classic IPC handles are for: pools and address ranges that were
+// mapped piece by piece may end sooner than the answer says.)
+size_t readable_bytes(const void* p) {
+  using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Query>(f);
+  }();
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  int whole = 0;
+  CUpointer_attribute ask[] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
+                               CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE};
+  void* answer[] = {&start, &size, &whole};
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  if (!query || query(3, ask, answer, at) != CUDA_SUCCESS || !whole || at < start || at - start >= size) return 0;
+  return size - (at - start);
 }
 
 static thread_local uint64_t t_launches = 0;

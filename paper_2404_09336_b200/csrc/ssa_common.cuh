@@ -17,6 +17,9 @@ constexpr float kLn2 = 0.6931471805599453f;
 void note_launches(int n);
 void take_kernel_events(cudaEvent_t* begin, cudaEvent_t* end);
 int sm_count();   // multiprocessors of the current device (cached; no synchronisation)
+// Bytes from p to the end of the allocation it lies in, as far as that is device memory mapped as a whole; else 0.  Reading
+// these is safe whatever offsets said that they are a list.
+size_t readable_bytes(const void* p);
 
 // Programmatic dependent launch.  Every kernel of the library is launched
 // with the programmatic-serialization attribute: its blocks may become
@@ -33,6 +36,11 @@ __device__ __forceinline__ int32_t load_early(const int32_t* p) {
   int32_t v;
   asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ int2 load_early(const int2* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return make_int2((int32_t)(uint32_t)v, (int32_t)(v >> 32));
 }
 // The 32 bytes around p into L2.
 __device__ __forceinline__ void prefetch_sector(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }

@@ -73,3 +73,55 @@ def test_lists_that_the_launch_in_front_still_writes(B, H, Hkv, D, rows, page_si
         assert torch.equal(cnt, sp[:, 1] - sp[:, 0])
         # fp32 rows: weights exact to 2^-16 (row-sharing kernel) or better, so 1e-4 of values of order 1 is ample
         assert float((out.double() - rows_of(q, k, v, idx, cnt)).abs().max()) < 1e-4
+
+
+# blocks of one head, of eight and sixteen warps, row-sharing (ordinary, wide, two chunks, above sixteen heads)
+@pytest.mark.parametrize("B,H,Hkv,D,dtype", [
+    (80, 8, 8, 128, "bf16"), (20, 8, 8, 128, "bf16"), (3, 8, 8, 64, "bf16"), (40, 32, 8, 128, "bf16"), (40, 8, 2, 128, "fp8"),
+    (3, 32, 8, 128, "bf16"), (20, 20, 1, 128, "bf16")])
+def test_lists_and_spans_that_an_attention_launch_in_front_writes(B, H, Hkv, D, dtype):
+    """An attention launch lets the next one's blocks move in as soon as its own have: they then read what it has yet to write.
+    Its lists are the next call's: as lists, and their pairs as spans, with its counts as contexts."""
+    gen = torch.Generator(device=DEV).manual_seed(B * H + D)
+    T, rows = 700, 300
+    q = torch.randn(B, H, D, device=DEV, generator=gen).bfloat16()
+    kv = torch.float8_e4m3fn if dtype == "fp8" else torch.bfloat16
+    k, v = (torch.randn(B, Hkv, T, D, device=DEV, generator=gen).bfloat16().to(kv) for _ in range(2))
+    i32 = dict(dtype=torch.int32, device=DEV)
+    n = 8
+    starts = torch.randint(0, 300, (n, B), device=DEV, generator=gen, dtype=torch.int32)
+    lengths = torch.randint(1, rows // 10, (n, B), device=DEV, generator=gen, dtype=torch.int32) * 10
+    lengths[0], lengths[1] = 60, 290                     # the same for all, then others everywhere
+    spans = torch.stack([starts, starts + lengths], -1).contiguous()
+    ctx, offsets = torch.full((B,), T, **i32), torch.arange(B + 1, **i32)
+    index, counts = torch.full((B, rows), 5, **i32), torch.zeros(B, **i32)
+    pairs = 29                                           # at most 32 are merged by a warp
+    status = torch.zeros(1, **i32)
+    out = [torch.full((n, B, H, D), 7.0, device=DEV) for _ in range(3)]
+    desc = ssa.make_desc(q, k, v, out[0][0])
+    ws = torch.empty(max(ssa.decode_spans_workspace_bytes(desc, rows, 150), 16), dtype=torch.uint8, device=DEV)
+    table, table_counts = torch.full((B, 2 * pairs), 3, **i32), torch.zeros(B, **i32)
+    kept, (kr, vr) = [], (k.bfloat16(), v.bfloat16())
+    torch.cuda.synchronize()
+    for i in range(n):
+        ssa.decode_attn_spans(desc, q, k, v, ctx, offsets, spans[i], 1, rows, out[0][i], index_out=index, counts_out=counts,
+                              workspace=ws, dev_status=status)
+        ssa.decode_attn_sparse(desc, q, k, v, ctx, index, counts, rows, out[1][i], None, ws, status)
+        # the first pairs of a list of 2 * pairs rows, as a table of spans without offsets
+        ssa.decode_attn_spans(desc, q, k, v, ctx, offsets, spans[i], 1, 2 * pairs, out[2][i], index_out=table,
+                              counts_out=table_counts, workspace=ws, dev_status=status)
+        ssa.decode_attn_spans(desc, q, k, v, counts, None, table, pairs, pairs, out[2][i], workspace=ws, dev_status=status)
+        kept.append((index.clone(), counts.clone(), table.clone()))
+    torch.cuda.synchronize()
+    for i, (idx, cnt, tab) in enumerate(kept):
+        assert torch.equal(cnt, lengths[i])
+        want = rows_of(q, kr, vr, idx, cnt)
+        for got in (out[0][i], out[1][i]):
+            assert float((got.double() - want).abs().max()) < 1e-4
+        # the pairs of the table are (p, p + 1), or (3, 3) where nothing has been written, below the contexts that the counts are
+        at, live = tab[:, 0::2], (tab[:, 1::2] > tab[:, 0::2]) & (tab[:, 0::2] < cnt[:, None])
+        chosen, num = torch.zeros(B, pairs, **i32), torch.zeros(B, **i32)
+        for b in range(B):
+            rows_b = at[b][live[b]].unique()
+            chosen[b, :len(rows_b)], num[b] = rows_b, len(rows_b)
+        assert float((out[2][i].double() - rows_of(q, kr, vr, chosen, num)).abs().max()) < 1e-4
