@@ -12,7 +12,7 @@ constexpr int kRefWarps = 4;
 
 __global__ void __launch_bounds__(kRefWarps * 32)
 refs_to_spans_kernel(const ssa_anchor_tables t, int32_t B, int32_t* __restrict__ span_offsets_out,
-                     int32_t* __restrict__ spans_out, int32_t span_stride, uint32_t* __restrict__ dev_status) {
+                     int32_t* __restrict__ spans_out, int32_t span_stride, uint32_t* __restrict__ dev_status, const Spare<40>) {
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * kRefWarps + (threadIdx.x >> 5);
   grid_dependency_wait();
@@ -43,7 +43,7 @@ extern "C" int32_t ssa_refs_to_spans(const ssa_anchor_tables* t, int32_t B, int3
   const unsigned blocks = (unsigned)((B + ssa::kRefWarps - 1) / ssa::kRefWarps);
   const cudaError_t err = ssa::launch_pdl(ssa::refs_to_spans_kernel, dim3(blocks), dim3(ssa::kRefWarps * 32),
                                           (cudaStream_t)stream, *t, B, span_offsets_out, spans_out, span_stride,
-                                          dev_status);
+                                          dev_status, ssa::Spare<40>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   ssa::note_launches(1);
   return SSA_OK;

@@ -21,7 +21,7 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
                           const int32_t* __restrict__ ctx_lens, int32_t block_size,
                           int32_t* __restrict__ block_idx, uint32_t* __restrict__ block_mask,
                           int32_t block_stride, int32_t* __restrict__ block_counts,
-                          uint32_t* __restrict__ dev_status) {
+                          uint32_t* __restrict__ dev_status, const Spare<16>) {
   __shared__ int2 s_span[kBmMaxSpans];
   __shared__ uint32_t s_word[kBmThreads];
   __shared__ int s_wcount[kBmThreads / 32];
@@ -108,7 +108,7 @@ extern "C" int32_t ssa_spans_to_blockmask(const int32_t* span_offsets, const int
   if (reinterpret_cast<uintptr_t>(spans) % 8 != 0) return SSA_ERR_ALIGN;
   const cudaError_t err = ssa::launch_pdl(ssa::spans_to_blockmask_kernel, dim3((unsigned)B), dim3(ssa::kBmThreads),
                                           (cudaStream_t)stream, span_offsets, spans, ctx_lens, block_size,
-                                          block_idx, block_mask, block_stride, block_counts, dev_status);
+                                          block_idx, block_mask, block_stride, block_counts, dev_status, ssa::Spare<16>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   ssa::note_launches(1);
   return SSA_OK;

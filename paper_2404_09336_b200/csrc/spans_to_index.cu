@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kIdxThreads)
 spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
                       int32_t index_stride, int32_t slice, int32_t* __restrict__ counts,
                       uint32_t* __restrict__ dev_status, const FetchJob job,
-                      int32_t capacity, int32_t span_cap) {
+                      int32_t capacity, int32_t span_cap, const Spare<48>) {
   // index_stride: distance between the rows of `index`; capacity <= index_stride: most positions a list keeps;
   // span_cap <= kMaxSpans: most spans a request may have
   if (kFetch && (int)blockIdx.y >= job.first_row) {
@@ -307,7 +307,7 @@ int32_t fetch_and_index(const int32_t* host_span_offsets, const int32_t* host_sp
   FetchJob job = {reinterpret_cast<uint4*>(dst), reinterpret_cast<const uint4*>(src), n16, B};
   dim3 grid((unsigned)slices, (unsigned)(B + std::max(copy_rows, 1)));
   const cudaError_t err = launch_pdl(spans_to_index_kernel<false, true>, grid, dim3(kIdxThreads), stream, s,
-                                     index, index_stride, slice, counts, dev_status, job, index_stride, kMaxSpans);
+                                     index, index_stride, slice, counts, dev_status, job, index_stride, kMaxSpans, Spare<48>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   note_launches(1);
   return SSA_OK;
@@ -328,7 +328,7 @@ int32_t spans_to_index_capped(const int32_t* span_offsets, const int32_t* spans,
   SpanSource src = {};
   src.span_offsets = span_offsets; src.spans = spans; src.ctx_lens = ctx_lens;
   const cudaError_t err = launch_pdl(spans_to_index_kernel<false>, grid, dim3(kIdxThreads), stream, src, index,
-                                     index_stride, slice, counts, dev_status, FetchJob{}, capacity, span_cap);
+                                     index_stride, slice, counts, dev_status, FetchJob{}, capacity, span_cap, Spare<48>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   note_launches(1);
   return SSA_OK;
@@ -358,7 +358,7 @@ extern "C" int32_t ssa_refs_to_index(const ssa_anchor_tables* tables, int32_t B,
   src.tables = *tables;
   const cudaError_t err = ssa::launch_pdl(ssa::spans_to_index_kernel<true>, grid, dim3(ssa::kIdxThreads),
                                           (cudaStream_t)stream, src, index, index_stride, slice, counts,
-                                          dev_status, ssa::FetchJob{}, index_stride, ssa::kMaxSpans);
+                                          dev_status, ssa::FetchJob{}, index_stride, ssa::kMaxSpans, ssa::Spare<48>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   ssa::note_launches(1);
   return SSA_OK;
