@@ -1037,7 +1037,8 @@ static void plan_early(const ssa_attn_desc* d, const Plan& pl, int max_selected,
                                                                (long long)d->B * d->H * pl.n_chunks > SSA_MIN_BLOCKS * sms)))
     p->early_blocks = sms * SSA_MIN_BLOCKS * 5 / 8;
   p->guess_blocks = pl.share ? 2 * sms : kWarpSlots / pl.warps * sms;
-  p->spans_readable = mode == kSpans ? (int)std::min<size_t>(readable_bytes(p->spans) / sizeof(int2), 0x7fffffff) : 0;
+  Allocation known = {};
+  p->spans_readable = mode == kSpans ? readable_entries<int2>(p->spans, &known) : 0;
 }
 
 // mode kDense: index/counts unused.  kIndex: the index list.  kBlockMask: `counts`

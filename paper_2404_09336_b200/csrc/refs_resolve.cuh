@@ -11,17 +11,24 @@ struct RefTables {
   int l0, n_lines, a0, n_anchors, r0, n_refs;
   int2 prefix, current;                     // the instruction prefix and the line being generated
 };
+// kEarly: as they stand before grid_dependency_wait().
+template <bool kEarly = false>
 __device__ __forceinline__ RefTables locate_refs(const ssa_anchor_tables& t, int b) {
+  auto load = [](const int32_t* p) { return kEarly ? load_early(p) : *p; };
   RefTables r;
-  r.l0 = t.line_offsets[b];
-  r.a0 = t.anchor_offsets[b];
-  r.r0 = t.ref_offsets[b];
-  r.n_lines = max(t.line_offsets[b + 1] - r.l0, 0);
-  r.n_anchors = max(t.anchor_offsets[b + 1] - r.a0, 0);
-  r.n_refs = max(t.ref_offsets[b + 1] - r.r0, 0);
-  r.prefix = make_int2(0, t.prefix_len[b]);
-  r.current = make_int2(t.line_start[b], t.ctx_lens[b]);
+  r.l0 = load(t.line_offsets + b);
+  r.a0 = load(t.anchor_offsets + b);
+  r.r0 = load(t.ref_offsets + b);
+  r.n_lines = max(load(t.line_offsets + b + 1) - r.l0, 0);
+  r.n_anchors = max(load(t.anchor_offsets + b + 1) - r.a0, 0);
+  r.n_refs = max(load(t.ref_offsets + b + 1) - r.r0, 0);
+  r.prefix = make_int2(0, load(t.prefix_len + b));
+  r.current = make_int2(load(t.line_start + b), load(t.ctx_lens + b));
   return r;
+}
+__device__ __forceinline__ bool same_tables(const RefTables& a, const RefTables& b) {
+  return a.l0 == b.l0 && a.n_lines == b.n_lines && a.a0 == b.a0 && a.n_anchors == b.n_anchors && a.r0 == b.r0 &&
+         a.n_refs == b.n_refs && a.prefix.y == b.prefix.y && a.current.x == b.current.x && a.current.y == b.current.y;
 }
 
 // The tables as they lie in global memory.

@@ -16,42 +16,21 @@ constexpr int kBmThreads = 256;
 constexpr int kWindowBits = kBmThreads * 32;           // positions per sweep window
 constexpr int kBmMaxSpans = SSA_MAX_SPANS_PER_SEQ;
 
-__global__ void __launch_bounds__(kBmThreads)
+__global__ void __launch_bounds__(kBmThreads, 4)
 spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_t* __restrict__ spans,
                           const int32_t* __restrict__ ctx_lens, int32_t block_size,
                           int32_t* __restrict__ block_idx, uint32_t* __restrict__ block_mask,
                           int32_t block_stride, int32_t* __restrict__ block_counts,
-                          uint32_t* __restrict__ dev_status, const Spare<16>) {
+                          uint32_t* __restrict__ dev_status, int32_t spans_readable, const Spare<12>) {
   __shared__ int2 s_span[kBmMaxSpans];
   __shared__ uint32_t s_word[kBmThreads];
   __shared__ int s_wcount[kBmThreads / 32];
   __shared__ uint32_t s_flags;
 
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  grid_dependency_wait();
-  const int n = max(ctx_lens[b], 0);
-  const int first = span_offsets[b];
-  int S = span_offsets[b + 1] - first;
-  uint32_t flags = 0;
-  if (S < 0) S = 0;
-  if (S > kBmMaxSpans) { S = kBmMaxSpans; flags |= SSA_DEV_TOO_MANY_SPANS; }
-  if (tid == 0) s_flags = 0;
-  for (int i = tid; i < S; i += kBmThreads) {
-    const int2 se = reinterpret_cast<const int2*>(spans)[first + i];
-    if (se.x < 0 || se.x > se.y) flags |= SSA_DEV_BAD_SPAN;
-    if (se.y > n) flags |= SSA_DEV_CLIPPED;
-    s_span[i] = make_int2(max(se.x, 0), min(se.y, n));  // empty when end <= start
-  }
-  __syncthreads();
-  if (flags) atomicOr(&s_flags, flags);
-
-  const int wpb = block_size / 32;                      // words per block
-  const int blocks_per_window = kBmThreads / wpb;
-  int listed = 0;                                       // non-empty blocks found so far
-  for (int w0 = 0; w0 < n; w0 += kWindowBits) {
-    // word t of the window's bitmap covers positions [w0 + 32 t, w0 + 32 t + 32).  A warp takes a span at a
-    // time and its lanes OR the span's overlap into the words it touches, so the work follows the total
-    // length of the spans, not spans x words.
+  // word t of the bitmap of the window at w0 covers positions [w0 + 32 t, w0 + 32 t + 32).  A warp takes a span at a time and its
+  // lanes OR the span's overlap into the words it touches, so the work follows the total length of the spans, not spans x words.
+  auto mark_window = [&](int w0, int S) {
     s_word[tid] = 0u;
     __syncthreads();
     for (int i = warp; i < S; i += kBmThreads / 32) {
@@ -66,6 +45,55 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
       }
     }
     __syncthreads();
+  };
+  // The first window is marked while the kernel in front drains, by the list as it stands (one span per thread, inside the
+  // allocation: spans_readable), and again only if the list has changed by then.  us, spans -> blocked lists and attention: 64
+  // requests of 32 heads, 1024 of 2048 rows 168.0 -> 166.0; 34 of 8 heads, up to 350 rows 27.2 -> 26.8.
+  bool guess = spans_readable > 0;
+  if (!guess) grid_dependency_wait();
+  int n, S;
+  uint32_t flags;
+  while (true) {
+    const int length = guess ? load_early(ctx_lens + b) : ctx_lens[b];
+    const int first = guess ? load_early(span_offsets + b) : span_offsets[b];
+    const int listed_spans = (guess ? load_early(span_offsets + b + 1) : span_offsets[b + 1]) - first;
+    if (guess && !(first >= 0 && listed_spans >= 0 && listed_spans <= kBmThreads && first <= spans_readable - listed_spans)) {
+      grid_dependency_wait();                           // (block-uniform) no guess
+      guess = false;
+      continue;
+    }
+    n = max(length, 0);
+    S = max(listed_spans, 0);
+    flags = 0;
+    if (S > kBmMaxSpans) { S = kBmMaxSpans; flags |= SSA_DEV_TOO_MANY_SPANS; }
+    if (tid == 0) s_flags = 0;
+    const int2* list = reinterpret_cast<const int2*>(spans) + first;
+    int2 own = make_int2(0, 0);                         // span tid
+    for (int i = tid; i < S; i += kBmThreads) {
+      const int2 se = guess ? load_early(list + i) : list[i];
+      if (i == tid) own = se;
+      if (se.x < 0 || se.x > se.y) flags |= SSA_DEV_BAD_SPAN;
+      if (se.y > n) flags |= SSA_DEV_CLIPPED;
+      s_span[i] = make_int2(max(se.x, 0), min(se.y, n));  // empty when end <= start
+    }
+    mark_window(0, S);
+    if (!guess) break;
+    grid_dependency_wait();
+    guess = false;
+    bool changed = ctx_lens[b] != length || span_offsets[b] != first || span_offsets[b + 1] - first != listed_spans;
+    if (tid < S) {
+      const int2 now = list[tid];
+      changed |= now.x != own.x || now.y != own.y;
+    }
+    if (!__syncthreads_or(changed)) break;
+  }
+  if (flags) atomicOr(&s_flags, flags);
+
+  const int wpb = block_size / 32;                      // words per block
+  const int blocks_per_window = kBmThreads / wpb;
+  int listed = 0;                                       // non-empty blocks found so far
+  for (int w0 = 0; w0 < n; w0 += kWindowBits) {
+    if (w0 > 0) mark_window(w0, S);
     // thread t < blocks_per_window owns block t of the window
     bool nonempty = false;
     if (tid < blocks_per_window)
@@ -106,9 +134,12 @@ extern "C" int32_t ssa_spans_to_blockmask(const int32_t* span_offsets, const int
   if (B <= 0 || block_stride <= 0) return SSA_ERR_SHAPE;
   if (block_size != 32 && block_size != 64 && block_size != 128 && block_size != 256) return SSA_ERR_UNSUPPORTED;
   if (reinterpret_cast<uintptr_t>(spans) % 8 != 0) return SSA_ERR_ALIGN;
+  ssa::Allocation known = {};
+  const int32_t readable = B < 8 ? 0 : ssa::readable_entries<int2>(spans, &known);   // (fewer: the host bounds such calls)
   const cudaError_t err = ssa::launch_pdl(ssa::spans_to_blockmask_kernel, dim3((unsigned)B), dim3(ssa::kBmThreads),
                                           (cudaStream_t)stream, span_offsets, spans, ctx_lens, block_size,
-                                          block_idx, block_mask, block_stride, block_counts, dev_status, ssa::Spare<16>{});
+                                          block_idx, block_mask, block_stride, block_counts, dev_status,
+                                          readable, ssa::Spare<12>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   ssa::note_launches(1);
   return SSA_OK;

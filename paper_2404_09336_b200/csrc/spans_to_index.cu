@@ -37,6 +37,7 @@ constexpr int kIdxThreads = 128;
 constexpr int kMaxSpans = SSA_MAX_SPANS_PER_SEQ;   // power of two
 constexpr int kRankSpans = 2 * kIdxThreads;        // most spans ranked by counting: two per thread
 constexpr int kTable = 512;                        // most entries of an anchor table that are copied to shared memory
+constexpr int kEarlyBlocks = 4;                    // per SM: the first of a launch guess
 constexpr unsigned long long kEmptyKey = 0xffffffffffffffffull;
 
 // Where the spans of a request come from: a span list in global memory, or the anchor tables.
@@ -45,6 +46,8 @@ struct SpanSource {
   const int32_t* spans;
   const int32_t* ctx_lens;
   ssa_anchor_tables tables;
+  // entries that may be read from these on before their offsets can be trusted (0: none); for blocks below early_blocks
+  int32_t spans_readable, lines_readable, anchors_readable, refs_readable, early_blocks;
 };
 
 // kFetch: rows of the grid from first_row on do not expand a request but copy n16 16-byte words from page-locked
@@ -62,7 +65,7 @@ __global__ void __launch_bounds__(kIdxThreads)
 spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
                       int32_t index_stride, int32_t slice, int32_t* __restrict__ counts,
                       uint32_t* __restrict__ dev_status, const FetchJob job,
-                      int32_t capacity, int32_t span_cap, const Spare<48>) {
+                      int32_t capacity, int32_t span_cap, const Spare<24>) {
   // index_stride: distance between the rows of `index`; capacity <= index_stride: most positions a list keeps;
   // span_cap <= kMaxSpans: most spans a request may have
   if (kFetch && (int)blockIdx.y >= job.first_row) {
@@ -88,9 +91,19 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
 
   const int b = blockIdx.y;
   const int tid = threadIdx.x;
-  grid_dependency_wait();      // dependents are released when this grid completes: blocks of a large
-                               // attention grid parked on the SMs during this kernel slowed it down
-  const int n = max(ctx_lens[b], 0);
+  // Steps 1-3 run while the kernel in front drains, on the lists as they stand, and again only if they have changed by then:
+  // seeing that they have not takes one trip to memory, the steps two to four and half a microsecond.  Spans to lists and
+  // attention, 64 requests 28.8 -> 28.1 us; references and attention, 2 requests of ~25 spans 11.6 -> 9.5, 36 of ~38, 8 heads,
+  // 23.9 -> 21.3, 16 of 2 to 50, 32 heads, 41.6 -> 40.5.  (A merge in front is too short to do it all in: 51 of ~20 77.5 -> 77.9.)
+  bool guess = (int)(blockIdx.y * gridDim.x + blockIdx.x) < src.early_blocks;
+  if (!guess) grid_dependency_wait();   // dependents are released when this grid completes: blocks of a large
+                                        // attention grid parked on the SMs during this kernel slowed it down
+  int2* const guess_room = reinterpret_cast<int2*>(keys + 2 * kRankSpans);
+  static_assert(2 * kRankSpans * 8 + kTable * 20 <= kMaxSpans * 8, "a guess's copies lie behind its keys and starts");
+  int P;
+  while (true) {
+  const int length = guess ? load_early(ctx_lens + b) : ctx_lens[b];
+  const int n = max(length, 0);
   uint32_t flags = 0;
   if (tid == 0) s_flags = 0;
 
@@ -103,6 +116,8 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   };
 
   int first = 0, S;
+  int2 raw[2] = {make_int2(0, 0), make_int2(0, 0)};   // spans tid and tid + kIdxThreads of a list of up to kRankSpans
+  RefTables r = {};
   if constexpr (kFromRefs) {
     // 1 (references): warp 0 resolves them and leaves the packed spans, unsorted, in keys[0, S)
     static_assert(4 * kTable <= kMaxSpans, "the copies lie in arrays that step 3 fills");
@@ -113,17 +128,25 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
       __device__ __forceinline__ int2 ref(int i) const { return refs[i]; }
       __device__ __forceinline__ int anchor(int i) const { return anchors[i]; }
     };
-    const RefTables r = locate_refs(src.tables, b);
+    r = guess ? locate_refs<true>(src.tables, b) : locate_refs(src.tables, b);
     const RefsInMemory far(src.tables, r);
-    const Copied near = {reinterpret_cast<int2*>(new_start), reinterpret_cast<int2*>(new_start) + kTable, offs};
+    // (a guess needs its copies for the comparison: behind the keys of a list of up to kRankSpans, where nothing else comes)
+    int2* const room = guess ? guess_room : reinterpret_cast<int2*>(new_start);
+    const Copied near = {room, room + kTable, guess ? reinterpret_cast<int32_t*>(room + 2 * kTable) : offs};
     const bool copied = r.n_lines <= kTable && r.n_anchors <= kTable && r.n_refs <= kTable;
+    if (guess && !(copied && r.l0 >= 0 && r.a0 >= 0 && r.r0 >= 0 && r.l0 <= src.lines_readable - r.n_lines &&
+                   r.a0 <= src.anchors_readable - r.n_anchors && r.r0 <= src.refs_readable - r.n_refs)) {
+      grid_dependency_wait();                         // (block-uniform) no guess
+      guess = false;
+      continue;
+    }
     if (copied) {
       for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
         int2 line = make_int2(0, 0), ref = line;        // all three requested before any is stored
         int anchor = 0;
-        if (i < r.n_lines) line = far.line(i);
-        if (i < r.n_anchors) anchor = far.anchor(i);
-        if (i < r.n_refs) ref = far.ref(i);
+        if (i < r.n_lines) line = guess ? load_early(far.lines + i) : far.line(i);
+        if (i < r.n_anchors) anchor = guess ? load_early(far.anchors + i) : far.anchor(i);
+        if (i < r.n_refs) ref = guess ? load_early(far.refs + i) : far.ref(i);
         if (i < r.n_lines) near.lines[i] = line;
         if (i < r.n_anchors) near.anchors[i] = anchor;
         if (i < r.n_refs) near.refs[i] = ref;
@@ -132,27 +155,49 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
     }
     if (tid < 32) {
       auto put = [&](int at, int2 span) {
-        if (at < kMaxSpans) keys[at] = pack(span);
+        if (at < (guess ? kRankSpans : kMaxSpans)) keys[at] = pack(span);
       };
       const int resolved = copied ? resolve_refs_warp(r, near, tid, flags, put) : resolve_refs_warp(r, far, tid, flags, put);
       if (tid == 0) s_resolved = resolved;
     }
     __syncthreads();
     S = s_resolved;
+    if (guess && S > kRankSpans) {
+      __syncthreads();                                // every thread has read s_resolved
+      grid_dependency_wait();
+      guess = false;
+      continue;
+    }
   } else {
-    first = span_offsets[b];
-    S = span_offsets[b + 1] - first;
+    first = guess ? load_early(span_offsets + b) : span_offsets[b];
+    S = (guess ? load_early(span_offsets + b + 1) : span_offsets[b + 1]) - first;
+    if (guess && !(first >= 0 && S >= 0 && S <= min(span_cap, kRankSpans) && first <= src.spans_readable - S)) {
+      grid_dependency_wait();
+      guess = false;
+      continue;
+    }
   }
   if (S < 0) S = 0;
   if (S > span_cap) { S = span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
-  int P = (max(S, 1) + 31) & ~31;
+  P = (max(S, 1) + 31) & ~31;
   if (S > kRankSpans)
     for (P = 2 * kRankSpans; P < S;) P <<= 1;
-  if constexpr (!kFromRefs) __syncthreads();            // s_flags
+  if constexpr (!kFromRefs) {
+    if (S <= kRankSpans) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int i = tid + k * kIdxThreads;
+        if (i < S) raw[k] = guess ? load_early(reinterpret_cast<const int2*>(spans) + first + i)
+                                  : reinterpret_cast<const int2*>(spans)[first + i];
+      }
+    }
+    __syncthreads();                                    // s_flags
+  }
 
   auto load_key = [&](int i) -> unsigned long long {
     if (i >= S) return kEmptyKey;
     if (kFromRefs) return keys[i];
+    if (S <= kRankSpans) return pack(raw[i / kIdxThreads]);   // i is tid or tid + kIdxThreads
     return pack(reinterpret_cast<const int2*>(spans)[first + i]);
   };
 
@@ -252,6 +297,38 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   }
   if (flags) atomicOr(&s_flags, flags);
   __syncthreads();
+  if (!guess) break;
+
+  grid_dependency_wait();
+  guess = false;
+  bool changed = false;
+  if constexpr (kFromRefs) {
+    const RefsInMemory far(src.tables, r);
+    changed = !same_tables(r, locate_refs(src.tables, b));
+    const int2 *lines = guess_room, *refs = guess_room + kTable;
+    const int32_t* anchors = reinterpret_cast<const int32_t*>(guess_room + 2 * kTable);
+    for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
+      int2 line = make_int2(0, 0), ref = line;
+      int anchor = 0;
+      if (i < r.n_lines) line = far.line(i);
+      if (i < r.n_anchors) anchor = far.anchor(i);
+      if (i < r.n_refs) ref = far.ref(i);
+      changed |= i < r.n_lines && (line.x != lines[i].x || line.y != lines[i].y);
+      changed |= i < r.n_anchors && anchor != anchors[i];
+      changed |= i < r.n_refs && (ref.x != refs[i].x || ref.y != refs[i].y);
+    }
+  } else {
+    const int2* list = reinterpret_cast<const int2*>(spans) + first;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (tid + k * kIdxThreads >= S) continue;
+      const int2 now = list[tid + k * kIdxThreads];
+      changed |= now.x != raw[k].x || now.y != raw[k].y;
+    }
+    changed |= ctx_lens[b] != length || span_offsets[b] != first || span_offsets[b + 1] - first != S;
+  }
+  if (!__syncthreads_or(changed)) break;
+  }
 
   const int total = offs[P];
   const int c = min(total, capacity);
@@ -286,7 +363,8 @@ static int32_t slice_of(int32_t B, int32_t capacity, int* slices) {
 }
 
 // ssa_spans_to_index with the span lists read from page-locked host memory (host_* are host addresses the
-// device can use), fused with the copy of `bytes` bytes from src (the same kind of memory) to dst (device).
+// device can use), fused with the copy of `bytes` bytes from src (the same kind of memory) to dst (device).  (No guess: two
+// readings across the bus, 43 -> 92 us.)
 int32_t fetch_and_index(const int32_t* host_span_offsets, const int32_t* host_spans, const int32_t* host_ctx_lens,
                         int32_t B, int32_t* index, int32_t index_stride, int32_t* counts, uint32_t* dev_status,
                         void* dst, const void* src, size_t bytes, cudaStream_t stream) {
@@ -307,7 +385,7 @@ int32_t fetch_and_index(const int32_t* host_span_offsets, const int32_t* host_sp
   FetchJob job = {reinterpret_cast<uint4*>(dst), reinterpret_cast<const uint4*>(src), n16, B};
   dim3 grid((unsigned)slices, (unsigned)(B + std::max(copy_rows, 1)));
   const cudaError_t err = launch_pdl(spans_to_index_kernel<false, true>, grid, dim3(kIdxThreads), stream, s,
-                                     index, index_stride, slice, counts, dev_status, job, index_stride, kMaxSpans, Spare<48>{});
+                                     index, index_stride, slice, counts, dev_status, job, index_stride, kMaxSpans, Spare<24>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   note_launches(1);
   return SSA_OK;
@@ -327,8 +405,11 @@ int32_t spans_to_index_capped(const int32_t* span_offsets, const int32_t* spans,
   dim3 grid((unsigned)slices, (unsigned)B);
   SpanSource src = {};
   src.span_offsets = span_offsets; src.spans = spans; src.ctx_lens = ctx_lens;
+  Allocation known = {};
+  src.spans_readable = readable_entries<int2>(spans, &known);
+  src.early_blocks = src.spans_readable > 0 ? kEarlyBlocks * sm_count() : 0;
   const cudaError_t err = launch_pdl(spans_to_index_kernel<false>, grid, dim3(kIdxThreads), stream, src, index,
-                                     index_stride, slice, counts, dev_status, FetchJob{}, capacity, span_cap, Spare<48>{});
+                                     index_stride, slice, counts, dev_status, FetchJob{}, capacity, span_cap, Spare<24>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   note_launches(1);
   return SSA_OK;
@@ -356,9 +437,14 @@ extern "C" int32_t ssa_refs_to_index(const ssa_anchor_tables* tables, int32_t B,
   dim3 grid((unsigned)slices, (unsigned)B);
   ssa::SpanSource src = {};
   src.tables = *tables;
+  ssa::Allocation known = {};
+  src.lines_readable = ssa::readable_entries<int2>(tables->lines, &known);
+  src.anchors_readable = ssa::readable_entries<int32_t>(tables->anchor_line, &known);
+  src.refs_readable = ssa::readable_entries<int2>(tables->refs, &known);
+  src.early_blocks = ssa::kEarlyBlocks * ssa::sm_count();
   const cudaError_t err = ssa::launch_pdl(ssa::spans_to_index_kernel<true>, grid, dim3(ssa::kIdxThreads),
                                           (cudaStream_t)stream, src, index, index_stride, slice, counts,
-                                          dev_status, ssa::FetchJob{}, index_stride, ssa::kMaxSpans, ssa::Spare<48>{});
+                                          dev_status, ssa::FetchJob{}, index_stride, ssa::kMaxSpans, ssa::Spare<24>{});
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SSA_ERR_CUDA;
   ssa::note_launches(1);
   return SSA_OK;

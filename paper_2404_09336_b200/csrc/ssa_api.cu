@@ -28,9 +28,11 @@ int sm_count() {
   return n;
 }
 
-// One driver query, 35 ns.  (Only cudaMalloc's memory, what classic IPC handles are for: pools and address ranges that were
+// One driver query, 35 to 150 ns.  (Only cudaMalloc's memory, what classic IPC handles are for: pools and address ranges that were
 // mapped piece by piece may end sooner than the answer says.)
-size_t readable_bytes(const void* p) {
+size_t readable_bytes(const void* p, Allocation* known) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+  if (at >= known->begin && at < known->end) return known->end - at;
   using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
   static const Query query = [] {
     void* f = nullptr;
@@ -48,9 +50,9 @@ size_t readable_bytes(const void* p) {
   CUpointer_attribute ask[] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
                                CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE};
   void* answer[] = {&start, &size, &whole};
-  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
-  if (!query || query(3, ask, answer, at) != CUDA_SUCCESS || !whole || at < start || at - start >= size) return 0;
-  return size - (at - start);
+  if (!query || query(3, ask, answer, (CUdeviceptr)at) != CUDA_SUCCESS || !whole || at < start || at - start >= size) return 0;
+  *known = {(uintptr_t)start, (uintptr_t)(start + size)};
+  return known->end - at;
 }
 
 static thread_local uint64_t t_launches = 0;

@@ -18,8 +18,14 @@ void note_launches(int n);
 void take_kernel_events(cudaEvent_t* begin, cudaEvent_t* end);
 int sm_count();   // multiprocessors of the current device (cached; no synchronisation)
 // Bytes from p to the end of the allocation it lies in, as far as that is device memory mapped as a whole; else 0.  Reading
-// these is safe whatever offsets said that they are a list.
-size_t readable_bytes(const void* p);
+// these is safe whatever offsets said that they are a list.  `known`: an allocation asked for before, which may hold p too.
+struct Allocation { uintptr_t begin, end; };
+size_t readable_bytes(const void* p, Allocation* known);
+template <typename Entry>
+inline int32_t readable_entries(const void* p, Allocation* known) {
+  const size_t n = readable_bytes(p, known) / sizeof(Entry);
+  return n < 0x7fffffff ? (int32_t)n : 0x7fffffff;
+}
 
 // Programmatic dependent launch.  Every kernel of the library is launched
 // with the programmatic-serialization attribute: its blocks may become

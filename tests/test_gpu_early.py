@@ -98,10 +98,14 @@ def test_lists_and_spans_that_an_attention_launch_in_front_writes(B, H, Hkv, D, 
     pairs = 29                                           # at most 32 are merged by a warp
     status = torch.zeros(1, **i32)
     out = [torch.full((n, B, H, D), 7.0, device=DEV) for _ in range(3)]
-    desc = ssa.make_desc(q, k, v, out[0][0])
+    scratch = torch.empty_like(out[0][0])
+    desc = ssa.make_desc(q, k, v, scratch)
     ws = torch.empty(max(ssa.decode_spans_workspace_bytes(desc, rows, 150), 16), dtype=torch.uint8, device=DEV)
     table, table_counts = torch.full((B, 2 * pairs), 3, **i32), torch.zeros(B, **i32)
-    kept, (kr, vr) = [], (k.bfloat16(), v.bfloat16())
+    pair_offsets = torch.arange(B + 1, **i32) * pairs
+    index2, counts2 = torch.full((B, pairs), 5, **i32), torch.zeros(B, **i32)
+    block_idx, block_mask, counts3 = torch.zeros(B, 24, **i32), torch.zeros(B, 24, 1, **i32), torch.zeros(B, **i32)
+    kept, lists, (kr, vr) = [], [], (k.bfloat16(), v.bfloat16())
     torch.cuda.synchronize()
     for i in range(n):
         ssa.decode_attn_spans(desc, q, k, v, ctx, offsets, spans[i], 1, rows, out[0][i], index_out=index, counts_out=counts,
@@ -112,6 +116,12 @@ def test_lists_and_spans_that_an_attention_launch_in_front_writes(B, H, Hkv, D, 
                               counts_out=table_counts, workspace=ws, dev_status=status)
         ssa.decode_attn_spans(desc, q, k, v, counts, None, table, pairs, pairs, out[2][i], workspace=ws, dev_status=status)
         kept.append((index.clone(), counts.clone(), table.clone()))
+        # and as span lists of the kernels that make lists of them
+        for call, got in ((ssa.spans_to_index, (index2, counts2)), (ssa.spans_to_blockmask, (32, block_idx, block_mask, counts3))):
+            ssa.decode_attn_spans(desc, q, k, v, ctx, offsets, spans[i], 1, 2 * pairs, scratch, index_out=table,
+                                  counts_out=table_counts, workspace=ws, dev_status=status)
+            call(pair_offsets, table.view(-1, 2), counts, *got, status)
+        lists.append([x.clone() for x in (index2, counts2, block_idx, block_mask, counts3)])
     torch.cuda.synchronize()
     for i, (idx, cnt, tab) in enumerate(kept):
         assert torch.equal(cnt, lengths[i])
@@ -124,4 +134,10 @@ def test_lists_and_spans_that_an_attention_launch_in_front_writes(B, H, Hkv, D, 
         for b in range(B):
             rows_b = at[b][live[b]].unique()
             chosen[b, :len(rows_b)], num[b] = rows_b, len(rows_b)
+            index2, counts2, block_idx, block_mask, counts3 = (x[b] for x in lists[i])
+            assert int(counts2) == len(rows_b) and torch.equal(index2[:len(rows_b)], rows_b)
+            blocks = (rows_b // 32).unique()
+            words = [sum(1 << int(t) % 32 for t in rows_b if int(t) // 32 == int(w)) for w in blocks]
+            assert int(counts3) == len(blocks) and torch.equal(block_idx[:len(blocks)], blocks)
+            assert [int(w) & 0xFFFFFFFF for w in block_mask[:len(blocks), 0]] == words
         assert float((out[2][i].double() - rows_of(q, kr, vr, chosen, num)).abs().max()) < 1e-4
