@@ -332,15 +332,14 @@ decode_partial_kernel(const DecodeParams p) {
   int span_first = 0, span_n = 0;
   int2 my_span = make_int2(0, 0);
   if constexpr (kMode == kSpans) {
-    if (guess.there && lane < guess.S) my_span = __ldg(p.spans + guess.first + lane);
+    if (guess.there && lane < guess.S) my_span = load_now(p.spans + guess.first + lane);
     if (p.span_offsets) {
-      span_first = __ldg(p.span_offsets + b);
-      span_n = __ldg(p.span_offsets + b + 1) - span_first;
+      span_first = load_now(p.span_offsets + b);
+      span_n = load_now(p.span_offsets + b + 1) - span_first;
     } else {
       span_first = b * p.span_cap;
       span_n = p.span_cap;
     }
-    if (warp_merge && !guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
   }
   // blocked lists: every warp takes all words of the block's entries, one per lane (those beyond the list are ignored below)
   int mask_block = -1;
@@ -357,13 +356,14 @@ decode_partial_kernel(const DecodeParams p) {
   int n, c;
   request_sizes(p, b, n, c, flags);
   if constexpr (kMode == kSpans) {
+    if (warp_merge && !guess.there && lane < min(span_n, p.span_cap)) my_span = load_now(p.spans + span_first + lane);
     // the request's spans -> disjoint ascending runs in shared memory (every block of the request repeats this)
     int total;
     if (warp_merge && still_the_spans(guess, span_first, span_n, n, my_span)) {
       total = guess.total;
       flags |= guess.flags;
     } else if (warp_merge) {                          // up to 32 spans: every warp merges them for itself, no barrier
-      if (guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
+      if (guess.there && lane < min(span_n, p.span_cap)) my_span = load_now(p.spans + span_first + lane);
       int S = max(span_n, 0);
       if (S > p.span_cap) { S = p.span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
       total = merge_spans_warp(s_wruns[warp], my_span, S, warp_runs, n, flags);

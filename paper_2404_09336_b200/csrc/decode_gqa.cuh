@@ -457,21 +457,27 @@ decode_partial_gqa_kernel(const DecodeParams p) {
     int span_first = 0, span_n = 0;
     int2 my_span = make_int2(0, 0);
     if constexpr (kMode == kSpans) {
-      if (guess.there && lane < guess.S) my_span = __ldg(p.spans + guess.first + lane);
-      span_first = p.span_offsets ? __ldg(p.span_offsets + b) : b * p.span_cap;
-      span_n = p.span_offsets ? __ldg(p.span_offsets + b + 1) - span_first : p.span_cap;
-      if (warp_merge && !guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
+      if (guess.there && lane < guess.S) my_span = load_now(p.spans + guess.first + lane);
+      span_first = p.span_offsets ? load_now(p.span_offsets + b) : b * p.span_cap;
+      span_n = p.span_offsets ? load_now(p.span_offsets + b + 1) - span_first : p.span_cap;
     }
+    // (8-bit rows: in front of the sizes.  32 requests, 32 heads over 8: 15.05 us, 15.33 behind them, 16-bit rows, 17 requests, 12.92
+    // and 12.32)
+    auto ask_span = [&]() {
+      if (warp_merge && !guess.there && lane < min(span_n, p.span_cap)) my_span = load_now(p.spans + span_first + lane);
+    };
+    if (kMode == kSpans && kFp8) ask_span();
     int n, c;
     if constexpr (kEven) n = c = s_line.rows[b];
     else request_sizes(p, b, n, c, flags);
     if constexpr (kMode == kSpans) {
+      if (!kFp8) ask_span();
       int total;
       if (warp_merge && still_the_spans(guess, span_first, span_n, n, my_span)) {
         total = guess.total;
         flags |= guess.flags;
       } else if (warp_merge) {
-        if (guess.there && lane < min(span_n, p.span_cap)) my_span = __ldg(p.spans + span_first + lane);
+        if (guess.there && lane < min(span_n, p.span_cap)) my_span = load_now(p.spans + span_first + lane);
         int S = max(span_n, 0);
         if (S > p.span_cap) { S = p.span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
         total = merge_spans_warp(s_wruns[warp], my_span, S, runs, n, flags);

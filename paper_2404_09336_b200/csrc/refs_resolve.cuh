@@ -14,7 +14,7 @@ struct RefTables {
 // kEarly: as they stand before grid_dependency_wait().
 template <bool kEarly = false>
 __device__ __forceinline__ RefTables locate_refs(const ssa_anchor_tables& t, int b) {
-  auto load = [](const int32_t* p) { return kEarly ? load_early(p) : *p; };
+  auto load = [](const int32_t* p) { return kEarly ? load_early(p) : load_now(p); };
   RefTables r;
   r.l0 = load(t.line_offsets + b);
   r.a0 = load(t.anchor_offsets + b);

@@ -54,9 +54,8 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
   int n, S;
   uint32_t flags;
   while (true) {
-    const int length = guess ? load_early(ctx_lens + b) : ctx_lens[b];
-    const int first = guess ? load_early(span_offsets + b) : span_offsets[b];
-    const int listed_spans = (guess ? load_early(span_offsets + b + 1) : span_offsets[b + 1]) - first;
+    auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
+    const int length = load(ctx_lens + b), first = load(span_offsets + b), listed_spans = load(span_offsets + b + 1) - first;
     if (guess && !(first >= 0 && listed_spans >= 0 && listed_spans <= kBmThreads && first <= spans_readable - listed_spans)) {
       grid_dependency_wait();                           // (block-uniform) no guess
       guess = false;
@@ -70,7 +69,7 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
     const int2* list = reinterpret_cast<const int2*>(spans) + first;
     int2 own = make_int2(0, 0);                         // span tid
     for (int i = tid; i < S; i += kBmThreads) {
-      const int2 se = guess ? load_early(list + i) : list[i];
+      const int2 se = load(list + i);
       if (i == tid) own = se;
       if (se.x < 0 || se.x > se.y) flags |= SSA_DEV_BAD_SPAN;
       if (se.y > n) flags |= SSA_DEV_CLIPPED;
@@ -80,9 +79,10 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
     if (!guess) break;
     grid_dependency_wait();
     guess = false;
-    bool changed = ctx_lens[b] != length || span_offsets[b] != first || span_offsets[b + 1] - first != listed_spans;
+    bool changed = load_now(ctx_lens + b) != length || load_now(span_offsets + b) != first ||
+                   load_now(span_offsets + b + 1) - first != listed_spans;
     if (tid < S) {
-      const int2 now = list[tid];
+      const int2 now = load_now(list + tid);
       changed |= now.x != own.x || now.y != own.y;
     }
     if (!__syncthreads_or(changed)) break;

@@ -102,7 +102,8 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   static_assert(2 * kRankSpans * 8 + kTable * 20 <= kMaxSpans * 8, "a guess's copies lie behind its keys and starts");
   int P;
   while (true) {
-  const int length = guess ? load_early(ctx_lens + b) : ctx_lens[b];
+  auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
+  const int length = load(ctx_lens + b);
   const int n = max(length, 0);
   uint32_t flags = 0;
   if (tid == 0) s_flags = 0;
@@ -128,7 +129,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
       __device__ __forceinline__ int2 ref(int i) const { return refs[i]; }
       __device__ __forceinline__ int anchor(int i) const { return anchors[i]; }
     };
-    r = guess ? locate_refs<true>(src.tables, b) : locate_refs(src.tables, b);
+    r = guess ? locate_refs<true>(src.tables, b) : locate_refs<false>(src.tables, b);
     const RefsInMemory far(src.tables, r);
     // (a guess needs its copies for the comparison: behind the keys of a list of up to kRankSpans, where nothing else comes)
     int2* const room = guess ? guess_room : reinterpret_cast<int2*>(new_start);
@@ -144,9 +145,9 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
       for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
         int2 line = make_int2(0, 0), ref = line;        // all three requested before any is stored
         int anchor = 0;
-        if (i < r.n_lines) line = guess ? load_early(far.lines + i) : far.line(i);
-        if (i < r.n_anchors) anchor = guess ? load_early(far.anchors + i) : far.anchor(i);
-        if (i < r.n_refs) ref = guess ? load_early(far.refs + i) : far.ref(i);
+        if (i < r.n_lines) line = load(far.lines + i);
+        if (i < r.n_anchors) anchor = load(far.anchors + i);
+        if (i < r.n_refs) ref = load(far.refs + i);
         if (i < r.n_lines) near.lines[i] = line;
         if (i < r.n_anchors) near.anchors[i] = anchor;
         if (i < r.n_refs) near.refs[i] = ref;
@@ -169,8 +170,8 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
       continue;
     }
   } else {
-    first = guess ? load_early(span_offsets + b) : span_offsets[b];
-    S = (guess ? load_early(span_offsets + b + 1) : span_offsets[b + 1]) - first;
+    first = load(span_offsets + b);
+    S = load(span_offsets + b + 1) - first;
     if (guess && !(first >= 0 && S >= 0 && S <= min(span_cap, kRankSpans) && first <= src.spans_readable - S)) {
       grid_dependency_wait();
       guess = false;
@@ -187,8 +188,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const int i = tid + k * kIdxThreads;
-        if (i < S) raw[k] = guess ? load_early(reinterpret_cast<const int2*>(spans) + first + i)
-                                  : reinterpret_cast<const int2*>(spans)[first + i];
+        if (i < S) raw[k] = load(reinterpret_cast<const int2*>(spans) + first + i);
       }
     }
     __syncthreads();                                    // s_flags
@@ -304,15 +304,15 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   bool changed = false;
   if constexpr (kFromRefs) {
     const RefsInMemory far(src.tables, r);
-    changed = !same_tables(r, locate_refs(src.tables, b));
+    changed = !same_tables(r, locate_refs<false>(src.tables, b));
     const int2 *lines = guess_room, *refs = guess_room + kTable;
     const int32_t* anchors = reinterpret_cast<const int32_t*>(guess_room + 2 * kTable);
     for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
       int2 line = make_int2(0, 0), ref = line;
       int anchor = 0;
-      if (i < r.n_lines) line = far.line(i);
-      if (i < r.n_anchors) anchor = far.anchor(i);
-      if (i < r.n_refs) ref = far.ref(i);
+      if (i < r.n_lines) line = load_now(far.lines + i);
+      if (i < r.n_anchors) anchor = load_now(far.anchors + i);
+      if (i < r.n_refs) ref = load_now(far.refs + i);
       changed |= i < r.n_lines && (line.x != lines[i].x || line.y != lines[i].y);
       changed |= i < r.n_anchors && anchor != anchors[i];
       changed |= i < r.n_refs && (ref.x != refs[i].x || ref.y != refs[i].y);
@@ -322,10 +322,11 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       if (tid + k * kIdxThreads >= S) continue;
-      const int2 now = list[tid + k * kIdxThreads];
+      const int2 now = load_now(list + tid + k * kIdxThreads);
       changed |= now.x != raw[k].x || now.y != raw[k].y;
     }
-    changed |= ctx_lens[b] != length || span_offsets[b] != first || span_offsets[b + 1] - first != S;
+    changed |= load_now(ctx_lens + b) != length || load_now(span_offsets + b) != first ||
+               load_now(span_offsets + b + 1) - first != S;
   }
   if (!__syncthreads_or(changed)) break;
   }

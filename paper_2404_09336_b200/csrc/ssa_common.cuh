@@ -48,6 +48,18 @@ __device__ __forceinline__ int2 load_early(const int2* p) {
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return make_int2((int32_t)(uint32_t)v, (int32_t)(v >> 32));
 }
+// The same after the wait, for what a guess is compared with: an ordinary load, but volatile, so that it stays behind the wait
+// whatever the compiler makes of read-only memory.
+__device__ __forceinline__ int32_t load_now(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int2 load_now(const int2* p) {
+  int2 v;
+  asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
 // The 32 bytes around p into L2.
 __device__ __forceinline__ void prefetch_sector(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
