@@ -127,6 +127,25 @@ __device__ __forceinline__ void store_row_value(const DecodeParams& p, int b, in
   if (d == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L == 0.f ? neg_inf() : (M + log2f(L)) * kLn2;
 }
 
+// The same for elements d..d + 3, d a multiple of four (rows start on 16 bytes: check_desc).
+template <typename T>
+__device__ __forceinline__ void store_row_values(const DecodeParams& p, int b, int h, int d, float M, float L, const float (&A)[4]) {
+  const int64_t o = (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + d;
+  float r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) r[i] = L == 0.f ? 0.f : A[i] / L;
+  if (p.out_f32) {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + o) = make_float4(r[0], r[1], r[2], r[3]);
+  } else {
+    const T x[4] = {from_float<T>(r[0]), from_float<T>(r[1]), from_float<T>(r[2]), from_float<T>(r[3])};
+    uint2 w;
+    w.x = (uint32_t)*reinterpret_cast<const uint16_t*>(&x[0]) | (uint32_t)*reinterpret_cast<const uint16_t*>(&x[1]) << 16;
+    w.y = (uint32_t)*reinterpret_cast<const uint16_t*>(&x[2]) | (uint32_t)*reinterpret_cast<const uint16_t*>(&x[3]) << 16;
+    *reinterpret_cast<uint2*>(reinterpret_cast<T*>(p.out) + o) = w;
+  }
+  if (d == 0 && p.lse) p.lse[(int64_t)b * p.H + h] = L == 0.f ? neg_inf() : (M + log2f(L)) * kLn2;
+}
+
 // A lane's piece of a cache row: 16 values as eight pairs.  16-bit storage: 32 bytes, a pair per word; 8-bit
 // storage: 16 bytes in w[0..3], two pairs per word.
 struct Piece { uint32_t w[8]; };
