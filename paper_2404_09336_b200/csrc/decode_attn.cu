@@ -762,6 +762,15 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
            5 * units >= (max_selected * d->D <= 768 * 128 ? sms : 2 * sms) &&
            (d->kv_dtype != SSA_FP8_E4M3 || (d->H == d->H_kv && (units <= sms || 5 * units >= 7 * sms))))
     chunk = kMaxWideChunk;
+  // Longer chunks where there are blocks enough without (us, 256 / 512 entries; 32 heads a request).  Rows of 128 16-bit values: 64
+  // requests of 4000 rows 612 / 598, 32 of them 307 / 303, of 2000 154.9 / 154.5, 64 of up to 1024, most of 141, 45.3 / 44.5; but 32 of
+  // 1500 121 / 123, 50 of 900 113 / 114, 64 of 600 98.4 / 99.5.  Rows of half the bytes, or less, are half a chunk: 8-bit, 32 of 900
+  // rows 49.7 / 47.4, 64 94 / 87, 16-bit of 64 52 / 51 (40) and 81 / 78.  (Fewer would make one-kernel steps of some that gain nothing by
+  // it: 24 of 600, 8-bit, 31.6 / 33.3.)
+  else if (!share && (d->D == 64 || d->kv_dtype == SSA_FP8_E4M3
+                          ? max_selected > kMaxChunk && units > 6 * sms
+                          : max_selected > 768 && units * ((max_selected + kMaxChunk - 1) / kMaxChunk) >= 27 * sms))
+    chunk = kMaxChunk;
   else while (chunk > 64 && units * ((max_selected + chunk - 1) / chunk) < want) chunk >>= 1;
   pl->share = share;
   pl->wide = false;
