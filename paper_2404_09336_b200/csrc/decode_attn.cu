@@ -756,7 +756,7 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   // measured with chunks.
   const long long sms = sm_count();
   const long long want = sms * 2;
-  int chunk = 256;
+  int chunk = 256, sized_for = 0;
   if (max_selected <= kMaxChunk && (units >= sms || max_selected <= 256)) chunk = kMaxChunk;
   else if (!share && max_selected <= staged_entries(block_warps(d, units, max_selected)) && units <= want &&
            5 * units >= (max_selected * d->D <= 768 * 128 ? sms : 2 * sms) &&
@@ -769,8 +769,10 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   // it: 24 of 600, 8-bit, 31.6 / 33.3.)
   else if (!share && (d->D == 64 || d->kv_dtype == SSA_FP8_E4M3
                           ? max_selected > kMaxChunk && units > 6 * sms
-                          : max_selected > 768 && units * ((max_selected + kMaxChunk - 1) / kMaxChunk) >= 27 * sms))
+                          : max_selected > 768 && units * ((max_selected + kMaxChunk - 1) / kMaxChunk) >= 27 * sms)) {
+    sized_for = chunk;                                   // (the workspace asked for stays that of chunks of 256)
     chunk = kMaxChunk;
+  }
   else while (chunk > 64 && units * ((max_selected + chunk - 1) / chunk) < want) chunk >>= 1;
   pl->share = share;
   pl->wide = false;
@@ -799,6 +801,8 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
   pl->chunk = chunk;
   pl->n_chunks = n_chunks;
   pl->total_bytes = triples_bytes(d, (size_t)out_units * n_chunks, &pl->acc_bytes);
+  size_t acc = 0;
+  if (sized_for > 0) pl->total_bytes = triples_bytes(d, (size_t)out_units * ((max_selected + sized_for - 1) / sized_for), &acc);
   return true;
 }
 

@@ -30,8 +30,9 @@ inline int32_t readable_entries(const void* p, Allocation* known) {
 // Programmatic dependent launch.  Every kernel of the library is launched
 // with the programmatic-serialization attribute: its blocks may become
 // resident while the preceding kernel of the stream is still draining, and
-// they call grid_dependency_wait() before touching any global memory, which
-// returns once that kernel has completed and its writes are visible.
+// they call grid_dependency_wait(), which returns once that kernel has
+// completed and its writes are visible, before they write anything or rely
+// on anything they read (see load_early).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
