@@ -18,6 +18,10 @@
  *    the default stream).  No call synchronises or reads device memory back,
  *    so everything data-dependent (selected counts, context lengths) stays on
  *    the device and host-side sizes are upper bounds.
+ *  - Kernels may read a call's inputs before the kernel in front of them in
+ *    the stream has ended, for guesses only: which cache rows to prefetch,
+ *    lists made ahead and compared with the inputs afterwards.  Results are
+ *    those of the inputs as that kernel leaves them.
  *  - Return value: an ssa_status.  Non-zero means nothing was launched.
  *  - Data-dependent problems never fault: they set bits in the caller's
  *    device status word (`dev_status`, may be NULL) and take the defined
