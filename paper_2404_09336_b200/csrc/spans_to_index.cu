@@ -102,233 +102,233 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   static_assert(2 * kRankSpans * 8 + kTable * 20 <= kMaxSpans * 8, "a guess's copies lie behind its keys and starts");
   int P;
   while (true) {
-  auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
-  const int length = load(ctx_lens + b);
-  const int n = max(length, 0);
-  uint32_t flags = 0;
-  if (tid == 0) s_flags = 0;
+    auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
+    const int length = load(ctx_lens + b);
+    const int n = max(length, 0);
+    uint32_t flags = 0;
+    if (tid == 0) s_flags = 0;
 
-  // clamp a span to the context and pack it; empty spans get the sentinel
-  auto pack = [&](int2 se) -> unsigned long long {
-    if (se.x < 0 || se.x > se.y) flags |= SSA_DEV_BAD_SPAN;
-    if (se.y > n) flags |= SSA_DEV_CLIPPED;
-    const int s = max(se.x, 0), e = min(se.y, n);
-    return e > s ? ((unsigned long long)(uint32_t)s << 32) | (uint32_t)e : kEmptyKey;
-  };
-
-  int first = 0, S;
-  int2 raw[2] = {make_int2(0, 0), make_int2(0, 0)};   // spans tid and tid + kIdxThreads of a list of up to kRankSpans
-  RefTables r = {};
-  if constexpr (kFromRefs) {
-    // 1 (references): warp 0 resolves them and leaves the packed spans, unsorted, in keys[0, S)
-    static_assert(4 * kTable <= kMaxSpans, "the copies lie in arrays that step 3 fills");
-    struct Copied {
-      int2 *lines, *refs;
-      int32_t* anchors;
-      __device__ __forceinline__ int2 line(int i) const { return lines[i]; }
-      __device__ __forceinline__ int2 ref(int i) const { return refs[i]; }
-      __device__ __forceinline__ int anchor(int i) const { return anchors[i]; }
+    // clamp a span to the context and pack it; empty spans get the sentinel
+    auto pack = [&](int2 se) -> unsigned long long {
+      if (se.x < 0 || se.x > se.y) flags |= SSA_DEV_BAD_SPAN;
+      if (se.y > n) flags |= SSA_DEV_CLIPPED;
+      const int s = max(se.x, 0), e = min(se.y, n);
+      return e > s ? ((unsigned long long)(uint32_t)s << 32) | (uint32_t)e : kEmptyKey;
     };
-    r = guess ? locate_refs<true>(src.tables, b) : locate_refs<false>(src.tables, b);
-    const RefsInMemory far(src.tables, r);
-    // (a guess needs its copies for the comparison: behind the keys of a list of up to kRankSpans, where nothing else comes)
-    int2* const room = guess ? guess_room : reinterpret_cast<int2*>(new_start);
-    const Copied near = {room, room + kTable, guess ? reinterpret_cast<int32_t*>(room + 2 * kTable) : offs};
-    const bool copied = r.n_lines <= kTable && r.n_anchors <= kTable && r.n_refs <= kTable;
-    if (guess && !(copied && r.l0 >= 0 && r.a0 >= 0 && r.r0 >= 0 && r.l0 <= src.lines_readable - r.n_lines &&
-                   r.a0 <= src.anchors_readable - r.n_anchors && r.r0 <= src.refs_readable - r.n_refs)) {
-      grid_dependency_wait();                         // (block-uniform) no guess
-      guess = false;
-      continue;
-    }
-    if (copied) {
-      for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
-        int2 line = make_int2(0, 0), ref = line;        // all three requested before any is stored
-        int anchor = 0;
-        if (i < r.n_lines) line = load(far.lines + i);
-        if (i < r.n_anchors) anchor = load(far.anchors + i);
-        if (i < r.n_refs) ref = load(far.refs + i);
-        if (i < r.n_lines) near.lines[i] = line;
-        if (i < r.n_anchors) near.anchors[i] = anchor;
-        if (i < r.n_refs) near.refs[i] = ref;
-      }
-      __syncthreads();
-    }
-    if (tid < 32) {
-      auto put = [&](int at, int2 span) {
-        if (at < (guess ? kRankSpans : kMaxSpans)) keys[at] = pack(span);
+
+    int first = 0, S;
+    int2 raw[2] = {make_int2(0, 0), make_int2(0, 0)};   // spans tid and tid + kIdxThreads of a list of up to kRankSpans
+    RefTables r = {};
+    if constexpr (kFromRefs) {
+      // 1 (references): warp 0 resolves them and leaves the packed spans, unsorted, in keys[0, S)
+      static_assert(4 * kTable <= kMaxSpans, "the copies lie in arrays that step 3 fills");
+      struct Copied {
+        int2 *lines, *refs;
+        int32_t* anchors;
+        __device__ __forceinline__ int2 line(int i) const { return lines[i]; }
+        __device__ __forceinline__ int2 ref(int i) const { return refs[i]; }
+        __device__ __forceinline__ int anchor(int i) const { return anchors[i]; }
       };
-      const int resolved = copied ? resolve_refs_warp(r, near, tid, flags, put) : resolve_refs_warp(r, far, tid, flags, put);
-      if (tid == 0) s_resolved = resolved;
-    }
-    __syncthreads();
-    S = s_resolved;
-    if (guess && S > kRankSpans) {
-      __syncthreads();                                // every thread has read s_resolved
-      grid_dependency_wait();
-      guess = false;
-      continue;
-    }
-  } else {
-    first = load(span_offsets + b);
-    S = load(span_offsets + b + 1) - first;
-    if (guess && !(first >= 0 && S >= 0 && S <= min(span_cap, kRankSpans) && first <= src.spans_readable - S)) {
-      grid_dependency_wait();
-      guess = false;
-      continue;
-    }
-  }
-  if (S < 0) S = 0;
-  if (S > span_cap) { S = span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
-  P = (max(S, 1) + 31) & ~31;
-  if (S > kRankSpans)
-    for (P = 2 * kRankSpans; P < S;) P <<= 1;
-  if constexpr (!kFromRefs) {
-    if (S <= kRankSpans) {
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int i = tid + k * kIdxThreads;
-        if (i < S) raw[k] = load(reinterpret_cast<const int2*>(spans) + first + i);
+      r = guess ? locate_refs<true>(src.tables, b) : locate_refs<false>(src.tables, b);
+      const RefsInMemory far(src.tables, r);
+      // (a guess needs its copies for the comparison: behind the keys of a list of up to kRankSpans, where nothing else comes)
+      int2* const room = guess ? guess_room : reinterpret_cast<int2*>(new_start);
+      const Copied near = {room, room + kTable, guess ? reinterpret_cast<int32_t*>(room + 2 * kTable) : offs};
+      const bool copied = r.n_lines <= kTable && r.n_anchors <= kTable && r.n_refs <= kTable;
+      if (guess && !(copied && r.l0 >= 0 && r.a0 >= 0 && r.r0 >= 0 && r.l0 <= src.lines_readable - r.n_lines &&
+                     r.a0 <= src.anchors_readable - r.n_anchors && r.r0 <= src.refs_readable - r.n_refs)) {
+        grid_dependency_wait();                         // (block-uniform) no guess
+        guess = false;
+        continue;
       }
-    }
-    __syncthreads();                                    // s_flags
-  }
-
-  auto load_key = [&](int i) -> unsigned long long {
-    if (i >= S) return kEmptyKey;
-    if (kFromRefs) return keys[i];
-    if (S <= kRankSpans) return pack(raw[i / kIdxThreads]);   // i is tid or tid + kIdxThreads
-    return pack(reinterpret_cast<const int2*>(spans)[first + i]);
-  };
-
-  if (P == 32) {
-    // 1+2 (up to 32 spans, the usual case): one warp ranks its starts with shuffles, no block barrier needed.  (The ends do
-    // not order: the walk of step 3 trims by the largest end so far.)
-    if (tid < 32) {
-      const unsigned long long key = load_key(tid);
-      if (kFromRefs) __syncwarp();                  // every lane has read its key before any is overwritten
-      const uint32_t start = (uint32_t)(key >> 32);
-      int rank = 0;
-      for (int j = 0; j < S; ++j) {
-        const uint32_t sj = __shfl_sync(0xffffffffu, start, j);
-        rank += (sj < start || (sj == start && j < tid)) ? 1 : 0;
-      }
-      keys[tid < S ? rank : tid] = key;
-      __syncwarp();
-    }
-  } else if (P <= kRankSpans) {
-    uint32_t* starts = reinterpret_cast<uint32_t*>(keys + kRankSpans);   // the unsorted starts, read four at a time
-    unsigned long long key[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int i = tid + k * kIdxThreads;
-      key[k] = i < P ? load_key(i) : kEmptyKey;
-      if (i < P) starts[i] = (uint32_t)(key[k] >> 32);
-    }
-    __syncthreads();                                // also: every key of the references has been read
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int i = tid + k * kIdxThreads;
-      if (i < P) {
-        const uint32_t start = (uint32_t)(key[k] >> 32);
-        int rank = 0;
-        for (int j = 0; j < P; j += 4) {
-          const uint4 s4 = *reinterpret_cast<const uint4*>(starts + j);
-          rank += (s4.x < start || (s4.x == start && j < i)) ? 1 : 0;
-          rank += (s4.y < start || (s4.y == start && j + 1 < i)) ? 1 : 0;
-          rank += (s4.z < start || (s4.z == start && j + 2 < i)) ? 1 : 0;
-          rank += (s4.w < start || (s4.w == start && j + 3 < i)) ? 1 : 0;
-        }
-        keys[rank] = key[k];
-      }
-    }
-    __syncthreads();
-  } else {
-    // 1. load, clamp, pack (references: the keys are in place, only the padding is missing)
-    for (int i = tid; i < P; i += kIdxThreads)
-      if (!kFromRefs || i >= S) keys[i] = load_key(i);
-    __syncthreads();
-    // 2. bitonic sort, ascending by (start, end); empty keys sink to the end
-    for (int k = 2; k <= P; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int i = tid; i < P; i += kIdxThreads) {
-          const int ixj = i ^ j;
-          if (ixj > i) {
-            const unsigned long long a = keys[i], c = keys[ixj];
-            const bool up = (i & k) == 0;
-            if ((a > c) == up) { keys[i] = c; keys[ixj] = a; }
-          }
+      if (copied) {
+        for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
+          int2 line = make_int2(0, 0), ref = line;        // all three requested before any is stored
+          int anchor = 0;
+          if (i < r.n_lines) line = load(far.lines + i);
+          if (i < r.n_anchors) anchor = load(far.anchors + i);
+          if (i < r.n_refs) ref = load(far.refs + i);
+          if (i < r.n_lines) near.lines[i] = line;
+          if (i < r.n_anchors) near.anchors[i] = anchor;
+          if (i < r.n_refs) near.refs[i] = ref;
         }
         __syncthreads();
       }
-    }
-  }
-
-  // 3. trim against the running maximum end and prefix-sum the lengths
-  if (tid < 32) {
-    int run_max = 0, run_sum = 0;
-    for (int base = 0; base < P; base += 32) {
-      const unsigned long long key = keys[base + tid];
-      const bool live = key != kEmptyKey;
-      const int s = live ? (int)(key >> 32) : 0;
-      const int e = live ? (int)(uint32_t)key : 0;
-      int mx = e;                                   // inclusive max-scan of ends
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, mx, d);
-        if (tid >= d) mx = max(mx, o);
+      if (tid < 32) {
+        auto put = [&](int at, int2 span) {
+          if (at < (guess ? kRankSpans : kMaxSpans)) keys[at] = pack(span);
+        };
+        const int resolved = copied ? resolve_refs_warp(r, near, tid, flags, put) : resolve_refs_warp(r, far, tid, flags, put);
+        if (tid == 0) s_resolved = resolved;
       }
-      int prev = __shfl_up_sync(0xffffffffu, mx, 1);
-      prev = (tid == 0) ? run_max : max(prev, run_max);
-      const int ns = max(s, prev);
-      const int len = live ? max(e - ns, 0) : 0;
-      int sum = len;                                // inclusive sum-scan of lengths
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, sum, d);
-        if (tid >= d) sum += o;
+      __syncthreads();
+      S = s_resolved;
+      if (guess && S > kRankSpans) {
+        __syncthreads();                                // every thread has read s_resolved
+        grid_dependency_wait();
+        guess = false;
+        continue;
       }
-      new_start[base + tid] = ns;
-      offs[base + tid] = run_sum + sum - len;
-      run_max = max(run_max, __shfl_sync(0xffffffffu, mx, 31));
-      run_sum += __shfl_sync(0xffffffffu, sum, 31);
+    } else {
+      first = load(span_offsets + b);
+      S = load(span_offsets + b + 1) - first;
+      if (guess && !(first >= 0 && S >= 0 && S <= min(span_cap, kRankSpans) && first <= src.spans_readable - S)) {
+        grid_dependency_wait();
+        guess = false;
+        continue;
+      }
     }
-    if (tid == 0) offs[P] = run_sum;
-  }
-  if (flags) atomicOr(&s_flags, flags);
-  __syncthreads();
-  if (!guess) break;
-
-  grid_dependency_wait();
-  guess = false;
-  bool changed = false;
-  if constexpr (kFromRefs) {
-    const RefsInMemory far(src.tables, r);
-    changed = !same_tables(r, locate_refs<false>(src.tables, b));
-    const int2 *lines = guess_room, *refs = guess_room + kTable;
-    const int32_t* anchors = reinterpret_cast<const int32_t*>(guess_room + 2 * kTable);
-    for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
-      int2 line = make_int2(0, 0), ref = line;
-      int anchor = 0;
-      if (i < r.n_lines) line = load_now(far.lines + i);
-      if (i < r.n_anchors) anchor = load_now(far.anchors + i);
-      if (i < r.n_refs) ref = load_now(far.refs + i);
-      changed |= i < r.n_lines && (line.x != lines[i].x || line.y != lines[i].y);
-      changed |= i < r.n_anchors && anchor != anchors[i];
-      changed |= i < r.n_refs && (ref.x != refs[i].x || ref.y != refs[i].y);
-    }
-  } else {
-    const int2* list = reinterpret_cast<const int2*>(spans) + first;
+    if (S < 0) S = 0;
+    if (S > span_cap) { S = span_cap; flags |= SSA_DEV_TOO_MANY_SPANS; }
+    P = (max(S, 1) + 31) & ~31;
+    if (S > kRankSpans)
+      for (P = 2 * kRankSpans; P < S;) P <<= 1;
+    if constexpr (!kFromRefs) {
+      if (S <= kRankSpans) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      if (tid + k * kIdxThreads >= S) continue;
-      const int2 now = load_now(list + tid + k * kIdxThreads);
-      changed |= now.x != raw[k].x || now.y != raw[k].y;
+        for (int k = 0; k < 2; ++k) {
+          const int i = tid + k * kIdxThreads;
+          if (i < S) raw[k] = load(reinterpret_cast<const int2*>(spans) + first + i);
+        }
+      }
+      __syncthreads();                                    // s_flags
     }
-    changed |= load_now(ctx_lens + b) != length || load_now(span_offsets + b) != first ||
-               load_now(span_offsets + b + 1) - first != S;
-  }
-  if (!__syncthreads_or(changed)) break;
+
+    auto load_key = [&](int i) -> unsigned long long {
+      if (i >= S) return kEmptyKey;
+      if (kFromRefs) return keys[i];
+      if (S <= kRankSpans) return pack(raw[i / kIdxThreads]);   // i is tid or tid + kIdxThreads
+      return pack(reinterpret_cast<const int2*>(spans)[first + i]);
+    };
+
+    if (P == 32) {
+      // 1+2 (up to 32 spans, the usual case): one warp ranks its starts with shuffles, no block barrier needed.  (The ends do
+      // not order: the walk of step 3 trims by the largest end so far.)
+      if (tid < 32) {
+        const unsigned long long key = load_key(tid);
+        if (kFromRefs) __syncwarp();                  // every lane has read its key before any is overwritten
+        const uint32_t start = (uint32_t)(key >> 32);
+        int rank = 0;
+        for (int j = 0; j < S; ++j) {
+          const uint32_t sj = __shfl_sync(0xffffffffu, start, j);
+          rank += (sj < start || (sj == start && j < tid)) ? 1 : 0;
+        }
+        keys[tid < S ? rank : tid] = key;
+        __syncwarp();
+      }
+    } else if (P <= kRankSpans) {
+      uint32_t* starts = reinterpret_cast<uint32_t*>(keys + kRankSpans);   // the unsorted starts, read four at a time
+      unsigned long long key[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int i = tid + k * kIdxThreads;
+        key[k] = i < P ? load_key(i) : kEmptyKey;
+        if (i < P) starts[i] = (uint32_t)(key[k] >> 32);
+      }
+      __syncthreads();                                // also: every key of the references has been read
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int i = tid + k * kIdxThreads;
+        if (i < P) {
+          const uint32_t start = (uint32_t)(key[k] >> 32);
+          int rank = 0;
+          for (int j = 0; j < P; j += 4) {
+            const uint4 s4 = *reinterpret_cast<const uint4*>(starts + j);
+            rank += (s4.x < start || (s4.x == start && j < i)) ? 1 : 0;
+            rank += (s4.y < start || (s4.y == start && j + 1 < i)) ? 1 : 0;
+            rank += (s4.z < start || (s4.z == start && j + 2 < i)) ? 1 : 0;
+            rank += (s4.w < start || (s4.w == start && j + 3 < i)) ? 1 : 0;
+          }
+          keys[rank] = key[k];
+        }
+      }
+      __syncthreads();
+    } else {
+      // 1. load, clamp, pack (references: the keys are in place, only the padding is missing)
+      for (int i = tid; i < P; i += kIdxThreads)
+        if (!kFromRefs || i >= S) keys[i] = load_key(i);
+      __syncthreads();
+      // 2. bitonic sort, ascending by (start, end); empty keys sink to the end
+      for (int k = 2; k <= P; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+          for (int i = tid; i < P; i += kIdxThreads) {
+            const int ixj = i ^ j;
+            if (ixj > i) {
+              const unsigned long long a = keys[i], c = keys[ixj];
+              const bool up = (i & k) == 0;
+              if ((a > c) == up) { keys[i] = c; keys[ixj] = a; }
+            }
+          }
+          __syncthreads();
+        }
+      }
+    }
+
+    // 3. trim against the running maximum end and prefix-sum the lengths
+    if (tid < 32) {
+      int run_max = 0, run_sum = 0;
+      for (int base = 0; base < P; base += 32) {
+        const unsigned long long key = keys[base + tid];
+        const bool live = key != kEmptyKey;
+        const int s = live ? (int)(key >> 32) : 0;
+        const int e = live ? (int)(uint32_t)key : 0;
+        int mx = e;                                   // inclusive max-scan of ends
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int o = __shfl_up_sync(0xffffffffu, mx, d);
+          if (tid >= d) mx = max(mx, o);
+        }
+        int prev = __shfl_up_sync(0xffffffffu, mx, 1);
+        prev = (tid == 0) ? run_max : max(prev, run_max);
+        const int ns = max(s, prev);
+        const int len = live ? max(e - ns, 0) : 0;
+        int sum = len;                                // inclusive sum-scan of lengths
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int o = __shfl_up_sync(0xffffffffu, sum, d);
+          if (tid >= d) sum += o;
+        }
+        new_start[base + tid] = ns;
+        offs[base + tid] = run_sum + sum - len;
+        run_max = max(run_max, __shfl_sync(0xffffffffu, mx, 31));
+        run_sum += __shfl_sync(0xffffffffu, sum, 31);
+      }
+      if (tid == 0) offs[P] = run_sum;
+    }
+    if (flags) atomicOr(&s_flags, flags);
+    __syncthreads();
+    if (!guess) break;
+
+    grid_dependency_wait();
+    guess = false;
+    bool changed = false;
+    if constexpr (kFromRefs) {
+      const RefsInMemory far(src.tables, r);
+      changed = !same_tables(r, locate_refs<false>(src.tables, b));
+      const int2 *lines = guess_room, *refs = guess_room + kTable;
+      const int32_t* anchors = reinterpret_cast<const int32_t*>(guess_room + 2 * kTable);
+      for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
+        int2 line = make_int2(0, 0), ref = line;
+        int anchor = 0;
+        if (i < r.n_lines) line = load_now(far.lines + i);
+        if (i < r.n_anchors) anchor = load_now(far.anchors + i);
+        if (i < r.n_refs) ref = load_now(far.refs + i);
+        changed |= i < r.n_lines && (line.x != lines[i].x || line.y != lines[i].y);
+        changed |= i < r.n_anchors && anchor != anchors[i];
+        changed |= i < r.n_refs && (ref.x != refs[i].x || ref.y != refs[i].y);
+      }
+    } else {
+      const int2* list = reinterpret_cast<const int2*>(spans) + first;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (tid + k * kIdxThreads >= S) continue;
+        const int2 now = load_now(list + tid + k * kIdxThreads);
+        changed |= now.x != raw[k].x || now.y != raw[k].y;
+      }
+      changed |= load_now(ctx_lens + b) != length || load_now(span_offsets + b) != first ||
+                 load_now(span_offsets + b + 1) - first != S;
+    }
+    if (!__syncthreads_or(changed)) break;
   }
 
   const int total = offs[P];
