@@ -298,6 +298,39 @@ __device__ __forceinline__ void scan_even_line(EvenLine& line, const DecodeParam
   __syncthreads();
 }
 
+// What block chunk_id of the launch begins with: a request, a K/V head, a row, and its pieces [piece, piece_end) (of the line, or
+// of the slice).  False if nothing.  kEarly: sum_even_line's.
+struct EvenCut { int b, kvh, start, piece, piece_end; };
+template <int kThreads, bool kEarly>
+__device__ __forceinline__ bool cut_even(EvenLine& line, const DecodeParams& p, int chunk_id, EvenCut& c, uint32_t& flags) {
+  const int kv_heads = p.H / p.kv_group;
+  int total, longest;
+  const int at = sum_even_line<kThreads, kEarly>(line, p, flags, total, longest);
+  total *= kv_heads;
+  if (even_by_slices(p, total, longest)) {
+    const int unit = chunk_id / p.n_chunks, slice = chunk_id - unit * p.n_chunks;
+    if (unit >= p.B * kv_heads) return false;
+    c.b = unit / kv_heads;
+    c.kvh = unit - c.b * kv_heads;
+    c.start = slice * p.chunk;
+    c.piece = 0;
+    c.piece_end = min(p.chunk / kEvenRows, even_pieces(line.rows[c.b]) - c.start / kEvenRows);
+    return c.piece_end > 0;
+  }
+  const int share = even_share(p, total);
+  if ((int64_t)chunk_id * share >= total) return false;
+  c.piece = chunk_id * share;
+  c.piece_end = min(total - c.piece, share) + c.piece;
+  scan_even_line<kThreads>(line, p, at);
+  c.b = 0;                                               // the last request that begins at or before the share
+  for (int step = kEvenMaxBatch / 2; step > 0; step >>= 1)
+    if (c.b + step < p.B && line.before[c.b + step] * kv_heads <= c.piece) c.b += step;
+  const int in_request = c.piece - line.before[c.b] * kv_heads, of_unit = even_pieces(line.rows[c.b]);
+  c.kvh = in_request / of_unit;
+  c.start = (in_request - c.kvh * of_unit) * kEvenRows;
+  return true;
+}
+
 // What the rows of V whose value at `v` is not finite add to it: infinities of their sign, or a NaN.  Called by one thread for
 // its dim where the split weights (kSplit) have made a NaN of it; the scores as the kernel has them, the weights whole.
 template <typename T, typename Position>
@@ -402,48 +435,24 @@ decode_partial_gqa_kernel(const DecodeParams p) {
   uint32_t flags = 0;
   int kvh = blockIdx.y, b = blockIdx.z, start = chunk_id * p.chunk;
   int piece = 0, piece_end = 0;                        // kEven: what is left of this block's share
-  // What this block begins with; false if nothing.
-  auto cut = [&](auto early, uint32_t& flags) -> bool {
-    if constexpr (kEven) {
-      const int kv_heads = p.H / G;
-      int total, longest;
-      const int at = sum_even_line<kThreads, decltype(early)::value>(s_line, p, flags, total, longest);
-      total *= kv_heads;
-      if (even_by_slices(p, total, longest)) {
-        const int unit = chunk_id / p.n_chunks, slice = chunk_id - unit * p.n_chunks;
-        if (unit >= p.B * kv_heads) return false;
-        b = unit / kv_heads;
-        kvh = unit - b * kv_heads;
-        start = slice * p.chunk;
-        piece_end = min(p.chunk / kEvenRows, even_pieces(s_line.rows[b]) - start / kEvenRows);
-        if (piece_end <= 0) return false;
-      } else {
-        const int share = even_share(p, total);
-        if ((int64_t)chunk_id * share >= total) return false;
-        piece = chunk_id * share;
-        piece_end = min(total - piece, share) + piece;
-        scan_even_line<kThreads>(s_line, p, at);
-        b = 0;                                           // the last request that begins at or before the share
-        for (int step = kEvenMaxBatch / 2; step > 0; step >>= 1)
-          if (b + step < p.B && s_line.before[b + step] * kv_heads <= piece) b += step;
-        const int in_request = piece - s_line.before[b] * kv_heads, of_unit = even_pieces(s_line.rows[b]);
-        kvh = in_request / of_unit;
-        start = (in_request - kvh * of_unit) * kEvenRows;
-      }
-    }
-    return true;
-  };
   if constexpr (kEven) {
     if (block < (unsigned)p.early_blocks) {
       // (34 requests of 5000 rows, 8 heads on each of 4 K/V heads: 58.2 -> 57.2 us; 15 of 7972, two tokens, 78.4 -> 77.1)
       uint32_t unused = 0;
-      if (cut(std::true_type(), unused) && warp < p.early_warps && part == 0)
-        prefetch_early<T, D, kDense, false>(p, b, kvh, start, warp);
+      EvenCut guessed;                                 // (nothing of it is used behind the wait)
+      if (cut_even<kThreads, true>(s_line, p, chunk_id, guessed, unused) && warp < p.early_warps && part == 0)
+        prefetch_early<T, D, kDense, false>(p, guessed.b, guessed.kvh, guessed.start, warp);
       __syncthreads();                                 // the lengths are gathered anew
     }
     grid_dependency_wait();
     if (p.early_release) grid_launch_dependents();
-    if (!cut(std::false_type(), flags)) return;
+    EvenCut c;
+    if (!cut_even<kThreads, false>(s_line, p, chunk_id, c, flags)) return;
+    b = c.b;
+    kvh = c.kvh;
+    start = c.start;
+    piece = c.piece;
+    piece_end = c.piece_end;
   }
 
   while (true) {                                       // kEven: once per unit of the share; else once

@@ -141,3 +141,84 @@ def test_lists_and_spans_that_an_attention_launch_in_front_writes(B, H, Hkv, D, 
             assert int(counts3) == len(blocks) and torch.equal(block_idx[:len(blocks)], blocks)
             assert [int(w) & 0xFFFFFFFF for w in block_mask[:len(blocks), 0]] == words
         assert float((out[2][i].double() - rows_of(q, kr, vr, chosen, num)).abs().max()) < 1e-4
+
+
+class Writer:
+    """An attention launch that lets the next launch's blocks in as soon as its own have begun, and leaves at its end what that one
+    reads: `numbers` int32 (below 0x7c00) in `words`.  Its output rows are fp16; a request's list holds 255 rows whose weight is
+    0 and one row of V that is the numbers: each the bits of a value, and a zero for the upper half."""
+    ROWS = 256
+
+    def __init__(self, numbers, turns, before):
+        heads = -(-numbers // 64)
+        assert heads <= 74                               # SMs are left for the next launch's blocks
+        half = dict(dtype=torch.float16, device=DEV)
+        self.q = torch.ones(1, heads, 128, **half)
+        self.k = torch.full((1, heads, turns + self.ROWS - 1, 128), -60.0, **half)
+        self.k[:, :, :turns] = 0
+        self.v = torch.zeros_like(self.k)
+        rows = torch.arange(turns, turns + self.ROWS - 1, dtype=torch.int32, device=DEV)
+        self.index = torch.stack([torch.cat([rows, torch.full_like(rows[:1], t)])[None] for t in range(turns)])
+        self.count, self.ctx = (torch.full((1,), n, dtype=torch.int32, device=DEV) for n in (self.ROWS, self.k.shape[2]))
+        self.out = torch.empty(1, heads, 128, **half)
+        self.words = self.out.view(torch.int32).view(-1)
+        self.words.fill_(before)
+        self.desc = ssa.make_desc(self.q, self.k, self.v, self.out)
+        self.ws = torch.empty(ssa.decode_workspace_bytes(self.desc, self.ROWS), dtype=torch.uint8, device=DEV)
+
+    def set(self, turn, numbers):
+        """What the launch of that turn leaves."""
+        words = np.zeros(len(self.words), np.int32)
+        words[:len(numbers)] = numbers
+        assert 0 <= words.min() and words.max() < 0x7C00
+        self.v[0, :, turn] = torch.from_numpy(words).to(DEV).view(torch.float16).view(-1, 128)
+
+    def write(self, turn):
+        ssa.decode_attn_sparse(self.desc, self.q, self.k, self.v, self.ctx, self.index[turn], self.count, self.ROWS, self.out, None,
+                               self.ws)
+
+
+def keep_busy():
+    """So that the launches that follow stand in line, and begin as soon as the one in front lets them."""
+    big = torch.empty(2 << 30, dtype=torch.uint8, device=DEV)
+    torch.cuda.synchronize()
+    for i in range(3):
+        big.fill_(i)
+
+
+# rows shared by 4 heads (and tokens), over 8-bit rows, by 20 heads: by two blocks side by side
+@pytest.mark.parametrize("B,H,Hkv,T,n_q,dtype", [
+    (17, 32, 8, 2560, 1, "bf16"), (17, 16, 8, 2560, 2, "f16"), (17, 32, 8, 2560, 1, "fp8"), (34, 40, 2, 8190, 1, "bf16")])
+def test_full_contexts_cut_by_lengths_that_the_launch_in_front_writes(B, H, Hkv, T, n_q, dtype):
+    """Full contexts are cut on the device, alike ones otherwise than ragged ones: the lengths change from one to the other."""
+    gen, rng = torch.Generator(device=DEV).manual_seed(B + H), np.random.default_rng(T + H)
+    tq = torch.float16 if dtype == "f16" else torch.bfloat16
+    q = torch.randn(B, H, n_q, 128, device=DEV, generator=gen).to(tq)
+    k, v = (torch.randn(B, Hkv, T, 128, device=DEV, generator=gen).to(tq) for _ in range(2))
+    if dtype == "fp8":
+        k, v = k.to(torch.float8_e4m3fn), v.to(torch.float8_e4m3fn)
+    turns = 8
+    writer, lengths = Writer(B, turns, 3), []
+    for t in range(turns):
+        alike, ragged = rng.integers(T - 64, T + 1, B), rng.integers(1, T // 16, B)
+        ragged[rng.integers(0, B)] = T
+        lengths.append((ragged, alike)[t % 2])
+        writer.set(t, lengths[t])
+    outs, again = (torch.full((turns, B, H, n_q, 128), 7.0, device=DEV) for _ in range(2))
+    desc, *tokens = ssa.make_desc_multiq(q, k, v, outs[0])
+    ws = torch.empty(ssa.decode_multiq_workspace_bytes(desc, n_q, T), dtype=torch.uint8, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    keep_busy()
+    for t in range(turns):
+        writer.write(t)
+        ssa.decode_attn_dense_multiq(desc, *tokens, q, k, v, writer.words[:B], outs[t], None, ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    everything = torch.arange(T, device=DEV).expand(B, T)
+    for t in range(turns):
+        ctx = torch.from_numpy(lengths[t].astype(np.int32)).to(DEV)
+        ssa.decode_attn_dense_multiq(desc, *tokens, q, k, v, ctx, again[t], None, ws, status)
+        torch.cuda.synchronize()
+        want = rows_of(q.reshape(B, H * n_q, 128), k.to(tq), v.to(tq), everything, ctx)
+        assert float((outs[t].reshape(B, H * n_q, 128).double() - want).abs().max()) < 1e-4, t
+        assert torch.equal(outs[t], again[t]), t
