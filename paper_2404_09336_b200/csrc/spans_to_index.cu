@@ -87,7 +87,6 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   __shared__ int s_resolved;
   const int32_t* __restrict__ span_offsets = src.span_offsets;
   const int32_t* __restrict__ spans = src.spans;
-  const int32_t* __restrict__ ctx_lens = kFromRefs ? src.tables.ctx_lens : src.ctx_lens;
 
   const int b = blockIdx.y;
   const int tid = threadIdx.x;
@@ -103,7 +102,9 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   int P;
   while (true) {
     auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
-    const int length = load(ctx_lens + b);
+    RefTables r = {};
+    if constexpr (kFromRefs) r = guess ? locate_refs<true>(src.tables, b) : locate_refs<false>(src.tables, b);
+    const int length = kFromRefs ? r.current.y : load(src.ctx_lens + b);   // read once: what is compared is what was used
     const int n = max(length, 0);
     uint32_t flags = 0;
     if (tid == 0) s_flags = 0;
@@ -118,7 +119,6 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
 
     int first = 0, S;
     int2 raw[2] = {make_int2(0, 0), make_int2(0, 0)};   // spans tid and tid + kIdxThreads of a list of up to kRankSpans
-    RefTables r = {};
     if constexpr (kFromRefs) {
       // 1 (references): warp 0 resolves them and leaves the packed spans, unsorted, in keys[0, S)
       static_assert(4 * kTable <= kMaxSpans, "the copies lie in arrays that step 3 fills");
@@ -129,7 +129,6 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
         __device__ __forceinline__ int2 ref(int i) const { return refs[i]; }
         __device__ __forceinline__ int anchor(int i) const { return anchors[i]; }
       };
-      r = guess ? locate_refs<true>(src.tables, b) : locate_refs<false>(src.tables, b);
       const RefsInMemory far(src.tables, r);
       // (a guess needs its copies for the comparison: behind the keys of a list of up to kRankSpans, where nothing else comes)
       int2* const room = guess ? guess_room : reinterpret_cast<int2*>(new_start);
@@ -325,7 +324,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
         const int2 now = load_now(list + tid + k * kIdxThreads);
         changed |= now.x != raw[k].x || now.y != raw[k].y;
       }
-      changed |= load_now(ctx_lens + b) != length || load_now(span_offsets + b) != first ||
+      changed |= load_now(src.ctx_lens + b) != length || load_now(span_offsets + b) != first ||
                  load_now(span_offsets + b + 1) - first != S;
     }
     if (!__syncthreads_or(changed)) break;
