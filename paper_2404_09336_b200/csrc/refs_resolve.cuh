@@ -6,29 +6,39 @@
 
 namespace ssa {
 
-// Where request b's tables begin and how long they are, and its first two spans: one trip to memory.
+// Where request b's tables begin and how long they are, and its first two spans.
 struct RefTables {
   int l0, n_lines, a0, n_anchors, r0, n_refs;
   int2 prefix, current;                     // the instruction prefix and the line being generated
 };
-// kEarly: as they stand before grid_dependency_wait().
-template <bool kEarly = false>
-__device__ __forceinline__ RefTables locate_refs(const ssa_anchor_tables& t, int b) {
-  auto load = [](const int32_t* p) { return kEarly ? load_early(p) : load_now(p); };
-  RefTables r;
-  r.l0 = load(t.line_offsets + b);
-  r.a0 = load(t.anchor_offsets + b);
-  r.r0 = load(t.ref_offsets + b);
-  r.n_lines = max(load(t.line_offsets + b + 1) - r.l0, 0);
-  r.n_anchors = max(load(t.anchor_offsets + b + 1) - r.a0, 0);
-  r.n_refs = max(load(t.ref_offsets + b + 1) - r.r0, 0);
-  r.prefix = make_int2(0, load(t.prefix_len + b));
-  r.current = make_int2(load(t.line_start + b), load(t.ctx_lens + b));
-  return r;
+// They follow from nine words: one trip to memory.
+constexpr int kRefWords = 9;
+__device__ __forceinline__ const int32_t* ref_word(const ssa_anchor_tables& t, int b, int i) {
+  switch (i) {
+    case 0: return t.line_offsets + b;
+    case 1: return t.line_offsets + b + 1;
+    case 2: return t.anchor_offsets + b;
+    case 3: return t.anchor_offsets + b + 1;
+    case 4: return t.ref_offsets + b;
+    case 5: return t.ref_offsets + b + 1;
+    case 6: return t.prefix_len + b;
+    case 7: return t.line_start + b;
+    default: return t.ctx_lens + b;
+  }
 }
-__device__ __forceinline__ bool same_tables(const RefTables& a, const RefTables& b) {
-  return a.l0 == b.l0 && a.n_lines == b.n_lines && a.a0 == b.a0 && a.n_anchors == b.n_anchors && a.r0 == b.r0 &&
-         a.n_refs == b.n_refs && a.prefix.y == b.prefix.y && a.current.x == b.current.x && a.current.y == b.current.y;
+// word(i): the value of the i-th.
+template <typename Word>
+__device__ __forceinline__ RefTables locate_refs(Word word) {
+  RefTables r;
+  r.l0 = word(0);
+  r.n_lines = max(word(1) - r.l0, 0);
+  r.a0 = word(2);
+  r.n_anchors = max(word(3) - r.a0, 0);
+  r.r0 = word(4);
+  r.n_refs = max(word(5) - r.r0, 0);
+  r.prefix = make_int2(0, word(6));
+  r.current = make_int2(word(7), word(8));
+  return r;
 }
 
 // The tables as they lie in global memory.

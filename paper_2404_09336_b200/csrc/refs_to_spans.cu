@@ -22,7 +22,7 @@ refs_to_spans_kernel(const ssa_anchor_tables t, int32_t B, int32_t* __restrict__
   uint32_t flags = 0;
   if (lane == 0) span_offsets_out[b] = b * span_stride;
   // spans beyond the row are counted, not stored (overflow)
-  const RefTables r = locate_refs(t, b);
+  const RefTables r = locate_refs([&](int i) { return load_now(ref_word(t, b, i)); });
   const int written = resolve_refs_warp(r, RefsInMemory(t, r), lane, flags, [&](int at, int2 span) {
     if (at < span_stride) row[at] = span;
   });

@@ -85,7 +85,8 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   __shared__ __align__(16) int32_t offs[kMaxSpans + 1];
   __shared__ uint32_t s_flags;
   __shared__ int s_resolved;
-  const int32_t* __restrict__ span_offsets = src.span_offsets;
+  constexpr int kWords = kFromRefs ? kRefWords : 3;
+  __shared__ int32_t s_words[kWords];
   const int32_t* __restrict__ spans = src.spans;
 
   const int b = blockIdx.y;
@@ -99,13 +100,23 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
                                         // attention grid parked on the SMs during this kernel slowed it down
   int2* const guess_room = reinterpret_cast<int2*>(keys + 2 * kRankSpans);
   static_assert(2 * kRankSpans * 8 + kTable * 20 <= kMaxSpans * 8, "a guess's copies lie behind its keys and starts");
+  // The words that say where the request's list or tables lie, and its context, decide about barriers below.  The kernel in
+  // front may be writing them, so that threads could see different ones: for a guess one warp reads them, once, and hands them out.
+  auto word_at = [&](int i) -> const int32_t* {
+    if constexpr (kFromRefs) return ref_word(src.tables, b, i);
+    else return i == 0 ? src.ctx_lens + b : src.span_offsets + b + (i - 1);
+  };
+  if (guess) {
+    if (tid < kWords) s_words[tid] = load_early(word_at(tid));
+    __syncthreads();
+  }
   int P;
   while (true) {
     auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
+    auto word = [&](int i) { return guess ? s_words[i] : load_now(word_at(i)); };
     RefTables r = {};
-    if constexpr (kFromRefs) r = guess ? locate_refs<true>(src.tables, b) : locate_refs<false>(src.tables, b);
-    const int length = kFromRefs ? r.current.y : load(src.ctx_lens + b);   // read once: what is compared is what was used
-    const int n = max(length, 0);
+    if constexpr (kFromRefs) r = locate_refs(word);
+    const int n = max(kFromRefs ? r.current.y : word(0), 0);
     uint32_t flags = 0;
     if (tid == 0) s_flags = 0;
 
@@ -136,7 +147,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
       const bool copied = r.n_lines <= kTable && r.n_anchors <= kTable && r.n_refs <= kTable;
       if (guess && !(copied && r.l0 >= 0 && r.a0 >= 0 && r.r0 >= 0 && r.l0 <= src.lines_readable - r.n_lines &&
                      r.a0 <= src.anchors_readable - r.n_anchors && r.r0 <= src.refs_readable - r.n_refs)) {
-        grid_dependency_wait();                         // (block-uniform) no guess
+        grid_dependency_wait();                         // no guess; the same for all threads, as r is
         guess = false;
         continue;
       }
@@ -169,8 +180,8 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
         continue;
       }
     } else {
-      first = load(span_offsets + b);
-      S = load(span_offsets + b + 1) - first;
+      first = word(1);
+      S = word(2) - first;
       if (guess && !(first >= 0 && S >= 0 && S <= min(span_cap, kRankSpans) && first <= src.spans_readable - S)) {
         grid_dependency_wait();
         guess = false;
@@ -300,10 +311,9 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
 
     grid_dependency_wait();
     guess = false;
-    bool changed = false;
+    bool changed = tid < kWords && load_now(word_at(tid)) != s_words[tid];
     if constexpr (kFromRefs) {
       const RefsInMemory far(src.tables, r);
-      changed = !same_tables(r, locate_refs<false>(src.tables, b));
       const int2 *lines = guess_room, *refs = guess_room + kTable;
       const int32_t* anchors = reinterpret_cast<const int32_t*>(guess_room + 2 * kTable);
       for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
@@ -324,8 +334,6 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
         const int2 now = load_now(list + tid + k * kIdxThreads);
         changed |= now.x != raw[k].x || now.y != raw[k].y;
       }
-      changed |= load_now(src.ctx_lens + b) != length || load_now(span_offsets + b) != first ||
-                 load_now(span_offsets + b + 1) - first != S;
     }
     if (!__syncthreads_or(changed)) break;
   }

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import ssa_oracle as O
 from paper_2404_09336_b200 import ssa
 
 from gpu_util import DEV
@@ -222,3 +223,129 @@ def test_full_contexts_cut_by_lengths_that_the_launch_in_front_writes(B, H, Hkv,
         want = rows_of(q.reshape(B, H * n_q, 128), k.to(tq), v.to(tq), everything, ctx)
         assert float((outs[t].reshape(B, H * n_q, 128).double() - want).abs().max()) < 1e-4, t
         assert torch.equal(outs[t], again[t]), t
+
+
+GPU_BITS = {O.ST_BAD_SPAN: ssa.DEV_BAD_SPAN, O.ST_CLIPPED: ssa.DEV_CLIPPED, O.ST_OVERFLOW: ssa.DEV_OVERFLOW,
+            O.ST_BAD_REF: ssa.DEV_BAD_REF}
+LIST_LENGTHS = [0, 1, 5, 30, 31, 32, 33, 64, 100, 255, 256, 257, 300]   # spans: about where the ways to rank them change
+
+
+def random_spans(rng, n, top):
+    starts = rng.integers(0, top, n)
+    return np.stack([starts, starts + rng.integers(0, 40, n)], -1)
+
+
+@pytest.mark.parametrize("before", [-1, 0x7FFFFFFF, 0])
+@pytest.mark.parametrize("written", ["offsets", "contexts", "offsets and contexts", "all"])
+@pytest.mark.parametrize("block_size", [0])               # 0: index lists; else blocked lists
+def test_span_lists_whose_places_the_launch_in_front_writes(block_size, written, before):
+    """Offsets, contexts and spans rewritten in place between calls: every block works by what the launch in front leaves."""
+    rng = np.random.default_rng(len(written))
+    B, T, turns, stride = 13, 3000, 8, 3000
+    i32 = dict(dtype=torch.int32, device=DEV)
+    n_spans = sum(LIST_LENGTHS) + 20
+    turn = []
+    for t in range(turns):
+        lengths = rng.permutation(LIST_LENGTHS) if t % 3 else rng.permutation(LIST_LENGTHS[:6] + [2] * 7)
+        offsets = np.concatenate([[0], np.cumsum(lengths)]) + rng.integers(0, 20)
+        turn.append(dict(offsets=offsets, contexts=rng.integers(0, T, B), spans=random_spans(rng, n_spans, T)))
+    for x in turn[1:]:
+        for name in ("offsets", "contexts", "spans"):
+            if name not in written and written != "all":
+                x[name] = turn[0][name]
+    at = {"offsets": slice(0, B + 1), "contexts": slice(32, 32 + B), "spans": slice(64, 64 + 2 * n_spans)}
+    writer = Writer(64 + 2 * n_spans, turns, before)
+    for t, x in enumerate(turn):
+        words = np.zeros(64 + 2 * n_spans, np.int32)
+        for name, where in at.items():
+            words[where] = x[name].reshape(-1)
+        writer.set(t, words)
+    tensors = {name: writer.words[where] if name in written or written == "all" else
+               torch.from_numpy(turn[0][name].reshape(-1).astype(np.int32)).to(DEV) for name, where in at.items()}
+    counts, status = torch.full((turns, B), -7, **i32), torch.zeros(turns, **i32)
+    bs = block_size or 32
+    listed = torch.full((turns, B, T // bs + 1 if block_size else stride), -7, **i32)
+    masks = torch.full((turns, B, T // bs + 1, bs // 32), -7, **i32)
+    args = tensors["offsets"], tensors["spans"], tensors["contexts"]
+    keep_busy()
+    for t in range(turns):
+        writer.write(t)
+        if block_size:
+            ssa.spans_to_blockmask(*args, bs, listed[t], masks[t], counts[t], status[t:])
+        else:
+            ssa.spans_to_index(*args, listed[t], counts[t], status[t:])
+    torch.cuda.synchronize()
+    listed, masks, counts, status = (x.cpu().numpy() for x in (listed, masks, counts, status))
+    for t, x in enumerate(turn):
+        want_status = 0
+        for b in range(B):
+            spans, n = x["spans"][x["offsets"][b]:x["offsets"][b + 1]], int(x["contexts"][b])
+            want_status |= O.spans_status(spans, n, stride)
+            want, words = O.spans_to_blockmask(spans, n, bs) if block_size else (O.spans_to_index(spans, n), None)
+            assert counts[t, b] == len(want) and listed[t, b, :len(want)].tolist() == want.tolist(), (t, b)
+            assert np.all(listed[t, b, len(want):] == -7)
+            if block_size:
+                assert np.array_equal(masks[t, b, :len(want)].view(np.uint32), words), (t, b)
+        assert status[t] == sum(v for k, v in GPU_BITS.items() if want_status & k)
+
+
+@pytest.mark.parametrize("before", [-1, 0x7FFFFFFF])
+@pytest.mark.parametrize("written", [
+    "line_offsets", "lines", "anchor_offsets", "anchors", "ref_offsets", "refs", "prefix", "start", "ctx", "all"])
+def test_references_whose_tables_the_launch_in_front_writes(written, before):
+    """Every table of ssa_refs_to_index, and all of them, rewritten in place between calls."""
+    rng = np.random.default_rng(len(written))
+    B, turns, stride, T = 9, 8, 3000, 3000
+    i32 = dict(dtype=torch.int32, device=DEV)
+    at, end = {}, 0
+    for name, size in dict(line_offsets=B + 1, anchor_offsets=B + 1, ref_offsets=B + 1, prefix=B, start=B, ctx=B, lines=1800,
+                           anchors=1400, refs=700).items():
+        at[name], end = slice(end, end + size), end + size + size % 2          # (pairs stay on 8 bytes)
+    turn = []
+    for t in range(turns):
+        n_lines, n_anchors = rng.choice([0, 20, 60, 90], B), rng.choice([1, 40, 150], B)
+        n_refs = rng.choice([0, 1, 2, 31, 33], B)
+        if t == turns - 2:
+            n_lines[0], n_anchors[1], n_refs[2] = 100, 560, 40                 # a table that is not copied
+            n_lines[1:], n_anchors[2:] = 60, 40
+        place = lambda n: np.concatenate([[0], np.cumsum(n)]) + 2
+        lo = rng.integers(0, 140, 350)
+        turn.append(dict(
+            line_offsets=place(n_lines), anchor_offsets=place(n_anchors), ref_offsets=place(n_refs),
+            prefix=rng.integers(0, 80, B), start=rng.integers(T - 200, T, B), ctx=rng.integers(T // 2, T, B),
+            lines=random_spans(rng, 900, T), anchors=rng.integers(0, 100, 1400),
+            refs=np.stack([lo, lo + rng.integers(0, 12, 350)], -1)))
+    for x in turn[1:]:
+        for name in at:
+            if written not in (name, "all"):
+                x[name] = turn[0][name]
+    writer = Writer(end, turns, before)
+    for t, x in enumerate(turn):
+        words = np.zeros(end, np.int32)
+        for name, where in at.items():
+            words[where] = x[name].reshape(-1)
+        writer.set(t, words)
+    tables = [writer.words[where] if written in (name, "all") else
+              torch.from_numpy(turn[0][name].reshape(-1).astype(np.int32)).to(DEV)
+              for name, where in ((n, at[n]) for n in ("line_offsets", "lines", "anchor_offsets", "anchors", "ref_offsets", "refs",
+                                                       "prefix", "start", "ctx"))]
+    listed, counts = torch.full((turns, B, stride), -7, **i32), torch.full((turns, B), -7, **i32)
+    status = torch.zeros(turns, **i32)
+    keep_busy()
+    for t in range(turns):
+        writer.write(t)
+        ssa.refs_to_index(*tables, listed[t], counts[t], status[t:])
+    torch.cuda.synchronize()
+    listed, counts, status = listed.cpu().numpy(), counts.cpu().numpy(), status.cpu().numpy()
+    for t, x in enumerate(turn):
+        want_status = 0
+        for b in range(B):
+            own = lambda name, offsets: x[name][x[offsets][b]:x[offsets][b + 1]]
+            spans, bits = O.resolve_references(own("lines", "line_offsets"), own("anchors", "anchor_offsets"),
+                                               own("refs", "ref_offsets"), x["prefix"][b], x["start"][b], x["ctx"][b])
+            assert len(spans) <= 2048
+            want_status |= bits | O.spans_status(spans, x["ctx"][b], stride)
+            rows = O.spans_to_index(spans, x["ctx"][b])
+            assert counts[t, b] == len(rows) and listed[t, b, :len(rows)].tolist() == rows.tolist(), (t, b)
+            assert np.all(listed[t, b, len(rows):] == -7)
+        assert status[t] == sum(v for k, v in GPU_BITS.items() if want_status & k)
