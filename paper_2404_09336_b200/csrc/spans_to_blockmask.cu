@@ -26,6 +26,7 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
   __shared__ uint32_t s_word[kBmThreads];
   __shared__ int s_wcount[kBmThreads / 32];
   __shared__ uint32_t s_flags;
+  __shared__ int32_t s_words[3];
 
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // word t of the bitmap of the window at w0 covers positions [w0 + 32 t, w0 + 32 t + 32).  A warp takes a span at a time and its
@@ -51,17 +52,24 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
   // requests of 32 heads, 1024 of 2048 rows 168.0 -> 166.0; 34 of 8 heads, up to 350 rows 27.2 -> 26.8.
   bool guess = spans_readable > 0;
   if (!guess) grid_dependency_wait();
+  // (the words that decide about barriers may be about to change: for a guess one warp reads them, once, and hands them out)
+  auto word_at = [&](int i) { return i == 0 ? ctx_lens + b : span_offsets + b + (i - 1); };
+  if (guess) {
+    if (tid < 3) s_words[tid] = load_early(word_at(tid));
+    __syncthreads();
+  }
   int n, S;
   uint32_t flags;
   while (true) {
     auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
-    const int length = load(ctx_lens + b), first = load(span_offsets + b), listed_spans = load(span_offsets + b + 1) - first;
+    auto word = [&](int i) { return guess ? s_words[i] : load_now(word_at(i)); };
+    const int first = word(1), listed_spans = word(2) - first;
     if (guess && !(first >= 0 && listed_spans >= 0 && listed_spans <= kBmThreads && first <= spans_readable - listed_spans)) {
-      grid_dependency_wait();                           // (block-uniform) no guess
+      grid_dependency_wait();                           // no guess; the same for all threads, as the words are
       guess = false;
       continue;
     }
-    n = max(length, 0);
+    n = max(word(0), 0);
     S = max(listed_spans, 0);
     flags = 0;
     if (S > kBmMaxSpans) { S = kBmMaxSpans; flags |= SSA_DEV_TOO_MANY_SPANS; }
@@ -79,8 +87,7 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
     if (!guess) break;
     grid_dependency_wait();
     guess = false;
-    bool changed = load_now(ctx_lens + b) != length || load_now(span_offsets + b) != first ||
-                   load_now(span_offsets + b + 1) - first != listed_spans;
+    bool changed = tid < 3 && load_now(word_at(tid)) != s_words[tid];
     if (tid < S) {
       const int2 now = load_now(list + tid);
       changed |= now.x != own.x || now.y != own.y;

@@ -237,7 +237,7 @@ def random_spans(rng, n, top):
 
 @pytest.mark.parametrize("before", [-1, 0x7FFFFFFF, 0])
 @pytest.mark.parametrize("written", ["offsets", "contexts", "offsets and contexts", "all"])
-@pytest.mark.parametrize("block_size", [0])               # 0: index lists; else blocked lists
+@pytest.mark.parametrize("block_size", [0, 32, 256])      # 0: index lists; else blocked lists
 def test_span_lists_whose_places_the_launch_in_front_writes(block_size, written, before):
     """Offsets, contexts and spans rewritten in place between calls: every block works by what the launch in front leaves."""
     rng = np.random.default_rng(len(written))
