@@ -180,8 +180,9 @@ __device__ __forceinline__ int merge_spans_warp(WarpRuns& w, int2 my_span, int S
 // A request's spans merged ahead of grid_dependency_wait() (merge_spans_early), for a guess that is checked after it
 // (still_the_spans): the kernel in front may yet write the list.
 struct EarlySpans {
-  bool there;                               // warp-uniform: the list could be read
-  int first, S, n, total;                   // where it was, how long; the context; what merge_spans_warp returned
+  bool there;                               // the list could be read
+  int first, S, n, total;                   // where it was, how long; the context; what merge_spans_warp returned (all the same
+                                            // for every lane)
   int2 span;                                // lane i < S: span i
   uint32_t flags;
 };
@@ -191,9 +192,15 @@ __device__ __forceinline__ EarlySpans merge_spans_early(WarpRuns& w, const int32
                                                         const int32_t* ctx_lens, int max_ctx, int b, int cap, int P) {
   EarlySpans e;
   const int lane = threadIdx.x & 31;
-  e.first = span_offsets ? load_early(span_offsets + b) : b * cap;
-  e.S = span_offsets ? load_early(span_offsets + b + 1) - e.first : cap;
-  e.n = max(min(load_early(ctx_lens + b), max_ctx), 0);
+  // (a lane per word, and handed out: lanes that read a word for themselves while it is written need not agree on it)
+  int word = 0;
+  if (lane == 0) word = load_early(ctx_lens + b);
+  else if (lane < 3 && span_offsets) word = load_early(span_offsets + b + (lane - 1));
+  const int length = __shfl_sync(0xffffffffu, word, 0), first = __shfl_sync(0xffffffffu, word, 1);
+  const int end = __shfl_sync(0xffffffffu, word, 2);
+  e.first = span_offsets ? first : b * cap;
+  e.S = span_offsets ? end - first : cap;
+  e.n = max(min(length, max_ctx), 0);
   e.there = e.first >= 0 && e.S >= 0 && e.S <= cap && e.first <= readable - e.S;
   e.span = make_int2(0, 0);
   e.flags = 0;

@@ -349,3 +349,50 @@ def test_references_whose_tables_the_launch_in_front_writes(written, before):
             assert counts[t, b] == len(rows) and listed[t, b, :len(rows)].tolist() == rows.tolist(), (t, b)
             assert np.all(listed[t, b, len(rows):] == -7)
         assert status[t] == sum(v for k, v in GPU_BITS.items() if want_status & k)
+
+
+# blocks of one head, of eight and sixteen warps, row-sharing (ordinary, two chunks, 8-bit rows, above sixteen heads)
+@pytest.mark.parametrize("B,H,Hkv,D,dtype", [
+    (40, 8, 8, 128, "bf16"), (20, 8, 8, 128, "f16"), (3, 8, 8, 64, "bf16"), (40, 32, 8, 128, "bf16"), (3, 32, 8, 128, "bf16"),
+    (40, 8, 2, 128, "fp8"), (20, 20, 1, 128, "bf16")])
+@pytest.mark.parametrize("before", [-1, 0])
+def test_attention_over_spans_whose_places_the_launch_in_front_writes(B, H, Hkv, D, dtype, before):
+    """Offsets, contexts and spans of ssa_decode_attn_spans rewritten in place between calls."""
+    gen, rng = torch.Generator(device=DEV).manual_seed(B * H + D), np.random.default_rng(B)
+    T, turns, cap, most = 900, 8, 30, 900
+    tq = torch.float16 if dtype == "f16" else torch.bfloat16
+    q = torch.randn(B, H, D, device=DEV, generator=gen).to(tq)
+    k, v = (torch.randn(B, Hkv, T, D, device=DEV, generator=gen).to(tq) for _ in range(2))
+    if dtype == "fp8":
+        k, v = k.to(torch.float8_e4m3fn), v.to(torch.float8_e4m3fn)
+    n_spans = 18 * B + 40
+    ends = 3 * B + 1 + (3 * B + 1) % 2                   # (spans lie on 8 bytes)
+    writer, turn = Writer(ends + 2 * n_spans, turns, before), []
+    for t in range(turns):
+        lengths = np.minimum(rng.choice([0, 1, 3, 14, cap], B), 18 if t % 2 else cap)
+        while lengths.sum() > n_spans - 20:
+            lengths[rng.integers(B)] = 1
+        offsets, spans = np.concatenate([[0], np.cumsum(lengths)]) + rng.integers(0, 20), random_spans(rng, n_spans, T - 40)
+        ctx = rng.integers(1, T + 1, B)
+        turn.append((offsets, spans, ctx))
+        words = np.zeros(ends + 2 * n_spans, np.int32)
+        words[:B + 1], words[2 * B:3 * B], words[ends:] = offsets, ctx, spans.reshape(-1)
+        writer.set(t, words)
+    i32 = dict(dtype=torch.int32, device=DEV)
+    outs, status = torch.full((turns, B, H, D), 7.0, device=DEV), torch.zeros(1, **i32)
+    listed, counts = torch.full((turns, B, most), -7, **i32), torch.full((turns, B), -7, **i32)
+    desc = ssa.make_desc(q, k, v, outs[0])
+    ws = torch.empty(max(ssa.decode_spans_workspace_bytes(desc, most, cap), 16), dtype=torch.uint8, device=DEV)
+    keep_busy()
+    for t in range(turns):
+        writer.write(t)
+        ssa.decode_attn_spans(desc, q, k, v, writer.words[2 * B:3 * B], writer.words[:B + 1], writer.words[ends:], cap, most, outs[t],
+                              index_out=listed[t], counts_out=counts[t], workspace=ws, dev_status=status)
+    torch.cuda.synchronize()
+    got_lists, got_counts = listed.cpu().numpy(), counts.cpu().numpy()
+    for t, (offsets, spans, ctx) in enumerate(turn):
+        for b in range(B):
+            rows = O.spans_to_index(spans[offsets[b]:offsets[b + 1]], int(ctx[b]))
+            assert got_counts[t, b] == len(rows) and got_lists[t, b, :len(rows)].tolist() == rows.tolist(), (t, b)
+        want = rows_of(q, k.to(tq), v.to(tq), listed[t], counts[t])
+        assert float((outs[t].double() - want).abs().max()) < 1e-4, t
