@@ -1,5 +1,6 @@
-"""What blocks do before the launch in front of theirs has ended: they prefetch by lists, lengths and page tables that may still be
-a former step's, or no list at all.  Whatever these say, results are those of the lists as the launch in front leaves them."""
+"""What blocks do before the launch in front of theirs has ended: they prefetch by lists, lengths and page tables, cut full contexts
+and make lists by what may still be a former step's, or nothing at all.  Results are those of the inputs as the launch in front
+leaves them."""
 import numpy as np
 import pytest
 import torch
@@ -31,7 +32,7 @@ def rows_of(q, k, v, index, counts):
     (74, 8, 8, 128, 65, 0), (75, 8, 8, 128, 129, 0), (47, 8, 8, 128, 200, 0), (37, 32, 32, 64, 257, 0),
     (40, 8, 8, 128, 130, 16), (9, 32, 8, 128, 193, 0), (37, 32, 8, 128, 300, 0), (37, 32, 8, 128, 129, 16)])
 @pytest.mark.parametrize("before", [-1, 0x7FFFFFFF, -0x80000000])
-def test_lists_that_the_launch_in_front_still_writes(B, H, Hkv, D, rows, page_size, before):
+def test_lists_of_an_index_launch_in_front(B, H, Hkv, D, rows, page_size, before):
     gen = torch.Generator(device=DEV).manual_seed(B * rows + D)
     T = 1024
     q = torch.randn(B, H, D, device=DEV, generator=gen).bfloat16()
@@ -61,7 +62,7 @@ def test_lists_that_the_launch_in_front_still_writes(B, H, Hkv, D, rows, page_si
         table.copy_(full_table)
         paging = ssa.make_paging(table, page_size, B * (T // page_size))
     lists = []
-    for sp, out in zip(spans, outs):                     # every launch's lists are written by the one in front
+    for sp, out in zip(spans, outs):                     # (the index launch has ended when attention blocks begin)
         ssa.spans_to_index(offsets, sp, ctx, index, counts, status)
         if page_size:
             ssa.decode_attn_sparse_paged(desc, q, kc, vc, paging, ctx, index, counts, rows, out, None, ws, status)
@@ -179,12 +180,15 @@ class Writer:
                                self.ws)
 
 
-def keep_busy():
-    """So that the launches that follow stand in line, and begin as soon as the one in front lets them."""
+def in_line(turns):
+    """The turns, twice: the first time round kernels may have to be loaded, which parts launches.  What is launched meanwhile
+    stands in line, and begins as soon as the launch in front lets it."""
     big = torch.empty(2 << 30, dtype=torch.uint8, device=DEV)
-    torch.cuda.synchronize()
-    for i in range(3):
-        big.fill_(i)
+    for _ in range(2):
+        torch.cuda.synchronize()
+        for i in range(3):
+            big.fill_(i)
+        yield from range(turns)
 
 
 # rows shared by 4 heads (and tokens), over 8-bit rows, by 20 heads: by two blocks side by side
@@ -209,8 +213,7 @@ def test_full_contexts_cut_by_lengths_that_the_launch_in_front_writes(B, H, Hkv,
     desc, *tokens = ssa.make_desc_multiq(q, k, v, outs[0])
     ws = torch.empty(ssa.decode_multiq_workspace_bytes(desc, n_q, T), dtype=torch.uint8, device=DEV)
     status = torch.zeros(1, dtype=torch.int32, device=DEV)
-    keep_busy()
-    for t in range(turns):
+    for t in in_line(turns):
         writer.write(t)
         ssa.decode_attn_dense_multiq(desc, *tokens, q, k, v, writer.words[:B], outs[t], None, ws, status)
     torch.cuda.synchronize()
@@ -267,8 +270,7 @@ def test_span_lists_whose_places_the_launch_in_front_writes(block_size, written,
     listed = torch.full((turns, B, T // bs + 1 if block_size else stride), -7, **i32)
     masks = torch.full((turns, B, T // bs + 1, bs // 32), -7, **i32)
     args = tensors["offsets"], tensors["spans"], tensors["contexts"]
-    keep_busy()
-    for t in range(turns):
+    for t in in_line(turns):
         writer.write(t)
         if block_size:
             ssa.spans_to_blockmask(*args, bs, listed[t], masks[t], counts[t], status[t:])
@@ -331,8 +333,7 @@ def test_references_whose_tables_the_launch_in_front_writes(written, before):
                                                        "prefix", "start", "ctx"))]
     listed, counts = torch.full((turns, B, stride), -7, **i32), torch.full((turns, B), -7, **i32)
     status = torch.zeros(turns, **i32)
-    keep_busy()
-    for t in range(turns):
+    for t in in_line(turns):
         writer.write(t)
         ssa.refs_to_index(*tables, listed[t], counts[t], status[t:])
     torch.cuda.synchronize()
@@ -383,8 +384,7 @@ def test_attention_over_spans_whose_places_the_launch_in_front_writes(B, H, Hkv,
     listed, counts = torch.full((turns, B, most), -7, **i32), torch.full((turns, B), -7, **i32)
     desc = ssa.make_desc(q, k, v, outs[0])
     ws = torch.empty(max(ssa.decode_spans_workspace_bytes(desc, most, cap), 16), dtype=torch.uint8, device=DEV)
-    keep_busy()
-    for t in range(turns):
+    for t in in_line(turns):
         writer.write(t)
         ssa.decode_attn_spans(desc, q, k, v, writer.words[2 * B:3 * B], writer.words[:B + 1], writer.words[ends:], cap, most, outs[t],
                               index_out=listed[t], counts_out=counts[t], workspace=ws, dev_status=status)
@@ -396,3 +396,55 @@ def test_attention_over_spans_whose_places_the_launch_in_front_writes(B, H, Hkv,
             assert got_counts[t, b] == len(rows) and got_lists[t, b, :len(rows)].tolist() == rows.tolist(), (t, b)
         want = rows_of(q, k.to(tq), v.to(tq), listed[t], counts[t])
         assert float((outs[t].double() - want).abs().max()) < 1e-4, t
+
+
+# one head per block, rows shared by four heads; contiguous and paged
+@pytest.mark.parametrize("B,H,Hkv,D,rows,page_size", [
+    (24, 32, 32, 128, 150, 0), (24, 32, 32, 64, 150, 0), (24, 32, 8, 128, 150, 0), (24, 32, 32, 128, 120, 16),
+    (12, 32, 8, 128, 300, 16)])
+@pytest.mark.parametrize("before", [-1, 0x7FFFFFFF, -0x80000000])
+def test_lists_that_an_attention_launch_in_front_writes(B, H, Hkv, D, rows, page_size, before):
+    """Lists, counts, contexts and page tables rewritten in place between calls over lists and over full contexts."""
+    gen, rng = torch.Generator(device=DEV).manual_seed(B * rows + D), np.random.default_rng(D)
+    T, turns = 1024, 4
+    per = T // page_size if page_size else 0
+    q = torch.randn(B, H, D, device=DEV, generator=gen).bfloat16()
+    shape = (B * per, page_size, Hkv, D) if page_size else (B, Hkv, T, D)
+    k, v = (torch.randn(shape, device=DEV, generator=gen).bfloat16() for _ in range(2))
+    at, end = {}, 0
+    for name, size in dict(ctx=B, counts=B, index=B * rows, table=B * per).items():
+        at[name], end = slice(end, end + size), end + size
+    writer, turn = Writer(end, turns, before), []
+    for t in range(turns):
+        ctx, counts = rng.integers(rows, T + 1, B), rng.integers(0, rows + 1, B)
+        index = np.stack([rng.permutation(n)[:rows] for n in ctx])
+        turn.append(dict(ctx=ctx, counts=counts, index=index, table=rng.permutation(B * per)))
+        writer.set(t, np.concatenate([turn[t][name].reshape(-1) for name in at]))
+    ctx, counts, index, table = (writer.words[where] for where in at.values())
+    index = index.view(B, rows)
+    outs, status = torch.full((2, turns, B, H, D), 7.0, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    desc = ssa.make_desc_paged(q, k, v, outs[0, 0], T) if page_size else ssa.make_desc(q, k, v, outs[0, 0])
+    ws = torch.empty(max(ssa.decode_workspace_bytes(desc, n) for n in (rows, T)), dtype=torch.uint8, device=DEV)
+    paging = ssa.make_paging(table.view(B, per), page_size, B * per) if page_size else None
+    for t in in_line(turns):
+        writer.write(t)
+        if page_size:
+            ssa.decode_attn_sparse_paged(desc, q, k, v, paging, ctx, index, counts, rows, outs[0, t], None, ws, status)
+        else:
+            ssa.decode_attn_sparse(desc, q, k, v, ctx, index, counts, rows, outs[0, t], None, ws, status)
+        t = (t + 1) % turns                              # other words again
+        writer.write(t)
+        if page_size:
+            ssa.decode_attn_dense_paged(desc, q, k, v, paging, ctx, outs[1, t], None, ws, status)
+        else:
+            ssa.decode_attn_dense(desc, q, k, v, ctx, outs[1, t], None, ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    everything = torch.arange(T, device=DEV).expand(B, T)
+    for t, x in enumerate(turn):
+        x = {name: torch.from_numpy(a).to(DEV) for name, a in x.items()}
+        kc, vc = k, v
+        if page_size:                                    # the requests' rows in order
+            kc, vc = (pool[x["table"].view(B, per)].reshape(B, T, Hkv, D).transpose(1, 2) for pool in (k, v))
+        for out, idx, n in ((outs[0, t], x["index"], x["counts"]), (outs[1, t], everything, x["ctx"])):
+            assert float((out.double() - rows_of(q, kc, vc, idx, n)).abs().max()) < 1e-4, t
