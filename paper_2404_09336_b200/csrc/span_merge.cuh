@@ -192,15 +192,12 @@ __device__ __forceinline__ EarlySpans merge_spans_early(WarpRuns& w, const int32
                                                         const int32_t* ctx_lens, int max_ctx, int b, int cap, int P) {
   EarlySpans e;
   const int lane = threadIdx.x & 31;
-  // (a lane per word, and handed out: lanes that read a word for themselves while it is written need not agree on it)
-  int word = 0;
-  if (lane == 0) word = load_early(ctx_lens + b);
-  else if (lane < 3 && span_offsets) word = load_early(span_offsets + b + (lane - 1));
-  const int length = __shfl_sync(0xffffffffu, word, 0), first = __shfl_sync(0xffffffffu, word, 1);
-  const int end = __shfl_sync(0xffffffffu, word, 2);
-  e.first = span_offsets ? first : b * cap;
-  e.S = span_offsets ? end - first : cap;
-  e.n = max(min(length, max_ctx), 0);
+  // (lanes that read a word while it is written need not agree on it: lane 0's counts.  With a lane per word instead the one-head
+  // kernel comes out up to 2 us slower: 34 requests of 32 heads, up to 7 spans, 18.0 / 19.8)
+  auto word = [](const int32_t* p) { return __shfl_sync(0xffffffffu, load_early(p), 0); };
+  e.first = span_offsets ? word(span_offsets + b) : b * cap;
+  e.S = span_offsets ? word(span_offsets + b + 1) - e.first : cap;
+  e.n = max(min(word(ctx_lens + b), max_ctx), 0);
   e.there = e.first >= 0 && e.S >= 0 && e.S <= cap && e.first <= readable - e.S;
   e.span = make_int2(0, 0);
   e.flags = 0;
