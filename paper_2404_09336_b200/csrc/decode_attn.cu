@@ -739,7 +739,8 @@ static size_t triples_bytes(const ssa_attn_desc* d, size_t triples, size_t* acc_
   return *acc_bytes + (triples * sizeof(float2) + 255) / 256 * 256;
 }
 
-static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan* pl) {
+// full: contexts that are read as they lie, without a list or a page table.
+static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, bool full, Plan* pl) {
   if (!d || d->B <= 0 || d->H <= 0 || max_selected <= 0) return false;
   if (d->D != 64 && d->D != 128) return false;
   const long long out_units = (long long)d->B * d->H;                  // triples per chunk
@@ -762,14 +763,18 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
            5 * units >= (max_selected * d->D <= 768 * 128 ? sms : 2 * sms) &&
            (d->kv_dtype != SSA_FP8_E4M3 || (d->H == d->H_kv && (units <= sms || 5 * units >= 7 * sms))))
     chunk = kMaxWideChunk;
-  // Longer chunks where there are blocks enough without (us, 256 / 512 entries; 32 heads a request).  Rows of 128 16-bit values: 64
-  // requests of 4000 rows 612 / 598, 32 of them 307 / 303, of 2000 154.9 / 154.5, 64 of up to 1024, most of 141, 45.3 / 44.5; but 32 of
-  // 1500 121 / 123, 50 of 900 113 / 114, 64 of 600 98.4 / 99.5.  Rows of half the bytes, or less, are half a chunk: 8-bit, 32 of 900
-  // rows 49.7 / 47.4, 64 94 / 87, 16-bit of 64 52 / 51 (40) and 81 / 78.  (Fewer would make one-kernel steps of some that gain nothing by
-  // it: 24 of 600, 8-bit, 31.6 / 33.3.)
-  else if (!share && (d->D == 64 || d->kv_dtype == SSA_FP8_E4M3
-                          ? max_selected > kMaxChunk && units > 6 * sms
-                          : max_selected > 768 && units * ((max_selected + kMaxChunk - 1) / kMaxChunk) >= 27 * sms)) {
+  // Longer chunks where there are blocks enough without (us, 256 / 512 entries; 32 heads a request).  Rows of 128 16-bit values:
+  // lists and page tables gain, most of all where they are ragged (a paged context of 64 x 2048 307 / 304, of 64 x 512..2048 181 /
+  // 177; 72 requests of up to 1024, every eighth full, 49.6 / 47.1, 64 44.9 / 43.7), but below 27 chunks of 512 per SM as often lose
+  // (44 of them 34.6 / 35.0, 36 30.2 / 30.9; 56 41.2 / 40.3).  Contexts read as they lie do only in the longest launches (64 x 1024
+  // 151 / 154, 32 x 512..2048 97 / 99, 32 x 4096 292 / 295; 32 x 8192 602 / 601, 32 x 2048..8192 395 / 388, on another GPU 581 / 584
+  // and 384 / 384).  Rows of half the bytes, or less, are half a chunk: 8-bit, 32 x 900 49.7 / 47.4, 64 94 / 87, 16-bit of 64 52 / 51
+  // (40) and 81 / 78 (fewer would make one-kernel steps of some that gain nothing by it: 24 x 600, 8-bit, 31.6 / 33.3); contexts
+  // read as they lie from 20 chunks per SM on (rows of 64: 32 x 1024 42.7 / 45.0, 48 x 256..1024 42.7 / 41.5; 8-bit, 64 x 1024 90 / 86).
+  else if (const long long long_chunks = units * ((max_selected + kMaxChunk - 1) / kMaxChunk);
+           !share && (d->D == 64 || d->kv_dtype == SSA_FP8_E4M3
+                          ? max_selected > kMaxChunk && units > 6 * sms && (!full || long_chunks >= 20 * sms)
+                          : max_selected > 768 && long_chunks >= (full ? 80 : 27) * sms)) {
     sized_for = chunk;                                   // (the workspace asked for stays that of chunks of 256)
     chunk = kMaxChunk;
   }
@@ -808,7 +813,7 @@ static bool make_plan(const ssa_attn_desc* d, int max_selected, bool share, Plan
 
 // The plan every workspace holds: grouped heads share rows.
 static bool make_plan(const ssa_attn_desc* d, int max_selected, Plan* pl) {
-  return make_plan(d, max_selected, d && can_share_rows(d), pl);
+  return make_plan(d, max_selected, d && can_share_rows(d), false, pl);
 }
 
 // Small launches over an 8-bit cache, grouped heads: a row-sharing block starts up slower (ring, Q fragments), combines G
@@ -836,10 +841,10 @@ static bool one_head_blocks_pay(const ssa_attn_desc* d, int max_selected, const 
 // The plan of a call with a workspace of ws_bytes: one head per block where that pays and the workspace, which callers may
 // have sized by another bound, holds its partial results; otherwise the plan above.  (Above kGqaHeads heads per K/V head
 // that is also the plan for a workspace too small for the one above.)
-static bool choose_plan(const ssa_attn_desc* d, int max_selected, size_t ws_bytes, Plan* pl) {
-  if (!make_plan(d, max_selected, pl)) return false;
+static bool choose_plan(const ssa_attn_desc* d, int max_selected, size_t ws_bytes, Plan* pl, bool full = false) {
+  if (!make_plan(d, max_selected, d && can_share_rows(d), full, pl)) return false;
   Plan single;
-  if (pl->share && make_plan(d, max_selected, false, &single) && single.total_bytes <= ws_bytes &&
+  if (pl->share && make_plan(d, max_selected, false, full, &single) && single.total_bytes <= ws_bytes &&
       (one_head_blocks_pay(d, max_selected, *pl, single) || (head_splits(d) > 1 && pl->total_bytes > ws_bytes)))
     *pl = single;
   return true;
@@ -1128,7 +1133,7 @@ static int32_t run(const ssa_attn_desc* d, const void* q, const void* k, const v
     if (bl->block_size != 32 && bl->block_size != 64 && bl->block_size != 128 && bl->block_size != 256)
       return SSA_ERR_UNSUPPORTED;
     if (!make_plan_blockmask(d, bl->block_size, max_selected, &pl)) return SSA_ERR_SHAPE;
-  } else if (!choose_plan(d, max_selected, ws_bytes - std::min(ws_bytes, list_bytes), &pl)) {
+  } else if (!choose_plan(d, max_selected, ws_bytes - std::min(ws_bytes, list_bytes), &pl, mode == kDense)) {
     return SSA_ERR_SHAPE;
   }
   if (!ws || ws_bytes < pl.total_bytes + list_bytes) return SSA_ERR_WORKSPACE;
@@ -1278,7 +1283,7 @@ int32_t ssa_decode_attn_sparse_noalloc(const ssa_attn_desc* desc, const void* q,
   ssa::Plan pl;
   // (groups above kGqaHeads are taken as far as their one-head-per-block plan fits, like multi-head calls)
   const bool share = ssa::can_share_rows(desc) && ssa::head_splits(desc) == 1;
-  if (!ssa::make_plan(desc, max_selected, share, &pl)) return SSA_ERR_SHAPE;
+  if (!ssa::make_plan(desc, max_selected, share, false, &pl)) return SSA_ERR_SHAPE;
   if (pl.total_bytes > SSA_STATIC_SCRATCH_BYTES) return SSA_ERR_WORKSPACE;   // beyond the built-in scratch
   void* scratch = ssa::static_scratch_address();
   if (!scratch) return SSA_ERR_CUDA;

@@ -1054,3 +1054,43 @@ def test_lists_taken_whole_by_large_blocks(H, D, sel, launches):
     ref, ref_lse = O.decode_attn_sparse(p.q_bits, p.k_bits, p.v_bits, [1100], index, [sel], scale_of(D), "bf16", heads=heads)
     assert_parity(out[:, heads], ref[:, heads], False, "lists taken whole")
     np.testing.assert_allclose(lse[:, heads], ref_lse[:, heads], rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("B,D,rows,dtype", [
+    (62, 128, 800, "bf16"), (63, 128, 800, "bf16"),          # 16-bit rows of 128: 27 chunks of 512 per SM
+    (27, 128, 600, "fp8"), (28, 128, 600, "fp8"), (27, 64, 513, "f16"), (28, 64, 513, "f16"),   # six units per SM
+    (46, 128, 600, "fp8"), (47, 128, 600, "fp8"), (46, 64, 1024, "f16"), (47, 64, 1025, "f16"),    # full contexts: 20 chunks per SM
+    (61, 128, 2561, "bf16"), (62, 128, 2600, "bf16")])       # ... of 16-bit rows of 128: 80
+def test_chunks_on_both_sides_of_the_lines_for_longer_ones(B, D, rows, dtype):
+    """Ragged lists and full contexts (148 SMs) whose chunks are 256 rows on one side of a line, 512 on the other: empty ones,
+    ends of chunks, lists in reverse."""
+    H, gen = 32, torch.Generator(device=DEV).manual_seed(B * rows)
+    tq = torch.float16 if dtype == "f16" else torch.bfloat16
+    q = torch.randn(B, H, D, device=DEV, generator=gen).to(tq)
+    k, v = (torch.randn(B, H, rows, D, device=DEV, generator=gen).to(tq) for _ in range(2))
+    if dtype == "fp8":
+        k, v = k.to(torch.float8_e4m3fn), v.to(torch.float8_e4m3fn)
+    lens = torch.randint(0, rows + 1, (B,), device=DEV, generator=gen, dtype=torch.int32)
+    lens[:7] = torch.tensor([0, 1, 256, 257, 512, min(513, rows), rows])
+    index = torch.arange(rows - 1, -1, -1, dtype=torch.int32, device=DEV).expand(B, rows).contiguous()
+    ctx, status = torch.full_like(lens, rows), torch.zeros(1, dtype=torch.int32, device=DEV)
+    outs, lses = torch.full((2, B, H, D), 7.0, device=DEV), torch.full((2, B, H), 7.0, device=DEV)
+    desc = ssa.make_desc(q, k, v, outs[0])
+    nbytes = ssa.decode_workspace_bytes(desc, rows)
+    ws = torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device=DEV)
+    ssa.decode_attn_sparse(desc, q, k, v, ctx, index, lens, rows, outs[0], lses[0], ws[:nbytes], status)
+    ssa.decode_attn_dense(desc, q, k, v, lens, outs[1], lses[1], ws[:nbytes], status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and bool((ws[nbytes:] == 0xA5).all())
+    for b in range(B):
+        n = int(lens[b])
+        scores = torch.einsum("hd,htd->ht", q[b].double(), k[b].to(tq).double()) / D ** 0.5
+        for i, part in enumerate((scores[:, rows - n:], scores[:, :n])):
+            if n == 0:
+                assert bool((outs[i, b] == 0).all()) and bool(torch.isneginf(lses[i, b]).all())
+                continue
+            vs = v[b].to(tq).double()
+            want = torch.einsum("ht,htd->hd", torch.softmax(part, -1), vs[:, rows - n:] if i == 0 else vs[:, :n])
+            # fp32 throughout: sums of up to 2600 terms of order 1
+            assert float((outs[i, b].double() - want).abs().max()) < 1e-5, (b, i)
+            assert float((lses[i, b].double() - torch.logsumexp(part, -1)).abs().max()) < 1e-5, (b, i)
