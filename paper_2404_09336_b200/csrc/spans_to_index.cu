@@ -92,7 +92,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   const int b = blockIdx.y;
   const int tid = threadIdx.x;
   // Steps 1-3 run while the kernel in front drains, on the lists as they stand, and again only if they have changed by then:
-  // seeing that they have not takes one trip to memory, the steps two to four and half a microsecond.  Spans to lists and
+  // seeing that they have not takes one trip to memory, the steps two or three and half a microsecond.  Spans to lists and
   // attention, 64 requests 28.8 -> 28.1 us; references and attention, 2 requests of ~25 spans 11.6 -> 9.5, 36 of ~38, 8 heads,
   // 23.9 -> 21.3, 16 of 2 to 50, 32 heads, 41.6 -> 40.5.  (A merge in front is too short to do it all in: 51 of ~20 77.5 -> 77.9.)
   bool guess = (int)(blockIdx.y * gridDim.x + blockIdx.x) < src.early_blocks;
@@ -199,6 +199,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
         for (int k = 0; k < 2; ++k) {
           const int i = tid + k * kIdxThreads;
           if (i < S) raw[k] = load(reinterpret_cast<const int2*>(spans) + first + i);
+          if (guess && i < S) guess_room[i] = raw[k];
         }
       }
       __syncthreads();                                    // s_flags
@@ -275,6 +276,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
     }
 
     // 3. trim against the running maximum end and prefix-sum the lengths
+    bool changed = false;
     if (tid < 32) {
       int run_max = 0, run_sum = 0;
       for (int base = 0; base < P; base += 32) {
@@ -304,37 +306,44 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
         run_sum += __shfl_sync(0xffffffffu, sum, 31);
       }
       if (tid == 0) offs[P] = run_sum;
+    } else if (guess) {
+      // Meanwhile the other warps see whether the guess still holds, so that its trip is not one more where there was no time in
+      // front of the wait.  us, references and attention behind an elementwise kernel, compared after the lists have been made /
+      // meanwhile / without guesses: 1 request of 32 heads 16.6 / 15.3 / 14.8, 9 29.2 / 28.6 / 28.0; between such calls 6 of 8 heads
+      // 13.6 / 12.9 / 13.4.
+      grid_dependency_wait();
+      const int t = tid - 32;
+      constexpr int kStep = kIdxThreads - 32;
+      changed = t < kWords && load_now(word_at(t)) != s_words[t];
+      if constexpr (kFromRefs) {
+        const RefsInMemory far(src.tables, r);
+        const int2 *lines = guess_room, *refs = guess_room + kTable;
+        const int32_t* anchors = reinterpret_cast<const int32_t*>(guess_room + 2 * kTable);
+        for (int i = t; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kStep) {
+          int2 line = make_int2(0, 0), ref = line;
+          int anchor = 0;
+          if (i < r.n_lines) line = load_now(far.lines + i);
+          if (i < r.n_anchors) anchor = load_now(far.anchors + i);
+          if (i < r.n_refs) ref = load_now(far.refs + i);
+          changed |= i < r.n_lines && (line.x != lines[i].x || line.y != lines[i].y);
+          changed |= i < r.n_anchors && anchor != anchors[i];
+          changed |= i < r.n_refs && (ref.x != refs[i].x || ref.y != refs[i].y);
+        }
+      } else {
+        const int2* list = reinterpret_cast<const int2*>(spans) + first;
+        for (int i = t; i < S; i += kStep) {
+          const int2 now = load_now(list + i), then = guess_room[i];
+          changed |= now.x != then.x || now.y != then.y;
+        }
+      }
     }
     if (flags) atomicOr(&s_flags, flags);
-    __syncthreads();
-    if (!guess) break;
-
+    if (!guess) {
+      __syncthreads();
+      break;
+    }
     grid_dependency_wait();
     guess = false;
-    bool changed = tid < kWords && load_now(word_at(tid)) != s_words[tid];
-    if constexpr (kFromRefs) {
-      const RefsInMemory far(src.tables, r);
-      const int2 *lines = guess_room, *refs = guess_room + kTable;
-      const int32_t* anchors = reinterpret_cast<const int32_t*>(guess_room + 2 * kTable);
-      for (int i = tid; i < max(max(r.n_lines, r.n_anchors), r.n_refs); i += kIdxThreads) {
-        int2 line = make_int2(0, 0), ref = line;
-        int anchor = 0;
-        if (i < r.n_lines) line = load_now(far.lines + i);
-        if (i < r.n_anchors) anchor = load_now(far.anchors + i);
-        if (i < r.n_refs) ref = load_now(far.refs + i);
-        changed |= i < r.n_lines && (line.x != lines[i].x || line.y != lines[i].y);
-        changed |= i < r.n_anchors && anchor != anchors[i];
-        changed |= i < r.n_refs && (ref.x != refs[i].x || ref.y != refs[i].y);
-      }
-    } else {
-      const int2* list = reinterpret_cast<const int2*>(spans) + first;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        if (tid + k * kIdxThreads >= S) continue;
-        const int2 now = load_now(list + tid + k * kIdxThreads);
-        changed |= now.x != raw[k].x || now.y != raw[k].y;
-      }
-    }
     if (!__syncthreads_or(changed)) break;
   }
 
