@@ -458,7 +458,9 @@ extern "C" int32_t ssa_refs_to_index(const ssa_anchor_tables* tables, int32_t B,
   src.lines_readable = ssa::readable_entries<int2>(tables->lines, &known);
   src.anchors_readable = ssa::readable_entries<int32_t>(tables->anchor_line, &known);
   src.refs_readable = ssa::readable_entries<int2>(tables->refs, &known);
-  src.early_blocks = ssa::kEarlyBlocks * ssa::sm_count();
+  // (tables elsewhere than in one allocation of device memory, across the bus for instance, are not read twice)
+  const bool readable = src.lines_readable > 0 && src.anchors_readable > 0 && src.refs_readable > 0;
+  src.early_blocks = readable ? ssa::kEarlyBlocks * ssa::sm_count() : 0;
   const cudaError_t err = ssa::launch_pdl(ssa::spans_to_index_kernel<true>, grid, dim3(ssa::kIdxThreads),
                                           (cudaStream_t)stream, src, index, index_stride, slice, counts,
                                           dev_status, ssa::FetchJob{}, index_stride, ssa::kMaxSpans, ssa::Spare<24>{});

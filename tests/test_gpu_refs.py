@@ -285,3 +285,22 @@ def test_one_launch_where_the_sort_or_the_table_copy_changes(n_spans, n_lines):
     for stride in (40, 3 * n_lines + 3):
         compare_index([one_each, empty, in_ranges], stride)
         compare_index([in_ranges] * 80 + [one_each], stride)
+
+
+@pytest.mark.parametrize("seed", range(3))
+def test_tables_in_page_locked_memory(seed):
+    """Tables that the device reads across the bus: not read ahead, the same lists."""
+    reqs, stride = fuzz_requests(seed), 600
+    want, want_counts, want_status = run_refs_index(reqs, stride)
+    here = []
+    for name, width in (("lines", 2), ("anchors", 1), ("refs", 2)):
+        lists = [[(a,) for a in r[name]] if width == 1 else r[name] for r in reqs]
+        here += [t.cpu().pin_memory() for t in flat(lists, width)]
+    i32 = lambda k: torch.tensor([r[k] for r in reqs], dtype=torch.int32).pin_memory()
+    index = torch.full((len(reqs), stride), -7, dtype=torch.int32, device=DEV)
+    counts, status = torch.full((len(reqs),), -7, dtype=torch.int32, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    rest = i32("prefix"), i32("start"), i32("ctx")
+    ssa.refs_to_index(here[0], here[1], here[2], here[3].view(-1), here[4], here[5], *rest, index, counts, status)
+    torch.cuda.synchronize()
+    assert np.array_equal(index.cpu().numpy(), want) and np.array_equal(counts.cpu().numpy(), want_counts)
+    assert int(status.item()) == want_status
