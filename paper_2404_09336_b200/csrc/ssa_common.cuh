@@ -64,22 +64,14 @@ __device__ __forceinline__ int2 load_now(const int2* p) {
 // The 32 bytes around p into L2.
 __device__ __forceinline__ void prefetch_sector(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// Bytes of a kernel's parameters.
-template <typename... KArgs>
-constexpr size_t param_bytes() {
-  size_t at = 0;
-  ((at = (at + alignof(KArgs) - 1) / alignof(KArgs) * alignof(KArgs) + sizeof(KArgs)), ...);
-  return at;
-}
-// A launch takes the host 1.9 us where these are 17 to 32 more than a multiple of 64, and 2.2..2.3 us where they are not (measured
-// over 8..512 bytes, driver 580): kernels with other needs take some
-// more bytes.
+// A launch takes the host 1.9 us where a kernel's parameters are 17 to 32 bytes more than a multiple of 64, and 2.2..2.3 us where
+// they are not (measured over 8..512 bytes, driver 580): kernels with other needs take some more bytes.  Another driver may have
+// other sizes, and no kernel depends on them.
 template <int kBytes> struct Spare { char unused[kBytes]; };
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t dynamic_smem,
                                    cudaStream_t stream, Args... args) {
-  static_assert((param_bytes<KArgs...>() - 17) % 64 < 16, "a size that launches fast: see Spare");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
