@@ -1049,14 +1049,14 @@ static size_t counts_bytes(const ssa_attn_desc* d) { return ((size_t)d->B * size
 // turn 26.9, with two 28.3, 370 with four 28.2, all four warps asking 28.1; 16 x 32 heads x 200 rows 12.1 / 10.0, 37 x 32 x 100
 // 15.0 / 13.1, 20 x 32 x 400 28.3 / 27.0.  A launch of a wave or less over lists of one turn has nothing to gain (16 x 32 x 40
 // 4.55 / 4.65; 37 x 32 x 40 9.1 / 8.2), nor have the shortest lists behind an index launch (61 x 32 x 15 14.2 / 14.4) and launches
-// of larger blocks, two per SM at most (7 requests of 8 heads and up to 900 rows 11.7 / 13.2).  Behind a merge launch, which is soon
-// over, never more than 128 rows: two turns of 8-bit rows, or of rows of 64, are a whole chunk of 256 (without / with two turns /
-// with 128 rows, steps over 8-bit rows, 30 spans, 7 x 8 heads 12.2 / 13.4 / 11.8, 1 x 32 12.1 / 13.4 / 11.9; index lists of 2000 of them,
-// 16 x 8 heads 20.3 / 19.0 / 18.2).  Span lists, which are merged first, are late as it is: one turn where all blocks begin at once
-// (without / two / one, 4 x 8 heads, 30 spans of 45 11.5 / 11.2 / 10.1, 7 x 8, 19 of 45 11.7 / 11.6 / 10.4, but 14 x 8, 30 of 110
-// 33.3 / 31.1 / 31.6; index lists 7 x 8 heads, 2000 rows, 15.4 / 13.1 / 14.0, though behind an index launch two turns lose there, too:
-// references of 8 requests, 8 heads, 14.8 / 15.9 / 14.8).  Lists of one chunk keep two
-// (16 x 32 heads of 64, 400 rows, 11.8 / 10.3 / 10.7).
+// of larger blocks, two per SM at most (7 requests of 8 heads and up to 900 rows 11.7 / 13.2).
+// Behind a merge launch, which is soon over, never more than 128 rows: two turns of 8-bit rows, or of rows of 64, are a whole chunk
+// of 256 (without / two turns / 128 rows; steps over 8-bit rows, 30 spans, 7 x 8 heads 12.2 / 13.4 / 11.8, 1 x 32 12.1 / 13.4 / 11.9;
+// index lists of 2000 of them, 16 x 8 heads 20.3 / 19.0 / 18.2).  Lists of one chunk keep two turns (16 x 32 heads of 64, 400 rows,
+// 11.8 / 10.3 / 10.7).  Span lists, which are merged first, are late as it is: one turn where all blocks begin at once (without / two
+// turns / one; 4 x 8 heads, 30 spans of 45, 11.5 / 11.2 / 10.1, 7 x 8, 19 spans, 11.7 / 11.6 / 10.4; but 14 x 8, 30 spans of 110, 33.3 /
+// 31.1 / 31.6).  Index lists keep two there (7 x 8 heads, 2000 rows, 15.4 / 13.1 / 14.0), which lose behind an index launch: references
+// of 8 requests, 8 heads, 14.8 / 15.9 / 14.8; the call does not know what is in front of it.
 // Row-sharing launches are a wave: three of four blocks, the rows that fill the rings, by four warps, or what these ask for at once
 // where there are fewer blocks than SMs.  us, 32 heads over 8, 32 requests of 820 rows 21.9 / 18.6, of 400 13.6 / 11.2, 8-bit rows
 // 15.6 / 14.1; 4 requests of 820 9.2 / 8.7, of 100 4.9 / 4.9; one warp asking 19.4 for the first of these, for 512 rows 20.3; 2 full contexts of 300 rows, 12

@@ -48,8 +48,9 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
     __syncthreads();
   };
   // The first window is marked while the kernel in front drains, by the list as it stands (one span per thread, inside the
-  // allocation: spans_readable), and again only if the list has changed by then.  us, spans -> blocked lists and attention: 64
-  // requests of 32 heads, 1024 of 2048 rows 168.0 -> 166.0; 34 of 8 heads, up to 350 rows 27.2 -> 26.8.
+  // allocation: spans_readable), and again only if the list has changed by then.  us, spans -> blocked lists and attention: 8
+  // requests of 32 heads, 200 of 2048 rows 14.6 -> 14.1, 12 of 8 heads 12.7 -> 12.3; 64 of 32 heads, 1024 of 2048, 1 % at most, no more
+  // than runs of one side differ.
   bool guess = spans_readable > 0;
   if (!guess) grid_dependency_wait();
   // (the words that decide about barriers may be about to change: for a guess one warp reads them, once, and hands them out)
