@@ -95,7 +95,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   // seeing that they have not takes one trip to memory, the steps two or three and half a microsecond.  Spans to lists and
   // attention, 64 requests 28.8 -> 28.1 us; references and attention, 2 requests of ~25 spans 11.6 -> 9.5, 36 of ~38, 8 heads,
   // 23.9 -> 21.3, 16 of 2 to 50, 32 heads, 41.6 -> 40.5.  (A merge in front is too short to do it all in: 51 of ~20 77.5 -> 77.9.)
-  bool guess = (int)(blockIdx.y * gridDim.x + blockIdx.x) < src.early_blocks;
+  bool guess = !kFetch && (int)(blockIdx.y * gridDim.x + blockIdx.x) < src.early_blocks;
   if (!guess) grid_dependency_wait();   // dependents are released when this grid completes: blocks of a large
                                         // attention grid parked on the SMs during this kernel slowed it down
   int2* const guess_room = reinterpret_cast<int2*>(keys + 2 * kRankSpans);
@@ -112,8 +112,8 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   }
   int P;
   while (true) {
-    auto load = [&](auto* p) { return guess ? load_early(p) : load_now(p); };
-    auto word = [&](int i) { return guess ? s_words[i] : load_now(word_at(i)); };
+    auto load = [&](auto* p) { return !kFetch && guess ? load_early(p) : load_now(p); };
+    auto word = [&](int i) { return !kFetch && guess ? s_words[i] : load_now(word_at(i)); };
     RefTables r = {};
     if constexpr (kFromRefs) r = locate_refs(word);
     const int n = max(kFromRefs ? r.current.y : word(0), 0);
@@ -306,7 +306,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
         run_sum += __shfl_sync(0xffffffffu, sum, 31);
       }
       if (tid == 0) offs[P] = run_sum;
-    } else if (guess) {
+    } else if (!kFetch && guess) {
       // Meanwhile the other warps see whether the guess still holds, so that its trip is not one more where there was no time in
       // front of the wait.  us, references and attention behind an elementwise kernel, compared after the lists have been made /
       // meanwhile / without guesses: 1 request of 32 heads 16.6 / 15.3 / 14.8, 9 29.2 / 28.6 / 28.0; between such calls 6 of 8 heads
@@ -338,7 +338,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
       }
     }
     if (flags) atomicOr(&s_flags, flags);
-    if (!guess) {
+    if (kFetch || !guess) {
       __syncthreads();
       break;
     }
