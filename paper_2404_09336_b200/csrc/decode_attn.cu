@@ -257,7 +257,9 @@ __device__ __forceinline__ void prefetch_early(const DecodeParams& p, int b, int
 // asks for its row (D/8 threads, 16 bytes each) before anything else, so that the trip across the bus overlaps
 // the block's start-up, shares it through shared memory and writes the device copy the caller expects at q.
 // kWarps: see block_warps.
-template <typename T, int D, int kMode, bool kAligned32, bool kPaged = false, bool kHostQ = false, int kWarps = kSmallBlock>
+// kGuess (span lists): the lists are merged before the wait (see plan_early for who does without).
+template <typename T, int D, int kMode, bool kAligned32, bool kPaged = false, bool kHostQ = false, int kWarps = kSmallBlock,
+          bool kGuess = kMode == kSpans>
 __global__ void __launch_bounds__(kWarps * 32, kWarpSlots / kWarps)
 decode_partial_kernel(const DecodeParams p) {
   constexpr int kThreads = kWarps * 32, kStage = staged_entries(kWarps);
@@ -300,7 +302,7 @@ decode_partial_kernel(const DecodeParams p) {
   while (warp_merge && warp_runs < p.span_cap) warp_runs <<= 1;
   EarlySpans guess;
   guess.there = false;
-  if constexpr (kMode == kSpans) {
+  if constexpr (kGuess) {
     const unsigned block = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     if (warp_merge && p.spans_readable > 0 && block < (unsigned)p.guess_blocks) {
       guess = merge_spans_early(s_wruns[warp], p.span_offsets, p.spans, p.spans_readable, p.ctx_lens, p.max_ctx, b, p.span_cap, warp_runs);
@@ -359,6 +361,7 @@ decode_partial_kernel(const DecodeParams p) {
       span_first = b * p.span_cap;
       span_n = p.span_cap;
     }
+    if (!kGuess && warp_merge && lane < min(span_n, p.span_cap)) my_span = load_now(p.spans + span_first + lane);
   }
   // blocked lists: every warp takes all words of the block's entries, one per lane (those beyond the list are ignored below)
   int mask_block = -1;
@@ -375,7 +378,8 @@ decode_partial_kernel(const DecodeParams p) {
   int n, c;
   request_sizes(p, b, n, c, flags);
   if constexpr (kMode == kSpans) {
-    if (warp_merge && !guess.there && lane < min(span_n, p.span_cap)) my_span = load_now(p.spans + span_first + lane);
+    if (kGuess && warp_merge && !guess.there && lane < min(span_n, p.span_cap))
+      my_span = load_now(p.spans + span_first + lane);
     // the request's spans -> disjoint ascending runs in shared memory (every block of the request repeats this)
     int total;
     if (warp_merge && still_the_spans(guess, span_first, span_n, n, my_span)) {
@@ -999,6 +1003,8 @@ static int32_t launch(const DecodeParams& p, int B, int mode, bool aligned32, cu
                : mode == kBlockMask ? decode_partial_kernel<T, D, kBlockMask, kA, false, false, kW>
                : mode == kSpans     ? decode_partial_kernel<T, D, kSpans, kA, false, false, kW>
                                     : decode_partial_kernel<T, D, kDense, kA, false, false, kW>;
+      if constexpr (D == 128 && !kFp8 && kW > kSmallBlock)
+        if (mode == kSpans && p.guess_blocks == 0) kernel = decode_partial_kernel<T, D, kSpans, kA, false, false, kW, false>;
     };
     auto by_warps = [&](auto aligned_tag) {
       if (p.warps == kWarpSlots) pick(aligned_tag, std::integral_constant<int, kWarpSlots>{});
@@ -1065,6 +1071,10 @@ static size_t counts_bytes(const ssa_attn_desc* d) { return ((size_t)d->B * size
 // Span lists of up to 32 are merged before the wait by every block that fits the chip, and by the others as before: checking
 // that the list is still the same takes one trip, reading and merging it two and 0.4 us.  us, one-kernel steps, merged after / before
 // the wait: 16 requests, 32 heads, three spans of 40: 10.9 / 8.9, 48 x 8 heads, 14 of 20: 13.7 / 12.3, 4 x 8, six of 20 5.1 / 4.6.
+// In blocks of 8 and 16 warps over 16-bit rows of 128 the turns come out slower where the kernel has the code to do so, which lists
+// of more than 384 rows lose by unless merging more than 16 spans takes longer: 8 requests of 32 heads, two of them full contexts of
+// up to 1024, 16.0 / 17.5, 32 units of up to 514 rows, 3 spans, 7.0 / 7.4; but 64 of 264 rows, 10 spans, 6.2 / 5.6, of 664, 30 spans, 8.4 /
+// 8.0.  These have a kernel without it.
 // What then is left for row-sharing blocks to prefetch in pays for lists of one chunk that take them longest: 32 heads over 8, 32
 // requests of six spans of 100 15.9 / 13.3, 8-bit rows 12.4 / 11.4; but with a merge launch in front, which is short, 4 requests of
 // 14 spans 10.0 / 11.0, and 16 of three, 8-bit rows, 7.3 / 7.6.
@@ -1081,9 +1091,11 @@ static void plan_early(const ssa_attn_desc* d, const Plan& pl, int max_selected,
   else if (pl.warps == kSmallBlock && (max_selected > turn || (2 * max_selected > turn &&
                                                                (long long)d->B * d->H * pl.n_chunks > SSA_MIN_BLOCKS * sms)))
     p->early_blocks = sms * SSA_MIN_BLOCKS * 5 / 8;
-  p->guess_blocks = pl.share ? 2 * sms : kWarpSlots / pl.warps * sms;
+  const bool long_turns = !pl.share && pl.warps > kSmallBlock && d->D == 128 && d->kv_dtype != SSA_FP8_E4M3;
+  p->guess_blocks = long_turns && p->span_cap <= 16 && std::min(pl.chunk, max_selected) > 384 ? 0
+                    : pl.share ? 2 * sms : kWarpSlots / pl.warps * sms;
   Allocation known = {};
-  p->spans_readable = mode == kSpans ? readable_entries<int2>(p->spans, &known) : 0;
+  p->spans_readable = mode == kSpans && p->guess_blocks > 0 ? readable_entries<int2>(p->spans, &known) : 0;
 }
 
 // mode kDense: index/counts unused.  kIndex: the index list.  kBlockMask: `counts`

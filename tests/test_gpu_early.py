@@ -353,14 +353,17 @@ def test_references_whose_tables_the_launch_in_front_writes(written, before):
 
 
 # blocks of one head, of eight and sixteen warps, row-sharing (ordinary, two chunks, 8-bit rows, above sixteen heads)
-@pytest.mark.parametrize("B,H,Hkv,D,dtype", [
-    (40, 8, 8, 128, "bf16"), (20, 8, 8, 128, "f16"), (3, 8, 8, 64, "bf16"), (40, 32, 8, 128, "bf16"), (3, 32, 8, 128, "bf16"),
-    (40, 8, 2, 128, "fp8"), (20, 20, 1, 128, "bf16")])
+# and large blocks on both sides of the line for merging early: rows and spans a request may have
+@pytest.mark.parametrize("B,H,Hkv,D,dtype,most,cap", [
+    (40, 8, 8, 128, "bf16", 900, 30), (20, 8, 8, 128, "f16", 900, 30), (3, 8, 8, 64, "bf16", 900, 30),
+    (40, 32, 8, 128, "bf16", 900, 30), (3, 32, 8, 128, "bf16", 900, 30), (40, 8, 2, 128, "fp8", 900, 30),
+    (20, 20, 1, 128, "bf16", 900, 30), (20, 8, 8, 128, "bf16", 384, 16), (20, 8, 8, 128, "bf16", 385, 16),
+    (10, 8, 8, 128, "f16", 900, 16), (10, 8, 8, 128, "f16", 900, 17)])
 @pytest.mark.parametrize("before", [-1, 0])
-def test_attention_over_spans_whose_places_the_launch_in_front_writes(B, H, Hkv, D, dtype, before):
+def test_attention_over_spans_whose_places_the_launch_in_front_writes(B, H, Hkv, D, dtype, most, cap, before):
     """Offsets, contexts and spans of ssa_decode_attn_spans rewritten in place between calls."""
     gen, rng = torch.Generator(device=DEV).manual_seed(B * H + D), np.random.default_rng(B)
-    T, turns, cap, most = 900, 8, 30, 900
+    T, turns = 900, 8
     tq = torch.float16 if dtype == "f16" else torch.bfloat16
     q = torch.randn(B, H, D, device=DEV, generator=gen).to(tq)
     k, v = (torch.randn(B, Hkv, T, D, device=DEV, generator=gen).to(tq) for _ in range(2))
@@ -370,7 +373,7 @@ def test_attention_over_spans_whose_places_the_launch_in_front_writes(B, H, Hkv,
     ends = 3 * B + 1 + (3 * B + 1) % 2                   # (spans lie on 8 bytes)
     writer, turn = Writer(ends + 2 * n_spans, turns, before), []
     for t in range(turns):
-        lengths = np.minimum(rng.choice([0, 1, 3, 14, cap], B), 18 if t % 2 else cap)
+        lengths = np.minimum(rng.choice([0, 1, 3, 14, cap], B), min(18, cap) if t % 2 else cap)
         while lengths.sum() > n_spans - 20:
             lengths[rng.integers(B)] = 1
         offsets, spans = np.concatenate([[0], np.cumsum(lengths)]) + rng.integers(0, 20), random_spans(rng, n_spans, T - 40)
@@ -392,7 +395,7 @@ def test_attention_over_spans_whose_places_the_launch_in_front_writes(B, H, Hkv,
     got_lists, got_counts = listed.cpu().numpy(), counts.cpu().numpy()
     for t, (offsets, spans, ctx) in enumerate(turn):
         for b in range(B):
-            rows = O.spans_to_index(spans[offsets[b]:offsets[b + 1]], int(ctx[b]))
+            rows = O.spans_to_index(spans[offsets[b]:offsets[b + 1]], int(ctx[b]))[:most]
             assert got_counts[t, b] == len(rows) and got_lists[t, b, :len(rows)].tolist() == rows.tolist(), (t, b)
         want = rows_of(q, k.to(tq), v.to(tq), listed[t], counts[t])
         assert float((outs[t].double() - want).abs().max()) < 1e-4, t
