@@ -49,8 +49,8 @@ spans_to_blockmask_kernel(const int32_t* __restrict__ span_offsets, const int32_
   };
   // The first window is marked while the kernel in front drains, by the list as it stands (one span per thread, inside the
   // allocation: spans_readable), and again only if the list has changed by then.  us, spans -> blocked lists and attention: 8
-  // requests of 32 heads, 200 of 2048 rows 14.6 -> 14.1, 12 of 8 heads 12.7 -> 12.3; 64 of 32 heads, 1024 of 2048, 1 % at most, no more
-  // than runs of one side differ.
+  // requests of 32 heads, 200 of 2048 rows 14.6 -> 14.1, 12 of 8 heads 12.7 -> 12.3, 3 of 32 12.5 -> 12.0; 64 of 32 heads, 1024 of 2048,
+  // 1 % at most, no more than runs of one side differ.
   bool guess = spans_readable > 0;
   if (!guess) grid_dependency_wait();
   // (the words that decide about barriers may be about to change: for a guess one warp reads them, once, and hands them out)
@@ -143,7 +143,7 @@ extern "C" int32_t ssa_spans_to_blockmask(const int32_t* span_offsets, const int
   if (block_size != 32 && block_size != 64 && block_size != 128 && block_size != 256) return SSA_ERR_UNSUPPORTED;
   if (reinterpret_cast<uintptr_t>(spans) % 8 != 0) return SSA_ERR_ALIGN;
   ssa::Allocation known = {};
-  const int32_t readable = B < 8 ? 0 : ssa::readable_entries<int2>(spans, &known);   // (fewer: the host bounds such calls)
+  const int32_t readable = ssa::readable_entries<int2>(spans, &known);
   const cudaError_t err = ssa::launch_pdl(ssa::spans_to_blockmask_kernel, dim3((unsigned)B), dim3(ssa::kBmThreads),
                                           (cudaStream_t)stream, span_offsets, spans, ctx_lens, block_size,
                                           block_idx, block_mask, block_stride, block_counts, dev_status,
