@@ -94,7 +94,7 @@ spans_to_index_kernel(const SpanSource src, int32_t* __restrict__ index,
   // Steps 1-3 run while the kernel in front drains, on the lists as they stand, and again only if they have changed by then:
   // seeing that they have not takes one trip to memory, the steps two or three and half a microsecond.  Spans to lists and
   // attention, 64 requests 28.8 -> 28.1 us; references and attention, 2 requests of ~25 spans 11.6 -> 9.5, 36 of ~38, 8 heads,
-  // 23.9 -> 21.3, 16 of 2 to 50, 32 heads, 41.6 -> 40.5.  (A merge in front is too short to do it all in: 51 of ~20 77.5 -> 77.9.)
+  // 23.9 -> 21.3, 16 of 2 to 50, 32 heads, 41.6 -> 40.5; 51 of ~20, behind a merge, 89.6 -> 88.1.
   bool guess = !kFetch && (int)(blockIdx.y * gridDim.x + blockIdx.x) < src.early_blocks;
   if (!guess) grid_dependency_wait();   // dependents are released when this grid completes: blocks of a large
                                         // attention grid parked on the SMs during this kernel slowed it down
